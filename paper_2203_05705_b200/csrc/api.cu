@@ -114,6 +114,14 @@ ard_status tc_eligible(ard_ctx* ctx, const ard_pattern* pat, ard_dtype dtype, in
   return ARD_OK;
 }
 
+// Calls the TMA kernels cannot take run on the tensor cores all the same when their operands can be staged by the
+// CTA's threads (gemm_ldg_sm100.cu); layers of a handful of neurons have CUDA-core kernels of their own.
+bool staged_by_threads(const ard_ctx* ctx, const ard_pattern* pat, GemmOp op, ard_dtype dtype, const GemmArgs& g) {
+  if (ctx->path != ARD_PATH_AUTO || dtype != ARD_BF16) return false;
+  if (pat->kind == ARD_ROW && op != OP_BWD_DATA && g.N <= ARD_SKINNY_N) return false;
+  return ldg_takes(ctx, pat->kind, g, pat->ts);
+}
+
 }  // namespace
 
 ard_status ard_encode_tcmap(ard_ctx* ctx, const void* base, int rows, int cols, int ld, int units, int variant,
@@ -191,7 +199,7 @@ ard_status ard_create(ard_ctx** out, int device, size_t workspace_bytes) {
   ctx->sk_min_gain = 24;
   ctx->d_sk_ws = nullptr;
   ctx->d_sk_cnt = nullptr;
-  ctx->last_gather = {nullptr, 0, 0, 0, nullptr, 0ull, nullptr};
+  ctx->last_gather = {nullptr, 0, 0, 0, nullptr, 0ull, nullptr, 0};
   ctx->workspace_bytes = workspace_bytes;
   ctx->d_workspace = nullptr;
   ctx->d_status = nullptr;
@@ -532,6 +540,7 @@ static ard_status fwd_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_patte
   if (el == ARD_OK && out_f32 && pat->kind == ARD_ROW && mode == ARD_OUT_SCATTER_ZEROFILL) el = ARD_ERR_UNSUPPORTED;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
+    if (staged_by_threads(ctx, pat, OP_FWD, dtype, g)) return launch_gemm_ldg(ctx, pat->kind, OP_FWD, g, pat->ts, s);
     return launch_gemm_cc(ctx, pat->kind, OP_FWD, dtype, g, pat->ts, s);
   }
   TcArgs t = {};
@@ -578,9 +587,10 @@ ard_status ard_layer_fwd(ard_ctx* ctx, const ard_pattern* pat, const ard_pattern
 
 // Produces the operand the tensor-core backward GEMMs read for dY: the caller's compact matrix, or
 // a compacted copy of the full-width one in the context workspace (row patterns only).
+// with_dense: a dense pattern is copied too (the caller reads the copy in every case).
 static ard_status compact_dy(ard_ctx* ctx, const ard_pattern* pat, int B, int N, const void* dY, int lddy,
                              int dy_is_compact, const void** out_ptr, int* out_ld, const void** dense_ptr,
-                             int* dense_ld, cudaStream_t s) {
+                             int* dense_ld, cudaStream_t s, int with_dense = 0) {
   *dense_ptr = nullptr;
   *dense_ld = 0;
   if (dy_is_compact) {
@@ -597,13 +607,31 @@ static ard_status compact_dy(ard_ctx* ctx, const ard_pattern* pat, int B, int N,
   *out_ld = ldc;
   auto& lg = ctx->last_gather;
   if (ctx->reuse_compact && lg.src == dY && lg.ld == lddy && lg.B == B && lg.N == N && lg.pat == pat &&
-      lg.gen == pat->generation && lg.stream == s)
+      lg.gen == pat->generation && lg.stream == s && lg.with_dense >= with_dense)
     return ARD_OK;  // the previous backward call on this stream already compacted this dY for this pattern
-  lg = {dY, lddy, B, N, pat, pat->generation, s};
-  ard_status st = launch_gather_cols(ctx, pat->d_hdr, pat->d_idx, dY, lddy, ctx->d_workspace, ldc, B, 2, N, 1, s);
+  lg = {dY, lddy, B, N, pat, pat->generation, s, with_dense};
+  ard_status st = launch_gather_cols(ctx, pat->d_hdr, pat->d_idx, dY, lddy, ctx->d_workspace, ldc, B, 2, N, !with_dense, s);
   *out_ptr = ctx->d_workspace;
   *out_ld = ldc;
   return st;
+}
+
+// The backward products on operands staged by the CTA's threads: dY compact (row patterns), then the product.
+// Returns ARD_ERR_UNSUPPORTED with nothing enqueued when this call has to go to the CUDA cores.
+static ard_status bwd_staged_by_threads(ard_ctx* ctx, const ard_pattern* pat, GemmOp op, ard_dtype dtype, GemmArgs g,
+                                        cudaStream_t s) {
+  if (!staged_by_threads(ctx, pat, op, dtype, g)) return ARD_ERR_UNSUPPORTED;
+  if (pat->kind == ARD_ROW && !g.flag0) {
+    if ((size_t)g.B * ((g.N + 7) / 8 * 8) * 2 > ctx->workspace_bytes) return ARD_ERR_UNSUPPORTED;
+    const void *dyc, *dense;
+    int ldc, dense_ld;
+    ard_status st = compact_dy(ctx, pat, g.B, g.N, g.A0, g.lda0, 0, &dyc, &ldc, &dense, &dense_ld, s, 1);
+    if (st != ARD_OK) return st;
+    g.A0 = dyc;
+    g.lda0 = ldc;
+    g.flag0 = 1;
+  }
+  return launch_gemm_ldg(ctx, pat->kind, op, g, pat->ts, s);
 }
 
 static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_pattern* in_pat, ard_dtype dtype, int B,
@@ -648,7 +676,8 @@ static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_
     el = ARD_ERR_NOMEM;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
-    return launch_gemm_cc(ctx, pat->kind, OP_BWD_DATA, dtype, g, pat->ts, s);
+    st = bwd_staged_by_threads(ctx, pat, OP_BWD_DATA, dtype, g, s);
+    return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_DATA, dtype, g, pat->ts, s);
   }
   TcArgs t = {};
   t.ts = pat->ts;
@@ -734,7 +763,12 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     el = ARD_ERR_NOMEM;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
-    return launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
+    if (staged_by_threads(ctx, pat, OP_BWD_WEIGHT, dtype, g) && pat->kind == ARD_TILE && zero_fill_dropped) {
+      st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
+      if (st != ARD_OK) return st;
+    }
+    st = bwd_staged_by_threads(ctx, pat, OP_BWD_WEIGHT, dtype, g, s);
+    return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
   }
   TcArgs t = {};
   t.ts = pat->ts;

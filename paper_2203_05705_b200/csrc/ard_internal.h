@@ -94,6 +94,9 @@ static inline size_t tm_slots_bytes() {
   return ((size_t)ARD_TM_SM_MAX * ARD_TM_SLOTS + (size_t)ARD_TM_LSTM_BLOCKS * ARD_TM_LSTM_SLOTS) * sizeof(CUtensorMap);
 }
 
+// Row-pattern layers of at most this many neurons have CUDA-core kernels of their own (an output layer).
+constexpr int ARD_SKINNY_N = 16;
+
 constexpr int ARD_MLP_EVENTS = 104;  // fork, forward done, two joins, and three per layer (up to 32 layers)
 
 struct ard_ctx {
@@ -116,7 +119,7 @@ struct ard_ctx {
   int sk_min_gain;    // fewest blocks the sharing must save per worker to be used
   void* d_sk_ws;      // partial accumulators of the shared tail, sk_ws_bytes(sm_count)
   int* d_sk_cnt;      // arrival counters, zero between launches
-  struct { const void* src; int ld, B, N; const ard_pattern* pat; unsigned long long gen; cudaStream_t stream; } last_gather;
+  struct { const void* src; int ld, B, N; const ard_pattern* pat; unsigned long long gen; cudaStream_t stream; int with_dense; } last_gather;
   size_t workspace_bytes;
   void* d_workspace;
   int* d_status;
@@ -217,6 +220,11 @@ enum GemmOp { OP_FWD = 0, OP_BWD_DATA = 1, OP_BWD_WEIGHT = 2 };
 // CUDA-core family (fp32 or bf16 operands, fp32 accumulate).
 ard_status launch_gemm_cc(ard_ctx* ctx, ard_kind kind, GemmOp op, ard_dtype dtype, const GemmArgs& a, int ts,
                           cudaStream_t s);
+
+// tcgen05 products whose operands the CTA's threads stage themselves: bf16 operands of any alignment under a row pattern
+// (dY compact), pattern tiles of 8 to 64 columns.  ldg_takes: can it take these operands?
+bool ldg_takes(const ard_ctx* ctx, ard_kind kind, const GemmArgs& g, int ts);
+ard_status launch_gemm_ldg(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
 
 // tcgen05 family (bf16 operands, fp32 accumulate in TMEM).
 struct TcArgs {
@@ -327,6 +335,30 @@ inline cudaError_t ard_launch(const ard_ctx* ctx, void (*kern)(P...), dim3 grid,
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+  }
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
+// The same for a grid of clusters of `cluster` CTAs.
+template <typename... P, typename... A>
+inline cudaError_t ard_launch_cluster(const ard_ctx* ctx, void (*kern)(P...), int cluster, dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (ard_pdl_allowed(ctx, s)) {
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.numAttrs = 2;
   }
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }

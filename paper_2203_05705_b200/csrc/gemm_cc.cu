@@ -175,7 +175,7 @@ __global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(GemmArgs g, int ts)
 // Forward: one CTA per batch row; every thread walks a strided share of the fan-in with one accumulator
 // per kept neuron, then the CTA adds the shares (fixed order).  Backward-weight: 32 fan-in columns per CTA,
 // the batch rows dealt to its 8 warps, one accumulator per kept neuron, warp sums added in warp order.
-constexpr int SKINNY_N = 16;
+constexpr int SKINNY_N = ARD_SKINNY_N;
 
 template <typename T>
 __global__ void __launch_bounds__(256) skinny_fwd_kernel(GemmArgs g) {

@@ -1,0 +1,249 @@
+// What the product kernels whose threads stage the operands themselves have in common (gemm_ldg_sm100.cu on the tensor
+// cores, gemm_cc.cu on the CUDA cores): the tiling worked out from the pattern header on the device, the sum of the
+// partial tiles of a cut contraction, and the rows' way out.  Everything is static to the including translation unit.
+//
+// A tile pattern (Sec. 3.2) keeps tile (r, c) iff r * Tc + c = b - 1 (mod dp), so tile-columns with equal c mod dp share
+// one kept list, and tile-rows with equal r mod dp / gcd(Tc mod dp, dp) another: the members of such a class side by
+// side are one dense product over their common list, whatever the size of a pattern tile.
+//
+// Work is dealt in clusters of SP_CLUSTER CTAs.  A product with fewer output tiles than the device has room for is cut
+// along its contraction over S = 2, 4 or 8 CTAs of a cluster; S follows from the sampled pattern.
+#pragma once
+
+#include "ard_internal.h"
+#include "sm100_ptx.h"
+
+namespace {
+
+constexpr int SP_CLUSTER = 8;
+
+struct ProductPlan {
+  int dp, bb, n_keep;
+  int M, N, K;         // extents of the product (tile patterns: K is the batch for the weight gradient, else unused)
+  int Mt;              // tiles along M
+  int tiles;           // output tiles (weight gradient of a tile pattern: an upper bound, some may turn out empty)
+  int S;               // CTAs per output tile
+  // tile patterns: class c (tiles with equal number mod cstep) has q + (c < rmd) members
+  int ts, lts;         // pattern tile, its log2 (-1: not a power of two)
+  int cstep, q, rmd, nclass;
+  int nH, nL;          // output tiles of a class with q + 1 / q members
+  int a, c0, mmax, nmax;       // weight gradient: non-empty classes c0, c0 + a, ...; tiles per class mmax x nmax
+
+  __device__ __forceinline__ int tile_of(int i) const { return lts >= 0 ? i >> lts : i / ts; }
+};
+
+struct ProductTile {
+  int m0, n0;           // tile patterns: along the gathered dimension a position among the class's members
+  int nkb;              // contraction blocks (-1: no such tile)
+  const int32_t* list;  // tile patterns: kept tiles along the contraction (weight gradient: along N)
+  int len;
+  int c, cnt;           // class and its members
+  int kext;             // contraction length
+
+  // coordinate of position i among the class's members / in the kept list
+  __device__ __forceinline__ int class_pos(const ProductPlan& s, int i) const {
+    const int m = s.tile_of(i);
+    return (c + m * s.cstep) * s.ts + i - m * s.ts;
+  }
+  __device__ __forceinline__ int list_pos(const ProductPlan& s, int i) const {
+    const int m = s.tile_of(i);
+    return list[m] * s.ts + i - m * s.ts;
+  }
+};
+
+__device__ __forceinline__ int sp_cdiv(int a, int b) { return (a + b - 1) / b; }
+
+// want: CTAs the device has room for at once.
+template <int KIND, int OP, int BM, int BN, int BK>
+__device__ __forceinline__ ProductPlan make_plan(const GemmArgs& g, int ts, int want) {
+  ProductPlan s = {};
+  s.dp = g.hdr[HDR_DP];
+  s.bb = g.hdr[HDR_B] - 1;
+  s.n_keep = g.hdr[HDR_NKEEP];
+  int nkb;
+  if (KIND == 0) {
+    // fan-in extent: all K inputs, or the kept outputs of the layer that produced the input
+    const int kin = g.hdr_in != nullptr ? g.hdr_in[HDR_NKEEP] : g.K;
+    s.M = OP == OP_BWD_WEIGHT ? s.n_keep : g.B;
+    s.N = OP == OP_FWD ? s.n_keep : kin;
+    s.K = OP == OP_FWD ? kin : (OP == OP_BWD_DATA ? s.n_keep : g.B);
+    s.Mt = sp_cdiv(s.M, BM);
+    s.tiles = s.Mt * sp_cdiv(s.N, BN);
+    nkb = sp_cdiv(s.K, BK);
+  } else {
+    const int Tr = g.hdr[HDR_TR], Tc = g.hdr[HDR_TC];
+    s.ts = ts;
+    s.lts = (ts & (ts - 1)) == 0 ? 31 - __clz(ts) : -1;
+    int gg = Tc % s.dp, a = s.dp;
+    while (gg) { const int t = a % gg; a = gg; gg = t; }  // a = gcd(Tc mod dp, dp)
+    const int extent = OP == OP_BWD_DATA ? Tr : Tc;
+    s.cstep = OP == OP_BWD_DATA ? s.dp / a : s.dp;
+    s.nclass = min(s.cstep, extent);
+    s.q = extent / s.cstep;
+    s.rmd = extent % s.cstep;
+    s.nH = sp_cdiv((s.q + 1) * ts, BN);
+    s.nL = sp_cdiv(s.q * ts, BN);
+    s.M = OP == OP_BWD_WEIGHT ? g.N : g.B;
+    s.N = OP == OP_FWD ? g.N : g.K;
+    s.K = g.B;
+    s.Mt = sp_cdiv(s.M, BM);
+    if (OP == OP_BWD_WEIGHT) {
+      s.a = a;
+      s.c0 = s.bb % a;
+      const int ncl = s.c0 < s.nclass ? (s.nclass - 1 - s.c0) / a + 1 : 0;
+      s.mmax = sp_cdiv(sp_cdiv(extent, s.cstep) * ts, BM);
+      s.nmax = sp_cdiv(sp_cdiv(Tr, s.dp / a) * ts, BN);
+      s.tiles = ncl * s.mmax * s.nmax;
+      nkb = sp_cdiv(g.B, BK);
+    } else {
+      s.tiles = s.Mt * (s.rmd * s.nH + (s.nclass - s.rmd) * s.nL);
+      // longest kept list
+      nkb = sp_cdiv(sp_cdiv(OP == OP_FWD ? Tr : Tc, OP == OP_FWD ? s.dp / a : s.dp) * ts, BK);
+    }
+  }
+  // Cut the contraction only while the pieces still find an idle place and hold at least two blocks: a cut costs
+  // two cluster barriers and a pass of the partial tiles through shared memory.
+  s.S = SP_CLUSTER;
+  while (s.S > 1 && (s.tiles * s.S > want || nkb < 2 * s.S)) s.S >>= 1;
+  return s;
+}
+
+template <int KIND, int OP, int BM, int BN, int BK>
+__device__ __forceinline__ ProductTile make_tile(const GemmArgs& g, const ProductPlan& s, int t) {
+  ProductTile ti = {};
+  if (KIND == 0) {
+    ti.m0 = (t % s.Mt) * BM;
+    ti.n0 = (t / s.Mt) * BN;
+    ti.kext = s.K;
+  } else if (OP == OP_BWD_WEIGHT) {
+    const int per = s.mmax * s.nmax, ci = t / per, r = t - ci * per;
+    ti.c = s.c0 + ci * s.a;
+    ti.cnt = s.q + (ti.c < s.rmd ? 1 : 0);
+    ti.m0 = (r % s.mmax) * BM;
+    ti.n0 = (r / s.mmax) * BN;
+    const int off = g.col_ptr[ti.c];
+    ti.len = g.col_ptr[ti.c + 1] - off;
+    ti.list = g.col_idx + off;
+    ti.kext = s.K;
+    if (ti.m0 >= ti.cnt * s.ts || ti.n0 >= ti.len * s.ts) { ti.nkb = -1; return ti; }
+  } else {
+    ti.m0 = (t % s.Mt) * BM;
+    int j = t / s.Mt, v;
+    if (j < s.rmd * s.nH) { ti.c = j / s.nH; v = j - ti.c * s.nH; }
+    else { j -= s.rmd * s.nH; const int i = j / s.nL; ti.c = s.rmd + i; v = j - i * s.nL; }
+    ti.cnt = s.q + (ti.c < s.rmd ? 1 : 0);
+    ti.n0 = v * BN;
+    const int32_t* ptr = OP == OP_FWD ? g.col_ptr : g.row_ptr;
+    const int off = ptr[ti.c];
+    ti.len = ptr[ti.c + 1] - off;
+    ti.list = (OP == OP_FWD ? g.col_idx : g.row_idx) + off;
+    ti.kext = ti.len * s.ts;
+  }
+  ti.nkb = sp_cdiv(ti.kext, BK);
+  return ti;
+}
+
+__device__ __forceinline__ float4 ld_cluster_f4(uint32_t a) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+  return v;
+}
+// Adds the S partial tiles at `off` (the same shared-memory offset in CTAs lead .. lead + S - 1) in contraction order.
+template <int S>
+__device__ __forceinline__ float4 sum_shares(uint32_t off, int lead) {
+  float4 v[S];
+#pragma unroll
+  for (int j = 0; j < S; ++j) v[j] = ld_cluster_f4(mapa_u32(off, (uint32_t)(lead + j)));
+#pragma unroll
+  for (int j = 1; j < S; ++j) { v[0].x += v[j].x; v[0].y += v[j].y; v[0].z += v[j].z; v[0].w += v[j].w; }
+  return v[0];
+}
+
+// The CTA's rows of a finished tile (fp32, PITCH words per row in shared memory at T / address t_addr): rows
+// [part * BM / S, (part + 1) * BM / S), dealt to NW warps.  With S > 1 the group's shares are added into this CTA's
+// own copy first.  T_: operand type (the saved activation's).
+template <int KIND, int OP, int BM, int BN, int PITCH, int NW, typename T_>
+__device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan& s, const ProductTile& ti, float* T, uint32_t t_addr,
+                                           int part, int lead, int warp, int lane) {
+  const int rows_per = BM / s.S, r0 = part * rows_per;
+  if (s.S > 1) {
+    for (int i = lane; i < rows_per / NW * (BN / 4); i += 32) {  // this warp's rows r0 + warp, r0 + warp + NW, ...
+      const int row = r0 + warp + NW * (i / (BN / 4)), w = row * PITCH + 4 * (i % (BN / 4));
+      const uint32_t off = t_addr + (uint32_t)w * 4u;
+      *reinterpret_cast<float4*>(T + w) = s.S == 8 ? sum_shares<8>(off, lead) : (s.S == 4 ? sum_shares<4>(off, lead) : sum_shares<2>(off, lead));
+    }
+    __syncwarp();
+  }
+  auto put = [&](size_t off, float val) {
+    if (g.out_is_f32) {
+      float* o = reinterpret_cast<float*>(g.out) + off;
+      *o = g.accumulate ? *o + val : val;
+    } else {
+      __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(g.out) + off;
+      *o = __float2bfloat16_rn(g.accumulate ? __bfloat162float(*o) + val : val);
+    }
+  };
+  for (int r = r0 + warp; r < r0 + rows_per; r += NW) {
+    const int m = ti.m0 + r;
+    const float* row = T + r * PITCH;
+    if (KIND == 0) {
+      if (m >= s.M) break;
+      auto fwd_value = [&](int j) {  // compact column j of the tile: bias, then the activation, then the rescale (Sec. 3.2)
+        float z = row[j];
+        if (g.bias != nullptr) z += g.bias[s.bb + (ti.n0 + j) * s.dp];
+        if (g.relu) z = fmaxf(z, 0.f);
+        return z * g.alpha;
+      };
+      if (OP == OP_FWD && g.flag0 == ARD_OUT_SCATTER_ZEROFILL) {
+        // output columns [n0 * dp, (n0 + BN) * dp), the last tile up to N: kept ones and the zeros between
+        const int lo = ti.n0 * s.dp, hi = ti.n0 + BN >= s.N ? g.N : (ti.n0 + BN) * s.dp;
+        for (int col = lo + lane; col < hi; col += 32) {
+          const int rel = col - s.bb, j = rel >= 0 ? rel / s.dp : -1;
+          const bool kept = j >= 0 && j * s.dp == rel && j < s.n_keep;
+          put((size_t)m * g.ldo + col, kept ? fwd_value(j - ti.n0) : 0.f);
+        }
+        continue;
+      }
+      const size_t orow = OP == OP_BWD_WEIGHT && g.hdr_in == nullptr ? (size_t)s.bb + (size_t)m * s.dp : (size_t)m;
+#pragma unroll
+      for (int j0 = 0; j0 < BN; j0 += 32) {
+        const int j = j0 + lane, n = ti.n0 + j;
+        if (n >= s.N) continue;
+        float val;
+        if (OP == OP_FWD) {
+          val = fwd_value(j);
+        } else {
+          val = row[j] * g.alpha;
+          // adjoint of the producing layer's ReLU: nothing flows where its output was not positive
+          if (OP == OP_BWD_DATA && g.act != nullptr && !((float)reinterpret_cast<const T_*>(g.act)[(size_t)m * g.ldact + n] > 0.f)) val = 0.f;
+        }
+        put(orow * g.ldo + n, val);
+      }
+      if (OP == OP_BWD_WEIGHT && g.flag1) {
+        // compact row m owns output rows [m * dp, (m + 1) * dp), the last one the tail: zeros but for its own
+        const long long first = (long long)m * s.dp;
+        const long long last = m == s.M - 1 ? g.N : min((long long)g.N, first + s.dp);
+        for (long long z = first; z < last; ++z)
+          if (z != (long long)orow)
+            for (int n = ti.n0 + lane; n < min(ti.n0 + BN, s.N); n += 32) put((size_t)z * g.ldo + n, 0.f);
+      }
+    } else {
+      size_t orow = m;
+      if (OP == OP_BWD_WEIGHT) {
+        if (m >= ti.cnt * s.ts) break;
+        orow = (size_t)ti.class_pos(s, m);
+      } else if (m >= s.M) {
+        break;
+      }
+      const int next = (OP == OP_BWD_WEIGHT ? ti.len : ti.cnt) * s.ts;
+#pragma unroll
+      for (int j0 = 0; j0 < BN; j0 += 32) {
+        const int j = j0 + lane, n = ti.n0 + j;
+        if (n >= next) continue;
+        put(orow * g.ldo + (size_t)(OP == OP_BWD_WEIGHT ? ti.list_pos(s, n) : ti.class_pos(s, n)), row[j] * g.alpha);
+      }
+    }
+  }
+}
+
+}  // namespace
