@@ -752,7 +752,13 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
   g.out_is_f32 = dW_dtype == ARD_F32;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
   if (in_pat && zero_fill_dropped) return ARD_ERR_INVALID_ARG;  // the packed gradient has no rows of dropped neurons
+  // The kernels write the zeros of dropped rows themselves, those of dropped pattern tiles are written first.
+  const bool zero_tiles = pat->kind == ARD_TILE && zero_fill_dropped;
   // Empty batch: the gradient of every kept weight is zero; the CUDA-core kernel writes exactly that.
+  if (B == 0 && zero_tiles) {
+    st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
+    if (st != ARD_OK) return st;
+  }
   if (B == 0) return launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
 
   ard_status el = ctx->path == ARD_PATH_CUDA_CORE
@@ -763,7 +769,7 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     el = ARD_ERR_NOMEM;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
-    if (staged_by_threads(ctx, pat, OP_BWD_WEIGHT, dtype, g) && pat->kind == ARD_TILE && zero_fill_dropped) {
+    if (zero_tiles) {
       st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
       if (st != ARD_OK) return st;
     }

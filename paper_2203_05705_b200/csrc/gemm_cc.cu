@@ -1,15 +1,13 @@
 // CUDA-core family of the compacted GEMMs: fp32 (or bf16) operands, fp32 FFMA accumulation.
 //
 // This is the path of the fp32 layers (a single tcgen05 tf32 pass keeps 10 mantissa bits and
-// cannot reach 1e-5) and the fall-back for bf16 shapes whose alignment the TMA path cannot take.
-// One generic 32x32x32 shared-memory tiled kernel; what differs per product is only how the
-// logical operand element (m, k), (n, k) maps to memory and which contraction indices exist:
-// dropped neurons / tiles are skipped through the index lists, never multiplied by zero.
-#include "ard_internal.h"
+// cannot reach 1e-5) and the fall-back for bf16 shapes whose alignment no tensor-core kernel can take.
+// One shared-memory tiled kernel; what differs per product is only how the logical operand element (m, k), (n, k)
+// maps to memory and which contraction indices exist: dropped neurons / tiles are skipped through the pattern,
+// never multiplied by zero.  Tiling, cut contractions and the rows' way out: staged_product.h.
+#include "staged_product.h"
 
 namespace {
-
-constexpr int T_M = 32, T_N = 32, T_K = 32, CC_THREADS = 256;
 
 template <typename T> __device__ __forceinline__ float to_f(T v);
 template <> __device__ __forceinline__ float to_f<float>(float v) { return v; }
@@ -25,149 +23,179 @@ __device__ __forceinline__ void store_out(void* out, size_t off, float v, int ou
   }
 }
 
-// KIND: 0 row, 1 tile.  OP: GemmOp.
-template <typename T, int KIND, int OP>
-__global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(GemmArgs g, int ts) {
-  __shared__ float As[T_K][T_M + 1];
-  __shared__ float Bs[T_K][T_N + 1];
+// Four consecutive elements at p as fp32; the address is a multiple of four elements.
+__device__ __forceinline__ float4 load4(const float* p) {
+  float4 v;
+  asm volatile("ld.global.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
+  uint32_t a, b;
+  asm volatile("ld.global.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "l"(p));
+  return make_float4(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u), __uint_as_float(b << 16), __uint_as_float(b & 0xffff0000u));
+}
 
-  pdl_launch_dependents();
-  pdl_wait_prior_grids();
-  const int dp = g.hdr[HDR_DP], b = g.hdr[HDR_B], n_keep = g.hdr[HDR_NKEEP];
-  const int Tc = g.hdr[HDR_TC];
+constexpr int CC_THREADS = 64;
+constexpr double CC_WIDE_FLOPS = 2e8;  // 64 x 64 tiles from here on, see launch_one
+struct CcParams {
+  GemmArgs g;
+  int ts;
+  int want;      // CTAs the device has room for at once
+  int vec;       // bit 0 / 1: rows of operand A / B start on four-element boundaries
+};
+
+// R: rows and columns of the output tile (64 or 32); a thread of the 8 x 8 grid owns R / 8 by R / 8 of it.  The
+// operands of a KT-deep block are staged k-major as fp32, [k][row], through registers, one block ahead of the
+// products.  KIND: 0 row, 1 tile.  OP: GemmOp.
+// Bound: FFMA issue for the 64 x 64 tile (64 FFMA per four 16-byte shared-memory reads and thread), latency for the
+// 32 x 32 one, which is for products that would otherwise occupy a few SMs.
+template <typename T, int KIND, int OP, int R>
+__global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(const __grid_constant__ CcParams p) {
+  constexpr int KT = R == 64 ? 16 : 32, Q = R / 8, PITCH = R + 4;
+  constexpr bool A_MN = OP == OP_BWD_WEIGHT, B_MN = OP != OP_FWD;
+  constexpr int NCH = R * KT / 4 / CC_THREADS;  // four-element pieces per thread, operand and block
+  __shared__ __align__(16) float sm[4 * KT * PITCH];  // [buffer][operand][k][row]; the finished tile overlays it
+  static_assert(R <= 4 * KT, "the tile overlays the stages");
+  const GemmArgs& g = p.g;
   // No __restrict__ / read-only loads on anything an earlier kernel of the stream wrote: this kernel may
   // become resident before that kernel has finished (see pdl_wait_prior_grids), and the non-coherent
   // load path may then serve a line another resident kernel brought in before the data was rewritten.
-  const T* P0 = reinterpret_cast<const T*>(g.A0);
-  const T* P1 = reinterpret_cast<const T*>(g.A1);
+  pdl_launch_dependents();
+  pdl_wait_prior_grids();
 
-  int M, N, nk;
-  const int m0 = blockIdx.y * T_M, n0 = blockIdx.x * T_N;
-  const int32_t* klist = nullptr;  // tile patterns: contraction runs over ts-wide blocks klist[0..]
-  if (KIND == 0) {
-    // fan-in extent: all K inputs, or the kept outputs of the layer that produced the input
-    const int kin = g.hdr_in != nullptr ? g.hdr_in[HDR_NKEEP] : g.K;
-    if (OP == OP_FWD) { M = g.B; N = n_keep; nk = kin; }
-    else if (OP == OP_BWD_DATA) { M = g.B; N = kin; nk = n_keep; }
-    else { M = n_keep; N = kin; nk = g.B; }
-  } else {
-    if (OP == OP_FWD) {
-      M = g.B; N = g.N;
-      if (n0 >= N) return;
-      const int c = n0 / ts;
-      klist = g.col_idx + g.col_ptr[c];
-      nk = (g.col_ptr[c + 1] - g.col_ptr[c]) * ts;
-    } else if (OP == OP_BWD_DATA) {
-      M = g.B; N = g.K;
-      if (n0 >= N) return;
-      const int r = n0 / ts;
-      klist = g.row_idx + g.row_ptr[r];
-      nk = (g.row_ptr[r + 1] - g.row_ptr[r]) * ts;
-    } else {
-      M = g.N; N = g.K; nk = g.B;
-    }
-  }
-  if (m0 >= M || n0 >= N) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = tid & 7, ty = tid >> 3;
+  const ProductPlan s = make_plan<KIND, OP, R, R, KT>(g, p.ts, p.want);
+  const int rank = (int)cluster_ctarank();
+  const int part = rank & (s.S - 1), lead = rank - part;
+  const int group = rank / s.S, groups = SP_CLUSTER / s.S;
+  const int n_cl = (int)gridDim.x / SP_CLUSTER, units = (s.tiles + groups - 1) / groups;
+  const T* PA = reinterpret_cast<const T*>(g.A0);
+  const T* PB = reinterpret_cast<const T*>(g.A1);
+  // Kept neurons are bb + i * dp: columns of a full-width dY, rows of the weight (unless packed for a feeding pattern).
+  const bool strided_a = KIND == 0 && OP != OP_FWD && !g.flag0;
+  const size_t step_a = strided_a ? (size_t)s.dp : 1, off_a = strided_a ? (size_t)s.bb : 0;
+  const bool strided_b = KIND == 0 && OP != OP_BWD_WEIGHT && g.hdr_in == nullptr;
+  const size_t ldb = strided_b ? (size_t)g.lda1 * s.dp : (size_t)g.lda1;
+  if (strided_b) PB += (size_t)s.bb * g.lda1;
+  const bool whole = KIND == 0 || (p.ts & 3) == 0;  // four consecutive positions never leave a pattern tile
+  const bool vec_a = (p.vec & 1) && step_a == 1 && whole, vec_b = (p.vec & 2) && whole;
 
-  if (KIND == 1 && OP == OP_BWD_WEIGHT) {
-    const int lin = (n0 / ts) * Tc + (m0 / ts);  // tile (r, c) = (k-block, neuron-block), 0-based t-1
-    const bool kept = lin >= b - 1 && (lin - (b - 1)) % dp == 0;
-    if (!kept) {
-      if (g.flag1) {
-        for (int e = threadIdx.x; e < T_M * T_N; e += CC_THREADS) {
-          const int m = m0 + e / T_N, n = n0 + e % T_N;
-          if (m < M && n < N) store_out(g.out, (size_t)m * g.ldo + n, 0.f, g.out_is_f32);
-        }
-      }
-      return;
-    }
-  }
+  for (int u = (int)blockIdx.x / SP_CLUSTER; u < units; u += n_cl) {
+    const int t = u * groups + group;
+    ProductTile ti = {};
+    ti.nkb = -1;
+    if (t < s.tiles) ti = make_tile<KIND, OP, R, R, KT>(g, s, t);
+    const bool live = ti.nkb >= 0;
+    const int kb0 = live ? (int)((long long)ti.nkb * part / s.S) : 0;
+    const int kb1 = live ? (int)((long long)ti.nkb * (part + 1) / s.S) : 0;
 
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  float acc[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+    // Element offsets of operand elements; r = row inside the tile, k = contraction index.
+    auto a_off = [&](int r, int k) -> size_t {
+      const int m = ti.m0 + r;
+      if (KIND == 0) return A_MN ? (size_t)k * g.lda0 + off_a + (size_t)m * step_a : (size_t)m * g.lda0 + off_a + (size_t)k * step_a;
+      return A_MN ? (size_t)k * g.lda0 + ti.class_pos(s, m) : (size_t)m * g.lda0 + ti.list_pos(s, k);
+    };
+    auto b_off = [&](int r, int k) -> size_t {
+      const int n = ti.n0 + r;
+      if (KIND == 0) return B_MN ? (size_t)k * ldb + n : (size_t)n * ldb + k;
+      if (OP == OP_FWD) return (size_t)ti.class_pos(s, n) * ldb + ti.list_pos(s, k);
+      if (OP == OP_BWD_DATA) return (size_t)ti.list_pos(s, k) * ldb + ti.class_pos(s, n);
+      return (size_t)k * ldb + ti.list_pos(s, n);
+    };
+    const int a_lim = (KIND == 0 || OP != OP_BWD_WEIGHT ? s.M : ti.cnt * s.ts) - ti.m0;
+    const int b_lim = (KIND == 0 ? s.N : (OP == OP_BWD_WEIGHT ? ti.len : ti.cnt) * s.ts) - ti.n0;
 
-  for (int k0 = 0; k0 < nk; k0 += T_K) {
-    for (int e = threadIdx.x; e < T_K * T_M; e += CC_THREADS) {
-      // operand A: element (m, kk)
-      int kk, m;
-      if ((KIND == 0 && OP == OP_BWD_WEIGHT) || (KIND == 1 && OP == OP_BWD_WEIGHT)) { m = e % T_M; kk = e / T_M; }
-      else { kk = e % T_K; m = e / T_K; }
-      float v = 0.f;
-      const int gm = m0 + m, gk = k0 + kk;
-      if (gm < M && gk < nk) {
-        size_t off;
-        if (KIND == 0) {
-          if (OP == OP_FWD) off = (size_t)gm * g.lda0 + gk;
-          else if (OP == OP_BWD_DATA) off = (size_t)gm * g.lda0 + (g.flag0 ? gk : g.idx[gk]);
-          else off = (size_t)gk * g.lda0 + (g.flag0 ? gm : g.idx[gm]);
-        } else {
-          if (OP == OP_BWD_WEIGHT) off = (size_t)gk * g.lda0 + gm;
-          else off = (size_t)gm * g.lda0 + (size_t)klist[gk / ts] * ts + gk % ts;
-        }
-        v = to_f<T>(P0[off]);
-      }
-      As[kk][m] = v;
-    }
-    for (int e = threadIdx.x; e < T_K * T_N; e += CC_THREADS) {
-      // operand B: element (n, kk)
-      int kk, n;
-      if (OP == OP_FWD) { kk = e % T_K; n = e / T_K; }
-      else { n = e % T_N; kk = e / T_N; }
-      float v = 0.f;
-      const int gn = n0 + n, gk = k0 + kk;
-      if (gn < N && gk < nk) {
-        size_t off;
-        if (KIND == 0) {
-          // with a feeding pattern the weight is packed in both dimensions (row j = j-th kept neuron)
-          if (OP == OP_FWD) off = (size_t)(g.hdr_in != nullptr ? gn : g.idx[gn]) * g.lda1 + gk;
-          else if (OP == OP_BWD_DATA) off = (size_t)(g.hdr_in != nullptr ? gk : g.idx[gk]) * g.lda1 + gn;
-          else off = (size_t)gk * g.lda1 + gn;
-        } else {
-          const size_t kidx = (OP == OP_BWD_WEIGHT) ? (size_t)gk : (size_t)klist[gk / ts] * ts + gk % ts;
-          if (OP == OP_FWD) off = (size_t)gn * g.lda1 + kidx;
-          else if (OP == OP_BWD_DATA) off = kidx * g.lda1 + gn;
-          else off = kidx * g.lda1 + gn;
-        }
-        v = to_f<T>(P1[off]);
-      }
-      Bs[kk][n] = v;
-    }
-    __syncthreads();
+    float4 va[NCH], vb[NCH];
+    // Piece i of this thread: four k of one row (K-major) or four rows of one k (MN-major).
+    auto load = [&](int kb) {
+      const int kbase = kb * KT;
 #pragma unroll
-    for (int kk = 0; kk < T_K; ++kk) {
-      const float a0 = As[kk][ty * 2], a1 = As[kk][ty * 2 + 1];
-      const float b0 = Bs[kk][tx * 2], b1 = Bs[kk][tx * 2 + 1];
-      acc[0][0] = fmaf(a0, b0, acc[0][0]);
-      acc[0][1] = fmaf(a0, b1, acc[0][1]);
-      acc[1][0] = fmaf(a1, b0, acc[1][0]);
-      acc[1][1] = fmaf(a1, b1, acc[1][1]);
-    }
-    __syncthreads();
-  }
+      for (int i = 0; i < NCH; ++i) {
+        const int id = tid + i * CC_THREADS;
+        auto fetch = [&](const T* P, bool mn, bool vec, int lim, auto off) {
+          const int r = mn ? 4 * (id % (R / 4)) : id / (KT / 4), k = kbase + (mn ? id / (R / 4) : 4 * (id % (KT / 4)));
+          const int n = mn ? (k < ti.kext ? lim - r : 0) : (r < lim ? ti.kext - k : 0);  // elements that exist
+          float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+          if (vec && n >= 4) {
+            v = load4(P + off(r, k));
+          } else {
+            if (n > 0) v.x = to_f<T>(P[off(r, k)]);
+            if (n > 1) v.y = to_f<T>(P[mn ? off(r + 1, k) : off(r, k + 1)]);
+            if (n > 2) v.z = to_f<T>(P[mn ? off(r + 2, k) : off(r, k + 2)]);
+            if (n > 3) v.w = to_f<T>(P[mn ? off(r + 3, k) : off(r, k + 3)]);
+          }
+          return v;
+        };
+        va[i] = fetch(PA, A_MN, vec_a, a_lim, a_off);
+        vb[i] = fetch(PB, B_MN, vec_b, b_lim, b_off);
+      }
+    };
+    auto stage = [&](int buf) {
+      float* SA = sm + buf * 2 * KT * PITCH;
+      float* SB = SA + KT * PITCH;
+#pragma unroll
+      for (int i = 0; i < NCH; ++i) {
+        const int id = tid + i * CC_THREADS;
+        auto put = [&](float* S, bool mn, const float4& v) {
+          if (mn) {
+            *reinterpret_cast<float4*>(S + (id / (R / 4)) * PITCH + 4 * (id % (R / 4))) = v;
+          } else {
+            float* d = S + 4 * (id % (KT / 4)) * PITCH + id / (KT / 4);
+            d[0] = v.x; d[PITCH] = v.y; d[2 * PITCH] = v.z; d[3 * PITCH] = v.w;
+          }
+        };
+        put(SA, A_MN, va[i]);
+        put(SB, B_MN, vb[i]);
+      }
+    };
 
+    float acc[Q][Q];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < Q; ++i)
 #pragma unroll
-    for (int j = 0; j < 2; ++j) {
-      const int m = m0 + ty * 2 + i, n = n0 + tx * 2 + j;
-      if (m >= M || n >= N) continue;
-      size_t off;
-      if (KIND == 0 && OP == OP_FWD) off = (size_t)m * g.ldo + (g.flag0 == ARD_OUT_SCATTER_ZEROFILL ? g.idx[n] : n);
-      else if (KIND == 0 && OP == OP_BWD_WEIGHT) off = (size_t)(g.hdr_in != nullptr ? m : g.idx[m]) * g.ldo + n;
-      else off = (size_t)m * g.ldo + n;
-      float v = acc[i][j];
-      if (KIND == 0 && OP == OP_FWD) {
-        // layer step: bias, then the activation, then the rescale (Sec. 3.2, last paragraph)
-        if (g.bias != nullptr) v += g.bias[g.idx[n]];
-        if (g.relu) v = fmaxf(v, 0.f);
+      for (int j = 0; j < Q; ++j) acc[i][j] = 0.f;
+    if (kb1 > kb0) {
+      load(kb0);
+      stage(0);
+      __syncthreads();
+      for (int kb = kb0; kb < kb1; ++kb) {
+        const int buf = (kb - kb0) & 1;
+        const bool more = kb + 1 < kb1;
+        if (more) load(kb + 1);
+        const float* SA = sm + buf * 2 * KT * PITCH;
+        const float* SB = SA + KT * PITCH;
+#pragma unroll
+        for (int k = 0; k < KT; ++k) {
+          float a[Q], b[Q];
+#pragma unroll
+          for (int h = 0; h < Q / 4; ++h) {
+            *reinterpret_cast<float4*>(a + 4 * h) = *reinterpret_cast<const float4*>(SA + k * PITCH + 32 * h + 4 * ty);
+            *reinterpret_cast<float4*>(b + 4 * h) = *reinterpret_cast<const float4*>(SB + k * PITCH + 32 * h + 4 * tx);
+          }
+#pragma unroll
+          for (int i = 0; i < Q; ++i)
+#pragma unroll
+            for (int j = 0; j < Q; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
+        }
+        if (more) stage(buf ^ 1);
+        __syncthreads();
       }
-      v *= g.alpha;
-      if (KIND == 0 && OP == OP_BWD_DATA && g.act != nullptr) {
-        // adjoint of the producing layer's ReLU: nothing flows where its output was not positive
-        if (!(to_f<T>(reinterpret_cast<const T*>(g.act)[(size_t)m * g.ldact + n]) > 0.f)) v = 0.f;
-      }
-      store_out(g.out, off, v, g.out_is_f32, g.accumulate);
     }
+    if (live) {
+#pragma unroll
+      for (int i = 0; i < Q; ++i)
+#pragma unroll
+        for (int h = 0; h < Q / 4; ++h)
+          *reinterpret_cast<float4*>(sm + (32 * (i / 4) + 4 * ty + i % 4) * PITCH + 32 * h + 4 * tx) =
+              make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
+    }
+    if (s.S > 1) cluster_sync_all();  // the partial tiles of the group are complete
+    else __syncthreads();
+    if (live) write_tile<KIND, OP, R, R, PITCH, CC_THREADS / 32, T>(g, s, ti, sm, smem_u32(sm), part, lead, warp, lane);
+    __syncwarp();
+    if (s.S > 1) cluster_sync_all();  // no CTA of the group reads this one's partial tile any more
+    else __syncthreads();
+  }
 }
 
 // ---- layers with at most 16 neurons (an output layer) -----------------------------------------------
@@ -278,24 +306,38 @@ __global__ void __launch_bounds__(256) skinny_bwd_weight_kernel(GemmArgs g) {
   }
 }
 
+inline int cdiv(int a, int b) { return (a + b - 1) / b; }
+
 template <typename T, int KIND, int OP>
-void launch_one(const ard_ctx* ctx, const GemmArgs& a, int ts, int Mmax, int Nmax, cudaStream_t s) {
-  dim3 grid((Nmax + T_N - 1) / T_N, (Mmax + T_M - 1) / T_M);
-  (void)ard_launch(ctx, gemm_cc_kernel<T, KIND, OP>, grid, dim3(CC_THREADS), 0, s, a, ts);  // errors: cudaGetLastError
-}
+void launch_one(const ard_ctx* ctx, const GemmArgs& g, int ts, cudaStream_t s) {
+  CcParams p = {};
+  p.g = g;
+  p.ts = ts;
+  p.want = 4 * ctx->sm_count;
+  const uintptr_t four = 4 * sizeof(T) - 1;
+  p.vec = ((reinterpret_cast<uintptr_t>(g.A0) & four) == 0 && g.lda0 % 4 == 0 ? 1 : 0) |
+          ((reinterpret_cast<uintptr_t>(g.A1) & four) == 0 && g.lda1 % 4 == 0 ? 2 : 0);
+  const int M = OP == OP_BWD_WEIGHT ? g.N : g.B, N = OP == OP_FWD ? g.N : g.K;
+  const double flops = 2.0 * g.B * g.K * g.N;
+  // The grid covers the tiles of the densest pattern, cut or not; CTAs without work read the header and leave.
+  auto grid = [&](int R) {
+    const int n = min(16 * ctx->sm_count, max(p.want, cdiv(M, R) * cdiv(N, R)));
+    return dim3(cdiv(n, SP_CLUSTER) * SP_CLUSTER);
+  };
+  if (flops > CC_WIDE_FLOPS) (void)ard_launch_cluster(ctx, gemm_cc_kernel<T, KIND, OP, 64>, SP_CLUSTER, grid(64), dim3(CC_THREADS), 0, s, p);
+  else (void)ard_launch_cluster(ctx, gemm_cc_kernel<T, KIND, OP, 32>, SP_CLUSTER, grid(32), dim3(CC_THREADS), 0, s, p);
+}  // errors: cudaGetLastError
 
 template <typename T>
 void dispatch(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& a, int ts, cudaStream_t s) {
-  // The grid covers the largest problem any pattern can produce (dp = 1); CTAs beyond the
-  // sampled extent read the header and exit.
   if (kind == ARD_ROW) {
-    if (op == OP_FWD) launch_one<T, 0, OP_FWD>(ctx, a, ts, a.B, a.N, s);
-    else if (op == OP_BWD_DATA) launch_one<T, 0, OP_BWD_DATA>(ctx, a, ts, a.B, a.K, s);
-    else launch_one<T, 0, OP_BWD_WEIGHT>(ctx, a, ts, a.N, a.K, s);
+    if (op == OP_FWD) launch_one<T, 0, OP_FWD>(ctx, a, ts, s);
+    else if (op == OP_BWD_DATA) launch_one<T, 0, OP_BWD_DATA>(ctx, a, ts, s);
+    else launch_one<T, 0, OP_BWD_WEIGHT>(ctx, a, ts, s);
   } else {
-    if (op == OP_FWD) launch_one<T, 1, OP_FWD>(ctx, a, ts, a.B, a.N, s);
-    else if (op == OP_BWD_DATA) launch_one<T, 1, OP_BWD_DATA>(ctx, a, ts, a.B, a.K, s);
-    else launch_one<T, 1, OP_BWD_WEIGHT>(ctx, a, ts, a.N, a.K, s);
+    if (op == OP_FWD) launch_one<T, 1, OP_FWD>(ctx, a, ts, s);
+    else if (op == OP_BWD_DATA) launch_one<T, 1, OP_BWD_DATA>(ctx, a, ts, s);
+    else launch_one<T, 1, OP_BWD_WEIGHT>(ctx, a, ts, s);
   }
 }
 
@@ -304,17 +346,6 @@ void dispatch(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& a, i
 ard_status launch_gemm_cc(ard_ctx* ctx, ard_kind kind, GemmOp op, ard_dtype dtype, const GemmArgs& a, int ts,
                           cudaStream_t s) {
   if ((a.B == 0 && op != OP_BWD_WEIGHT) || a.K == 0 || a.N == 0) return ARD_OK;
-  const size_t es_out = a.out_is_f32 ? 4 : 2;
-  // Row patterns: dropped outputs are cleared by a strided memset before the kept ones are written.
-  const bool small_layer = kind == ARD_ROW && a.N <= SKINNY_N && (op == OP_FWD ? a.B > 0 : op == OP_BWD_WEIGHT);
-  if (small_layer) {
-    // the kernels for a handful of neurons write their own zeros
-  } else if (kind == ARD_ROW && op == OP_FWD && a.flag0 == ARD_OUT_SCATTER_ZEROFILL) {
-    ARD_CUDA_OK(cudaMemset2DAsync(a.out, (size_t)a.ldo * es_out, 0, (size_t)a.N * es_out, a.B, s));
-  }
-  if (!small_layer && kind == ARD_ROW && op == OP_BWD_WEIGHT && a.flag1) {
-    ARD_CUDA_OK(cudaMemset2DAsync(a.out, (size_t)a.ldo * es_out, 0, (size_t)a.K * es_out, a.N, s));
-  }
   if (kind == ARD_ROW && a.N <= SKINNY_N && op == OP_FWD && a.B > 0) {
     if (dtype == ARD_F32) (void)ard_launch(ctx, skinny_fwd_kernel<float>, dim3(a.B), dim3(256), 0, s, a);
     else (void)ard_launch(ctx, skinny_fwd_kernel<__nv_bfloat16>, dim3(a.B), dim3(256), 0, s, a);
