@@ -575,8 +575,8 @@ ard_status ard_lstm_gate_gemm_bwd(ard_ctx* ctx, const ard_pattern* pat, int B, i
                                   void* cuda_stream);
 
 /* Whole-sequence forward: for t = 0..T-1, the gate product on XH[t] followed by the cell update, which writes
- * h_t into the h half of XH[t+1].  When the layer fits (B <= 128, the weight rows of 8 hidden units times
- * (I+H) columns fit in shared memory, H/8 <= number of SMs, operands aligned for the tensor-core path) this
+ * h_t into the h half of XH[t+1].  When the layer fits (B <= 128; 8 or 12 hidden units per SM, whose recurrent weight
+ * rows fit in shared memory beside part of h; any alignment with ARD_PATH_AUTO) this
  * is ONE cooperative kernel that keeps the weight in shared memory and the cell state in registers for the
  * whole sequence and synchronises the SMs once per step (every wait bounded, see ARD_ERR_TIMEOUT); Z is
  * then not used.  Otherwise, or after ard_set_lstm_persistent(ctx, 0), it is a loop in native code that
@@ -596,17 +596,22 @@ ard_status ard_lstm_forward(ard_ctx* ctx, const ard_pattern* pat, int T, int B, 
  * half of D[0] the gradient of h_0.  dH_last [B][H] fp32 is the gradient of h_{T-1}; dc [B][H] fp32 must be
  * zero on entry (or hold the gradient of c_T) and returns the gradient of c_0; DZ [T][B][4H] bf16 scratch;
  * dW [4H][I+H] fp32 receives the weight gradient (dropped units' rows zero).
- * When the layer fits (B <= 128, H <= 1024, 8*ceil(H/64) <= number of SMs, operands aligned) and
+ * When the layer fits (as for ard_lstm_forward) and
  * ard_set_lstm_persistent is on, the recurrence dh_{t-1} = upstream + dz_t W_h with the cell adjoint is ONE
- * cooperative kernel (weight slices resident in shared memory, dc in registers, two bounded grid-wide
- * synchronisations per step; one, and no partial sums, when the drawn pattern keeps at most 256 units, see
- * ARD_OPT_LSTM_COMPACT_H) and the x halves come from one product over all T*B rows; otherwise a loop
+ * cooperative kernel (weight slices resident in shared memory, dc in registers; one bounded grid-wide synchronisation
+ * per step, or, where the gate gradients of a step are too many to stream through shared memory, two and partial sums,
+ * see ARD_OPT_LSTM_COMPACT_H) and the x halves come from one product over all T*B rows; otherwise a loop
  * in native code enqueues ard_lstm_gates_bwd and ard_lstm_gate_gemm_bwd per step.  In both cases the h
  * halves of D[1..T-1] are overwritten (kept units: the total gradient of h_{t-1}; dropped units:
  * unspecified), and the h half of D[0] is meaningful at kept units only. */
 ard_status ard_lstm_backward(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                              const void* XH, const void* W, int ldw, const float* C, const float* G,
                              const float* dH_last, float* D, float* dc, void* DZ, float* dW, void* cuda_stream);
+/* The same with nothing prepared: dH [T][B][H] fp32 holds the upstream gradient of every h_t, no gradient arrives at
+ * c_T, and D and dc are outputs only (contents as above). */
+ard_status ard_lstm_backward_dh(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
+                                const void* XH, const void* W, int ldw, const float* C, const float* G, const float* dH,
+                                float* D, float* dc, void* DZ, float* dW, void* cuda_stream);
 
 /* ---- stacked LSTM with dropout on the layer OUTPUTS only (second reading of the LSTM experiment of Sec. 7) ----
  * The paper prints no LSTM equations; its LSTM networks are stacks of two and three layers.  In this reading every

@@ -232,6 +232,7 @@ ard_status ard_create(ard_ctx** out, int device, size_t workspace_bytes) {
         cudaMemset(ctx->d_sk_cnt, 0, cnt_bytes) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void**>(&ctx->d_tm_slots), tm_slots_bytes()) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void**>(&ctx->d_grid_bar), 256) != cudaSuccess ||
+        cudaMemset(ctx->d_grid_bar, 0, 256) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void**>(&ctx->d_lstm_partial), lstm_bwd_partial_bytes(ctx->sm_count)) != cudaSuccess ||
         cudaMalloc(&ctx->d_lstm_hc, lstm_hc_bytes()) != cudaSuccess ||
         cudaMemset(ctx->d_lstm_hc, 0, lstm_hc_bytes()) != cudaSuccess) {
@@ -1073,6 +1074,54 @@ ard_status ard_lstm_gates_bwd(ard_ctx* ctx, const ard_pattern* pat, ard_dtype dz
                                dc_inout, dZ, ldz_gate, (cudaStream_t)cuda_stream);
 }
 
+// One gate's share of a product over all T*B rows of a sequence, on operands that no descriptor can describe.
+static ard_status lstm_gate_product_staged(ard_ctx* ctx, const ard_pattern* pat, GemmOp op, int rows, int K, int H, const void* A0,
+                                           int lda0, const void* A1, int lda1, float* out, int ldo, int accumulate, cudaStream_t s) {
+  GemmArgs g = {};
+  fill_common(g, ctx, pat, rows, K, H, 1.0f);
+  g.A0 = A0; g.lda0 = lda0; g.A1 = A1; g.lda1 = lda1; g.out = out; g.ldo = ldo;
+  g.flag0 = op == OP_FWD ? (int)ARD_OUT_COMPACT : 1;
+  g.flag1 = 1;  // weight gradient: rows of dropped units are written as zero
+  g.out_is_f32 = 1;
+  g.accumulate = accumulate;
+  return launch_gemm_ldg(ctx, ARD_ROW, op, g, 0, s);
+}
+
+// Input half of every step's pre-activations: G[t][:, g*H + j] = x_t . W[g*H + keep[j]][0:I]  (T*B rows).
+static ard_status lstm_input_half(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, const void* XH, const void* W,
+                                  int ldw, float* G, cudaStream_t s) {
+  const int KH = I + H;
+  const char* Wc = reinterpret_cast<const char*>(W);
+  const bool tma = aligned16(XH) && aligned16(W) && aligned16(G) && KH % 8 == 0 && ldw % 8 == 0 && H % 4 == 0 &&
+                   pat->dp_bound <= ARD_MAX_NDP_TC;
+  ard_status st = ARD_OK;
+  if (!tma) {
+    for (int gate = 0; gate < 4 && st == ARD_OK; ++gate)
+      st = lstm_gate_product_staged(ctx, pat, OP_FWD, T * B, I, H, XH, KH, Wc + (size_t)gate * H * ldw * 2, ldw, G + (size_t)gate * H,
+                                    4 * H, 0, s);
+    return st;
+  }
+  TcArgs t = {};
+  GemmArgs g = {};
+  fill_common(g, ctx, pat, T * B, I, H, 1.0f);
+  g.A0 = XH; g.lda0 = KH; g.A1 = W; g.lda1 = ldw; g.out = G; g.ldo = 4 * H;
+  g.out_is_f32 = 1;
+  t.g = g;
+  t.ts = H;
+  t.bn = 0;
+  st = get_maps(ctx, XH, T * B, I, KH, 0, MAP_PLAIN, 0, 128, 64, &t.mapA);
+  if (st != ARD_OK) return st;
+  t.mapA_indexed = 0;
+  for (int gate = 0; gate < 4; ++gate) {
+    st = get_maps(ctx, Wc + (size_t)gate * H * ldw * 2, H, I, ldw, H, MAP_STRIDED_ROWS, pat->dp_bound, 64, 64, &t.mapB4[gate]);
+    if (st != ARD_OK) return st;
+    t.mapA4[gate] = t.mapA;
+  }
+  t.mapB = t.mapB4[0];
+  t.mapB_indexed = 1;
+  return launch_lstm_tc(ctx, 0, t, s);
+}
+
 // Whole-sequence drivers: the time loop runs here, in native code, and only enqueues kernels.
 // gates_ready: the input half of every step's pre-activations is already in G (the caller multiplied it, e.g. over
 // the kept outputs of the layer below); only the recurrence runs, which needs the one-kernel form.
@@ -1083,62 +1132,46 @@ static ard_status lstm_forward_impl(ard_ctx* ctx, const ard_pattern* pat, int T,
   if (T < 0 || B < 0 || I < 0 || H < 1) return ARD_ERR_INVALID_ARG;
   const int KH = I + H;
   __nv_bfloat16* xh = reinterpret_cast<__nv_bfloat16*>(XH);
-  // One cooperative kernel for the whole sequence when the layer fits it (the weight slice of 8 hidden
-  // units per CTA in shared memory, all CTAs resident, at most 128 batch rows) and the operands meet the
-  // TMA path's alignment rules; otherwise one gate product and one cell kernel per time step.
-  if (ctx->lstm_persistent && ctx->path != ARD_PATH_CUDA_CORE && T >= 1 && B >= 1) {
+  // One cooperative kernel for the whole sequence when the layer fits it (all units on the device at once, at most 128
+  // batch rows); otherwise one gate product and one cell kernel per time step.
+  if (ctx->lstm_persistent && ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && T >= 1 && B >= 1) {
     ard_status st = check_common(ctx, pat, B, KH, H);
     if (st != ARD_OK) return st;
     if (pat->kind != ARD_ROW) return ARD_ERR_INVALID_ARG;
     if (ldw < KH) return ARD_ERR_SHAPE;
     DeviceGuard guard(ctx->device);
     const char* Wc = reinterpret_cast<const char*>(W);
-    if (tc_eligible(ctx, pat, ARD_BF16, B, KH, H, XH, KH, W, ldw, C, H, 4) == ARD_OK &&
-        ((size_t)H * ldw * 2) % 16 == 0 && lstm_persistent_fits(ctx, B, H, H)) {
+    // operands that the TMA unit can read: 16-byte aligned rows, h starting on a 16-byte boundary
+    const bool tma = tc_eligible(ctx, pat, ARD_BF16, B, KH, H, XH, KH, W, ldw, C, H, 4) == ARD_OK &&
+                     ((size_t)H * ldw * 2) % 16 == 0 && I % 8 == 0;
+    if (lstm_persistent_fits(ctx, B, H, tma) && (tma || ctx->path == ARD_PATH_AUTO)) {
       cudaStream_t s = (cudaStream_t)cuda_stream;
-      TcMap mapXH;
+      TcMap mapXH, mapHc;
       TcMap mapW[4];
-      // 1. The input half for all steps at once: G[t][:, g*H + j] = x_t . W[g*H + keep[j]][0:I]  (T*B rows).
+      // 1. The input half for all steps at once.
       if (I > 0 && !gates_ready) {
-        TcArgs t = {};
-        GemmArgs g = {};
-        fill_common(g, ctx, pat, T * B, I, H, 1.0f);
-        g.A0 = XH; g.lda0 = KH; g.A1 = W; g.lda1 = ldw; g.out = G; g.ldo = 4 * H;
-        g.out_is_f32 = 1;
-        t.g = g;
-        t.ts = H;
-        t.bn = 0;
-        st = get_maps(ctx, XH, T * B, I, KH, 0, MAP_PLAIN, 0, 128, 64, &t.mapA);
-        if (st != ARD_OK) return st;
-        t.mapA_indexed = 0;
-        for (int gate = 0; gate < 4; ++gate) {
-          st = get_maps(ctx, Wc + (size_t)gate * H * ldw * 2, H, I, ldw, H, MAP_STRIDED_ROWS, pat->dp_bound, 64, 64,
-                        &t.mapB4[gate]);
-          if (st != ARD_OK) return st;
-          t.mapA4[gate] = t.mapA;
-        }
-        t.mapB = t.mapB4[0];
-        t.mapB_indexed = 1;
-        st = launch_lstm_tc(ctx, 0, t, s);
+        st = lstm_input_half(ctx, pat, T, B, I, H, XH, W, ldw, G, s);
         if (st != ARD_OK) return st;
       }
       // 2. The recurrence: one kernel, recurrent half of the weight resident in shared memory.
-      st = get_maps(ctx, XH, (T + 1) * B, KH, KH, 0, MAP_PLAIN, 0, 64, 64, &mapXH);
-      if (st != ARD_OK) return st;
-      for (int gate = 0; gate < 4; ++gate) {
-        st = get_maps(ctx, Wc + (size_t)gate * H * ldw * 2, H, KH, ldw, H, MAP_STRIDED_ROWS, pat->dp_bound, 8, 64,
-                      &mapW[gate]);
+      const int box = lstm_box_rows_of(B);
+      if (tma) {
+        st = get_maps(ctx, XH, (T + 1) * B, KH, KH, 0, MAP_PLAIN, 0, box, 64, &mapXH);
         if (st != ARD_OK) return st;
+        for (int gate = 0; gate < 4; ++gate) {
+          st = get_maps(ctx, Wc + (size_t)gate * H * ldw * 2, H, KH, ldw, H, MAP_STRIDED_ROWS, pat->dp_bound, 8, 64,
+                        &mapW[gate]);
+          if (st != ARD_OK) return st;
+        }
       }
-      // 2b. Under a pattern the recurrence contracts over the kept units of h_{t-1} alone: its operand is a compact
+      // Under a pattern the recurrence contracts over the kept units of h_{t-1} alone: its operand is a compact
       // copy of h in context scratch (two buffers, the kernel fills them).
-      TcMap mapHc;
-      const bool compact_h = ctx->lstm_compact_h && pat->dp_bound > 1 && ctx->d_lstm_hc != nullptr && H <= ARD_LSTM_HC_LD;
+      const bool compact_h = ctx->lstm_compact_h && ctx->d_lstm_hc != nullptr && H <= ARD_LSTM_HC_LD;
       if (compact_h) {
-        st = get_maps(ctx, ctx->d_lstm_hc, 2 * B, ARD_LSTM_HC_LD, ARD_LSTM_HC_LD, 0, MAP_PLAIN, 0, 64, 64, &mapHc);
+        st = get_maps(ctx, ctx->d_lstm_hc, 2 * B, ARD_LSTM_HC_LD, ARD_LSTM_HC_LD, 0, MAP_PLAIN, 0, box, 64, &mapHc);
         if (st != ARD_OK) return st;
       }
-      st = launch_lstm_forward_persistent(ctx, pat, T, B, I, H, I, H, I > 0 ? 1 : 0, alpha, mapXH, mapW,
+      st = launch_lstm_forward_persistent(ctx, pat, T, B, I, H, I > 0 ? 1 : 0, alpha, tma ? &mapXH : nullptr, mapW,
                                           compact_h ? &mapHc : nullptr, W, ldw, XH, bias, C, G, s);
       if (st != ARD_ERR_UNSUPPORTED) return st;
       // not launchable as one kernel right now: the per-step path below recomputes everything
@@ -1172,59 +1205,90 @@ ard_status ard_lstm_forward_from_gates(ard_ctx* ctx, const ard_pattern* pat, int
 
 // recurrent_only: the recurrence (gate gradients DZ) and the weight gradient of the recurrent half,
 // dW[:, I : I+H]; the input half (dx and dW[:, 0 : I]) is left to the caller.  Needs the one-kernel form.
+// dH: the gradient of every h_t, D and dc are then outputs only; nullptr: dH_last, D and dc prepared by the caller.
 static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                      const void* XH, const void* W, int ldw, const float* C, const float* G,
-                                     const float* dH_last, float* D, float* dc, void* DZ, float* dW,
+                                     const float* dH, const float* dH_last, float* D, float* dc, void* DZ, float* dW,
                                      int recurrent_only, void* cuda_stream) {
-  if (!ctx || !pat || !XH || !W || !C || !G || !dH_last || !D || !dc || !DZ || !dW) return ARD_ERR_INVALID_ARG;
+  if (!ctx || !pat || !XH || !W || !C || !G || (!dH && !dH_last) || !D || !dc || !DZ || !dW) return ARD_ERR_INVALID_ARG;
   if (T < 1 || B < 0 || I < 0 || H < 1) return ARD_ERR_INVALID_ARG;
   const int KH = I + H;
-  __nv_bfloat16* dz = reinterpret_cast<__nv_bfloat16*>(DZ);
+  const char* Wc = reinterpret_cast<const char*>(W);
+  cudaStream_t s = (cudaStream_t)cuda_stream;
+  // gate gradients: the caller's DZ, or a copy in context scratch whose rows are padded to the 16-byte grid
+  void* dz = DZ;
+  int gs = H;
   // One cooperative kernel for the recurrence of the whole sequence when the layer fits it, followed by the
   // input half of d[x, h] as one product over all T*B rows; otherwise the two kernels per time step below.
   bool recurrence_done = false;
-  if (ctx->lstm_persistent && ctx->path != ARD_PATH_CUDA_CORE && B >= 1 && I > 0) {
+  if (ctx->lstm_persistent && ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && B >= 1 && I > 0) {
     ard_status st = check_common(ctx, pat, B, KH, H);
     if (st != ARD_OK) return st;
     if (pat->kind != ARD_ROW) return ARD_ERR_INVALID_ARG;
     if (ldw < KH) return ARD_ERR_SHAPE;
     DeviceGuard guard(ctx->device);
-    cudaStream_t s = (cudaStream_t)cuda_stream;
-    const char* Wc = reinterpret_cast<const char*>(W);
-    const char* dZc = reinterpret_cast<const char*>(DZ);
-    if (tc_eligible(ctx, pat, ARD_BF16, T * B, KH, H, DZ, 4 * H, W, ldw, D, KH, 4) == ARD_OK &&
-        ((size_t)H * ldw * 2) % 16 == 0 && I % 8 == 0 && lstm_persistent_bwd_fits(ctx, B, H)) {
+    const bool tma = tc_eligible(ctx, pat, ARD_BF16, T * B, KH, H, DZ, 4 * H, W, ldw, D, KH, 4) == ARD_OK &&
+                     ((size_t)H * ldw * 2) % 16 == 0 && I % 8 == 0;
+    const int padded = (H + 7) / 8 * 8;
+    const bool room = tma || (size_t)T * B * 4 * padded * 2 <= sk_ws_bytes(ctx->sm_count);
+    if (lstm_persistent_bwd_fits(ctx, B, H, tma) && room && (tma || ctx->path == ARD_PATH_AUTO)) {
+      if (!tma) {
+        dz = ctx->d_sk_ws;
+        gs = padded;
+      }
       TcMap mapDZ[4];
       TcMap mapW[4];
       for (int gate = 0; gate < 4; ++gate) {
-        st = get_maps(ctx, dZc + (size_t)gate * H * 2, T * B, H, 4 * H, H, MAP_COMPACT_COLS, pat->dp_bound, 64, 64,
-                      &mapDZ[gate]);
+        st = get_maps(ctx, reinterpret_cast<const char*>(dz) + (size_t)gate * gs * 2, T * B, H, 4 * gs, H, MAP_COMPACT_COLS,
+                      pat->dp_bound, lstm_box_rows_of(B), 64, &mapDZ[gate]);
         if (st != ARD_OK) return st;
+        if (!tma) continue;
         st = get_maps(ctx, Wc + (size_t)gate * H * ldw * 2, H, KH, ldw, H, MAP_STRIDED_ROWS, pat->dp_bound, 64, 64,
                       &mapW[gate]);
         if (st != ARD_OK) return st;
       }
-      st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, mapW, W, ldw, C, G, dH_last, D, dc, DZ, s);
+      st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, tma ? mapW : nullptr, W, ldw, C, G, dH, dH_last, D, dc,
+                                           dz, gs, recurrent_only && dz != DZ ? DZ : nullptr, s);
       if (st == ARD_OK) {
-        // dx_t for all t: the x halves of D are overwritten
-        if (!recurrent_only) st = lstm_gate_gemm_bwd_tc(ctx, pat, T * B, I, H, DZ, H, W, ldw, D, KH, 0, s);
-        if (st != ARD_OK) return st;
         recurrence_done = true;
+        // dx_t for all t: the x halves of D are overwritten
+        if (!recurrent_only) {
+          if (aligned16(W) && aligned16(D) && ldw % 8 == 0 && KH % 4 == 0 && pat->dp_bound <= ARD_MAX_NDP_TC) {
+            st = lstm_gate_gemm_bwd_tc(ctx, pat, T * B, I, H, dz, gs, W, ldw, D, KH, 0, s);
+          } else {
+            for (int gate = 0; gate < 4 && st == ARD_OK; ++gate)
+              st = lstm_gate_product_staged(ctx, pat, OP_BWD_DATA, T * B, I, H, reinterpret_cast<const char*>(dz) + (size_t)gate * gs * 2,
+                                            4 * gs, Wc + (size_t)gate * H * ldw * 2, ldw, D, KH, gate > 0, s);
+          }
+        }
+        if (st != ARD_OK) return st;
       } else if (st != ARD_ERR_UNSUPPORTED) {
         return st;
+      } else {
+        dz = DZ;
+        gs = H;
       }
     }
   }
   if (recurrent_only && !recurrence_done) return ARD_ERR_UNSUPPORTED;
+  if (!recurrence_done && dH != nullptr) {
+    // what the steps below expect: upstream gradients of h_{t-1} in the h halves, zeros everywhere else
+    DeviceGuard guard(ctx->device);
+    ARD_CUDA_OK(cudaMemsetAsync(D, 0, (size_t)T * B * KH * sizeof(float), s));
+    ARD_CUDA_OK(cudaMemsetAsync(dc, 0, (size_t)B * H * sizeof(float), s));
+    if (T > 1)
+      ARD_CUDA_OK(cudaMemcpy2DAsync(D + (size_t)B * KH + I, (size_t)KH * sizeof(float), dH, (size_t)H * sizeof(float),
+                                    (size_t)H * sizeof(float), (size_t)(T - 1) * B, cudaMemcpyDeviceToDevice, s));
+    dH_last = dH + (size_t)(T - 1) * B * H;
+  }
   for (int t = T - 1; t >= 0 && !recurrence_done; --t) {
+    __nv_bfloat16* dz_t = reinterpret_cast<__nv_bfloat16*>(DZ) + (size_t)t * B * 4 * H;
     const float* dh = (t == T - 1) ? dH_last : D + (size_t)(t + 1) * B * KH + I;
     const int lddh = (t == T - 1) ? H : KH;
     ard_status st = ard_lstm_gates_bwd(ctx, pat, ARD_BF16, B, H, alpha, G + (size_t)t * B * 4 * H,
-                                       C + (size_t)t * B * H, C + (size_t)(t + 1) * B * H, H, dh, lddh, 1, dc,
-                                       dz + (size_t)t * B * 4 * H, H, cuda_stream);
+                                       C + (size_t)t * B * H, C + (size_t)(t + 1) * B * H, H, dh, lddh, 1, dc, dz_t, H, cuda_stream);
     if (st != ARD_OK) return st;
-    st = ard_lstm_gate_gemm_bwd(ctx, pat, B, KH, H, dz + (size_t)t * B * 4 * H, H, W, ldw, D + (size_t)t * B * KH, KH,
-                                1, cuda_stream);
+    st = ard_lstm_gate_gemm_bwd(ctx, pat, B, KH, H, dz_t, H, W, ldw, D + (size_t)t * B * KH, KH, 1, cuda_stream);
     if (st != ARD_OK) return st;
   }
   // Weight gradient over all T*B rows: the four gate blocks in one tensor-core launch when the operands
@@ -1233,21 +1297,21 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
   const int wcol0 = recurrent_only ? I : 0, wcols = recurrent_only ? H : KH;
   const void* XHw = reinterpret_cast<const __nv_bfloat16*>(XH) + wcol0;
   float* dWw = dW + wcol0;
-  const bool w_tc = ctx->path != ARD_PATH_CUDA_CORE && H % 8 == 0 && wcols % 8 == 0 && wcol0 % 8 == 0 &&
-                    tc_eligible(ctx, pat, ARD_BF16, T * B, KH, H, DZ, 4 * H, XH, KH, dW, KH, 4) == ARD_OK;
-  if (recurrent_only && !w_tc) return ARD_ERR_UNSUPPORTED;
+  const char* dzc = reinterpret_cast<const char*>(dz);
+  const bool w_tc = ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && B >= 1 && pat->kind == ARD_ROW &&
+                    pat->dp_bound <= ARD_MAX_NDP_TC && aligned16(dz) && gs % 8 == 0 && aligned16(XHw) && aligned16(dWw) && KH % 8 == 0;
+  DeviceGuard guard(ctx->device);
   if (w_tc) {
     TcArgs t = {};
     GemmArgs g = {};
     fill_common(g, ctx, pat, T * B, wcols, H, 1.0f);
-    g.A0 = DZ; g.lda0 = 4 * H; g.A1 = XHw; g.lda1 = KH; g.out = dWw; g.ldo = KH;
+    g.A0 = dz; g.lda0 = 4 * gs; g.A1 = XHw; g.lda1 = KH; g.out = dWw; g.ldo = KH;
     g.flag0 = 1;
     g.flag1 = 1;  // rows of dropped units are written as zero
     g.out_is_f32 = 1;
     ard_status st = ARD_OK;
-    const char* dZc = reinterpret_cast<const char*>(DZ);
     for (int gate = 0; gate < 4 && st == ARD_OK; ++gate)
-      st = get_maps(ctx, dZc + (size_t)gate * H * 2, T * B, H, 4 * H, H, MAP_COMPACT_COLS, pat->dp_bound, 64, 64,
+      st = get_maps(ctx, dzc + (size_t)gate * gs * 2, T * B, H, 4 * gs, H, MAP_COMPACT_COLS, pat->dp_bound, 64, 64,
                     &t.mapA4[gate]);
     if (st == ARD_OK) st = get_maps(ctx, XHw, T * B, wcols, KH, 0, MAP_PLAIN, 0, 64, 64, &t.mapB);
     if (st != ARD_OK) return st;
@@ -1257,10 +1321,17 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
     t.g = g;
     t.ts = 0;
     t.bn = ctx->force_bn;
-    return launch_lstm_tc(ctx, 2, t, (cudaStream_t)cuda_stream);
+    return launch_lstm_tc(ctx, 2, t, s);
+  }
+  if (recurrence_done) {
+    ard_status st = ARD_OK;
+    for (int gate = 0; gate < 4 && st == ARD_OK; ++gate)
+      st = lstm_gate_product_staged(ctx, pat, OP_BWD_WEIGHT, T * B, wcols, H, dzc + (size_t)gate * gs * 2, 4 * gs, XHw, KH,
+                                    dWw + (size_t)gate * H * KH, KH, 0, s);
+    return st;
   }
   for (int g = 0; g < 4; ++g) {  // one product per gate
-    ard_status st = ard_bwd_weight(ctx, pat, ARD_BF16, ARD_F32, T * B, KH, H, 1.0f, XH, KH, dz + (size_t)g * H, 4 * H,
+    ard_status st = ard_bwd_weight(ctx, pat, ARD_BF16, ARD_F32, T * B, KH, H, 1.0f, XH, KH, dzc + (size_t)g * H * 2, 4 * H,
                                    1, dW + (size_t)g * H * KH, KH, 1, cuda_stream);
     if (st != ARD_OK) return st;
   }
@@ -1270,14 +1341,21 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
 ard_status ard_lstm_backward(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                              const void* XH, const void* W, int ldw, const float* C, const float* G,
                              const float* dH_last, float* D, float* dc, void* DZ, float* dW, void* cuda_stream) {
-  return lstm_backward_impl(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH_last, D, dc, DZ, dW, 0, cuda_stream);
+  return lstm_backward_impl(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, nullptr, dH_last, D, dc, DZ, dW, 0, cuda_stream);
+}
+
+ard_status ard_lstm_backward_dh(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
+                                const void* XH, const void* W, int ldw, const float* C, const float* G, const float* dH,
+                                float* D, float* dc, void* DZ, float* dW, void* cuda_stream) {
+  if (!dH) return ARD_ERR_INVALID_ARG;
+  return lstm_backward_impl(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH, nullptr, D, dc, DZ, dW, 0, cuda_stream);
 }
 
 ard_status ard_lstm_backward_recurrent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                        const void* XH, const void* W, int ldw, const float* C, const float* G,
                                        const float* dH_last, float* D, float* dc, void* DZ, float* dW,
                                        void* cuda_stream) {
-  return lstm_backward_impl(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH_last, D, dc, DZ, dW, 1, cuda_stream);
+  return lstm_backward_impl(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, nullptr, dH_last, D, dc, DZ, dW, 1, cuda_stream);
 }
 
 ard_status ard_compact_cols(ard_ctx* ctx, const ard_pattern* pat, ard_dtype dtype, int rows, int N, const void* src,

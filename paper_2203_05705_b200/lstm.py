@@ -43,12 +43,9 @@ class LstmLayer:
     def backward(self, alpha, dH):
         """dH: fp32 [T][B][H], gradient with respect to every h_t.  Returns (dX [T][B][I] fp32 view, dW)."""
         ctx, pat, T, B, H, KH, I = self.ctx, self.pat, self.T, self.B, self.H, self.KH, self.I
-        self.D.zero_()
-        self.D[1:, :, I:] = dH[:-1]            # upstream gradient of h_{t-1}; the data GEMM of step t adds to it
-        self.dc.zero_()
-        dh_last = dH[T - 1].contiguous()
-        ard.ard_lstm_backward(ctx, pat, T, B, I, H, alpha, self.XH, self.W, KH, self.C, self.G, dh_last, self.D,
-                              self.dc, self.DZ, self.dW)
+        dH = dH.to(torch.float32).contiguous()
+        ard.ard_lstm_backward_dh(ctx, pat, T, B, I, H, alpha, self.XH, self.W, KH, self.C, self.G, dH, self.D, self.dc, self.DZ,
+                                 self.dW)
         return self.D[:, :, :I], self.dW
 
 
