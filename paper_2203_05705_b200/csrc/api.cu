@@ -206,10 +206,13 @@ ard_status ard_create(ard_ctx** out, int device, size_t workspace_bytes) {
   ctx->launches = 0;
   ctx->d_tm_slots = nullptr;
   ctx->encode_fn = nullptr;
-  cudaDeviceProp prop;
-  if (cudaGetDeviceProperties(&prop, device) != cudaSuccess) { delete ctx; return ARD_ERR_CUDA; }
-  ctx->sm_count = prop.multiProcessorCount;
-  if (prop.major == 10) {
+  int major = 0;  // single attributes: cudaGetDeviceProperties takes milliseconds
+  if (cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
+      cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, device) != cudaSuccess) {
+    delete ctx;
+    return ARD_ERR_CUDA;
+  }
+  if (major == 10) {
     void* fn = nullptr;
     cudaDriverEntryPointQueryResult qres;
     if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres) == cudaSuccess &&

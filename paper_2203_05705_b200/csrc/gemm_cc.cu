@@ -35,7 +35,7 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
   return make_float4(__uint_as_float(a << 16), __uint_as_float(a & 0xffff0000u), __uint_as_float(b << 16), __uint_as_float(b & 0xffff0000u));
 }
 
-constexpr int CC_THREADS = 64;
+__host__ __device__ constexpr int cc_threads(int R) { return R == 64 ? 128 : 64; }
 constexpr double CC_WIDE_FLOPS = 2e8;  // 64 x 64 tiles from here on, see launch_one
 struct CcParams {
   GemmArgs g;
@@ -44,14 +44,21 @@ struct CcParams {
   int vec;       // bit 0 / 1: rows of operand A / B start on four-element boundaries
 };
 
-// R: rows and columns of the output tile (64 or 32); a thread of the 8 x 8 grid owns R / 8 by R / 8 of it.  The
-// operands of a KT-deep block are staged k-major as fp32, [k][row], through registers, one block ahead of the
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
+
+// R: rows and columns of the output tile (64 or 32); a thread of the R / 4 x 8 grid owns 4 rows by R / 8 columns of it,
+// multiplied two columns an instruction.  The operands of a KT-deep block are staged k-major as fp32, [k][row], through registers, one block ahead of the
 // products.  KIND: 0 row, 1 tile.  OP: GemmOp.
-// Bound: FFMA issue for the 64 x 64 tile (64 FFMA per four 16-byte shared-memory reads and thread), latency for the
+// Bound: FFMA issue for the 64 x 64 tile (32 FFMA per three 16-byte shared-memory reads and thread), latency for the
 // 32 x 32 one, which is for products that would otherwise occupy a few SMs.
 template <typename T, int KIND, int OP, int R>
-__global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(const __grid_constant__ CcParams p) {
-  constexpr int KT = R == 64 ? 16 : 32, Q = R / 8, PITCH = R + 4;
+__global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_constant__ CcParams p) {
+  constexpr int CC_THREADS = cc_threads(R), KT = R == 64 ? 16 : 32, Q = R / 8, PITCH = R + 4;
   constexpr bool A_MN = OP == OP_BWD_WEIGHT, B_MN = OP != OP_FWD;
   constexpr int NCH = R * KT / 4 / CC_THREADS;  // four-element pieces per thread, operand and block
   __shared__ __align__(16) float sm[4 * KT * PITCH];  // [buffer][operand][k][row]; the finished tile overlays it
@@ -149,11 +156,11 @@ __global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(const __grid_consta
       }
     };
 
-    float acc[Q][Q];
+    uint64_t acc[4][Q / 2];  // column pairs
 #pragma unroll
-    for (int i = 0; i < Q; ++i)
+    for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < Q; ++j) acc[i][j] = 0.f;
+      for (int j = 0; j < Q / 2; ++j) acc[i][j] = 0ull;
     if (kb1 > kb0) {
       load(kb0);
       stage(0);
@@ -166,16 +173,17 @@ __global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(const __grid_consta
         const float* SB = SA + KT * PITCH;
 #pragma unroll
         for (int k = 0; k < KT; ++k) {
-          float a[Q], b[Q];
+          const float4 a = *reinterpret_cast<const float4*>(SA + k * PITCH + 4 * ty);
+          const uint64_t a2[4] = {pack2(a.x, a.x), pack2(a.y, a.y), pack2(a.z, a.z), pack2(a.w, a.w)};
 #pragma unroll
           for (int h = 0; h < Q / 4; ++h) {
-            *reinterpret_cast<float4*>(a + 4 * h) = *reinterpret_cast<const float4*>(SA + k * PITCH + 32 * h + 4 * ty);
-            *reinterpret_cast<float4*>(b + 4 * h) = *reinterpret_cast<const float4*>(SB + k * PITCH + 32 * h + 4 * tx);
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(SB + k * PITCH + 32 * h + 4 * tx);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              fma2(acc[i][2 * h], a2[i], b.x);
+              fma2(acc[i][2 * h + 1], a2[i], b.y);
+            }
           }
-#pragma unroll
-          for (int i = 0; i < Q; ++i)
-#pragma unroll
-            for (int j = 0; j < Q; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
         }
         if (more) stage(buf ^ 1);
         __syncthreads();
@@ -183,11 +191,10 @@ __global__ void __launch_bounds__(CC_THREADS) gemm_cc_kernel(const __grid_consta
     }
     if (live) {
 #pragma unroll
-      for (int i = 0; i < Q; ++i)
+      for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int h = 0; h < Q / 4; ++h)
-          *reinterpret_cast<float4*>(sm + (32 * (i / 4) + 4 * ty + i % 4) * PITCH + 32 * h + 4 * tx) =
-              make_float4(acc[i][4 * h], acc[i][4 * h + 1], acc[i][4 * h + 2], acc[i][4 * h + 3]);
+          *reinterpret_cast<ulonglong2*>(sm + (4 * ty + i) * PITCH + 32 * h + 4 * tx) = make_ulonglong2(acc[i][2 * h], acc[i][2 * h + 1]);
     }
     if (s.S > 1) cluster_sync_all();  // the partial tiles of the group are complete
     else __syncthreads();
@@ -313,19 +320,26 @@ void launch_one(const ard_ctx* ctx, const GemmArgs& g, int ts, cudaStream_t s) {
   CcParams p = {};
   p.g = g;
   p.ts = ts;
-  p.want = 4 * ctx->sm_count;
   const uintptr_t four = 4 * sizeof(T) - 1;
   p.vec = ((reinterpret_cast<uintptr_t>(g.A0) & four) == 0 && g.lda0 % 4 == 0 ? 1 : 0) |
           ((reinterpret_cast<uintptr_t>(g.A1) & four) == 0 && g.lda1 % 4 == 0 ? 2 : 0);
   const int M = OP == OP_BWD_WEIGHT ? g.N : g.B, N = OP == OP_FWD ? g.N : g.K;
   const double flops = 2.0 * g.B * g.K * g.N;
   // The grid covers the tiles of the densest pattern, cut or not; CTAs without work read the header and leave.
-  auto grid = [&](int R) {
-    const int n = min(16 * ctx->sm_count, max(p.want, cdiv(M, R) * cdiv(N, R)));
-    return dim3(cdiv(n, SP_CLUSTER) * SP_CLUSTER);
+  auto launch = [&](auto kern, int R, int KT) {
+    p.want = 4 * ctx->sm_count;
+    const int tiles = cdiv(M, R) * cdiv(N, R);
+    int n = min(16 * ctx->sm_count, max(p.want, tiles));
+    if (KIND == 0) {  // no pattern cuts a tile into more shares than its longest contraction allows
+      const int nkb = cdiv(OP == OP_FWD ? g.K : (OP == OP_BWD_DATA ? g.N : g.B), KT);
+      int S = SP_CLUSTER;
+      while (S > 1 && nkb < 2 * S) S >>= 1;
+      n = min(n, tiles * S);
+    }
+    (void)ard_launch_cluster(ctx, kern, SP_CLUSTER, dim3(cdiv(n, SP_CLUSTER) * SP_CLUSTER), dim3(cc_threads(R)), 0, s, p);
   };
-  if (flops > CC_WIDE_FLOPS) (void)ard_launch_cluster(ctx, gemm_cc_kernel<T, KIND, OP, 64>, SP_CLUSTER, grid(64), dim3(CC_THREADS), 0, s, p);
-  else (void)ard_launch_cluster(ctx, gemm_cc_kernel<T, KIND, OP, 32>, SP_CLUSTER, grid(32), dim3(CC_THREADS), 0, s, p);
+  if (flops > CC_WIDE_FLOPS) launch(gemm_cc_kernel<T, KIND, OP, 64>, 64, 16);
+  else launch(gemm_cc_kernel<T, KIND, OP, 32>, 32, 32);
 }  // errors: cudaGetLastError
 
 template <typename T>
