@@ -387,7 +387,14 @@ ard_status launch_gemm_ldg(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArg
   // 128 x 128 tiles once they fill the device without cutting the contraction, else 128 x 64
   const int M = op == OP_BWD_WEIGHT ? g.N : g.B, N = op == OP_FWD ? g.N : g.K;
   const bool wide = cdiv(M, UMMA_BM) * cdiv(N, 128) >= ctx->sm_count;
-  const int ctas = 2 * ctx->sm_count / SP_CLUSTER * SP_CLUSTER;
+  int ctas = 2 * ctx->sm_count / SP_CLUSTER * SP_CLUSTER;
+  if (kind == ARD_ROW) {  // no more than the densest pattern's tiles, cut as often as its contraction allows
+    const int nkb = cdiv(op == OP_FWD ? g.K : (op == OP_BWD_DATA ? g.N : g.B), LG_BK);
+    int S = SP_CLUSTER;
+    while (S > 1 && nkb < 2 * S) S >>= 1;
+    const int n = cdiv(M, UMMA_BM) * cdiv(N, wide ? 128 : 64) * S;
+    if (n < ctas) ctas = cdiv(n, SP_CLUSTER) * SP_CLUSTER;
+  }
   const bool on8 = ((reinterpret_cast<uintptr_t>(g.A0) | reinterpret_cast<uintptr_t>(g.A1)) & 7u) == 0 && g.lda0 % 4 == 0 && g.lda1 % 4 == 0;
 #define ARD_LDG(KIND_, OP_, AL_) \
   return wide ? launch_ldg<KIND_, OP_, 128, AL_>(ctx, p, ctas, s) : launch_ldg<KIND_, OP_, 64, AL_>(ctx, p, ctas, s)

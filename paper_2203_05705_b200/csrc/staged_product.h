@@ -174,6 +174,9 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
     }
     __syncwarp();
   }
+  const int es = g.out_is_f32 ? 4 : 2;
+  const bool vec = !g.accumulate && (reinterpret_cast<uintptr_t>(g.out) & (uintptr_t)(4 * es - 1)) == 0 && (g.ldo & 3) == 0 &&
+                   (KIND == 0 || (s.ts & 3) == 0);
   auto put = [&](size_t off, float val) {
     if (g.out_is_f32) {
       float* o = reinterpret_cast<float*>(g.out) + off;
@@ -183,65 +186,95 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
       *o = __float2bfloat16_rn(g.accumulate ? __bfloat162float(*o) + val : val);
     }
   };
-  for (int r = r0 + warp; r < r0 + rows_per; r += NW) {
-    const int m = ti.m0 + r;
+  // v, the first nv of them, to four consecutive elements; off is a multiple of four
+  auto put4 = [&](size_t off, const float (&v)[4], int nv) {
+    if (vec && nv >= 4) {
+      if (g.out_is_f32) {
+        *reinterpret_cast<float4*>(reinterpret_cast<float*>(g.out) + off) = make_float4(v[0], v[1], v[2], v[3]);
+      } else {
+        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(g.out) + off) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+      }
+      return;
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (i < nv) put(off + i, v[i]);
+  };
+  // compact column j of the tile: bias, then the activation, then the rescale (Sec. 3.2)
+  auto fwd_value = [&](const float* row, int j) {
+    float z = row[j];
+    if (g.bias != nullptr) z += g.bias[s.bb + (ti.n0 + j) * s.dp];
+    if (g.relu) z = fmaxf(z, 0.f);
+    return z * g.alpha;
+  };
+  if (KIND == 0 && OP == OP_FWD && g.flag0 == ARD_OUT_SCATTER_ZEROFILL && s.dp > 1) {
+    // output columns [n0 * dp, (n0 + BN) * dp), the last tile up to N: kept ones and the zeros between
+    const int lo = ti.n0 * s.dp, hi = ti.n0 + BN >= s.N ? g.N : (ti.n0 + BN) * s.dp;
+    for (int r = r0 + warp; r < r0 + rows_per && ti.m0 + r < s.M; r += NW) {
+      const float* row = T + r * PITCH;
+      const size_t base = (size_t)(ti.m0 + r) * g.ldo;
+      for (int c = lo + 4 * lane; c < hi; c += 128) {
+        const int rel = c - s.bb;
+        int j = rel <= 0 ? 0 : (rel + s.dp - 1) / s.dp;  // first kept column at or after c
+        int at = s.bb + j * s.dp - c;
+        float v[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          v[i] = 0.f;
+          if (i == at) {
+            if (j < s.n_keep) v[i] = fwd_value(row, j - ti.n0);
+            ++j;
+            at += s.dp;
+          }
+        }
+        put4(base + c, v, hi - c);
+      }
+    }
+    return;
+  }
+  // Four consecutive columns per lane.
+  constexpr int QR = BN / 4;
+  const int col_lim = KIND == 0 ? s.N : (OP == OP_BWD_WEIGHT ? ti.len : ti.cnt) * s.ts;
+  const int row_lim = KIND == 1 && OP == OP_BWD_WEIGHT ? ti.cnt * s.ts : s.M;
+  for (int e = lane; e < rows_per / NW * QR; e += 32) {
+    const int r = r0 + warp + NW * (e / QR), j0 = 4 * (e % QR);
+    const int m = ti.m0 + r, n = ti.n0 + j0, nv = col_lim - n;
+    if (m >= row_lim || nv <= 0) continue;
     const float* row = T + r * PITCH;
-    if (KIND == 0) {
-      if (m >= s.M) break;
-      auto fwd_value = [&](int j) {  // compact column j of the tile: bias, then the activation, then the rescale (Sec. 3.2)
-        float z = row[j];
-        if (g.bias != nullptr) z += g.bias[s.bb + (ti.n0 + j) * s.dp];
-        if (g.relu) z = fmaxf(z, 0.f);
-        return z * g.alpha;
-      };
-      if (OP == OP_FWD && g.flag0 == ARD_OUT_SCATTER_ZEROFILL) {
-        // output columns [n0 * dp, (n0 + BN) * dp), the last tile up to N: kept ones and the zeros between
-        const int lo = ti.n0 * s.dp, hi = ti.n0 + BN >= s.N ? g.N : (ti.n0 + BN) * s.dp;
-        for (int col = lo + lane; col < hi; col += 32) {
-          const int rel = col - s.bb, j = rel >= 0 ? rel / s.dp : -1;
-          const bool kept = j >= 0 && j * s.dp == rel && j < s.n_keep;
-          put((size_t)m * g.ldo + col, kept ? fwd_value(j - ti.n0) : 0.f);
-        }
-        continue;
-      }
-      const size_t orow = OP == OP_BWD_WEIGHT && g.hdr_in == nullptr ? (size_t)s.bb + (size_t)m * s.dp : (size_t)m;
+    float v[4];
+    const float4 x = *reinterpret_cast<const float4*>(row + j0);
+    v[0] = x.x * g.alpha; v[1] = x.y * g.alpha; v[2] = x.z * g.alpha; v[3] = x.w * g.alpha;
+    if (KIND == 0 && OP == OP_FWD && (g.bias != nullptr || g.relu)) {
 #pragma unroll
-      for (int j0 = 0; j0 < BN; j0 += 32) {
-        const int j = j0 + lane, n = ti.n0 + j;
-        if (n >= s.N) continue;
-        float val;
-        if (OP == OP_FWD) {
-          val = fwd_value(j);
-        } else {
-          val = row[j] * g.alpha;
-          // adjoint of the producing layer's ReLU: nothing flows where its output was not positive
-          if (OP == OP_BWD_DATA && g.act != nullptr && !((float)reinterpret_cast<const T_*>(g.act)[(size_t)m * g.ldact + n] > 0.f)) val = 0.f;
-        }
-        put(orow * g.ldo + n, val);
-      }
-      if (OP == OP_BWD_WEIGHT && g.flag1) {
-        // compact row m owns output rows [m * dp, (m + 1) * dp), the last one the tail: zeros but for its own
-        const long long first = (long long)m * s.dp;
-        const long long last = m == s.M - 1 ? g.N : min((long long)g.N, first + s.dp);
-        for (long long z = first; z < last; ++z)
-          if (z != (long long)orow)
-            for (int n = ti.n0 + lane; n < min(ti.n0 + BN, s.N); n += 32) put((size_t)z * g.ldo + n, 0.f);
-      }
+      for (int i = 0; i < 4; ++i)
+        if (i < nv) v[i] = fwd_value(row, j0 + i);
+    }
+    if (KIND == 0 && OP == OP_BWD_DATA && g.act != nullptr) {
+      // adjoint of the producing layer's ReLU: nothing flows where its output was not positive
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (i < nv && !((float)reinterpret_cast<const T_*>(g.act)[(size_t)m * g.ldact + n + i] > 0.f)) v[i] = 0.f;
+    }
+    size_t orow = m;
+    if (KIND == 0 && OP == OP_BWD_WEIGHT && g.hdr_in == nullptr) orow = (size_t)s.bb + (size_t)m * s.dp;
+    if (KIND == 1 && OP == OP_BWD_WEIGHT) orow = (size_t)ti.class_pos(s, m);
+    auto pos = [&](int i) { return KIND == 0 ? i : (OP == OP_BWD_WEIGHT ? ti.list_pos(s, i) : ti.class_pos(s, i)); };
+    if (KIND == 0 || (s.ts & 3) == 0) {
+      put4(orow * g.ldo + pos(n), v, nv);
     } else {
-      size_t orow = m;
-      if (OP == OP_BWD_WEIGHT) {
-        if (m >= ti.cnt * s.ts) break;
-        orow = (size_t)ti.class_pos(s, m);
-      } else if (m >= s.M) {
-        break;
-      }
-      const int next = (OP == OP_BWD_WEIGHT ? ti.len : ti.cnt) * s.ts;
 #pragma unroll
-      for (int j0 = 0; j0 < BN; j0 += 32) {
-        const int j = j0 + lane, n = ti.n0 + j;
-        if (n >= next) continue;
-        put(orow * g.ldo + (size_t)(OP == OP_BWD_WEIGHT ? ti.list_pos(s, n) : ti.class_pos(s, n)), row[j] * g.alpha);
-      }
+      for (int i = 0; i < 4; ++i)
+        if (i < nv) put(orow * g.ldo + pos(n + i), v[i]);
+    }
+    if (KIND == 0 && OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1) {
+      // compact row m owns output rows [m * dp, (m + 1) * dp), the last one the tail: zeros but for its own
+      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+      const long long first = (long long)m * s.dp;
+      const long long last = m == s.M - 1 ? g.N : min((long long)g.N, first + s.dp);
+      for (long long z = first; z < last; ++z)
+        if (z != (long long)orow) put4((size_t)z * g.ldo + n, zero, nv);
     }
   }
 }
