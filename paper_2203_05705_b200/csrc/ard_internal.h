@@ -365,6 +365,28 @@ inline cudaError_t ard_launch_cluster(const ard_ctx* ctx, void (*kern)(P...), in
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 
+// CTAs in clusters of `cl` that the occupancy query places at once (one cluster where it fails).
+template <typename K>
+inline int ard_cluster_room(const ard_ctx* ctx, K kern, int cl, int threads, int smem) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(ctx->sm_count / cl * cl);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n < 1) {
+    (void)cudaGetLastError();
+    n = 1;
+  }
+  return n * cl;
+}
+
 #define ARD_CUDA_OK(expr)                       \
   do {                                          \
     cudaError_t e__ = (expr);                   \

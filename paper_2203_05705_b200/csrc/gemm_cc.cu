@@ -36,6 +36,7 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16* p) {
 }
 
 __host__ __device__ constexpr int cc_threads(int R) { return R == 64 ? 128 : 64; }
+constexpr int CC_CLUSTER = 8;
 constexpr double CC_WIDE_FLOPS = 2e8;  // 64 x 64 tiles from here on, see launch_one
 struct CcParams {
   GemmArgs g;
@@ -71,11 +72,11 @@ __global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_con
   pdl_wait_prior_grids();
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, tx = tid & 7, ty = tid >> 3;
-  const ProductPlan s = make_plan<KIND, OP, R, R, KT>(g, p.ts, p.want);
+  const ProductPlan s = make_plan<KIND, OP, R, R, KT>(g, p.ts, p.want, CC_CLUSTER);
   const int rank = (int)cluster_ctarank();
   const int part = rank & (s.S - 1), lead = rank - part;
-  const int group = rank / s.S, groups = SP_CLUSTER / s.S;
-  const int n_cl = (int)gridDim.x / SP_CLUSTER, units = (s.tiles + groups - 1) / groups;
+  const int group = rank / s.S, groups = CC_CLUSTER / s.S;
+  const int n_cl = (int)gridDim.x / CC_CLUSTER, units = (s.tiles + groups - 1) / groups;
   const T* PA = reinterpret_cast<const T*>(g.A0);
   const T* PB = reinterpret_cast<const T*>(g.A1);
   // Kept neurons are bb + i * dp: columns of a full-width dY, rows of the weight (unless packed for a feeding pattern).
@@ -87,7 +88,7 @@ __global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_con
   const bool whole = KIND == 0 || (p.ts & 3) == 0;  // four consecutive positions never leave a pattern tile
   const bool vec_a = (p.vec & 1) && step_a == 1 && whole, vec_b = (p.vec & 2) && whole;
 
-  for (int u = (int)blockIdx.x / SP_CLUSTER; u < units; u += n_cl) {
+  for (int u = (int)blockIdx.x / CC_CLUSTER; u < units; u += n_cl) {
     const int t = u * groups + group;
     ProductTile ti = {};
     ti.nkb = -1;
@@ -327,16 +328,16 @@ void launch_one(const ard_ctx* ctx, const GemmArgs& g, int ts, cudaStream_t s) {
   const double flops = 2.0 * g.B * g.K * g.N;
   // The grid covers the tiles of the densest pattern, cut or not; CTAs without work read the header and leave.
   auto launch = [&](auto kern, int R, int KT) {
-    p.want = 4 * ctx->sm_count;
     const int tiles = cdiv(M, R) * cdiv(N, R);
+    p.want = 4 * ctx->sm_count;
     int n = min(16 * ctx->sm_count, max(p.want, tiles));
     if (KIND == 0) {  // no pattern cuts a tile into more shares than its longest contraction allows
       const int nkb = cdiv(OP == OP_FWD ? g.K : (OP == OP_BWD_DATA ? g.N : g.B), KT);
-      int S = SP_CLUSTER;
+      int S = CC_CLUSTER;
       while (S > 1 && nkb < 2 * S) S >>= 1;
       n = min(n, tiles * S);
     }
-    (void)ard_launch_cluster(ctx, kern, SP_CLUSTER, dim3(cdiv(n, SP_CLUSTER) * SP_CLUSTER), dim3(cc_threads(R)), 0, s, p);
+    (void)ard_launch_cluster(ctx, kern, CC_CLUSTER, dim3(cdiv(n, CC_CLUSTER) * CC_CLUSTER), dim3(cc_threads(R)), 0, s, p);
   };
   if (flops > CC_WIDE_FLOPS) launch(gemm_cc_kernel<T, KIND, OP, 64>, 64, 16);
   else launch(gemm_cc_kernel<T, KIND, OP, 32>, 32, 32);

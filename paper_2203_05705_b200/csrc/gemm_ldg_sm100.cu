@@ -2,16 +2,17 @@
 // memory): rows that do not start on 16-byte boundaries (a fan-in of 1500, an odd width), periods beyond the
 // TMA kernels' table, and pattern tiles narrower than the 64 columns of a swizzle row (the paper's 32 x 32 tiles).
 //
-// The CTA's own threads stage the operands: eight warps read 16-byte pieces of the operand rows into registers and
-// store them into the 128-byte-swizzled layout that tcgen05.mma reads, a ninth warp issues the products.  Rows on the
-// 8-byte grid are read in 8-byte pieces; a row that starts anywhere else is read as the aligned 16-byte units that
-// cover it and shifted into place with one exchange between neighbouring lanes.
+// The CTA's own threads stage the operands in the 128-byte-swizzled layout that tcgen05.mma reads, a ninth warp issues
+// the products.  Rows on the 4-, 8- or 16-byte grid are copied with asynchronous copies of that size, several blocks
+// ahead.  An odd width puts every second row between two elements of that grid: such rows are read into registers as
+// the aligned 16-byte units that cover them, one block ahead, and shifted into place with one exchange between
+// neighbouring lanes.
 // Tiling, cut contractions and the rows' way out: staged_product.h.
 //
-// Bound: latency of the staging loads (registers hold one 64-deep block per CTA, two CTAs share an SM); the tensor
+// Bound: the load unit and the latency of its copies (two CTAs share an SM); the tensor
 // pipe is nearly idle.  Three products of a layer, against the CUDA-core kernel that took these shapes before:
-// 700 x 1500 x 1500 under a row pattern of period 2 463 -> 93 us, 128 x 2048 x 2048 under 32 x 32 tiles of period 2
-// 519 -> 55 us.
+// 700 x 1500 x 1500 under a row pattern of period 2 463 -> 73 us, 128 x 2048 x 2048 under 32 x 32 tiles of period 2
+// 519 -> 51 us.
 #include "staged_product.h"
 
 namespace {
@@ -19,20 +20,21 @@ namespace {
 constexpr int LG_LOADERS = 256;             // warps 0..7: loads, then the epilogue
 constexpr int LG_THREADS = LG_LOADERS + 32; // warp 8: tensor memory, products
 constexpr int LG_BK = 64;
-constexpr int LG_STAGES = 3;
 
 struct LdgParams {
   GemmArgs g;
   int ts;
+  int cl;  // CTAs per cluster
 };
 
 template <int BN>
 struct LdgSmem {
+  static constexpr int STAGES = BN == 64 ? 4 : 3;
   static constexpr int A_BYTES = UMMA_BM * LG_BK * 2;
   static constexpr int B_BYTES = BN * LG_BK * 2;
   static constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
   static constexpr int PITCH = BN + 4;  // words per row of the fp32 tile (overlays the stages between two tiles)
-  static constexpr int BAR_OFF = LG_STAGES * STAGE_BYTES;
+  static constexpr int BAR_OFF = STAGES * STAGE_BYTES;
   static constexpr int TOTAL = BAR_OFF + 128 + 1024;
   static_assert(UMMA_BM * PITCH * 4 <= BAR_OFF, "the fp32 tile overlays the operand stages");
 };
@@ -45,13 +47,11 @@ __device__ __forceinline__ uint4 ldg16(uintptr_t a, bool pred) {
       : "=&r"(v.x), "=&r"(v.y), "=&r"(v.z), "=&r"(v.w) : "l"(a), "r"((int)pred));
   return v;
 }
-__device__ __forceinline__ uint2 ldg8(uintptr_t a, bool pred) {
-  uint2 v;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.b32 %0, 0;\n\tmov.b32 %1, 0;\n\t"
-      "@p ld.global.v2.u32 {%0, %1}, [%2];\n\t}"
-      : "=&r"(v.x), "=&r"(v.y) : "l"(a), "r"((int)pred));
-  return v;
+// AL bytes global -> shared, those beyond `bytes` zero (0: nothing is read)
+template <int AL>
+__device__ __forceinline__ void copy_async(uint32_t dst, uintptr_t src, int bytes) {
+  if (AL == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
+  else asm volatile("cp.async.ca.shared.global [%0], [%1], %3, %2;" ::"r"(dst), "l"(src), "r"(bytes), "n"(AL) : "memory");
 }
 __device__ __forceinline__ void sts16(uint32_t a, const uint4& v) {
   asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
@@ -78,10 +78,12 @@ __device__ __forceinline__ uint4 keep_first(uint4 v, int nv) {
 }
 
 // KIND: 0 row pattern, 1 tile pattern (ts a power of two from 8 to 64).  AL: every operand row starts on the AL-byte
-// grid (16 for tile patterns, 8 or 2 for row patterns).
+// grid (16 for tile patterns; 16, 8, 4 or 2 for row patterns).
 template <int KIND, int OP, int BN, int AL>
 __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_constant__ LdgParams p) {
   using L = LdgSmem<BN>;
+  constexpr int LG_STAGES = L::STAGES;
+  constexpr bool ASYNC = AL >= 4;
   constexpr bool A_MN = OP == OP_BWD_WEIGHT, B_MN = OP != OP_FWD;
   constexpr int NA = 4, NB = BN / 32;  // 16-byte pieces per loading thread and block, A and B
   const GemmArgs& g = p.g;
@@ -94,14 +96,14 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
   auto full_bar = [&](int s) { return bars + 8u * s; };
   auto empty_bar = [&](int s) { return bars + 8u * (LG_STAGES + s); };
   const uint32_t done_bar = bars + 8u * (2 * LG_STAGES);
-  volatile uint32_t* tmem_ptr = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 64);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::BAR_OFF + 68);
+  volatile uint32_t* tmem_ptr = reinterpret_cast<volatile uint32_t*>(smem + L::BAR_OFF + 96);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + L::BAR_OFF + 100);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_launch_dependents();
   if (tid == 0) {
     for (int s = 0; s < LG_STAGES; ++s) {
-      mbar_init(full_bar(s), LG_LOADERS / 32);
+      mbar_init(full_bar(s), ASYNC ? LG_LOADERS : LG_LOADERS / 32);
       mbar_init(empty_bar(s), 1);
     }
     mbar_init(done_bar, 1);
@@ -118,17 +120,17 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
   const uint32_t tmem = *tmem_ptr;
   pdl_wait_prior_grids();
 
-  const ProductPlan s = make_plan<KIND, OP, UMMA_BM, BN, LG_BK>(g, p.ts, (int)gridDim.x);
+  const ProductPlan s = make_plan<KIND, OP, UMMA_BM, BN, LG_BK>(g, p.ts, (int)gridDim.x, p.cl);
   const int rank = (int)cluster_ctarank();
   const int part = rank & (s.S - 1);          // this CTA's share of the contraction
   const int lead = rank - part;               // first CTA of the tile's group
-  const int group = rank / s.S, groups = SP_CLUSTER / s.S;
-  const int n_cl = (int)gridDim.x / SP_CLUSTER, units = (s.tiles + groups - 1) / groups;
+  const int group = rank / s.S, groups = p.cl / s.S;
+  const int n_cl = (int)gridDim.x / p.cl, units = (s.tiles + groups - 1) / groups;
   int blk = 0;        // blocks staged so far: stage = blk % STAGES
   int done = 0;       // accumulators finished so far
   bool ok = true;
 
-  for (int u = (int)blockIdx.x / SP_CLUSTER; u < units; u += n_cl) {
+  for (int u = (int)blockIdx.x / p.cl; u < units; u += n_cl) {
     const int t = u * groups + group;
     ProductTile ti = {};
     ti.nkb = -1;
@@ -147,6 +149,7 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
         for (int kb = kb0; kb < kb1; ++kb) {
           const int it = blk + kb - kb0, st = it % LG_STAGES;
           if (!mbar_wait(full_bar(st), (uint32_t)(it / LG_STAGES) & 1u, abort_flag, g.status)) { ok = false; break; }
+          if (ASYNC) fence_proxy_async_smem();  // the copies were made in the generic proxy
           tc_fence_after();
           const uint32_t sA = base + st * L::STAGE_BYTES;
           const uint64_t ad0 = desc_a | (uint64_t)((sA & 0x3FFFFu) >> 4);
@@ -224,8 +227,25 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
         const size_t kp = k < ti.kext ? (size_t)ti.list_pos(s, k) : 0;
         return ptr[j] + (mn ? kp * (size_t)g.lda1 : kp) * 2;
       };
-      // Loads of block kb.  A row on the 8-byte grid (AL == 8) is read in 8-byte pieces.  Any other is read in the
-      // aligned 16-byte units that cover it: each lane the unit of its piece's first byte, and the unit after
+      // K-major: row 32 jj + rsub; MN-major: box jj / 2 (8 KiB each), row 32 (jj & 1) + rsub: the same offset
+      auto place = [&](int j, uint32_t sA) {
+        const int row = (j < NA ? j : j - NA) * 32 + rsub;
+        return sA + (j < NA ? 0u : (uint32_t)L::A_BYTES) + (uint32_t)row * 128u + (uint32_t)((c ^ (row & 7)) << 4);
+      };
+      auto copy = [&](int kb, uint32_t sA) {
+#pragma unroll
+        for (int j = 0; j < NA + NB; ++j) {
+          const int bytes = 2 * max(0, exists(j, kb, c));
+          const uintptr_t a = bytes > 0 ? address(j, kb) : reinterpret_cast<uintptr_t>(j < NA ? g.A0 : g.A1);
+          const uint32_t d = place(j, sA);
+#pragma unroll
+          for (int o = 0; o < 16; o += AL) {
+            const int b = min(AL, max(0, bytes - o));
+            copy_async<AL>(d + o, b > 0 ? a + o : a, b);
+          }
+        }
+      };
+      // AL == 2: loads of block kb in the aligned 16-byte units that cover the row: each lane the unit of its piece's first byte, and the unit after
       // the row's last piece is fetched by lane j of the row's eight lanes for the j-th row (x).  A unit is read only if it holds
       // an element that exists, so no load leaves the 16-byte unit of such an element.
       auto issue = [&](int kb) {
@@ -233,20 +253,13 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
         for (int j = 0; j < NA + NB; ++j) {
           const int nv = exists(j, kb, c);
           const uintptr_t a = address(j, kb);
-          if (KIND == 1) {
-            v[j] = ldg16(a, nv > 0);
-          } else if (AL == 8) {
-            const uint2 lo = ldg8(a, nv > 0), hi = ldg8(a + 8, nv > 4);
-            v[j] = make_uint4(lo.x, lo.y, hi.x, hi.y);
-          } else {
-            // also when only the piece before it (same row) reaches into this unit
-            const int sh = (int)(a & 15u);
-            const int prev = exists(j, kb, c - 1);
-            const bool before = c > 0 && sh != 0 && prev > 0 && 2 * prev > 16 - sh;
-            v[j] = ldg16(a & ~(uintptr_t)15, nv > 0 || before);
-          }
+          // also when only the piece before it (same row) reaches into this unit
+          const int sh = (int)(a & 15u);
+          const int prev = exists(j, kb, c - 1);
+          const bool before = c > 0 && sh != 0 && prev > 0 && 2 * prev > 16 - sh;
+          v[j] = ldg16(a & ~(uintptr_t)15, nv > 0 || before);
         }
-        if (KIND == 0 && AL == 2) {
+        {
           // the j-th row's end: this lane stands in for piece 7 of row group j = c
           uintptr_t a = 0;
           int nv = 0;
@@ -264,31 +277,30 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
       auto store = [&](int kb, uint32_t sA) {
 #pragma unroll
         for (int j = 0; j < NA + NB; ++j) {
-          uint4 w = v[j];
-          if (KIND == 0) {
-            if (AL == 2) {
-              const int sh = (int)(address(j, kb) & 15u);
-              uint4 hi, e;
-              hi.x = __shfl_down_sync(0xffffffffu, v[j].x, 1, 8);
-              hi.y = __shfl_down_sync(0xffffffffu, v[j].y, 1, 8);
-              hi.z = __shfl_down_sync(0xffffffffu, v[j].z, 1, 8);
-              hi.w = __shfl_down_sync(0xffffffffu, v[j].w, 1, 8);
-              e.x = __shfl_sync(0xffffffffu, x.x, j, 8);
-              e.y = __shfl_sync(0xffffffffu, x.y, j, 8);
-              e.z = __shfl_sync(0xffffffffu, x.z, j, 8);
-              e.w = __shfl_sync(0xffffffffu, x.w, j, 8);
-              if (c == 7) hi = e;
-              w = shift_pair(v[j], hi, sh);
-            }
-            w = keep_first(w, exists(j, kb, c));
-          }
-          const bool isA = j < NA;
-          // K-major: row 32 jj + rsub; MN-major: box jj / 2 (8 KiB each), row 32 (jj & 1) + rsub: the same offset
-          const int row = (isA ? j : j - NA) * 32 + rsub;
-          sts16(sA + (isA ? 0u : (uint32_t)L::A_BYTES) + (uint32_t)row * 128u + (uint32_t)((c ^ (row & 7)) << 4), w);
+          const int sh = (int)(address(j, kb) & 15u);
+          uint4 hi, e;
+          hi.x = __shfl_down_sync(0xffffffffu, v[j].x, 1, 8);
+          hi.y = __shfl_down_sync(0xffffffffu, v[j].y, 1, 8);
+          hi.z = __shfl_down_sync(0xffffffffu, v[j].z, 1, 8);
+          hi.w = __shfl_down_sync(0xffffffffu, v[j].w, 1, 8);
+          e.x = __shfl_sync(0xffffffffu, x.x, j, 8);
+          e.y = __shfl_sync(0xffffffffu, x.y, j, 8);
+          e.z = __shfl_sync(0xffffffffu, x.z, j, 8);
+          e.w = __shfl_sync(0xffffffffu, x.w, j, 8);
+          if (c == 7) hi = e;
+          sts16(place(j, sA), keep_first(shift_pair(v[j], hi, sh), exists(j, kb, c)));
         }
       };
-      if (has_acc && ok) {
+      if (has_acc && ok && ASYNC) {
+        for (int kb = kb0; kb < kb1; ++kb) {
+          const int it = blk + kb - kb0, st = it % LG_STAGES;
+          if (!mbar_wait(empty_bar(st), ((uint32_t)(it / LG_STAGES) & 1u) ^ 1u, abort_flag, g.status)) ok = false;
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          copy(kb, base + st * L::STAGE_BYTES);
+          cp_async_mbar_arrive_noinc(full_bar(st));
+        }
+      } else if (has_acc && ok) {
         issue(kb0);
         for (int kb = kb0; kb < kb1; ++kb) {
           const int it = blk + kb - kb0, st = it % LG_STAGES;
@@ -355,7 +367,7 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
 }
 
 template <int KIND, int OP, int BN, int AL>
-ard_status launch_ldg(ard_ctx* ctx, const LdgParams& p, int ctas, cudaStream_t s) {
+ard_status launch_ldg(ard_ctx* ctx, LdgParams p, int M, int N, int nkb, cudaStream_t s) {
   auto kern = gemm_ldg_kernel<KIND, OP, BN, AL>;
   static bool attr_done[64] = {};
   const int dev = ctx->device & 63;
@@ -363,7 +375,23 @@ ard_status launch_ldg(ard_ctx* ctx, const LdgParams& p, int ctas, cudaStream_t s
     ARD_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LdgSmem<BN>::TOTAL));
     attr_done[dev] = true;
   }
-  ARD_CUDA_OK(ard_launch_cluster(ctx, kern, SP_CLUSTER, dim3(ctas), dim3(LG_THREADS), LdgSmem<BN>::TOTAL, s, p));
+  const int tiles = (M + UMMA_BM - 1) / UMMA_BM * ((N + BN - 1) / BN);
+  // A cluster lives inside one GPC, and what is left of a GPC behind the last whole cluster stays empty: of two CTAs per SM
+  // this GPU holds 37 clusters of 8 by count but 30 at once (15 by the occupancy query, which counts on one CTA per SM
+  // for a kernel that allocates tensor memory), and a grid of 37 ran in two waves.  Hence a grid of what fits at once,
+  // in clusters of 8 only where even eight shares of every tile find a place, else of 4.
+  p.cl = tiles * 8 <= 2 * ctx->sm_count ? 8 : 4;
+  static int room[2][64] = {};
+  int& r = room[p.cl == 8][dev];
+  if (r == 0) r = 2 * ard_cluster_room(ctx, kern, p.cl, LG_THREADS, LdgSmem<BN>::TOTAL);
+  int ctas = r;
+  if (KIND == 0) {  // no more than the densest pattern's tiles, cut as often as its contraction allows
+    int S = p.cl;
+    while (S > 1 && nkb < 2 * S) S >>= 1;
+    const int n = (tiles * S + p.cl - 1) / p.cl * p.cl;
+    if (n < ctas) ctas = n;
+  }
+  ARD_CUDA_OK(ard_launch_cluster(ctx, kern, p.cl, dim3(ctas), dim3(LG_THREADS), LdgSmem<BN>::TOTAL, s, p));
   ctx->launches++;
   ARD_CUDA_OK(cudaGetLastError());
   return ARD_OK;
@@ -387,21 +415,16 @@ ard_status launch_gemm_ldg(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArg
   // 128 x 128 tiles once they fill the device without cutting the contraction, else 128 x 64
   const int M = op == OP_BWD_WEIGHT ? g.N : g.B, N = op == OP_FWD ? g.N : g.K;
   const bool wide = cdiv(M, UMMA_BM) * cdiv(N, 128) >= ctx->sm_count;
-  int ctas = 2 * ctx->sm_count / SP_CLUSTER * SP_CLUSTER;
-  if (kind == ARD_ROW) {  // no more than the densest pattern's tiles, cut as often as its contraction allows
-    const int nkb = cdiv(op == OP_FWD ? g.K : (op == OP_BWD_DATA ? g.N : g.B), LG_BK);
-    int S = SP_CLUSTER;
-    while (S > 1 && nkb < 2 * S) S >>= 1;
-    const int n = cdiv(M, UMMA_BM) * cdiv(N, wide ? 128 : 64) * S;
-    if (n < ctas) ctas = cdiv(n, SP_CLUSTER) * SP_CLUSTER;
-  }
-  const bool on8 = ((reinterpret_cast<uintptr_t>(g.A0) | reinterpret_cast<uintptr_t>(g.A1)) & 7u) == 0 && g.lda0 % 4 == 0 && g.lda1 % 4 == 0;
+  const int nkb = cdiv(op == OP_FWD ? g.K : (op == OP_BWD_DATA ? g.N : g.B), LG_BK);
+  const uintptr_t grid = reinterpret_cast<uintptr_t>(g.A0) | reinterpret_cast<uintptr_t>(g.A1) | (uintptr_t)(2 * g.lda0) | (uintptr_t)(2 * g.lda1);
 #define ARD_LDG(KIND_, OP_, AL_) \
-  return wide ? launch_ldg<KIND_, OP_, 128, AL_>(ctx, p, ctas, s) : launch_ldg<KIND_, OP_, 64, AL_>(ctx, p, ctas, s)
+  return wide ? launch_ldg<KIND_, OP_, 128, AL_>(ctx, p, M, N, nkb, s) : launch_ldg<KIND_, OP_, 64, AL_>(ctx, p, M, N, nkb, s)
 #define ARD_LDG_ROW(OP_)             \
   do {                               \
-    if (on8) ARD_LDG(0, OP_, 8);     \
-    ARD_LDG(0, OP_, 2);              \
+    if (grid % 16 == 0) ARD_LDG(0, OP_, 16);  \
+    if (grid % 8 == 0) ARD_LDG(0, OP_, 8);    \
+    if (grid % 4 == 0) ARD_LDG(0, OP_, 4);    \
+    ARD_LDG(0, OP_, 2);                       \
   } while (0)
   if (kind == ARD_ROW) {
     if (op == OP_FWD) ARD_LDG_ROW(OP_FWD);

@@ -6,7 +6,7 @@
 // one kept list, and tile-rows with equal r mod dp / gcd(Tc mod dp, dp) another: the members of such a class side by
 // side are one dense product over their common list, whatever the size of a pattern tile.
 //
-// Work is dealt in clusters of SP_CLUSTER CTAs.  A product with fewer output tiles than the device has room for is cut
+// Work is dealt in clusters of 4 or 8 CTAs.  A product with fewer output tiles than the device has room for is cut
 // along its contraction over S = 2, 4 or 8 CTAs of a cluster; S follows from the sampled pattern.
 #pragma once
 
@@ -14,8 +14,6 @@
 #include "sm100_ptx.h"
 
 namespace {
-
-constexpr int SP_CLUSTER = 8;
 
 struct ProductPlan {
   int dp, bb, n_keep;
@@ -53,9 +51,9 @@ struct ProductTile {
 
 __device__ __forceinline__ int sp_cdiv(int a, int b) { return (a + b - 1) / b; }
 
-// want: CTAs the device has room for at once.
+// want: CTAs the device has room for at once; cl: CTAs per cluster.
 template <int KIND, int OP, int BM, int BN, int BK>
-__device__ __forceinline__ ProductPlan make_plan(const GemmArgs& g, int ts, int want) {
+__device__ __forceinline__ ProductPlan make_plan(const GemmArgs& g, int ts, int want, int cl) {
   ProductPlan s = {};
   s.dp = g.hdr[HDR_DP];
   s.bb = g.hdr[HDR_B] - 1;
@@ -103,7 +101,7 @@ __device__ __forceinline__ ProductPlan make_plan(const GemmArgs& g, int ts, int 
   }
   // Cut the contraction only while the pieces still find an idle place and hold at least two blocks: a cut costs
   // two cluster barriers and a pass of the partial tiles through shared memory.
-  s.S = SP_CLUSTER;
+  s.S = cl;
   while (s.S > 1 && (s.tiles * s.S > want || nkb < 2 * s.S)) s.S >>= 1;
   return s;
 }
