@@ -97,10 +97,10 @@ ard_status ard_set_path(ard_ctx* ctx, ard_path path);
  *                                 fits it (see ard_mlp_step); 0: always call by call
  *   ARD_OPT_LSTM_COMPACT_H [1]    the whole-sequence kernels of ard_lstm_forward / ard_lstm_backward contract over
  *                                 the kept units alone when the pattern drops any: forward over a compact copy of
- *                                 h_{t-1} in context scratch, BPTT (at most 256 kept units) with every block of
- *                                 dz_{t+1} in one CTA and one grid-wide barrier per step (0: forward over all H
- *                                 columns, the dropped ones being zero, BPTT always cut along the contraction
- *                                 with partial sums); same results up to the order of fp32 additions
+ *                                 h_{t-1} in context scratch, BPTT with whole contractions in every CTA where few
+ *                                 units are kept (0: forward over all H columns, the dropped ones being zero, BPTT's
+ *                                 contraction always shared by a cluster of CTAs); same results up to the order of
+ *                                 fp32 additions
  * Errors: ARD_ERR_INVALID_ARG (unknown option, negative value). */
 typedef enum { ARD_OPT_PDL = 0, ARD_OPT_PDL_IN_CAPTURE = 1, ARD_OPT_SIDE_STREAMS = 2, ARD_OPT_CTA_PAIRS = 3,
                ARD_OPT_BAND_ROWS = 4, ARD_OPT_MLP_PERSISTENT = 5, ARD_OPT_LSTM_COMPACT_H = 6 } ard_option;
@@ -598,9 +598,8 @@ ard_status ard_lstm_forward(ard_ctx* ctx, const ard_pattern* pat, int T, int B, 
  * dW [4H][I+H] fp32 receives the weight gradient (dropped units' rows zero).
  * When the layer fits (as for ard_lstm_forward) and
  * ard_set_lstm_persistent is on, the recurrence dh_{t-1} = upstream + dz_t W_h with the cell adjoint is ONE
- * cooperative kernel (weight slices resident in shared memory, dc in registers; one bounded grid-wide synchronisation
- * per step, or, where the gate gradients of a step are too many to stream through shared memory, two and partial sums,
- * see ARD_OPT_LSTM_COMPACT_H) and the x halves come from one product over all T*B rows; otherwise a loop
+ * cooperative kernel (weight slices resident in shared memory, dc in registers, one bounded grid-wide synchronisation
+ * per step) and the x halves come from one product over all T*B rows; otherwise a loop
  * in native code enqueues ard_lstm_gates_bwd and ard_lstm_gate_gemm_bwd per step.  In both cases the h
  * halves of D[1..T-1] are overwritten (kept units: the total gradient of h_{t-1}; dropped units:
  * unspecified), and the h half of D[0] is meaningful at kept units only. */
@@ -608,7 +607,7 @@ ard_status ard_lstm_backward(ard_ctx* ctx, const ard_pattern* pat, int T, int B,
                              const void* XH, const void* W, int ldw, const float* C, const float* G,
                              const float* dH_last, float* D, float* dc, void* DZ, float* dW, void* cuda_stream);
 /* The same with nothing prepared: dH [T][B][H] fp32 holds the upstream gradient of every h_t, no gradient arrives at
- * c_T, and D and dc are outputs only (contents as above). */
+ * c_T, and D and dc are outputs only: contents as above, the h halves of D[1..T-1] unspecified. */
 ard_status ard_lstm_backward_dh(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                 const void* XH, const void* W, int ldw, const float* C, const float* G, const float* dH,
                                 float* D, float* dc, void* DZ, float* dW, void* cuda_stream);

@@ -186,7 +186,6 @@ ard_status ard_create(ard_ctx** out, int device, size_t workspace_bytes) {
   ctx->use_pdl = 1;
   ctx->lstm_persistent = 1;
   ctx->d_grid_bar = nullptr;
-  ctx->d_lstm_partial = nullptr;
   ctx->d_lstm_hc = nullptr;
   ctx->lstm_compact_h = 1;
   ctx->pdl_in_capture = 1;
@@ -236,11 +235,9 @@ ard_status ard_create(ard_ctx** out, int device, size_t workspace_bytes) {
         cudaMalloc(reinterpret_cast<void**>(&ctx->d_tm_slots), tm_slots_bytes()) != cudaSuccess ||
         cudaMalloc(reinterpret_cast<void**>(&ctx->d_grid_bar), 256) != cudaSuccess ||
         cudaMemset(ctx->d_grid_bar, 0, 256) != cudaSuccess ||
-        cudaMalloc(reinterpret_cast<void**>(&ctx->d_lstm_partial), lstm_bwd_partial_bytes(ctx->sm_count)) != cudaSuccess ||
         cudaMalloc(&ctx->d_lstm_hc, lstm_hc_bytes()) != cudaSuccess ||
         cudaMemset(ctx->d_lstm_hc, 0, lstm_hc_bytes()) != cudaSuccess) {
       if (ctx->d_lstm_hc) cudaFree(ctx->d_lstm_hc);
-      if (ctx->d_lstm_partial) cudaFree(ctx->d_lstm_partial);
       if (ctx->d_grid_bar) cudaFree(ctx->d_grid_bar);
       if (ctx->d_tm_slots) cudaFree(ctx->d_tm_slots);
       if (ctx->d_sk_ws) cudaFree(ctx->d_sk_ws);
@@ -266,7 +263,6 @@ ard_status ard_destroy(ard_ctx* ctx) {
   if (ctx->d_sk_ws) cudaFree(ctx->d_sk_ws);
   if (ctx->d_sk_cnt) cudaFree(ctx->d_sk_cnt);
   if (ctx->d_grid_bar) cudaFree(ctx->d_grid_bar);
-  if (ctx->d_lstm_partial) cudaFree(ctx->d_lstm_partial);
   if (ctx->d_lstm_hc) cudaFree(ctx->d_lstm_hc);
   if (ctx->d_status) cudaFree(ctx->d_status);
   for (int i = 0; i < ctx->n_ev; ++i) cudaEventDestroy(ctx->ev[i]);
@@ -1234,24 +1230,18 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
                      ((size_t)H * ldw * 2) % 16 == 0 && I % 8 == 0;
     const int padded = (H + 7) / 8 * 8;
     const bool room = tma || (size_t)T * B * 4 * padded * 2 <= sk_ws_bytes(ctx->sm_count);
-    if (lstm_persistent_bwd_fits(ctx, B, H, tma) && room && (tma || ctx->path == ARD_PATH_AUTO)) {
+    if (lstm_persistent_bwd_fits(ctx, B, H) && room && (tma || ctx->path == ARD_PATH_AUTO)) {
       if (!tma) {
         dz = ctx->d_sk_ws;
         gs = padded;
       }
       TcMap mapDZ[4];
-      TcMap mapW[4];
       for (int gate = 0; gate < 4; ++gate) {
         st = get_maps(ctx, reinterpret_cast<const char*>(dz) + (size_t)gate * gs * 2, T * B, H, 4 * gs, H, MAP_COMPACT_COLS,
                       pat->dp_bound, lstm_box_rows_of(B), 64, &mapDZ[gate]);
         if (st != ARD_OK) return st;
-        if (!tma) continue;
-        st = get_maps(ctx, Wc + (size_t)gate * H * ldw * 2, H, KH, ldw, H, MAP_STRIDED_ROWS, pat->dp_bound, 64, 64,
-                      &mapW[gate]);
-        if (st != ARD_OK) return st;
       }
-      st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, tma ? mapW : nullptr, W, ldw, C, G, dH, dH_last, D, dc,
-                                           dz, gs, recurrent_only && dz != DZ ? DZ : nullptr, s);
+      st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, recurrent_only && dz != DZ ? DZ : nullptr, s);
       if (st == ARD_OK) {
         recurrence_done = true;
         // dx_t for all t: the x halves of D are overwritten

@@ -109,7 +109,6 @@ struct ard_ctx {
   int reuse_compact;  // opt-in: consecutive backward calls share one compacted dY
   int lstm_persistent; // ard_lstm_forward: one cooperative kernel for the whole sequence when the layer fits
   unsigned int* d_grid_bar;  // arrival counters of the cooperative kernels: word 0 ard_mlp_step, words 32, 33 LSTM (zero between launches)
-  float* d_lstm_partial;     // partial sums of the whole-sequence BPTT kernel, lstm_bwd_partial_bytes(sm_count)
   void* d_lstm_hc;           // compact copies of h_{t-1} and h_t of the whole-sequence forward kernel, lstm_hc_bytes()
   int lstm_compact_h;        // ... which contracts over the kept units of h alone under a pattern
   int use_pdl;        // launch kernels with programmatic stream serialization (see ard_launch)
@@ -244,15 +243,14 @@ ard_status launch_rows_tc(ard_ctx* ctx, GemmOp op, const TcArgs& a, const int32_
                           const void* gB, int ldgB, cudaStream_t s);
 
 // Whole-sequence LSTM kernels (lstm_persistent.cu).
-size_t lstm_bwd_partial_bytes(int sm_count);
 // tma: descriptors of [x | h], the weight and dz exist (16-byte aligned rows); without them only the compact form runs.
 int lstm_box_rows_of(int B);  // rows of a TMA box of the activations
 bool lstm_persistent_fits(ard_ctx* ctx, int B, int H, bool tma);
-bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H, bool tma);
+bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H);
 // dH: gradients of every h_t, D and dc are then outputs only; nullptr: dH_last, D and dc as ard_lstm_backward has them.
 // DZ: gate blocks of width gs; DZ_out: a second copy with the caller's layout, or nullptr.
 ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
-                                           const TcMap mapDZ[4], const TcMap* mapW, const void* W, int ldw,
+                                           const TcMap mapDZ[4], const void* W, int ldw,
                                            const float* C, const float* G, const float* dH, const float* dH_last, float* D,
                                            float* dc, void* DZ, int gs, void* DZ_out, cudaStream_t s);
 ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, int add_zx,

@@ -7,7 +7,11 @@
 //     x_t . W_x for all steps with one large product beforehand and leaves it where the gate activations
 //     of step t will be stored; the kernel adds it in its epilogue and handles the recurrent half only;
 //   - every CTA owns U kept hidden units, i.e. 4 U gate columns (i|f|g|o x U), and keeps its slice of
-//     the weight, [4 U rows][H] bf16, in shared memory.  U = 8; layers of more than 8 units per SM take U = 12;
+//     the weight, [4 U rows][H] bf16, in shared memory.  The grid is sized for nothing dropped with U = 8 (12 for layers
+//     of more than 8 units per SM); the drawn pattern then takes the smallest U of 4, 8, 12 with which the kept units
+//     fit the grid: the cell update is a serial chain per (batch row, unit) pair, and a second pair per thread costs
+//     more than the additional CTAs' reads of h (us per step: 64 rows, 512 of 1024 units kept, 4.7 with U = 8, 4.0 with
+//     4; 20 rows, 750 of 1500 kept, 5.4 with 12, 4.4 with 8; 128 rows, 64 kept, 4.6 with 8, 3.6 with 4);
 //   - per step it loads h_{t-1} (TMA boxes of up to 64 rows x 64 columns) into a ring of slots, one quarter of the
 //     blocks per loading warp.  Usually every block of a step has a slot of its own, so all loads of a step are in
 //     flight together; a slice so large that fewer slots fit re-uses them within the step.  The warp that loads a
@@ -139,15 +143,33 @@ __device__ __forceinline__ void grid_leave(unsigned int* bar) {
   }
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
+// Sums of the first `groups` issuing warps' accumulators (`stride` columns apart) over N consecutive columns of this
+// warp's 32 rows.
+template <int N>
+__device__ __forceinline__ void lstm_sum_groups(uint32_t taddr, int stride, int groups, float (&z)[N]) {
+  static_assert(N == 4 || N == 8);
+  uint32_t y[LP_GROUPS][N];
+#pragma unroll
+  for (int c = 0; c < LP_GROUPS; ++c) {
+    if (c >= groups) continue;
+    const uint32_t a = taddr + (uint32_t)(c * stride);
+    if constexpr (N == 8)
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                   : "=r"(y[c][0]), "=r"(y[c][1]), "=r"(y[c][2]), "=r"(y[c][3]), "=r"(y[c][4]), "=r"(y[c][5]), "=r"(y[c][6]), "=r"(y[c][7])
+                   : "r"(a) : "memory");
+    else
+      asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0, %1, %2, %3}, [%4];"
+                   : "=r"(y[c][0]), "=r"(y[c][1]), "=r"(y[c][2]), "=r"(y[c][3]) : "r"(a) : "memory");
+  }
+  tmem_ld_wait();
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    z[i] = __uint_as_float(y[0][i]);
+#pragma unroll
+    for (int c = 1; c < LP_GROUPS; ++c)
+      if (c < groups) z[i] += __uint_as_float(y[c][i]);
+  }
 }
-
 // One step's blocks [0, n) of a loading warp, called by all its lanes: lane i requests block i into slot i while slots
 // last; lane 0 multiplies the blocks as they arrive and requests the later ones into the slots that fell free.  A slot's
 // barriers are phased by how often it has been used: `step` steps before this one.  request(block, slot) issues the
@@ -183,68 +205,44 @@ __device__ __forceinline__ bool lstm_stream_blocks(int n, int cap, int step, int
 __device__ __forceinline__ float sigmoid_fast(float x) { return 1.f / (1.f + __expf(-x)); }
 __device__ __forceinline__ float tanh_fast(float x) { return 1.f - 2.f / (1.f + __expf(2.f * x)); }
 
+// Barriers behind the slots' full and free ones (byte offsets): accumulators complete / read (two each), weight slice
+// complete, h_{t-1} complete (relayed from the grid barrier); behind them the flags.
+constexpr uint32_t LF_TFULL = 8 * 2 * LP_GROUPS * LP_SLOTS;
+constexpr uint32_t LF_TEMPTY = LF_TFULL + 16;
+constexpr uint32_t LF_WFULL = LF_TEMPTY + 16;
+constexpr uint32_t LF_HREADY = LF_WFULL + 8;
+
+// The recurrence with U units per CTA.  compact: see below.
 template <int U>
-__global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const __grid_constant__ LstmFwdParams p) {
+__device__ __forceinline__ void lstm_forward_body(const LstmFwdParams& p, uint8_t* smem, uint32_t base, uint32_t tmem_base,
+                                                  volatile int* abort_flag, int dp, int bb, int n_keep, bool compact) {
   constexpr int N = 4 * U;                             // gate columns per CTA
   constexpr int W_BLOCK = N * LP_BK * 2;               // one contraction block of the resident weight slice
   constexpr int ZS_LD = N + 1;                         // staged pre-activations: [rows][N + 1] floats
   constexpr int PAIRS = (128 * U + LP_MATH - 1) / LP_MATH;  // (row, unit) pairs per thread
-  constexpr uint32_t TMEM_COLS = 2 * LP_GROUPS * N <= 256 ? 256 : 512;
-  extern __shared__ uint8_t smem_raw[];
-  const uint32_t raw_addr = smem_u32(smem_raw);
-  const uint32_t base = (raw_addr + 1023u) & ~1023u;
-  uint8_t* smem = smem_raw + (base - raw_addr);
-
   const int KH = p.I + p.H;
   const int box_rows = lstm_box_rows(p.B), row_boxes = (p.B + 63) / 64;
   const uint32_t a_block = (uint32_t)lstm_a_block(p.B);
   auto full_bar = [&](int g, int s) { return base + 8u * (g * LP_SLOTS + s); };
   auto free_bar = [&](int g, int s) { return base + 8u * ((LP_GROUPS + g) * LP_SLOTS + s); };
-  const uint32_t bar_base = base + 8u * (2 * LP_GROUPS * LP_SLOTS);
-  auto tfull_bar = [&](int a) { return bar_base + 8u * a; };
-  auto tempty_bar = [&](int a) { return bar_base + 8u * (2 + a); };
-  const uint32_t wfull_bar = bar_base + 8u * 4;
-  const uint32_t hready_bar = bar_base + 8u * 5;  // h_{t-1} is complete (relayed from the grid barrier)
-  uint8_t* misc = smem + (bar_base - base) + 8 * 6;
-  volatile uint32_t* tmem_ptr_smem = reinterpret_cast<volatile uint32_t*>(misc);
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
-
+  auto tfull_bar = [&](int a) { return base + LF_TFULL + 8u * a; };
+  auto tempty_bar = [&](int a) { return base + LF_TEMPTY + 8u * a; };
+  const uint32_t wfull_bar = base + LF_WFULL, hready_bar = base + LF_HREADY;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (threadIdx.x < LP_GROUPS * LP_SLOTS) {
-    mbar_init(full_bar(0, threadIdx.x), 1);
-    mbar_init(free_bar(0, threadIdx.x), 1);
-  }
-  if (threadIdx.x == 0) {
-    for (int a = 0; a < 2; ++a) {
-      mbar_init(tfull_bar(a), LP_GROUPS);  // one commit per MMA issuer
-      mbar_init(tempty_bar(a), 4);         // one arrival per TMEM-reading warp
-    }
-    mbar_init(wfull_bar, 1);
-    mbar_init(hready_bar, 1);
-    *abort_flag = 0;
-  }
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-  if (warp == 15) {
-    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_ptr_smem)), TMEM_COLS);
-    tmem_relinquish();
-  }
-  tc_fence_before();
-  __syncthreads();
-  tc_fence_after();
-  const uint32_t tmem_base = *tmem_ptr_smem;
-  pdl_wait_prior_grids();
-
-  const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP];
   const int n_active = (n_keep + U - 1) / U;       // CTAs that own units (the others only tear down)
   const int j0 = (int)blockIdx.x * U;              // first kept unit (compact index) of this CTA
   const bool active = (int)blockIdx.x < n_active;
+  // The dropped units of h_1 .. h_T, read by nobody before the kernel ends when the recurrence is compact: where enough
+  // of the grid's CTAs have no units, these write the zeros meanwhile; otherwise the threads of the cell update do after
+  // their CTA has signalled (as stores ahead of the signal they cost 0.3 us a step).
+  const int n_idle = (int)gridDim.x - n_active;
+  const bool idle_zeros = n_idle >= 8;
   // Under a pattern the dropped units of h_{t-1} are exact zeros (Sec. 3.1), so the recurrent contraction runs over
   // the kept units alone: the operand of a step is the compact copy of h_{t-1} (column j = j-th kept unit) that the
   // cell update writes beside the full-width one, and the weight slice holds the kept fan-in columns only.  Those
   // stride the weight's contiguous dimension, which no TMA box can follow, so the CTA gathers its slice itself,
   // once per sequence, straight into the swizzled layout the MMA reads.
-  const bool compact = p.Hc != nullptr && (dp > 1 || p.always_compact);
   const int hs = compact ? 1 : 0;  // the compact h_0 is made by the kernel: one more grid-wide hand-over, before step 0
   const int nkb = ((compact ? n_keep : p.H) + LP_BK - 1) / LP_BK;
   // The staged pre-activations share the start of the ring where they fit: they are written after the step's MMAs
@@ -412,33 +410,23 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
             }
           }
         }
-        if (warp < 4) {
-          // accumulator rows -> shared memory
+        if (warp < 8) {
+          // accumulator rows -> shared memory; warps 4-7 take the second half of the columns
           if (!mbar_wait(tfull_bar(acc), (uint32_t)(t >> 1) & 1u, abort_flag, p.status)) ok = false;
-          if (ok) {
+          if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
-            if (warp * 32 < p.B) {
-              const uint32_t t_row = tmem_base + ((uint32_t)(warp * 32) << 16) + (uint32_t)(acc * LP_GROUPS * N);
+            const int quadrant = warp & 3;
+            if (quadrant * 32 < p.B) {
+              const uint32_t t_row = tmem_base + ((uint32_t)(quadrant * 32) << 16) + (uint32_t)(acc * LP_GROUPS * N);
               const int ngroups = (nkb + gsz - 1) / gsz;  // accumulators that received MMAs
-              float* zr = zs + (warp * 32 + lane) * ZS_LD;
+              float* zr = zs + (quadrant * 32 + lane) * ZS_LD;
 #pragma unroll
-              for (int c0 = 0; c0 < N; c0 += 16) {
-                uint32_t y[LP_GROUPS][16];
+              for (int i0 = 0; i0 < N / 2; i0 += 8) {
+                const int c0 = (warp >> 2) * (N / 2) + i0;
+                float z[8];
+                lstm_sum_groups<8>(t_row + (uint32_t)c0, N, ngroups, z);
 #pragma unroll
-                for (int c = 0; c < LP_GROUPS; ++c)
-                  if (c < ngroups) tmem_ld16(t_row + (uint32_t)(c * N + c0), y[c]);
-                tmem_ld_wait();
-                float z[16];
-#pragma unroll
-                for (int i = 0; i < 16; ++i) z[i] = __uint_as_float(y[0][i]);
-#pragma unroll
-                for (int c = 1; c < LP_GROUPS; ++c)
-                  if (c < ngroups) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) z[i] += __uint_as_float(y[c][i]);
-                  }
-#pragma unroll
-                for (int i = 0; i < 16; ++i) zr[c0 + i] = z[i];
+                for (int i = 0; i < 8; ++i) zr[c0 + i] = z[i];
               }
             }
             tc_fence_before();
@@ -469,7 +457,7 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
             const __nv_bfloat16 h = __float2bfloat16_rn(p.alpha * go[i] * tanh_fast(creg[i]));
             p.XH[((size_t)(t + 1) * p.B + row) * ldxh + p.I + u] = h;
             if (compact) p.Hc[((size_t)((t + 1) & 1) * p.B + row) * p.ldhc + j0 + k] = h;
-            else if (dp > 1) zeros_of(row, t, j0 + k);  // operands of the next step's product (compact: see below)
+            else if (dp > 1) zeros_of(row, t, j0 + k);  // operands of the next step's product
           }
         }
         // publish h_t: all stores of the CTA, then one release-add for the CTA (the staged sums may lie in the
@@ -488,22 +476,62 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
             g_out[p.H] = gf[i];
             g_out[2 * p.H] = gg[i];
             g_out[3 * p.H] = go[i];
+            if (compact && dp > 1 && !idle_zeros) zeros_of(row, t, j0 + k);
           }
         }
       }
     }
   }
 
-  if (!active && compact && dp > 1) {
-    // The dropped units of h_1 .. h_T, read by nobody before the kernel ends: under a period of dp all but 1 / dp of
-    // the grid's CTAs have no units and write the zeros meanwhile (as stores of the cell update they cost 0.3 us a step).
-    const int n_idle = (int)gridDim.x - n_active, rows = p.T * p.B;
+  if (!active && compact && dp > 1 && idle_zeros) {
+    const int rows = p.T * p.B;
     for (int r = (int)blockIdx.x - n_active; r < rows; r += n_idle) {
       __nv_bfloat16* hrow = p.XH + ((size_t)p.B + r) * KH + p.I;
       for (int u = threadIdx.x; u < p.H; u += LP_THREADS)
         if (u < bb || (u - bb) % dp != 0) hrow[u] = __float2bfloat16_rn(0.f);
     }
   }
+}
+
+// U: units per CTA at most; the layer fits the grid with U units per CTA when nothing is dropped.
+template <int U>
+__global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const __grid_constant__ LstmFwdParams p) {
+  constexpr uint32_t TMEM_COLS = 2 * LP_GROUPS * 4 * U <= 256 ? 256 : 512;
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  const uint32_t base = (raw_addr + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (base - raw_addr);
+  uint8_t* misc = smem + LF_HREADY + 8;
+  volatile uint32_t* tmem_ptr_smem = reinterpret_cast<volatile uint32_t*>(misc);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
+  const int warp = threadIdx.x >> 5;
+
+  if (threadIdx.x < 2 * LP_GROUPS * LP_SLOTS) mbar_init(base + 8u * threadIdx.x, 1);  // slots: full, free
+  if (threadIdx.x == 0) {
+    for (int a = 0; a < 2; ++a) {
+      mbar_init(base + LF_TFULL + 8u * a, LP_GROUPS);  // one commit per MMA issuer
+      mbar_init(base + LF_TEMPTY + 8u * a, 8);       // one arrival per TMEM-reading warp
+    }
+    mbar_init(base + LF_WFULL, 1);
+    mbar_init(base + LF_HREADY, 1);
+    *abort_flag = 0;
+  }
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  if (warp == 15) {
+    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_ptr_smem)), TMEM_COLS);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem_base = *tmem_ptr_smem;
+  pdl_wait_prior_grids();
+
+  const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP], ctas = (int)gridDim.x;
+  const bool compact = p.Hc != nullptr && (dp > 1 || p.always_compact);
+  if (compact && n_keep <= 4 * ctas) lstm_forward_body<4>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
+  else if (U == 8 || (compact && n_keep <= 8 * ctas)) lstm_forward_body<8>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
+  else lstm_forward_body<U>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
 
   // ---- teardown ----
   tc_fence_before();
@@ -522,51 +550,54 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
 // Whole-sequence BPTT recurrence (Sec. 7), the counterpart of the kernel above.
 //
 // Per step t = T-1 .. 0 the recurrence needs  dh_t = upstream_t + dz_{t+1} . W_h  (contraction over the
-// 4 * n_keep kept gate rows, output over the hidden units), then the cell adjoint gives dz_t.  Every SM
-// would need all of dz_{t+1} if the output units were simply dealt out, so the product is cut both ways:
-// CTA (s, r) owns the 64 hidden-unit COLUMNS 64 s .. 64 s + 63 of the recurrent weight (all of them, kept
-// or not: the columns of a kept-unit set are strided and cannot be boxed) and the r-th eighth of the
-// contraction blocks; its slice of the weight (at most 8 boxes of 64 gate rows x 64 columns, MN-major B
-// operand straight from the neuron-major weight) stays in shared memory for the whole sequence.  A step is
-//   A. wait until dz_{t+1} is complete (grid barrier), TMA-load this CTA's blocks of it, multiply
-//      (tcgen05.mma M = 128, N = 64, four issuing warps with an accumulator each), park the 64-column
-//      partial sums in global memory, arrive;
-//   B. wait until all partial sums are there (grid barrier); the threads that own a kept unit among this
-//      CTA's 8 columns 64 s + 8 r .. + 7 add the 8 partial sums in a fixed order, add the upstream gradient,
-//      store the total (the caller's D holds it afterwards), apply the cell adjoint with dc in a register,
-//      store dz_t (bf16, the operand of the next step and of the weight-gradient products), arrive.
-// After t = 0 one more product gives the gradient of h_0.  The input half of d[x, h] and the weight
-// gradient are large products over all T*B rows that the caller runs afterwards.
-// Grid barriers are phases of one arrival counter: every CTA arrives exactly once per phase and only
-// after it has passed the previous phase, so the count p * (number of CTAs) identifies phase p.
-constexpr int LB_COLS = 64;    // weight columns (hidden units, kept or not) per CTA
-constexpr int LB_KPARTS = 8;   // CTAs sharing the contraction of one column slice
-constexpr int LB_OWN = LB_COLS / LB_KPARTS;  // columns whose cell adjoint this CTA computes
-constexpr int LB_MAX_BLOCKS = 8;             // contraction blocks of one CTA (64 gate rows each)
-constexpr int LB_W_BLOCK = 64 * LB_COLS * 2; // one resident weight box
-constexpr int LB_THREADS = 512;              // warps 0-10 adjoint (0-3 also read TMEM), 11 relay, 12-15 load + MMA
+// 4 * n_keep kept gate rows, output over the kept hidden units), then the cell adjoint gives dz_t.  A CTA owns U KEPT
+// units: it keeps their cell gradient in registers and writes their columns of dz_t.  If it contracted for its own
+// units only, every CTA would have to read all of dz_{t+1} in every step (256 KB at batch 64 and 512 kept units),
+// which is what bounds a step then.  So CTAs work in clusters of LB_CLUSTER: the cluster owns LB_CLUSTER * U units and
+// CTA r contracts the r-th share of the blocks of 64 gate rows for all of them.  A step is
+//   1. dz_{t+1} is complete (grid barrier, relayed): TMA-load this CTA's blocks of it into the ring of slots of the
+//      forward kernel and multiply (tcgen05.mma M = 128, N = LB_CLUSTER * U, four issuing warps with an accumulator
+//      each) by the resident weight slice: the fan-out weights of the cluster's units, [units][gate rows] (K-major),
+//      gathered by the kernel once per sequence;
+//   2. send the sums of every CTA's units to that CTA's shared memory (st.async: the bytes themselves complete the
+//      receiver's mbarrier, so the exchange costs one trip between SMs and no barrier);
+//   3. the owner adds the shares in a fixed order and the upstream gradient, applies the cell adjoint with dc in a
+//      register, stores dz_t (bf16, the operand of the next step and of the weight-gradient products), arrives.
+// A pattern that keeps so few units that all of a step's blocks fit beside the slice of one CTA's own units may do
+// without the exchange (see LB_WHOLE_BLOCKS): every CTA contracts whole rows for its own units.  The same form serves
+// layers whose CTAs do not all fit the device in clusters.  After t = 0 one more product gives the gradient of h_0.
+// The input half of d[x, h] and the weight gradient are large products over all T*B rows that the caller runs
+// afterwards.  No operand of the caller but dz is read through a descriptor, and dz lives in a padded copy in context
+// scratch where the caller's rows are off the 16-byte grid.
+// The grid barrier is one arrival counter: every CTA that takes part arrives once per step, after all of its stores.
+// us per step, before (partial sums through global memory and a second grid barrier, or whole contractions in every CTA;
+// the cell adjoint formed behind the wait; 8 units per CTA) and now: 64 rows, 512 of 1024 units kept 7.4 -> 4.2, all
+// kept 8.6 -> 6.3; 128 rows, 512 of 1024 kept 10.1 -> 5.6; 20 rows, 750 of 1500 kept 9.7 -> 4.9, all kept 25.4 -> 7.5.
+// About 2.9 of it are what a step of any size costs: stores, barrier, TMA, a few narrow MMAs, the exchange.
+constexpr int LB_CLUSTER = 4;     // of 148 SMs 132 can be used by clusters of 4, 120 by clusters of 8
+constexpr int LB_COLS = 64;       // tensor-memory columns of an issuing warp's accumulator (at most LB_CLUSTER * 12 used)
+constexpr int LB_THREADS = 512;   // warps 0-10 adjoint (0-7 also read TMEM), 11 relay, 12-15 load + MMA
 constexpr int LB_MATH = 352;
-constexpr int LB_PAIRS_MAX = (128 * LB_OWN + LB_MATH - 1) / LB_MATH;
-// The compact form drops the cut along the contraction: a CTA owns U KEPT units, holds their fan-out weights over all
-// 4 * n_keep kept gate rows (gathered by the kernel, K-major) and contracts the whole of dz_{t+1} itself, streamed
-// through the same ring of slots as in the forward kernel: one grid-wide barrier per step instead of two, no partial
-// sums through global memory.  Its slice needs only the rows of its U units: the instruction's columns beyond them
-// are read from whatever follows and never used, so U = 8 takes one KiB per block (U = 12, for layers of more than 8
-// units per SM, two).  It reads no operand of the caller through a descriptor but dz, which lives in a padded copy
-// in context scratch where the caller's rows are off the 16-byte grid.
-// Which form: the compact one while each of a step's blocks has a slot of its own (LB_ROUNDS; batch 64, H = 1024: up
-// to 320 kept units), or where the other form cannot run at all.  Every CTA reads all of dz_{t+1} (256 KB of it at a
-// period of 2): with slots re-used there the recurrence took 286 us against 264 with partial sums.
-constexpr int LC_N = 16;                       // MMA width (the instruction's minimum at 128 rows)
-constexpr int LB_ROUNDS = 1;
-constexpr int LB_SMEM_BYTES = 195 * 1024;      // one carve-out step higher the form with partial sums was measured 4 - 8 % slower
-constexpr int LC_TAIL = 1024;                  // the second 8-row group of the last block's read
-__host__ __device__ constexpr int lc_w_block(int U) { return (U + 7) / 8 * 1024; }
-__host__ __device__ inline int lc_zs_bytes(int U, int B) { return (B + 31) / 32 * 32 * (U + 1) * 4; }
+// A step of this many blocks is contracted whole by every CTA: one block per issuing warp either way, and no exchange
+// (64 rows, 64 of 1024 units kept: 3.22 us per step against 3.42 with it; 128 kept, 8 blocks: 3.68 against 3.44).
+constexpr int LB_WHOLE_BLOCKS = 4;
+constexpr uint32_t LB_TFULL = 8 * 2 * LP_GROUPS * LP_SLOTS;  // barriers behind the slots' full and free ones
+constexpr uint32_t LB_HREADY = LB_TFULL + 8;                 // dz of the previous step is complete
+constexpr uint32_t LB_PFULL = LB_TFULL + 16;                 // all shares of this CTA's sums are there; behind it: flags
+constexpr int LC_N = 16;          // MMA width without the exchange (the instruction's minimum at 128 rows)
+constexpr int LC_TAIL = 1024;     // ... whose slice has rows for the CTA's own units only: the read past its last block
+// Rows of the weight slice, bytes of it per block, bytes of the staged sums (cl: CTAs sharing a contraction, or 1).
+__host__ __device__ constexpr int lb_rows(int U, int cl) { return (cl * U + 7) / 8 * 8; }
+__host__ __device__ constexpr int lb_w_block(int U, int cl) { return lb_rows(U, cl) * 128; }
+__host__ __device__ inline LstmPlan lb_plan(int nblk, int B, int U, int cl, int smem_bytes) {
+  if (cl == 1)  // the sums may share the ring: written once a step's products are complete, read before the CTA arrives
+    return lstm_plan(nblk, lstm_a_block(B), lb_w_block(U, 1), LC_TAIL, (B + 31) / 32 * 32 * (U + 1) * 4, smem_bytes);
+  // the other CTAs write here while this one's products may still read the ring: behind the slice
+  return lstm_plan((nblk + cl - 1) / cl, lstm_a_block(B), lb_w_block(U, cl), cl * B * U * 4, 0, smem_bytes);
+}
 
 struct LstmBwdParams {
-  TcMap mapDZ[4];  // per gate: [T*B rows][H columns], boxes 64 x 64; the kernel limits them to the n_keep compact columns
-  TcMap mapW[4];   // per gate: [H rows][I+H columns], boxes 64 x 64; the kernel turns them into the kept rows
+  TcMap mapDZ[4];  // per gate: [T*B rows][H columns], boxes of box_rows x 64; the kernel limits them to the n_keep compact columns
   CUtensorMap* tm_slots;  // this launch's descriptor scratch: ARD_TM_LSTM_SLOTS slots per block
   const int32_t* hdr;
   int T, B, I, H;
@@ -580,13 +611,11 @@ struct LstmBwdParams {
   __nv_bfloat16* DZ;     // [T][B][4 * gs]: gate blocks of width gs, compact inside a block
   int gs;
   __nv_bfloat16* DZ_out; // a second copy for the caller, [T][B][4H] (nullptr: DZ is the caller's)
-  float* partial;        // [CTA][128][64]
   unsigned int* bar;     // arrival counter, zero at launch; [1]: CTAs that left
   int* status;
-  const __nv_bfloat16* W;  // the weight itself, [4H][ldw] (the compact form gathers its slice from it)
+  const __nv_bfloat16* W;  // [4H][ldw]
   int ldw;
-  int compact_ok;          // the compact form may be used when the drawn pattern allows it
-  int always_compact;      // the operands do not allow the other form
+  int whole_ok;            // a pattern that keeps few units may do without the exchange
   int smem_bytes;          // dynamic shared memory of this launch
 };
 
@@ -594,12 +623,7 @@ struct LstmBwdParams {
 struct AdjointIn {
   float gi, gf, gg, go, cp, c, up;
 };
-// Upstream gradient of h_t at (row, u).
-__device__ __forceinline__ float upstream(const LstmBwdParams& p, int t, int row, int u) {
-  if (p.dH != nullptr) return __ldcg(p.dH + ((size_t)t * p.B + row) * p.H + u);
-  return t == p.T - 1 ? p.dH_last[(size_t)row * p.H + u] : __ldcg(p.D + ((size_t)(t + 1) * p.B + row) * (p.I + p.H) + p.I + u);
-}
-__device__ __forceinline__ void fetch_saved(const LstmBwdParams& p, int t, int row, int j, AdjointIn& in) {
+__device__ __forceinline__ void fetch_saved(const LstmBwdParams& p, int t, int row, int j, int u, AdjointIn& in) {
   const float* gs = p.G + ((size_t)t * p.B + row) * 4 * p.H + j;
   in.gi = __ldcg(gs);
   in.gf = __ldcg(gs + p.H);
@@ -607,86 +631,159 @@ __device__ __forceinline__ void fetch_saved(const LstmBwdParams& p, int t, int r
   in.go = __ldcg(gs + 3 * p.H);
   in.cp = __ldcg(p.C + ((size_t)t * p.B + row) * p.H + j);
   in.c = __ldcg(p.C + ((size_t)(t + 1) * p.B + row) * p.H + j);
+  // upstream gradient of h_t (u: the unit's index in the layer)
+  if (p.dH != nullptr) in.up = __ldcg(p.dH + ((size_t)t * p.B + row) * p.H + u);
+  else if (t == p.T - 1) in.up = p.dH_last[(size_t)row * p.H + u];
+  else in.up = __ldcg(p.D + ((size_t)(t + 1) * p.B + row) * (p.I + p.H) + p.I + u);
 }
-// Cell adjoint: dz of the four gates from the total gradient dh of h_t; dc is updated to the gradient of c_{t-1}.
-__device__ __forceinline__ void cell_adjoint(const LstmBwdParams& p, const AdjointIn& in, float dh, float& dc, __nv_bfloat16 (&dz)[4]) {
+// The cell adjoint is linear in the total gradient dh of h_t: with dcv = dc + dh * c, the gradient of c_t, the gates'
+// dz are dcv * i, dcv * f, dcv * g and dh * o, and dcv * next is the gradient of c_{t-1}.  These factors are formed
+// while the recurrent sums are on their way
+// (64 rows, 512 kept units: 4.27 -> 4.21 us per step; 64 kept: 3.29 -> 3.22).
+struct Adjoint {
+  float c, i, f, g, o, next, up;
+};
+__device__ __forceinline__ Adjoint adjoint_factors(const AdjointIn& in, float alpha) {
+  Adjoint a;
   const float tc = tanh_fast(in.c);
-  const float d_o = dh * p.alpha * tc;
-  const float dcv = dc + dh * p.alpha * in.go * (1.f - tc * tc);
-  dc = dcv * in.gf;
-  dz[0] = __float2bfloat16_rn(dcv * in.gg * in.gi * (1.f - in.gi));
-  dz[1] = __float2bfloat16_rn(dcv * in.cp * in.gf * (1.f - in.gf));
-  dz[2] = __float2bfloat16_rn(dcv * in.gi * (1.f - in.gg * in.gg));
-  dz[3] = __float2bfloat16_rn(d_o * in.go * (1.f - in.go));
+  a.c = alpha * in.go * (1.f - tc * tc);
+  a.i = in.gg * in.gi * (1.f - in.gi);
+  a.f = in.cp * in.gf * (1.f - in.gf);
+  a.g = in.gi * (1.f - in.gg * in.gg);
+  a.o = alpha * tc * in.go * (1.f - in.go);
+  a.next = in.gf;
+  a.up = in.up;
+  return a;
+}
+__device__ __forceinline__ void cell_adjoint(const Adjoint& a, float dh, float& dc, __nv_bfloat16 (&dz)[4]) {
+  const float dcv = dc + dh * a.c;
+  dc = dcv * a.next;
+  dz[0] = __float2bfloat16_rn(dcv * a.i);
+  dz[1] = __float2bfloat16_rn(dcv * a.f);
+  dz[2] = __float2bfloat16_rn(dcv * a.g);
+  dz[3] = __float2bfloat16_rn(dh * a.o);
 }
 __device__ __forceinline__ void store_dz(__nv_bfloat16* dst, size_t gs, const __nv_bfloat16 (&dz)[4]) {
 #pragma unroll
   for (int g = 0; g < 4; ++g) dst[g * gs] = dz[g];
 }
 
-// The compact form of the BPTT recurrence (see LC_N).
+// 16 bytes into another CTA's shared memory, counted on that CTA's barrier.
+__device__ __forceinline__ void st_async_f4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%2, %3, %4, %5}, [%1];"
+               ::"r"(addr), "r"(bar), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+// Bounded wait for data that other CTAs of the cluster store into this one.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  unsigned long long t0 = 0;
+  for (int spin = 0;; ++spin) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2, %3;\n\t"
+        "selp.b32 %0, 1, 0, P;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity), "r"(1000000u) : "memory");
+    if (ok) return true;
+    if (*abort_flag) return false;
+    if (spin == 0) t0 = global_ns();
+    else if (global_ns() - t0 > WAIT_LIMIT_NS) {
+      *abort_flag = 1;
+      atomicMax(status, (int)ARD_ERR_TIMEOUT);
+      return false;
+    }
+  }
+}
+// Barrier ID of the LB_MATH adjoint threads; the same verdict for all of them: did anyone fail?
+template <int ID>
+__device__ __forceinline__ bool math_barrier_failed(bool failed) {
+  uint32_t r;
+  __syncwarp();
+  asm volatile(
+      "{\n\t.reg .pred P, Q;\n\t"
+      "setp.ne.b32 Q, %1, 0;\n\t"
+      "barrier.cta.red.or.pred.aligned P, %2, %3, Q;\n\t"
+      "selp.b32 %0, 1, 0, P;\n\t}"
+      : "=r"(r) : "r"((uint32_t)failed), "n"(ID), "n"(LB_MATH) : "memory");
+  return r != 0;
+}
+
+// The recurrence with U units per CTA.
 template <int U>
-__device__ __forceinline__ void lstm_backward_compact(const LstmBwdParams& p, uint8_t* smem, uint32_t base, uint32_t tfull_bar,
-                                                      uint32_t hready_bar, uint32_t tmem_base, volatile int* abort_flag, int dp,
-                                                      int bb, int n_keep) {
-  constexpr int W_BLOCK = lc_w_block(U), W_ROWS = W_BLOCK / 128;
-  constexpr int ZS_LD = U + 1;                               // staged recurrent sums: [rows][U + 1] floats
-  constexpr int PAIRS = (128 * U + LB_MATH - 1) / LB_MATH;
+__device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8_t* smem, uint32_t base, uint32_t tmem_base,
+                                                   volatile int* abort_flag, int cl, int dp, int bb, int n_keep) {
+  constexpr int PAIRS = (128 * U + LB_MATH - 1) / LB_MATH;  // (row, unit) pairs per thread
+  constexpr int GRAN = 4;                                   // columns read from tensor memory at a time
   auto full_bar = [&](int g, int s) { return base + 8u * (g * LP_SLOTS + s); };
   auto free_bar = [&](int g, int s) { return base + 8u * ((LP_GROUPS + g) * LP_SLOTS + s); };
+  const uint32_t tfull_bar = base + LB_TFULL, hready_bar = base + LB_HREADY, pfull_bar = base + LB_PFULL;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int KH = p.I + p.H, T = p.T;
   const int box_rows = lstm_box_rows(p.B), row_boxes = (p.B + 63) / 64;
   const uint32_t a_block = (uint32_t)lstm_a_block(p.B);
   const int nb = (n_keep + 63) / 64;                  // contraction blocks per gate
-  const int nblk = 4 * nb;                            // ... per step; block = gate * nb + jb
-  const LstmPlan plan = lstm_plan(nblk, (int)a_block, W_BLOCK, LC_TAIL, lc_zs_bytes(U, p.B), p.smem_bytes);
+  const int nblk_all = 4 * nb;                        // ... per step; block = gate * nb + jb
+  int share = cl;                                     // CTAs that share a contraction
+  LstmPlan plan = lb_plan(nblk_all, p.B, U, 1, p.smem_bytes);
+  if (p.whole_ok && nblk_all <= LB_WHOLE_BLOCKS && plan.cap >= plan.gsz) share = 1;
+  if (share > 1) plan = lb_plan(nblk_all, p.B, U, LB_CLUSTER, p.smem_bytes);
   const int gsz = plan.gsz, cap = plan.cap;
-  const int n_active = (n_keep + U - 1) / U;
-  const bool active = (int)blockIdx.x < n_active;
-  const int j0 = (int)blockIdx.x * U;                 // first kept unit (compact index) of this CTA
+  const int per = (nblk_all + share - 1) / share;     // blocks of one share
+  const int parts = (nblk_all + per - 1) / per;       // shares that have blocks
+  // Without the exchange the first CTA of every cluster takes units before the second of any does: the CTAs of a
+  // cluster are neighbours, and neighbours share their way to L2.
+  const int cta = share > 1 ? (int)blockIdx.x : (int)(blockIdx.x % cl * (gridDim.x / cl) + blockIdx.x / cl);
+  const int rank = cta % share;
+  const int blk0 = rank * per, nblk = max(0, min(per, nblk_all - blk0));
+  const int j0 = cta * U;                             // first kept unit (compact index) of this CTA
+  const int s0 = j0 - rank * U;                       // ... of those whose sums it forms
+  const int units = share * U;
+  const int n_active = (n_keep + units - 1) / units * share;
+  const bool active = cta < n_active;
+  const int w_rows = share > 1 ? lb_rows(U, LB_CLUSTER) : lb_rows(U, 1);
+  const uint32_t w_block = (uint32_t)w_rows * 128u;
   const uint32_t sA = base + LP_BAR_BYTES;            // the ring
   const uint32_t sW = sA + (uint32_t)(LP_GROUPS * cap) * a_block;  // the weight slice
-  // the sums share the ring where they fit: written once a step's products are complete, read before the CTA arrives
-  float* zs = reinterpret_cast<float*>(smem + (plan.zs_shared ? sA - base : sW - base + (uint32_t)plan.behind));
+  const uint32_t sZ = share > 1 ? sW + (uint32_t)per * w_block     // staged sums
+                                : (plan.zs_shared ? sA : sW + (uint32_t)plan.behind);
+  float* zs = reinterpret_cast<float*>(smem + (sZ - base));
 
   if (active) {
-    // Weight slice, K-major: row r = unit j0 + r, column (gate, i) = W[gate * H + keep[i]][I + keep[j0 + r]], in the
-    // 128-byte swizzle (16-byte piece c of row r of an 8-row group sits at piece c ^ r); rows beyond the CTA's units
-    // and what lies beyond the kept counts are zeros.
-    for (int task = threadIdx.x; task < nblk * W_ROWS * 8; task += LB_THREADS) {
-      const int kb = task / (W_ROWS * 8), c = (task / W_ROWS) & 7, r = task % W_ROWS;
-      const int g = kb / nb, jb = kb - g * nb;
+    // Weight slice, K-major: row r = unit s0 + r, column (gate, i) = W[gate * H + keep[i]][I + keep[s0 + r]], in the
+    // 128-byte swizzle (16-byte piece c of row r of an 8-row group sits at piece c ^ r); rows beyond the units and
+    // what lies beyond the kept counts are zeros.
+    for (int task = threadIdx.x; task < nblk * w_rows * 8; task += LB_THREADS) {
+      const int r = task % w_rows, c = task / w_rows & 7, kb = task / (w_rows * 8);
+      const int blk = blk0 + kb, g = blk / nb, jb = blk - g * nb;
       uint32_t w[4] = {0u, 0u, 0u, 0u};
-      if (r < U && j0 + r < n_keep) {
+      if (r < units && s0 + r < n_keep) {
         const int i0 = jb * 64 + c * 8;
         const unsigned short* src = reinterpret_cast<const unsigned short*>(p.W) +
-                                    ((size_t)g * p.H + bb + (size_t)i0 * dp) * p.ldw + p.I + bb + (size_t)(j0 + r) * dp;
+                                    ((size_t)g * p.H + bb + (size_t)i0 * dp) * p.ldw + p.I + bb + (size_t)(s0 + r) * dp;
         uint32_t e[8];
 #pragma unroll
         for (int q = 0; q < 8; ++q) e[q] = (i0 + q < n_keep) ? (uint32_t)__ldg(src + (size_t)q * dp * p.ldw) : 0u;
 #pragma unroll
         for (int q = 0; q < 4; ++q) w[q] = e[2 * q] | (e[2 * q + 1] << 16);
       }
-      uint8_t* dst = smem + (sW - base) + (size_t)kb * W_BLOCK + (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4);
+      uint8_t* dst = smem + (sW - base) + (size_t)kb * w_block + (r >> 3) * 1024 + (r & 7) * 128 + ((c ^ (r & 7)) << 4);
       *reinterpret_cast<uint4*>(dst) = make_uint4(w[0], w[1], w[2], w[3]);
     }
     fence_proxy_async_smem();  // generic-proxy stores -> the tensor core's reads
   }
   __syncthreads();
-  if (!active) return;
 
   CUtensorMap* slots = p.tm_slots + (size_t)blockIdx.x * ARD_TM_LSTM_SLOTS;
-  if (warp == 11) {
+  if (!active) {
+  } else if (warp == 11) {
     // ===================== descriptors of the compact gradient columns, barrier relay =====================
 #pragma unroll
     for (int g = 0; g < 4; ++g)  // the ring, still empty, is the work area
-      tensormap_specialise(&p.mapDZ[g], dp, bb + 1, n_keep, smem + LP_BAR_BYTES + 128 * g, slots + 4 + g, lane);
+      tensormap_specialise(&p.mapDZ[g], dp, bb + 1, n_keep, smem + LP_BAR_BYTES + 128 * g, slots + g, lane);
     fence_proxy_async_smem();
     __syncwarp();
     if (lane == 0) {
       for (int ph = 1; ph <= T; ++ph) {
-        // dz of time index T - ph is complete when every CTA with units has arrived ph times
+        // dz of time index T - ph is complete when every CTA that takes part has arrived ph times
         if (!grid_wait(p.bar, (unsigned)ph * (unsigned)n_active, abort_flag, p.status)) break;
         mbar_arrive(hready_bar);
       }
@@ -696,8 +793,8 @@ __device__ __forceinline__ void lstm_backward_compact(const LstmBwdParams& p, ui
     const int g4 = warp - 12;
     const int kb0 = g4 * gsz, n = max(0, min(nblk - kb0, gsz));
     // where dp == 1 the descriptors are used as encoded (tensormap_specialise returns the parameter)
-    auto map_of = [&](int gate) -> const CUtensorMap* { return dp == 1 ? &p.mapDZ[gate].tm : slots + 4 + gate; };
-    const uint32_t idesc = make_idesc(LC_N, false, false, 128);
+    auto map_of = [&](int gate) -> const CUtensorMap* { return dp == 1 ? &p.mapDZ[gate].tm : slots + gate; };
+    const uint32_t idesc = make_idesc(share > 1 ? LB_CLUSTER * U : LC_N, false, false, 128);
     const uint32_t d_tmem = tmem_base + (uint32_t)(g4 * LB_COLS);
     bool ok = true;
     for (int k = 1; k <= T; ++k) {
@@ -705,18 +802,18 @@ __device__ __forceinline__ void lstm_backward_compact(const LstmBwdParams& p, ui
       if (!__all_sync(0xffffffffu, ok)) break;
       if (k == 1 && dp > 1) {  // written by warp 11 ahead of its first arrival on hready_bar
 #pragma unroll
-        for (int g = 0; g < 4; ++g) tensormap_acquire(slots + 4 + g);
+        for (int g = 0; g < 4; ++g) tensormap_acquire(slots + g);
       }
       asm volatile("fence.proxy.async.global;" ::: "memory");  // generic-proxy stores of other CTAs -> TMA reads
       auto request = [&](int i, int slot) {
-        const int kb = kb0 + i, gate = kb / nb, jb = kb - gate * nb;
+        const int kb = blk0 + kb0 + i, gate = kb / nb, jb = kb - gate * nb;
         mbar_arrive_expect_tx(full_bar(g4, slot), a_block);
         for (int rb = 0; rb < row_boxes; ++rb)
           tma_load_2d(sA + (uint32_t)(g4 * cap + slot) * a_block + rb * LP_ROW_BOX, map_of(gate), full_bar(g4, slot), jb * 64,
                       (T - k) * p.B + rb * box_rows);
       };
       auto multiply = [&](int i, int slot, bool first) {
-        const uint64_t ad = make_desc(sA + (uint32_t)(g4 * cap + slot) * a_block, 16, 1024), bd = make_desc(sW + (kb0 + i) * W_BLOCK, 16, 1024);
+        const uint64_t ad = make_desc(sA + (uint32_t)(g4 * cap + slot) * a_block, 16, 1024), bd = make_desc(sW + (kb0 + i) * w_block, 16, 1024);
 #pragma unroll
         for (int s = 0; s < LP_BK / 16; ++s) tc_mma_bf16(d_tmem, ad + 2 * s, bd + 2 * s, idesc, (!first || s != 0) ? 1u : 0u);
       };
@@ -733,128 +830,145 @@ __device__ __forceinline__ void lstm_backward_compact(const LstmBwdParams& p, ui
     const int tid = threadIdx.x;
     const int npairs = p.B * U;  // (batch row, owned unit) pairs; pair q = row * U + kk
     const size_t ldd = (size_t)KH;
+    const int ngroups = (nblk + gsz - 1) / gsz;  // issuing warps with blocks
     float dcreg[PAIRS];
-    int jj[PAIRS];  // kept index of the pair's unit, -1 beyond the kept count or the batch
+    auto row_of = [&](int i) { return (tid + i * LB_MATH) / U; };
+    auto unit_of = [&](int i) { return j0 + (tid + i * LB_MATH) % U; };  // kept index
+    uint32_t own = 0;  // bit i: pair i exists (not beyond the kept count or the batch)
 #pragma unroll
     for (int i = 0; i < PAIRS; ++i) {
-      const int q = tid + i * LB_MATH;
-      const int row = q / U, j = j0 + q % U;
-      jj[i] = (q < npairs && j < n_keep) ? j : -1;
-      dcreg[i] = jj[i] >= 0 && p.dH == nullptr ? p.dc[(size_t)row * p.H + j] : 0.f;
+      if (tid + i * LB_MATH < npairs && unit_of(i) < n_keep) own |= 1u << i;
+      dcreg[i] = (own >> i & 1u) && p.dH == nullptr ? p.dc[(size_t)row_of(i) * p.H + unit_of(i)] : 0.f;
     }
     bool ok = true;
-    for (int k = 0; k <= T && ok; ++k) {
+    for (int k = 0; k <= T; ++k) {
       const int t = T - 1 - k;  // time index whose dh is formed in this round (-1: the gradient of h_0)
-      AdjointIn in[PAIRS];
+      // what does not depend on the recurrence is fetched before the waits
+      Adjoint adj[PAIRS];
 #pragma unroll
-      for (int i = 0; i < PAIRS; ++i) {
-        if (jj[i] >= 0 && t >= 0) {
-          const int row = (tid + i * LB_MATH) / U;
-          fetch_saved(p, t, row, jj[i], in[i]);
-          in[i].up = upstream(p, t, row, bb + jj[i] * dp);
-        }
+      for (int i0 = 0; i0 < PAIRS; i0 += 3) {  // three pairs at a time: what fits the registers
+        AdjointIn in[3];
+#pragma unroll
+        for (int i = i0; i < min(PAIRS, i0 + 3); ++i)
+          if ((own >> i & 1u) && t >= 0) fetch_saved(p, t, row_of(i), unit_of(i), bb + unit_of(i) * dp, in[i - i0]);
+#pragma unroll
+        for (int i = i0; i < min(PAIRS, i0 + 3); ++i)
+          if ((own >> i & 1u) && t >= 0) adj[i] = adjoint_factors(in[i - i0], p.alpha);
       }
-      if (k >= 1) {
-        if (warp < 4) {
-          if (!mbar_wait(tfull_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
-          if (ok) {
+      if (k >= 1 && share > 1) {
+        const uint32_t phase = (uint32_t)(k - 1) & 1u;
+        // j0 < n_keep: this CTA has units (the last ones of a cluster may have none: nobody sends to them)
+        if (tid == 0 && j0 < n_keep) mbar_arrive_expect_tx(pfull_bar, (uint32_t)(parts * p.B * U * 4));
+        if (warp < 8 && (warp & 3) * 32 < p.B && nblk > 0) {
+          if (!mbar_wait(tfull_bar, phase, abort_flag, p.status)) ok = false;
+          if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
-            if (warp * 32 < p.B) {
-              const uint32_t t_row = tmem_base + ((uint32_t)(warp * 32) << 16);
-              const int ngroups = (nblk + gsz - 1) / gsz;
-              uint32_t y[LP_GROUPS][16];
+            const int row = (warp & 3) * 32 + lane;
+            const uint32_t t_row = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll
-              for (int c = 0; c < LP_GROUPS; ++c)
-                if (c < ngroups) tmem_ld16(t_row + (uint32_t)(c * LB_COLS), y[c]);
-              tmem_ld_wait();
-              float* zr = zs + (warp * 32 + lane) * ZS_LD;
+            for (int h = 0; h < LB_CLUSTER / 2; ++h) {  // warps 0-3: the units of CTAs 0 and 1, warps 4-7: of CTAs 2 and 3
+              const int r = (warp >> 2) * (LB_CLUSTER / 2) + h;
+              if (s0 + r * U >= n_keep) break;
+              const uint32_t dst = mapa_u32(sZ + (uint32_t)((rank * p.B + row) * U * 4), (uint32_t)r), bar = mapa_u32(pfull_bar, (uint32_t)r);
 #pragma unroll
-              for (int i = 0; i < U; ++i) {
-                float z = __uint_as_float(y[0][i]);
+              for (int u0 = 0; u0 < U; u0 += GRAN) {
+                float z[GRAN];
+                lstm_sum_groups<GRAN>(t_row + (uint32_t)(r * U + u0), LB_COLS, ngroups, z);
+                if (row < p.B) {
 #pragma unroll
-                for (int c = 1; c < LP_GROUPS; ++c)
-                  if (c < ngroups) z += __uint_as_float(y[c][i]);
-                zr[i] = z;
+                  for (int i = 0; i < GRAN; i += 4) st_async_f4(dst + 4u * (u0 + i), bar, z[i], z[i + 1], z[i + 2], z[i + 3]);
+                }
               }
             }
             tc_fence_before();
           }
         }
-        asm volatile("bar.sync 2, 352;" ::: "memory");
-        if (*abort_flag) { ok = false; break; }
+        if (ok && j0 < n_keep && !mbar_wait_cluster(pfull_bar, phase, abort_flag, p.status)) ok = false;
+      } else if (k >= 1) {
+        if (warp < 4) {
+          if (!mbar_wait(tfull_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
+          if (__all_sync(0xffffffffu, ok)) {
+            tc_fence_after();
+            if (warp * 32 < p.B) {
+              const uint32_t t_row = tmem_base + ((uint32_t)(warp * 32) << 16);
+              float* zr = zs + (warp * 32 + lane) * (U + 1);
+#pragma unroll
+              for (int u0 = 0; u0 < U; u0 += GRAN) {
+                float z[GRAN];
+                lstm_sum_groups<GRAN>(t_row + (uint32_t)u0, LB_COLS, ngroups, z);
+#pragma unroll
+                for (int i = 0; i < GRAN; ++i) zr[u0 + i] = z[i];
+              }
+            }
+            tc_fence_before();
+          }
+        }
+        if (math_barrier_failed<2>(!ok)) { ok = false; break; }
       }
       float total[PAIRS];  // gradient of h_t, also handed back to the caller
 #pragma unroll
       for (int i = 0; i < PAIRS; ++i) {
-        if (jj[i] < 0) continue;
-        const int q = tid + i * LB_MATH;
-        const int row = q / U, j = jj[i];
-        const float rec = k >= 1 ? zs[row * ZS_LD + q % U] : 0.f;
+        if (!(own >> i & 1u)) continue;
+        const int row = row_of(i), j = unit_of(i);
+        float rec = 0.f;
+        if (k >= 1 && share > 1) {
+#pragma unroll
+          for (int r = 0; r < LB_CLUSTER; ++r)  // fixed order: same bits every launch
+            if (r < parts) rec += zs[r * p.B * U + tid + i * LB_MATH];
+        } else if (k >= 1) {
+          rec = zs[row * (U + 1) + j - j0];
+        }
         if (t < 0) {  // gradient of h_0, added to what the caller left in the h half of D[0]
           float* d0 = p.D + (size_t)row * ldd + p.I + bb + j * dp;
           *d0 = p.dH == nullptr ? *d0 + rec : rec;
           continue;
         }
-        total[i] = in[i].up + rec;  // upstream gradient of h_t plus the recurrent part (none at T - 1)
+        total[i] = adj[i].up + rec;  // upstream gradient of h_t plus the recurrent part (none at T - 1)
         __nv_bfloat16 dz[4];
-        cell_adjoint(p, in[i], total[i], dcreg[i], dz);
+        cell_adjoint(adj[i], total[i], dcreg[i], dz);
         store_dz(p.DZ + ((size_t)t * p.B + row) * 4 * p.gs + j, p.gs, dz);
         if (p.DZ_out != nullptr) store_dz(p.DZ_out + ((size_t)t * p.B + row) * 4 * p.H + j, p.H, dz);
       }
       if (t >= 0) {
         // the staged sums may lie in the ring, which the TMA unit overwrites next
         fence_proxy_async_smem();
-        asm volatile("bar.sync 1, 352;" ::: "memory");
+        if (math_barrier_failed<1>(!ok)) { ok = false; break; }
         if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
-        if (t < T - 1) {
+        if (t < T - 1 && p.dH == nullptr) {  // the caller's D holds the totals afterwards
 #pragma unroll
           for (int i = 0; i < PAIRS; ++i)
-            if (jj[i] >= 0) p.D[((size_t)(t + 1) * p.B + (tid + i * LB_MATH) / U) * ldd + p.I + bb + jj[i] * dp] = total[i];
+            if (own >> i & 1u) p.D[((size_t)(t + 1) * p.B + row_of(i)) * ldd + p.I + bb + unit_of(i) * dp] = total[i];
         }
       }
     }
     if (ok) {
 #pragma unroll
       for (int i = 0; i < PAIRS; ++i)
-        if (jj[i] >= 0) p.dc[(size_t)((tid + i * LB_MATH) / U) * p.H + jj[i]] = dcreg[i];
+        if (own >> i & 1u) p.dc[(size_t)row_of(i) * p.H + unit_of(i)] = dcreg[i];
     }
   }
+
 }
 
-// SUMS: the form with partial sums is available too (U = 8).
-template <int U, bool SUMS>
+// U: units per CTA at most; the layer fits the grid with U units per CTA when nothing is dropped.
+template <int U>
 __global__ void __launch_bounds__(LB_THREADS, 1) ard_lstm_backward_kernel(const __grid_constant__ LstmBwdParams p) {
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw_addr = smem_u32(smem_raw);
   const uint32_t base = (raw_addr + 1023u) & ~1023u;
   uint8_t* smem = smem_raw + (base - raw_addr);
-
-  const int KH = p.I + p.H;
-  const int box_rows = lstm_box_rows(p.B), row_boxes = (p.B + 63) / 64;
-  const uint32_t a_block = (uint32_t)lstm_a_block(p.B);
-  // slots' full and free barriers of the compact form, then tfull, hready, wfull, pready, gfull[4]; flags
-  const uint32_t bar_base = base + 8u * (2 * LP_GROUPS * LP_SLOTS);
-  const uint32_t sA = base + LP_BAR_BYTES;                      // LB_MAX_BLOCKS blocks of dz
-  const uint32_t sW = sA + LB_MAX_BLOCKS * a_block;             // LB_MAX_BLOCKS weight boxes (the MMA's 128-row read of
-                                                                 // the last dz block ends inside this region)
-  const uint32_t tfull_bar = bar_base;
-  const uint32_t hready_bar = bar_base + 8u;                     // dz of the previous step is complete
-  const uint32_t wfull_bar = bar_base + 8u * 2;
-  const uint32_t pready_bar = bar_base + 8u * 3;                 // all partial sums of this step are parked
-  auto gfull_bar = [&](int g) { return bar_base + 8u * (4 + g); };
-  uint8_t* misc = smem + (bar_base - base) + 8 * (LP_GROUPS + 4);
+  uint8_t* misc = smem + LB_PFULL + 8;
   volatile uint32_t* tmem_ptr_smem = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
-
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  uint32_t cl;
+  asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cl));
 
   if (threadIdx.x < 2 * LP_GROUPS * LP_SLOTS) mbar_init(base + 8u * threadIdx.x, 1);
   if (threadIdx.x == 0) {
-    for (int g = 0; g < LP_GROUPS; ++g) mbar_init(gfull_bar(g), 1);
-    mbar_init(tfull_bar, LP_GROUPS);
-    mbar_init(wfull_bar, 1);
-    mbar_init(hready_bar, 1);
-    mbar_init(pready_bar, 1);
+    mbar_init(base + LB_TFULL, LP_GROUPS);
+    mbar_init(base + LB_HREADY, 1);
+    mbar_init(base + LB_PFULL, 1);
     *abort_flag = 0;
   }
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -866,227 +980,15 @@ __global__ void __launch_bounds__(LB_THREADS, 1) ard_lstm_backward_kernel(const 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_smem;
+  if (cl > 1) cluster_sync_all();  // every CTA's barriers exist before anyone sends
   pdl_wait_prior_grids();
 
   const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP];
-  // Descriptors of this pattern: slots 0-3 the gates' kept weight rows, 4-7 the gates' compact gradient columns.
-  // Warp 11 writes them (below) before its first arrival on hready_bar; the loading lanes acquire them after
-  // their first wait on that barrier.
-  CUtensorMap* slots = p.tm_slots + (size_t)blockIdx.x * ARD_TM_LSTM_SLOTS;
-  auto map_of = [&](const TcMap* m, int slot) -> const CUtensorMap* { return dp == 1 ? &m->tm : slots + slot; };
-  const int n_cta = (int)gridDim.x;
-  const int s_idx = (int)blockIdx.x / LB_KPARTS, r_idx = (int)blockIdx.x % LB_KPARTS;
-  const int c0 = s_idx * LB_COLS;                       // first weight column (hidden unit) of the slice
-  const int nb = (n_keep + 63) / 64;                    // contraction blocks per gate
-  const int per = (4 * nb + LB_KPARTS - 1) / LB_KPARTS; // blocks per CTA (<= LB_MAX_BLOCKS, checked by the host)
-  const int blk0 = r_idx * per;
-  const int nblk = max(0, min(per, 4 * nb - blk0));     // this CTA's blocks blk0 .. blk0 + nblk - 1; block = gate * nb + jb
-  const int parts = (4 * nb + per - 1) / per;           // CTAs of a slice that have blocks
-  const int gsz = (nblk + LP_GROUPS - 1) / LP_GROUPS;   // blocks per loader / MMA warp
-  const int T = p.T;
-
-  bool compact = p.always_compact || !SUMS;
-  if (!compact && p.compact_ok && dp > 1) {
-    const LstmPlan plan = lstm_plan(4 * nb, lstm_a_block(p.B), lc_w_block(U), LC_TAIL, lc_zs_bytes(U, p.B), p.smem_bytes);
-    compact = LB_ROUNDS * plan.cap >= plan.gsz;
-  }
-  if (compact) {
-    lstm_backward_compact<U>(p, smem, base, tfull_bar, hready_bar, tmem_base, abort_flag, dp, bb, n_keep);
-  } else if (!SUMS) {
-  } else if (warp == 11) {
-    // ===================== weight loader and barrier relay =====================
-    // the weight area, still empty, is the work area of the eight descriptors
-#pragma unroll
-    for (int g = 0; g < 4; ++g) {
-      tensormap_specialise(&p.mapW[g], dp, bb + 1, n_keep, smem + (sW - base) + 128 * g, slots + g, lane);
-      tensormap_specialise(&p.mapDZ[g], dp, bb + 1, n_keep, smem + (sW - base) + 128 * (4 + g), slots + 4 + g, lane);
-    }
-    fence_proxy_async_smem();
-    const int kb = lane;
-    if (kb < nblk) {
-      const int blk = blk0 + kb, g = blk / nb, jb = blk - g * nb;
-      const CUtensorMap* mw = map_of(&p.mapW[g], g);
-      if (dp > 1) tensormap_acquire(mw);
-      if (lane == 0) mbar_arrive_expect_tx(wfull_bar, (uint32_t)nblk * LB_W_BLOCK);
-      __syncwarp(__activemask());
-      tma_load_2d(sW + kb * LB_W_BLOCK, mw, wfull_bar, p.I + c0, jb * 64);
-    }
-    __syncwarp();
-    if (lane == 0) {
-      for (int ph = 1; ph <= 2 * T; ++ph) {
-        if (!grid_wait(p.bar, (unsigned)ph * (unsigned)n_cta, abort_flag, p.status)) break;
-        mbar_arrive((ph & 1) ? hready_bar : pready_bar);
-      }
-    }
-  } else if (warp >= 12) {
-    // ===================== loaders and MMA issuers (group g = warp - 12) =====================
-    const int g4 = warp - 12;
-    const int kb0 = g4 * gsz, kb1 = min(nblk, kb0 + gsz);
-    const int kb = kb0 + lane;
-    const bool mine = kb < kb1;
-    int gate = 0, jb = 0;
-    if (mine) {
-      const int blk = blk0 + kb;
-      gate = blk / nb;
-      jb = blk - gate * nb;
-    }
-    const CUtensorMap* mdz = map_of(&p.mapDZ[gate], 4 + gate);
-    const uint32_t idesc = make_idesc(LB_COLS, false, true, 128);
-    bool ok = (lane != 0) || nblk == 0 || mbar_wait(wfull_bar, 0u, abort_flag, p.status);
-    for (int k = 1; k <= T; ++k) {
-      // dz of time index T - k is complete
-      if (ok && !mbar_wait(hready_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
-      if (!__all_sync(0xffffffffu, ok)) break;
-      if (k == 1 && mine && dp > 1) tensormap_acquire(mdz);  // written by warp 11 ahead of its first arrival on hready_bar
-      if (kb0 < kb1) {
-        asm volatile("fence.proxy.async.global;" ::: "memory");  // generic-proxy stores of other CTAs -> TMA reads
-        if (lane == 0) mbar_arrive_expect_tx(gfull_bar(g4), (uint32_t)(kb1 - kb0) * a_block);
-        __syncwarp();
-        if (mine)
-          for (int rb = 0; rb < row_boxes; ++rb)
-            tma_load_2d(sA + kb * a_block + rb * LP_ROW_BOX, mdz, gfull_bar(g4), jb * 64,
-                        (T - k) * p.B + rb * box_rows);
-        if (lane == 0) {
-          if (!mbar_wait(gfull_bar(g4), (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
-          if (ok) {
-            tc_fence_after();
-            const uint32_t d_tmem = tmem_base + (uint32_t)(g4 * LB_COLS);
-            for (int k2 = kb0; k2 < kb1; ++k2) {
-              const uint32_t a0 = sA + k2 * a_block, b0 = sW + k2 * LB_W_BLOCK;
-#pragma unroll
-              for (int s = 0; s < LP_BK / 16; ++s)  // A K-major: 32 bytes per step; B MN-major: 16 k-rows = 2048 bytes
-                tc_mma_bf16(d_tmem, make_desc(a0 + s * 32, 16, 1024), make_desc(b0 + s * 2048, 64 * LP_BK * 2, 1024), idesc,
-                            (k2 != kb0 || s != 0) ? 1u : 0u);
-            }
-          }
-        }
-      }
-      if (lane == 0 && ok && nblk > 0) {
-        if (kb0 < kb1) tc_commit(tfull_bar);
-        else mbar_arrive(tfull_bar);
-      }
-      __syncwarp();
-    }
-  } else {
-    // ===================== partial sums and cell adjoint (warps 0-10) =====================
-    const int tid = threadIdx.x;  // 0 .. LB_MATH-1
-    const int npairs = p.B * LB_OWN;  // (batch row, owned column) pairs; pair q = row * 8 + cc
-    const size_t ldd = (size_t)KH;
-    float dcreg[LB_PAIRS_MAX];
-    int jj[LB_PAIRS_MAX];  // kept index of the pair's unit, -1 if the column is a dropped unit or out of range
-#pragma unroll
-    for (int i = 0; i < LB_PAIRS_MAX; ++i) {
-      const int q = tid + i * LB_MATH;
-      const int row = q >> 3, u = c0 + r_idx * LB_OWN + (q & 7);
-      const int rel = u - bb;
-      jj[i] = (q < npairs && u < p.H && rel >= 0 && rel % dp == 0) ? rel / dp : -1;
-      dcreg[i] = jj[i] >= 0 && p.dH == nullptr ? p.dc[(size_t)row * p.H + jj[i]] : 0.f;
-    }
-    float* my_partial = p.partial + (size_t)blockIdx.x * 128 * LB_COLS;
-    const float* slice_partial = p.partial + (size_t)(s_idx * LB_KPARTS) * 128 * LB_COLS;
-    bool ok = true;
-    for (int k = 0; k <= T && ok; ++k) {
-      const int t = T - 1 - k;  // time index whose dh is formed in this round (-1: the gradient of h_0)
-      // what does not depend on the recurrence is fetched before the waits: gate activations, cell states
-      AdjointIn in[LB_PAIRS_MAX];
-#pragma unroll
-      for (int i = 0; i < LB_PAIRS_MAX; ++i)
-        if (jj[i] >= 0 && t >= 0) fetch_saved(p, t, (tid + i * LB_MATH) >> 3, jj[i], in[i]);
-      if (k >= 1) {
-        // ---- phase A: park this CTA's partial sums ----
-        // Every CTA passes the previous phase before it arrives for this one, also a CTA that has no
-        // contraction blocks: the arrival count identifies a phase only if nobody is two arrivals ahead.
-        if (!mbar_wait(hready_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
-        if (ok && warp < 4 && nblk > 0) {
-          if (!mbar_wait(tfull_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
-          if (ok) {
-            tc_fence_after();
-            const int row = warp * 32 + lane;
-            const uint32_t t_row = tmem_base + ((uint32_t)(warp * 32) << 16);
-            const int ngroups = (nblk + gsz - 1) / gsz;
-#pragma unroll 1
-            for (int half = 0; half < 2; ++half) {
-              uint32_t z[32], y[32];
-              tmem_ld32(t_row + (uint32_t)(half * 32), z);
-              tmem_ld_wait();
-              for (int c = 1; c < ngroups; ++c) {
-                tmem_ld32(t_row + (uint32_t)(c * LB_COLS + half * 32), y);
-                tmem_ld_wait();
-#pragma unroll
-                for (int i = 0; i < 32; ++i) z[i] = __float_as_uint(__uint_as_float(z[i]) + __uint_as_float(y[i]));
-              }
-              if (row < p.B) {
-                float4* dst = reinterpret_cast<float4*>(my_partial + (size_t)row * LB_COLS + half * 32);
-#pragma unroll
-                for (int i = 0; i < 8; ++i)
-                  __stcg(dst + i, make_float4(__uint_as_float(z[4 * i]), __uint_as_float(z[4 * i + 1]),
-                                              __uint_as_float(z[4 * i + 2]), __uint_as_float(z[4 * i + 3])));
-              }
-            }
-            tc_fence_before();
-          }
-        }
-        asm volatile("bar.sync 1, 352;" ::: "memory");
-        if (*abort_flag) { ok = false; break; }
-        if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
-        // ---- all partial sums of the slice are parked ----
-        if (!mbar_wait(pready_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
-        asm volatile("bar.sync 2, 352;" ::: "memory");
-        if (*abort_flag) { ok = false; break; }
-      }
-      // ---- phase B: total gradient of h_t, cell adjoint, dz_t ----
-      // All loads of all owned (row, unit) pairs are issued before the first is consumed: the partial sums
-      // come from L2 and a chain of dependent round trips would cost more than the whole product.
-      float total[LB_PAIRS_MAX];  // recurrent part, then the gradient of h_t, also handed back to the caller
-#pragma unroll
-      for (int i = 0; i < LB_PAIRS_MAX; ++i) {
-        total[i] = 0.f;
-        if (jj[i] < 0) continue;
-        const int q = tid + i * LB_MATH;
-        const int row = q >> 3, cc = r_idx * LB_OWN + (q & 7), u = c0 + cc;
-        float part[LB_KPARTS];
-#pragma unroll
-        for (int rp = 0; rp < LB_KPARTS; ++rp)
-          part[rp] = (k >= 1 && rp < parts) ? __ldcg(slice_partial + ((size_t)rp * 128 + row) * LB_COLS + cc) : 0.f;
-        in[i].up = t >= 0 ? upstream(p, t, row, u) : 0.f;
-        float rec = 0.f;
-#pragma unroll
-        for (int rp = 0; rp < LB_KPARTS; ++rp) rec += part[rp];  // fixed order: same bits every launch
-        total[i] = rec;
-      }
-#pragma unroll
-      for (int i = 0; i < LB_PAIRS_MAX; ++i) {
-        if (jj[i] < 0) continue;
-        const int q = tid + i * LB_MATH;
-        const int row = q >> 3, u = c0 + r_idx * LB_OWN + (q & 7), j = jj[i];
-        if (t < 0) {  // gradient of h_0, added to what the caller left in the h half of D[0]
-          float* d0 = p.D + (size_t)row * ldd + p.I + u;
-          *d0 = p.dH == nullptr ? *d0 + total[i] : total[i];
-          continue;
-        }
-        total[i] += in[i].up;  // upstream gradient of h_t plus the recurrent part (none at T - 1)
-        __nv_bfloat16 dz[4];
-        cell_adjoint(p, in[i], total[i], dcreg[i], dz);
-        store_dz(p.DZ + ((size_t)t * p.B + row) * 4 * p.gs + j, p.gs, dz);
-        if (p.DZ_out != nullptr) store_dz(p.DZ_out + ((size_t)t * p.B + row) * 4 * p.H + j, p.H, dz);
-      }
-      if (t >= 0) {
-        asm volatile("bar.sync 1, 352;" ::: "memory");
-        if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
-        if (t < T - 1) {
-#pragma unroll
-          for (int i = 0; i < LB_PAIRS_MAX; ++i)
-            if (jj[i] >= 0)
-              p.D[((size_t)(t + 1) * p.B + ((tid + i * LB_MATH) >> 3)) * ldd + p.I + c0 + r_idx * LB_OWN + ((tid + i * LB_MATH) & 7)] = total[i];
-        }
-      }
-    }
-    if (ok) {
-#pragma unroll
-      for (int i = 0; i < LB_PAIRS_MAX; ++i)
-        if (jj[i] >= 0) p.dc[(size_t)((tid + i * LB_MATH) >> 3) * p.H + jj[i]] = dcreg[i];
-    }
-  }
+  const int ctas = (int)gridDim.x;
+  // as few units per CTA as the grid allows (see the forward kernel; 64 rows, 512 kept: 4.9 us per step with 8, 4.2 with 4)
+  if (n_keep <= 4 * ctas) lstm_backward_body<4>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
+  else if (U == 8 || n_keep <= 8 * ctas) lstm_backward_body<8>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
+  else lstm_backward_body<U>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
 
   // ---- teardown ----
   tc_fence_before();
@@ -1098,6 +1000,8 @@ __global__ void __launch_bounds__(LB_THREADS, 1) ard_lstm_backward_kernel(const 
     tc_fence_after();
     tmem_dealloc(tmem_base, LP_GROUPS * LB_COLS);
   }
+  __syncwarp();
+  if (cl > 1) cluster_sync_all();  // nobody leaves while its peers may still send to it
 }
 
 }  // namespace
@@ -1115,8 +1019,9 @@ int lstm_fwd_smem_bytes(int B, int H, int U) {
   const int N = 4 * U;
   return lstm_smem_bytes((H + LP_BK - 1) / LP_BK, B, N * LP_BK * 2, 0, (B + 31) / 32 * 32 * (N + 1) * 4);
 }
-int lstm_bwd_compact_smem_bytes(int B, int n, int U) {
-  return lstm_smem_bytes(4 * ((n + 63) / 64), B, lc_w_block(U), LC_TAIL, lc_zs_bytes(U, B));
+int lstm_bwd_smem_bytes(int B, int H, int U, int cl) {
+  const LstmPlan r = lb_plan(4 * ((H + 63) / 64), B, U, cl, LP_SMEM_MAX);
+  return r.cap < 1 ? LP_SMEM_MAX + 1 : 1024 + LP_BAR_BYTES + r.bytes;
 }
 
 // A kernel's dynamic shared memory limit raised once per device; false where that fails.
@@ -1130,17 +1035,21 @@ bool lstm_probe(const ard_ctx* ctx, K kern, int* probed) {
 // ARD_ERR_UNSUPPORTED (nothing enqueued) when the device cannot hold all CTAs at once right now (SMs taken by another
 // context, a smaller partition).
 template <typename K, typename P>
-ard_status lstm_launch(ard_ctx* ctx, K kern, int grid, int smem, const P& p, cudaStream_t s) {
+ard_status lstm_launch(ard_ctx* ctx, K kern, int cluster, int grid, int smem, const P& p, cudaStream_t s) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(LP_THREADS);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeCooperative;  // all CTAs resident: they wait for one another
   attr[0].val.cooperative = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = cluster;
+  attr[1].val.clusterDim.y = 1;
+  attr[1].val.clusterDim.z = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   const cudaError_t err = cudaLaunchKernelEx(&cfg, kern, p);
   if (err == cudaErrorCooperativeLaunchTooLarge || err == cudaErrorLaunchOutOfResources) {
     (void)cudaGetLastError();
@@ -1169,7 +1078,7 @@ bool lstm_persistent_fits(ard_ctx* ctx, int B, int H, bool tma) {
 
 // tma: mapXH and mapW describe the operands (U = 8 only); otherwise they are not read and the compact form runs always.
 // 35 steps, batch 20, 1500 -> 1500 units at a period of 2, forward and backward: 3.47 ms step by step with the products of
-// gemm_ldg_sm100.cu.
+// gemm_ldg_sm100.cu, 0.45 ms with the whole-sequence kernels.
 ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, int add_zx, float alpha,
                                           const TcMap* mapXH, const TcMap* mapW, const TcMap* mapHc, const void* W, int ldw, void* XH,
                                           const float* bias, float* C, float* G, cudaStream_t s) {
@@ -1196,50 +1105,55 @@ ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, 
   p.bar = ctx->d_grid_bar + LP_BAR_WORD;
   p.status = ctx->d_status;
   p.smem_bytes = lstm_fwd_smem_bytes(B, H, U);
-  // Sized for dp = 1.  Under a period of 2 or more at least one CTA has no units: it writes the zeros of dropped ones.
-  const int grid = H > U ? (H + U - 1) / U : 2;
+  const int grid = (H + U - 1) / U;  // sized for dp = 1
   static int probed[2][64] = {};
   if (U == 8) {
     if (!lstm_probe(ctx, ard_lstm_forward_kernel<8>, probed[0])) return ARD_ERR_UNSUPPORTED;
-    return lstm_launch(ctx, ard_lstm_forward_kernel<8>, grid, p.smem_bytes, p, s);
+    return lstm_launch(ctx, ard_lstm_forward_kernel<8>, 1, grid, p.smem_bytes, p, s);
   }
   if (!lstm_probe(ctx, ard_lstm_forward_kernel<12>, probed[1])) return ARD_ERR_UNSUPPORTED;
-  return lstm_launch(ctx, ard_lstm_forward_kernel<12>, grid, p.smem_bytes, p, s);
+  return lstm_launch(ctx, ard_lstm_forward_kernel<12>, 1, grid, p.smem_bytes, p, s);
 }
 
 // ---- whole-sequence BPTT recurrence ----
-// Shared memory of the kernel with both forms.  The form is chosen on the device from the drawn pattern, so the launch
-// asks for what either may need: 8 row blocks and 8 weight boxes behind the barriers for the form with partial sums,
-// and below LB_SMEM_BYTES what the compact form can use.
-static int lstm_bwd_sums_smem_bytes(int B) {
-  static_assert((size_t)LB_MAX_BLOCKS * 2 * LP_ROW_BOX + (size_t)LB_MAX_BLOCKS * LB_W_BLOCK + LP_BAR_BYTES + 1024 <= LP_SMEM_MAX,
-                "the form with partial sums does not fit");
-  return LB_MAX_BLOCKS * lstm_a_block(B) + LB_MAX_BLOCKS * LB_W_BLOCK + LP_BAR_BYTES + 1024;
+namespace {
+struct LstmBwdForm {
+  int U, cl;  // units per CTA, cluster size; U == 0: the layer does not fit
+  int smem;
+};
+}  // namespace
+
+// In clusters while all CTAs of a dense draw can be resident that way, 8 units per CTA rather than 12; else without.
+static LstmBwdForm lstm_bwd_form(ard_ctx* ctx, int B, int H) {
+  static int probed[2][64] = {}, room[2][64] = {};
+  const int dev = ctx->device & 63;
+  for (int i = 0; i < 4; ++i) {
+    const int u = i & 1, U = u ? 12 : 8, cl = i < 2 ? LB_CLUSTER : 1;
+    auto kern = u ? ard_lstm_backward_kernel<12> : ard_lstm_backward_kernel<8>;
+    if (!lstm_probe(ctx, kern, probed[u])) continue;
+    int have = ctx->sm_count;
+    if (cl > 1) {
+      if (room[u][dev] == 0) room[u][dev] = ard_cluster_room(ctx, kern, cl, LB_THREADS, LP_SMEM_MAX);
+      have = room[u][dev];
+    }
+    const int grid = ((H + U - 1) / U + cl - 1) / cl * cl, smem = lstm_bwd_smem_bytes(B, H, U, cl);
+    if (grid <= have && grid <= ARD_TM_LSTM_BLOCKS && smem <= LP_SMEM_MAX) return LstmBwdForm{U, cl, smem};
+  }
+  return LstmBwdForm{0, 0, 0};
 }
 
-size_t lstm_bwd_partial_bytes(int sm_count) { return (size_t)sm_count * 128 * LB_COLS * sizeof(float); }
-
-// The form with partial sums needs descriptors of the weight (tma) and at most 8 contraction blocks per CTA.
-static bool lstm_bwd_sums_fits(const ard_ctx* ctx, int H, bool tma) {
-  return tma && H <= 1024 && ctx->d_lstm_partial != nullptr && (H + LB_COLS - 1) / LB_COLS * LB_KPARTS <= ctx->sm_count;
-}
-
-bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H, bool tma) {
-  if (B < 1 || B > 128 || H < 1) return false;
-  if (lstm_bwd_sums_fits(ctx, H, tma)) return true;
-  const int U = lstm_units(H, ctx->sm_count);
-  if ((H + U - 1) / U > ctx->sm_count || (H + U - 1) / U > ARD_TM_LSTM_BLOCKS || !ctx->lstm_compact_h) return false;
-  return lstm_bwd_compact_smem_bytes(B, H, U) <= LP_SMEM_MAX;
+bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H) {
+  return B >= 1 && B <= 128 && H >= 1 && lstm_bwd_form(ctx, B, H).U != 0;
 }
 
 ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
-                                           const TcMap mapDZ[4], const TcMap* mapW, const void* W, int ldw, const float* C,
-                                           const float* G, const float* dH, const float* dH_last, float* D, float* dc, void* DZ, int gs,
+                                           const TcMap mapDZ[4], const void* W, int ldw, const float* C, const float* G,
+                                           const float* dH, const float* dH_last, float* D, float* dc, void* DZ, int gs,
                                            void* DZ_out, cudaStream_t s) {
+  const LstmBwdForm f = lstm_bwd_form(ctx, B, H);
+  if (f.U == 0) return ARD_ERR_UNSUPPORTED;
   LstmBwdParams p = {};
-  const bool sums = lstm_bwd_sums_fits(ctx, H, mapW != nullptr);
-  const int U = sums ? 8 : lstm_units(H, ctx->sm_count);
-  for (int g = 0; g < 4; ++g) { p.mapDZ[g] = mapDZ[g]; p.mapW[g] = mapW ? mapW[g] : mapDZ[g]; }
+  for (int g = 0; g < 4; ++g) p.mapDZ[g] = mapDZ[g];
   p.tm_slots = ctx->d_tm_slots + (size_t)ARD_TM_SM_MAX * ARD_TM_SLOTS;
   p.hdr = pat->d_hdr;
   p.T = T; p.B = B; p.I = I; p.H = H;
@@ -1248,30 +1162,12 @@ ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat,
   p.DZ = reinterpret_cast<__nv_bfloat16*>(DZ);
   p.gs = gs;
   p.DZ_out = reinterpret_cast<__nv_bfloat16*>(DZ_out);
-  p.partial = ctx->d_lstm_partial;
   p.bar = ctx->d_grid_bar + LP_BAR_WORD;
   p.status = ctx->d_status;
   p.W = reinterpret_cast<const __nv_bfloat16*>(W);
   p.ldw = ldw;
-  p.compact_ok = ctx->lstm_compact_h;
-  p.always_compact = !sums;
-  static int probed[3][64] = {};
-  if (sums) {
-    p.smem_bytes = lstm_bwd_sums_smem_bytes(B);
-    // the compact form of as many kept units as fit below the carve-out step (see LB_SMEM_BYTES)
-    for (int nb = 1; p.compact_ok && pat->dp_bound > 1 && nb <= (H / 2 + 63) / 64; ++nb) {
-      const int c = lstm_bwd_compact_smem_bytes(B, 64 * nb, 8);
-      if (c > LB_SMEM_BYTES) break;
-      if (c > p.smem_bytes) p.smem_bytes = c;
-    }
-    if (!lstm_probe(ctx, ard_lstm_backward_kernel<8, true>, probed[0])) return ARD_ERR_UNSUPPORTED;
-    return lstm_launch(ctx, ard_lstm_backward_kernel<8, true>, (H + LB_COLS - 1) / LB_COLS * LB_KPARTS, p.smem_bytes, p, s);
-  }
-  p.smem_bytes = lstm_bwd_compact_smem_bytes(B, H, U);
-  if (U == 8) {
-    if (!lstm_probe(ctx, ard_lstm_backward_kernel<8, false>, probed[1])) return ARD_ERR_UNSUPPORTED;
-    return lstm_launch(ctx, ard_lstm_backward_kernel<8, false>, (H + U - 1) / U, p.smem_bytes, p, s);
-  }
-  if (!lstm_probe(ctx, ard_lstm_backward_kernel<12, false>, probed[2])) return ARD_ERR_UNSUPPORTED;
-  return lstm_launch(ctx, ard_lstm_backward_kernel<12, false>, (H + U - 1) / U, p.smem_bytes, p, s);
+  p.whole_ok = ctx->lstm_compact_h || f.cl == 1;
+  p.smem_bytes = f.smem;
+  const int grid = ((H + f.U - 1) / f.U + f.cl - 1) / f.cl * f.cl;
+  return lstm_launch(ctx, f.U == 8 ? ard_lstm_backward_kernel<8> : ard_lstm_backward_kernel<12>, f.cl, grid, f.smem, p, s);
 }

@@ -1,6 +1,7 @@
 """Whole-sequence LSTM kernels on layers off the 16-byte grid and of more than 8 units per SM, forward and backward against
-the oracle: gate blocks, h columns and rows at every phase, a ring of slots that is re-used within a step, 12 units per
-CTA, one and two row boxes; and a layer whose backward pass does not fit and runs step by step."""
+the oracle: gate blocks, h columns and rows at every phase, a ring of slots that is re-used within a step, 4, 8 and 12 units
+per CTA, shared and whole contractions of the gradients (clusters of CTAs with units for some of them only, a layer whose
+CTAs do not fit the device in clusters), one and two row boxes; and a layer whose backward pass does not fit and runs step by step."""
 import numpy as np
 import pytest
 import torch
@@ -16,9 +17,11 @@ pytestmark = pytest.mark.gpu
 BF = torch.bfloat16
 
 
-# (KH % 8 == 0, H % 8 == 4), odd everything, H % 4 == 2, > 1024 units at one and two row boxes, > 1184 units (12 per CTA)
+# (KH % 8 == 0, H % 8 == 4), odd everything, H % 4 == 2, > 1024 units at one and two row boxes, > 1184 units (12 per CTA),
+# does not fit; few CTAs, not a multiple of a cluster, two CTAs, more CTAs than clusters of them fit
 @pytest.mark.parametrize("T,B,I,H,fits", [(4, 20, 52, 204, 1), (3, 33, 57, 131, 1), (3, 8, 64, 98, 1), (3, 70, 36, 1100, 1),
-                                          (3, 128, 64, 1096, 1), (3, 20, 300, 1500, 1), (2, 100, 44, 1500, 0)])
+                                          (3, 128, 64, 1096, 1), (3, 20, 300, 1500, 1), (2, 100, 44, 1500, 0),
+                                          (4, 9, 24, 40, 1), (3, 40, 24, 604, 1), (3, 5, 16, 12, 1), (2, 8, 40, 1600, 1)])
 def test_any_shape_matches_the_oracle(T, B, I, H, fits):
     rng = np.random.default_rng(T * 100 + B + H)
     W = inputs.bf16_round(rng.uniform(-0.06, 0.06, size=(I + H, 4 * H)).astype(np.float32))
