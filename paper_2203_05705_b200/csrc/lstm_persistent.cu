@@ -15,7 +15,7 @@
 //   - per step it loads h_{t-1} (TMA boxes of up to 64 rows x 64 columns) into a ring of slots, one quarter of the
 //     blocks per loading warp.  Usually every block of a step has a slot of its own, so all loads of a step are in
 //     flight together; a slice so large that fewer slots fit re-uses them within the step.  The warp that loads a
-//     quarter also issues its products (tcgen05.mma, M = 128, N = 4 U, accumulators in tensor memory,
+//     quarter also issues its products (tcgen05.mma, M = 64 or 128, N = 4 U, accumulators in tensor memory,
 //     double-buffered over steps): one thread issuing box after box paces at ~410 SM cycles per box, the lanes of a
 //     warp ~70 cycles apart, and a tcgen05.mma this narrow costs its issuing thread ~110 cycles;
 //   - the accumulator rows move to shared memory, then all 11 compute warps apply the cell
@@ -83,6 +83,11 @@ __host__ __device__ inline LstmPlan lstm_plan(int blocks, int a_block, int w_blo
   r.bytes = LP_GROUPS * r.cap * a_block + r.behind + (r.zs_shared ? 0 : zs);
   return r;
 }
+
+// Rows of the products: an instruction of 64 reads half as much of the activations' slots as one of 128, and that is what
+// paces these narrow products (us per step, forward / BPTT: 20 rows, 512 of 1024 units kept, 3.65 / 3.86 with 128, 3.48 /
+// 3.65 with 64; 64 rows 4.02 / 4.20 and 3.95 / 4.10).  Its accumulator has 16 rows in each 32 lanes of tensor memory.
+__host__ __device__ inline int lstm_mma_rows(int B) { return B <= 64 ? 64 : 128; }
 
 struct LstmFwdParams {
   TcMap mapXH;    // [(T+1)*B][I+H], boxes of box_rows x 64 columns (used as encoded; not by the compact form)
@@ -319,7 +324,7 @@ __device__ __forceinline__ void lstm_forward_body(const LstmFwdParams& p, uint8_
       const int g = warp - 12;
       const int kb0 = g * gsz, n = max(0, min(nkb - kb0, gsz));
       const CUtensorMap* mapXH = compact ? &p.mapHc.tm : &p.mapXH.tm;  // kernel parameters, used as encoded
-      const uint32_t idesc = make_idesc(N, false, false, 128);
+      const uint32_t idesc = make_idesc(N, false, false, lstm_mma_rows(p.B));
       bool ok = (lane != 0) || mbar_wait(wfull_bar, 0u, abort_flag, p.status);
       for (int t = 0; t < p.T; ++t) {
         const int acc = t & 1;
@@ -356,6 +361,7 @@ __device__ __forceinline__ void lstm_forward_body(const LstmFwdParams& p, uint8_
       const size_t ldxh = (size_t)KH;
       const int npairs = p.B * U;                    // (batch row, unit) pairs of this CTA; pair q = row * U + k
       const int nvalid = min(U, n_keep - j0);        // units this CTA really owns (>= 1)
+      const int qrows = lstm_mma_rows(p.B) / 4;      // batch rows in each 32 lanes of tensor memory
       float creg[PAIRS];
 #pragma unroll
       for (int i = 0; i < PAIRS; ++i) {
@@ -416,17 +422,19 @@ __device__ __forceinline__ void lstm_forward_body(const LstmFwdParams& p, uint8_
           if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
             const int quadrant = warp & 3;
-            if (quadrant * 32 < p.B) {
+            if (quadrant * qrows < p.B) {
               const uint32_t t_row = tmem_base + ((uint32_t)(quadrant * 32) << 16) + (uint32_t)(acc * LP_GROUPS * N);
               const int ngroups = (nkb + gsz - 1) / gsz;  // accumulators that received MMAs
-              float* zr = zs + (quadrant * 32 + lane) * ZS_LD;
+              float* zr = zs + (quadrant * qrows + lane) * ZS_LD;
 #pragma unroll
               for (int i0 = 0; i0 < N / 2; i0 += 8) {
                 const int c0 = (warp >> 2) * (N / 2) + i0;
                 float z[8];
                 lstm_sum_groups<8>(t_row + (uint32_t)c0, N, ngroups, z);
+                if (lane < qrows) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) zr[c0 + i] = z[i];
+                  for (int i = 0; i < 8; ++i) zr[c0 + i] = z[i];
+                }
               }
             }
             tc_fence_before();
@@ -556,7 +564,7 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
 // which is what bounds a step then.  So CTAs work in clusters of LB_CLUSTER: the cluster owns LB_CLUSTER * U units and
 // CTA r contracts the r-th share of the blocks of 64 gate rows for all of them.  A step is
 //   1. dz_{t+1} is complete (grid barrier, relayed): TMA-load this CTA's blocks of it into the ring of slots of the
-//      forward kernel and multiply (tcgen05.mma M = 128, N = LB_CLUSTER * U, four issuing warps with an accumulator
+//      forward kernel and multiply (tcgen05.mma M = 64 or 128, N = LB_CLUSTER * U, four issuing warps with an accumulator
 //      each) by the resident weight slice: the fan-out weights of the cluster's units, [units][gate rows] (K-major),
 //      gathered by the kernel once per sequence;
 //   2. send the sums of every CTA's units to that CTA's shared memory (st.async: the bytes themselves complete the
@@ -571,9 +579,9 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
 // scratch where the caller's rows are off the 16-byte grid.
 // The grid barrier is one arrival counter: every CTA that takes part arrives once per step, after all of its stores.
 // us per step, before (partial sums through global memory and a second grid barrier, or whole contractions in every CTA;
-// the cell adjoint formed behind the wait; 8 units per CTA) and now: 64 rows, 512 of 1024 units kept 7.4 -> 4.2, all
-// kept 8.6 -> 6.3; 128 rows, 512 of 1024 kept 10.1 -> 5.6; 20 rows, 750 of 1500 kept 9.7 -> 4.9, all kept 25.4 -> 7.5.
-// About 2.9 of it are what a step of any size costs: stores, barrier, TMA, a few narrow MMAs, the exchange.
+// the cell adjoint formed behind the wait; 8 units per CTA) and now: 64 rows, 512 of 1024 units kept 7.4 -> 4.1, all
+// kept 8.6 -> 6.1; 128 rows, 512 of 1024 kept 10.1 -> 5.6; 20 rows, 750 of 1500 kept 9.7 -> 4.8, all kept 25.4 -> 7.3.
+// About 2.8 of it are what a step of any size costs: stores, barrier, TMA, a few narrow MMAs, the exchange.
 constexpr int LB_CLUSTER = 4;     // of 148 SMs 132 can be used by clusters of 4, 120 by clusters of 8
 constexpr int LB_COLS = 64;       // tensor-memory columns of an issuing warp's accumulator (at most LB_CLUSTER * 12 used)
 constexpr int LB_THREADS = 512;   // warps 0-10 adjoint (0-7 also read TMEM), 11 relay, 12-15 load + MMA
@@ -794,7 +802,7 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
     const int kb0 = g4 * gsz, n = max(0, min(nblk - kb0, gsz));
     // where dp == 1 the descriptors are used as encoded (tensormap_specialise returns the parameter)
     auto map_of = [&](int gate) -> const CUtensorMap* { return dp == 1 ? &p.mapDZ[gate].tm : slots + gate; };
-    const uint32_t idesc = make_idesc(share > 1 ? LB_CLUSTER * U : LC_N, false, false, 128);
+    const uint32_t idesc = make_idesc(share > 1 ? LB_CLUSTER * U : LC_N, false, false, lstm_mma_rows(p.B));
     const uint32_t d_tmem = tmem_base + (uint32_t)(g4 * LB_COLS);
     bool ok = true;
     for (int k = 1; k <= T; ++k) {
@@ -831,6 +839,7 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
     const int npairs = p.B * U;  // (batch row, owned unit) pairs; pair q = row * U + kk
     const size_t ldd = (size_t)KH;
     const int ngroups = (nblk + gsz - 1) / gsz;  // issuing warps with blocks
+    const int qrows = lstm_mma_rows(p.B) / 4;    // batch rows in each 32 lanes of tensor memory
     float dcreg[PAIRS];
     auto row_of = [&](int i) { return (tid + i * LB_MATH) / U; };
     auto unit_of = [&](int i) { return j0 + (tid + i * LB_MATH) % U; };  // kept index
@@ -859,11 +868,11 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
         const uint32_t phase = (uint32_t)(k - 1) & 1u;
         // j0 < n_keep: this CTA has units (the last ones of a cluster may have none: nobody sends to them)
         if (tid == 0 && j0 < n_keep) mbar_arrive_expect_tx(pfull_bar, (uint32_t)(parts * p.B * U * 4));
-        if (warp < 8 && (warp & 3) * 32 < p.B && nblk > 0) {
+        if (warp < 8 && (warp & 3) * qrows < p.B && nblk > 0) {
           if (!mbar_wait(tfull_bar, phase, abort_flag, p.status)) ok = false;
           if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
-            const int row = (warp & 3) * 32 + lane;
+            const int row = lane < qrows ? (warp & 3) * qrows + lane : p.B;
             const uint32_t t_row = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
 #pragma unroll
             for (int h = 0; h < LB_CLUSTER / 2; ++h) {  // warps 0-3: the units of CTAs 0 and 1, warps 4-7: of CTAs 2 and 3
@@ -889,15 +898,16 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
           if (!mbar_wait(tfull_bar, (uint32_t)(k - 1) & 1u, abort_flag, p.status)) ok = false;
           if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
-            if (warp * 32 < p.B) {
+            if (warp * qrows < p.B) {
               const uint32_t t_row = tmem_base + ((uint32_t)(warp * 32) << 16);
-              float* zr = zs + (warp * 32 + lane) * (U + 1);
+              float* zr = zs + (warp * qrows + lane) * (U + 1);
 #pragma unroll
               for (int u0 = 0; u0 < U; u0 += GRAN) {
                 float z[GRAN];
                 lstm_sum_groups<GRAN>(t_row + (uint32_t)u0, LB_COLS, ngroups, z);
 #pragma unroll
-                for (int i = 0; i < GRAN; ++i) zr[u0 + i] = z[i];
+                for (int i = 0; i < GRAN; ++i)
+                  if (lane < qrows) zr[u0 + i] = z[i];
               }
             }
             tc_fence_before();
