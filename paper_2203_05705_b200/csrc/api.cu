@@ -752,7 +752,8 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
   g.out_is_f32 = dW_dtype == ARD_F32;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
   if (in_pat && zero_fill_dropped) return ARD_ERR_INVALID_ARG;  // the packed gradient has no rows of dropped neurons
-  // The kernels write the zeros of dropped rows themselves, those of dropped pattern tiles are written first.
+  // The kernels write the zeros of dropped rows themselves; those of dropped pattern tiles are written first, except by
+  // the class form of the tensor-core kernels.
   const bool zero_tiles = pat->kind == ARD_TILE && zero_fill_dropped;
   // Empty batch: the gradient of every kept weight is zero; the CUDA-core kernel writes exactly that.
   if (B == 0 && zero_tiles) {
@@ -789,7 +790,7 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     st = get_maps(ctx, dyc, B, N, ldc, N, MAP_COMPACT_COLS, pat->dp_bound, 64, 64, &t.mapA, dense, dense_ld);
     t.mapA_indexed = 1;
   } else {
-    if (zero_fill_dropped) {
+    if (zero_fill_dropped && t.bn != 0) {  // the class form (0) writes them itself
       st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
       if (st != ARD_OK) return st;
     }
