@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(MP_THREADS, 1) ard_mlp_persistent_kernel(const
     } else if (warp <= MP_NI) {
       // ===================== MMA issuers: warp 1 + w takes blocks w, w + NI, ... of a tile =====================
       const int w = warp - 1;
-      {
+      if (lane == 0) {
         bool ok = true;
 #pragma unroll 1
         for (int q = 0; q < njobs && ok; ++q) {
@@ -775,35 +775,29 @@ __global__ void __launch_bounds__(MP_THREADS, 1) ard_mlp_persistent_kernel(const
 #pragma unroll 1
           for (int ti = 0; ti < j.mine && ok; ++ti, ++git, gblk += j.nkb) {
             // the epilogue warps have taken the previous tile's sums out of the accumulators
-            if (!__all_sync(0xffffffffu, mp_wait(tempty_bar, ((uint32_t)git & 1u) ^ 1u, abort_flag, p.status))) { ok = false; break; }
+            if (!mp_wait(tempty_bar, ((uint32_t)git & 1u) ^ 1u, abort_flag, p.status)) { ok = false; break; }
             tc_fence_after();
 #pragma unroll 1
             for (int kb = w; kb < j.nkb; kb += MP_NI) {
               const int g = gblk + kb;
               const int stage = g % MP_STAGES;
               const uint32_t phase = (uint32_t)(g / MP_STAGES) & 1u;
-              if (!__all_sync(0xffffffffu, mp_wait(full_bar(stage), phase, abort_flag, p.status))) { ok = false; break; }
+              if (!mp_wait(full_bar(stage), phase, abort_flag, p.status)) { ok = false; break; }
               tc_fence_after();
               const uint32_t sA = base + stage * MP_STAGE_BYTES;
               const uint64_t ad0 = desc_a_hi | (uint64_t)((sA & 0x3FFFFu) >> 4);
               const uint64_t bd0 = desc_b_hi | (uint64_t)(((sA + MP_A_BYTES) & 0x3FFFFu) >> 4);
-              if (elect_one()) {
 #pragma unroll
-                for (int s = 0; s < MP_BK / 16; ++s) {
-                  const uint64_t ad = ad0 + (uint64_t)(s * (a_mn ? 128 : 2));
-                  const uint64_t bd = bd0 + (uint64_t)(s * (b_mn ? 128 : 2));
-                  tc_mma_bf16(d_tmem, ad, bd, idesc, (kb != w || s != 0) ? 1u : 0u);
-                }
-                tc_commit(empty_bar(stage));
+              for (int s = 0; s < MP_BK / 16; ++s) {
+                const uint64_t ad = ad0 + (uint64_t)(s * (a_mn ? 128 : 2));
+                const uint64_t bd = bd0 + (uint64_t)(s * (b_mn ? 128 : 2));
+                tc_mma_bf16(d_tmem, ad, bd, idesc, (kb != w || s != 0) ? 1u : 0u);
               }
-              __syncwarp();
+              tc_commit(empty_bar(stage));
             }
             if (!ok) break;
-            if (elect_one()) {
-              if (w < j.nkb) tc_commit(tfull_bar(w));
-              else mbar_arrive(tfull_bar(w));  // no block of this tile was this warp's
-            }
-            __syncwarp();
+            if (w < j.nkb) tc_commit(tfull_bar(w));
+            else mbar_arrive(tfull_bar(w));  // no block of this tile was this warp's
           }
         }
       }

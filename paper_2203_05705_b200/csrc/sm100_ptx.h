@@ -83,7 +83,9 @@ __device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, vo
 // drops the loop over active lanes around each.  Cycles per instruction of one issuing thread: tcgen05.mma 136 behind
 // `lane == 0`, 63 - 75 behind this (the tensor core needs 64 for 128 x 128 x 16, 128 for 128 x 256 x 16), the commit of a
 // block 213 and 108.  Such a region uses registers that the whole warp shares, so it holds the instructions only: the
-// waits around it are the whole warp's, and a __syncwarp() follows it at once.
+// waits around it are the whole warp's, a __syncwarp() follows it at once, and nothing between two regions of a loop calls
+// a function that is not inlined (the iteration kernel, whose waits do, lost the context now and then: it keeps the test
+// of the lane number).
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
   asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.b32 %0, 1, 0, P;\n\t}" : "=r"(p) : : "memory");
