@@ -752,14 +752,9 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
   g.out_is_f32 = dW_dtype == ARD_F32;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
   if (in_pat && zero_fill_dropped) return ARD_ERR_INVALID_ARG;  // the packed gradient has no rows of dropped neurons
-  // The kernels write the zeros of dropped rows themselves; those of dropped pattern tiles are written first, except by
-  // the class form of the tensor-core kernels.
-  const bool zero_tiles = pat->kind == ARD_TILE && zero_fill_dropped;
+  // The kernels write the zeros of dropped rows and pattern tiles themselves, but for the tensor-core kernels of a fixed
+  // tile width (below).
   // Empty batch: the gradient of every kept weight is zero; the CUDA-core kernel writes exactly that.
-  if (B == 0 && zero_tiles) {
-    st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
-    if (st != ARD_OK) return st;
-  }
   if (B == 0) return launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
 
   ard_status el = ctx->path == ARD_PATH_CUDA_CORE
@@ -770,10 +765,6 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     el = ARD_ERR_NOMEM;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
-    if (zero_tiles) {
-      st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
-      if (st != ARD_OK) return st;
-    }
     st = bwd_staged_by_threads(ctx, pat, OP_BWD_WEIGHT, dtype, g, s);
     return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
   }

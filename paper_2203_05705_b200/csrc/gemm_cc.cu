@@ -88,6 +88,8 @@ __global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_con
   const bool whole = KIND == 0 || (p.ts & 3) == 0;  // four consecutive positions never leave a pattern tile
   const bool vec_a = (p.vec & 1) && step_a == 1 && whole, vec_b = (p.vec & 2) && whole;
 
+  if (KIND == 1 && OP == OP_BWD_WEIGHT && g.flag1)
+    sp_zero_dropped_tiles(g, p.ts, (int)blockIdx.x * (CC_THREADS / 32) + warp, (int)gridDim.x * (CC_THREADS / 32), lane);
   for (int u = (int)blockIdx.x / CC_CLUSTER; u < units; u += n_cl) {
     const int t = u * groups + group;
     ProductTile ti = {};

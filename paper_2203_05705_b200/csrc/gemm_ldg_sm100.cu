@@ -126,6 +126,8 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
   const int lead = rank - part;               // first CTA of the tile's group
   const int group = rank / s.S, groups = p.cl / s.S;
   const int n_cl = (int)gridDim.x / p.cl, units = (s.tiles + groups - 1) / groups;
+  if (KIND == 1 && OP == OP_BWD_WEIGHT && g.flag1 && warp < LG_LOADERS / 32)
+    sp_zero_dropped_tiles(g, p.ts, (int)blockIdx.x * (LG_LOADERS / 32) + warp, (int)gridDim.x * (LG_LOADERS / 32), lane);
   int blk = 0;        // blocks staged so far: stage = blk % STAGES
   int done = 0;       // accumulators finished so far
   bool ok = true;

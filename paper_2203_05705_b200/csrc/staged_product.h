@@ -51,6 +51,28 @@ struct ProductTile {
 
 __device__ __forceinline__ int sp_cdiv(int a, int b) { return (a + b - 1) / b; }
 
+// Tile patterns, weight gradient: zeros of the dropped tiles (Sec. 3.2), dealt to the grid's `warps` warps.  They go out
+// while the first blocks are on their way; a kernel of its own ahead of the product was one more dependent launch
+// (2048 x 2048, 32-wide tiles, batch 128, a period of 2, sampler and three products: 50.8 us with it, 48.5 without).  The j-th dropped tile: bb of them precede the first kept one, dp - 1 follow each kept one.
+__device__ __forceinline__ void sp_zero_dropped_tiles(const GemmArgs& g, int ts, int warp, int warps, int lane) {
+  const int dp = g.hdr[HDR_DP], bb = g.hdr[HDR_B] - 1, Tc = g.hdr[HDR_TC];
+  const int n_drop = g.hdr[HDR_TR] * Tc - g.hdr[HDR_NKEEP], es = g.out_is_f32 ? 4 : 2;
+  const size_t pitch = (size_t)g.ldo * es;
+  const bool wide = ((ts * es) & 15) == 0 && (pitch & 15) == 0 && (reinterpret_cast<uintptr_t>(g.out) & 15) == 0;
+  const int per_row = wide ? ts * es >> 4 : ts * es >> 1, piece = wide ? 16 : 2;
+  for (int j = warp; j < n_drop; j += warps) {
+    const int after = j - bb, lin = after < 0 ? j : bb + after / (dp - 1) * dp + 1 + after % (dp - 1);
+    const int r = lin / Tc, c = lin - r * Tc;  // tile-row along the fan-in, tile-column along the neurons
+    char* tile = reinterpret_cast<char*>(g.out) + (size_t)c * ts * pitch + (size_t)r * ts * es;
+    for (int e = lane; e < ts * per_row; e += 32) {
+      const int n = e / per_row, q = e - n * per_row;
+      char* d = tile + (size_t)n * pitch + (size_t)q * piece;
+      if (wide) *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
+      else *reinterpret_cast<uint16_t*>(d) = 0;
+    }
+  }
+}
+
 // want: CTAs the device has room for at once; cl: CTAs per cluster.
 template <int KIND, int OP, int BM, int BN, int BK>
 __device__ __forceinline__ ProductPlan make_plan(const GemmArgs& g, int ts, int want, int cl) {
