@@ -879,13 +879,13 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
     }
   } else if (warp == 0 || (has_second_producer(MODE) && warp == 10)) {
     // ===================== TMA producers =====================
-    // In the class form of the tile pattern (and in the tile-list kernels) two threads issue the copies, lane 0 of warp 0 the even contraction
-    // blocks (counted over all tiles of the CTA) and lane 0 of warp 10 the odd ones: there a thread spends ~160
-    // cycles in each copy instruction, three or four per block, and one thread alone paced the product (0.44 us per
-    // block where the MMAs need 0.34; -10 to -25 % per product with two).  Everywhere else one thread keeps up, and a
-    // second one gains nothing (the row form's weight gradient was 4 % slower with the eleventh warp merely present):
-    // only the class-form kernels and the tile-list kernels have warp 10, and it stays idle in the class form's
-    // dense draws.
+    // In the class form of the tile pattern (and in the tile-list kernels) two warps issue the copies, one thread each:
+    // warp 0 the even contraction blocks (counted over all tiles of the CTA) and warp 10 the odd ones.  Their blocks are
+    // three or four copies whose boxes lie in full-width matrices, and the copy unit pushes back while earlier ones are
+    // outstanding: three products of 8192 x 8192, 128-wide tiles, batch 4096, a period of 3: 447 us with two warps, 456
+    // with one.  Everywhere else one keeps up, and a second one gains nothing (the row form's weight gradient was 4 %
+    // slower with the eleventh warp merely present): only the class-form kernels and the tile-list kernels have warp 10,
+    // and it stays idle in the class form's dense draws.
     constexpr bool TWO = has_second_producer(MODE) && !(is_class_mode(MODE) && PLAIN);
     // Warp 0 first turns the descriptors it was given into those of the sampled pattern (the first
     // operand stage is free until the first load and serves as the 128-byte work area of each); warp 10 works out
