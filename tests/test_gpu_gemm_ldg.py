@@ -61,3 +61,18 @@ def test_narrow_pattern_tiles(ctx, ts, B, Tr, Tc):
         res = run_three_gemms(ctx, pat, ard.ARD_TILE, ard.ARD_BF16, X, W, dY, dp, b, 2.0, ts=ts, zero_fill=(i % 2 == 0),
                               dw_dtype=ard.ARD_F32 if i % 2 else ard.ARD_BF16)
         assert_ok(res, TOL[ard.ARD_BF16], (ts, B, Tr, Tc, dp, b))
+
+
+@pytest.mark.parametrize("B,N", [(9475, 131), (2402, 131), (1187, 515)])
+def test_compaction_of_tall_gradients(ctx, B, N):
+    """The pass that compacts dY off the 16-byte grid takes 8, 4 or 1 rows per block: a last group that is not full."""
+    rng = np.random.default_rng(B)
+    K = 26
+    X = inputs.bf16_round(rng.standard_normal((B, K)).astype(np.float32))
+    W = inputs.bf16_round((rng.standard_normal((K, N)) * 0.05).astype(np.float32))
+    dY = inputs.bf16_round(rng.standard_normal((B, N)).astype(np.float32))
+    pat = ctx.pattern(ard.ARD_ROW, K, N)
+    for dp, b in [(2, 2), (7, 3)]:
+        ard.ard_pattern_set(ctx.h, pat, dp, b)
+        res = run_three_gemms(ctx, pat, ard.ARD_ROW, ard.ARD_BF16, X, W, dY, dp, b, 2.0)
+        assert_ok(res, TOL[ard.ARD_BF16], (B, N, dp))
