@@ -144,29 +144,25 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
 
     if (warp == 8) {
       // ===================== products =====================
-      ok = __all_sync(0xffffffffu, ok);
-      if (has_acc && ok) {
+      if (lane == 0 && has_acc && ok) {
         const uint64_t desc_a = A_MN ? make_desc(0, 64 * LG_BK * 2, 1024) : make_desc(0, 16, 1024);
         const uint64_t desc_b = B_MN ? make_desc(0, 64 * LG_BK * 2, 1024) : make_desc(0, 16, 1024);
         const uint32_t idesc = make_idesc(BN, A_MN, B_MN);
         for (int kb = kb0; kb < kb1; ++kb) {
           const int it = blk + kb - kb0, st = it % LG_STAGES;
-          if (!mbar_wait_warp(full_bar(st), (uint32_t)(it / LG_STAGES) & 1u, abort_flag, g.status)) { ok = false; break; }
+          if (!mbar_wait(full_bar(st), (uint32_t)(it / LG_STAGES) & 1u, abort_flag, g.status)) { ok = false; break; }
           if (ASYNC) fence_proxy_async_smem();  // the copies were made in the generic proxy
           tc_fence_after();
           const uint32_t sA = base + st * L::STAGE_BYTES;
           const uint64_t ad0 = desc_a | (uint64_t)((sA & 0x3FFFFu) >> 4);
           const uint64_t bd0 = desc_b | (uint64_t)(((sA + L::A_BYTES) & 0x3FFFFu) >> 4);
-          if (elect_one()) {
 #pragma unroll
-            for (int k = 0; k < LG_BK / 16; ++k)
-              tc_mma_bf16(tmem, ad0 + (uint64_t)(k * (A_MN ? 128 : 2)), bd0 + (uint64_t)(k * (B_MN ? 128 : 2)), idesc,
-                          (kb != kb0 || k != 0) ? 1u : 0u);
-            tc_commit(empty_bar(st));
-          }
-          __syncwarp();
+          for (int k = 0; k < LG_BK / 16; ++k)
+            tc_mma_bf16(tmem, ad0 + (uint64_t)(k * (A_MN ? 128 : 2)), bd0 + (uint64_t)(k * (B_MN ? 128 : 2)), idesc,
+                        (kb != kb0 || k != 0) ? 1u : 0u);
+          tc_commit(empty_bar(st));
         }
-        if (ok && elect_one()) tc_commit(done_bar);
+        if (ok) tc_commit(done_bar);
       }
       __syncwarp();
     } else {

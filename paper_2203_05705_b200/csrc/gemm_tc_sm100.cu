@@ -826,22 +826,19 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
         const uint32_t sA = base + stage * L::STAGE_BYTES;
         const uint32_t sB = sA + L::A_BYTES;
         const int kx = kb * BK;
-        if (warp == 0) {
-          if (elect_one()) {
-            if (MODE == M_ROWS_BWD_WEIGHT) {
-              mbar_arrive(full_bar(stage));
-            } else {
-              mbar_arrive_expect_tx(full_bar(stage), (uint32_t)(L::A_BYTES + ti.nbox * 64 * BK * 2));
+        if (warp == 0 && lane == 0) {
+          if (MODE == M_ROWS_BWD_WEIGHT) {
+            mbar_arrive(full_bar(stage));
+          } else {
+            mbar_arrive_expect_tx(full_bar(stage), (uint32_t)(L::A_BYTES + ti.nbox * 64 * BK * 2));
 #pragma unroll
-              for (int bxi = 0; bxi < 4; ++bxi) {
-                if (bxi < ti.nbox) {
-                  if (MODE == M_ROWS_FWD) tma_load_2d(sB + bxi * (64 * BK * 2), mapB, full_bar(stage), kx, ti.bx[bxi]);
-                  else tma_load_2d(sB + bxi * (64 * BK * 2), mapB, full_bar(stage), ti.bx[bxi], kx);
-                }
+            for (int bxi = 0; bxi < 4; ++bxi) {
+              if (bxi < ti.nbox) {
+                if (MODE == M_ROWS_FWD) tma_load_2d(sB + bxi * (64 * BK * 2), mapB, full_bar(stage), kx, ti.bx[bxi]);
+                else tma_load_2d(sB + bxi * (64 * BK * 2), mapB, full_bar(stage), ti.bx[bxi], kx);
               }
             }
           }
-          __syncwarp();
         }
         if (MODE != M_ROWS_BWD_WEIGHT) {
           // [128 rows][64 k]: rows 4g .. 4g+3 at byte 512 g of the stage
@@ -915,24 +912,21 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
     if (has_second_producer(MODE)) asm volatile("bar.sync 3, 64;" ::: "memory");  // the rewritten descriptors are in global memory
     if (smid >= (uint32_t)ARD_TM_SM_MAX) {  // more SMs than the scratch was laid out for: refuse rather than share a slot
       if (lane == 0) { *abort_flag = 1; atomicMax(p.status, (int)ARD_ERR_UNSUPPORTED); }
-    } else {
+    } else if (lane == 0) {
       // only the rewritten copies live in global memory and need the tensor-map proxy's acquire; a descriptor
       // used as encoded is read from the kernel's parameters
       auto acquire = [&](const CUtensorMap* m, int mi) {
         if (m != &p.maps[mi].tm) tensormap_acquire(m);
       };
-      if (elect_one()) {  // the lane that issues the copies
-        acquire(mapA, 0);
-        acquire(mapB, 1);
-        if (is_lstm_mode(MODE)) {
+      acquire(mapA, 0);
+      acquire(mapB, 1);
+      if (is_lstm_mode(MODE)) {
 #pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            if (MODE == M_LSTM_BWD_DATA || MODE == M_LSTM_BWD_WEIGHT) acquire(mapA4[g], 2 + g);
-            if (MODE == M_LSTM_FWD || MODE == M_LSTM_BWD_DATA) acquire(mapB4[g], 6 + g);
-          }
+        for (int g = 0; g < 4; ++g) {
+          if (MODE == M_LSTM_BWD_DATA || MODE == M_LSTM_BWD_WEIGHT) acquire(mapA4[g], 2 + g);
+          if (MODE == M_LSTM_FWD || MODE == M_LSTM_BWD_DATA) acquire(mapB4[g], 6 + g);
         }
       }
-      __syncwarp();
       int stage = 0;
       uint32_t phase = 0;
       int turn = 0;  // whose block this is: blocks alternate between the two producers over all tiles
@@ -957,11 +951,12 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
             if (++stage == STAGES) { stage = 0; phase ^= 1u; }
             continue;
           }
-          if (!mbar_wait_warp(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+          if (!mbar_wait(empty_bar(stage), phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
           const uint32_t sA = base + stage * L::STAGE_BYTES;
           const uint32_t sB = sA + L::A_BYTES;
           // In a pair every load reports to the leader's barrier, which expects the bytes of both CTAs.
           const uint32_t fbar = (CTAS == 2) ? mapa_u32(full_bar(stage), 0u) : full_bar(stage);
+          if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), stage_tx);
           auto load = [&](uint32_t dst, const CUtensorMap* map, int x, int y) {
             if (CTAS == 2) tma_load_2d_pair(dst, map, fbar, x, y);
             else tma_load_2d(dst, map, fbar, x, y);
@@ -979,41 +974,37 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
             kx = kb * BK;
           }
           const CUtensorMap* mapBk = mapB;
-          if (elect_one()) {
-            if (rank == 0) mbar_arrive_expect_tx(full_bar(stage), stage_tx);
-            if (MODE == M_LSTM_BWD_DATA) {
-              // contraction runs gate by gate over the kept units: block kb = (gate, 64 kept units)
-              const int nkg = ti.nkb >> 2;
-              const int g = kb / nkg;
-              kx = (kb - g * nkg) * BK;
-              mapBk = mapB4[g];
-              load(sA, mapA4[g], kx, ti.m0);
-            } else if (!A_MN) {
-              load(sA, mapA, kx, ti.m0);  // [BM rows][64 k]
-            } else {
+          if (MODE == M_LSTM_BWD_DATA) {
+            // contraction runs gate by gate over the kept units: block kb = (gate, 64 kept units)
+            const int nkg = ti.nkb >> 2;
+            const int g = kb / nkg;
+            kx = (kb - g * nkg) * BK;
+            mapBk = mapB4[g];
+            load(sA, mapA4[g], kx, ti.m0);
+          } else if (!A_MN) {
+            load(sA, mapA, kx, ti.m0);  // [BM rows][64 k]
+          } else {
 #pragma unroll
-              for (int i = 0; i < BM / 64; ++i)  // [64 k rows][64 m] per box
-                load(sA + i * (64 * BK * 2), MODE == M_LSTM_BWD_WEIGHT ? sel_map(mapA4, ti.gate) : mapA, ti.ax[i], kx);
-            }
-            // B always moves in 64-wide boxes: K-major [64 rows][64 k] stacked, MN-major [64 k][64 n].
-            // In a pair this CTA stages the second half of the tile's B boxes if its rank is 1.
+            for (int i = 0; i < BM / 64; ++i)  // [64 k rows][64 m] per box
+              load(sA + i * (64 * BK * 2), MODE == M_LSTM_BWD_WEIGHT ? sel_map(mapA4, ti.gate) : mapA, ti.ax[i], kx);
+          }
+          // B always moves in 64-wide boxes: K-major [64 rows][64 k] stacked, MN-major [64 k][64 n].
+          // In a pair this CTA stages the second half of the tile's B boxes if its rank is 1.
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              if (i < ti.nbox) {
-                if (MODE == M_LSTM_FWD) load(sB + i * (64 * BK * 2), mapB4[i], kx, ti.bx[i]);
-                else if (!B_MN) load(sB + i * (64 * BK * 2), mapBk, kx, ti.bx[i]);
-                else load(sB + i * (64 * BK * 2), mapBk, ti.bx[i], kx);
-              }
+          for (int i = 0; i < 4; ++i) {
+            if (i < ti.nbox) {
+              if (MODE == M_LSTM_FWD) load(sB + i * (64 * BK * 2), mapB4[i], kx, ti.bx[i]);
+              else if (!B_MN) load(sB + i * (64 * BK * 2), mapBk, kx, ti.bx[i]);
+              else load(sB + i * (64 * BK * 2), mapBk, ti.bx[i], kx);
             }
           }
-          __syncwarp();
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
       }
     }
   } else if (warp == 1) {
     // ===================== MMA issuer =====================
-    if (rank == 0) {
+    if (lane == 0 && rank == 0) {
       // descriptors without the start address: K-major (LBO unused, SBO 1024) or MN-major (LBO 8 KiB, SBO 1024)
       const uint64_t desc_a_hi = A_MN ? make_desc(0, 64 * BK * 2, 1024) : make_desc(0, 16, 1024);
       const uint64_t desc_b_hi = B_MN ? make_desc(0, 64 * BK * 2, 1024) : make_desc(0, 16, 1024);
@@ -1031,44 +1022,38 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
         const int acc = nacc & 1;
         const uint32_t acc_phase = (uint32_t)(nacc >> 1) & 1u;
         ++nacc;
-        if (!mbar_wait_warp(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
+        if (!mbar_wait(tempty_bar(acc), acc_phase ^ 1u, abort_flag, p.status)) { ok = false; break; }
         tc_fence_after();
         const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
         for (int kb = kb_begin; kb < kb_end; ++kb) {
-          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, p.status)) { ok = false; break; }
+          if (!mbar_wait(full_bar(stage), phase, abort_flag, p.status)) { ok = false; break; }
           if (MODE == M_ROWS_BWD_WEIGHT) {
             // the gathered operands were written by ordinary asynchronous copies (generic proxy)
             fence_proxy_async_smem();
             tc_fence_after();
           }
-          // The issuing thread's instruction stream is what feeds the tensor pipe: the descriptors of a block are
+          // This thread's instruction stream is what feeds the tensor pipe: the descriptors of a block are
           // the stage's descriptor plus a constant per 16-deep step (the start-address field counts 16-byte
           // units: K-major 32 bytes = 2 per step, MN-major 16 k-rows = 2048 bytes = 128 per step).
           const uint32_t sA = base + stage * L::STAGE_BYTES;
           const uint64_t ad0 = desc_a_hi | (uint64_t)((sA & 0x3FFFFu) >> 4);
           const uint64_t bd0 = desc_b_hi | (uint64_t)(((sA + L::A_BYTES) & 0x3FFFFu) >> 4);
-          if (elect_one()) {
 #pragma unroll
-            for (int s = 0; s < BK / 16; ++s) {
-              const uint64_t ad = ad0 + (uint64_t)(s * (A_MN ? 128 : 2));
-              const uint64_t bd = bd0 + (uint64_t)(s * (B_MN ? 128 : 2));
-              const uint32_t accum = (kb != kb_begin || s != 0) ? 1u : 0u;
-              if (CTAS == 2) tc_mma_bf16_pair(d_tmem, ad, bd, idesc, accum);
-              else tc_mma_bf16(d_tmem, ad, bd, idesc, accum);
-            }
-            // frees the stage (in both CTAs of a pair) once these MMAs have read it
-            if (CTAS == 2) tc_commit2(empty_bar(stage), (uint16_t)3);
-            else tc_commit(empty_bar(stage));
+          for (int s = 0; s < BK / 16; ++s) {
+            const uint64_t ad = ad0 + (uint64_t)(s * (A_MN ? 128 : 2));
+            const uint64_t bd = bd0 + (uint64_t)(s * (B_MN ? 128 : 2));
+            const uint32_t accum = (kb != kb_begin || s != 0) ? 1u : 0u;
+            if (CTAS == 2) tc_mma_bf16_pair(d_tmem, ad, bd, idesc, accum);
+            else tc_mma_bf16(d_tmem, ad, bd, idesc, accum);
           }
-          __syncwarp();
+          // frees the stage (in both CTAs of a pair) once these MMAs have read it
+          if (CTAS == 2) tc_commit2(empty_bar(stage), (uint16_t)3);
+          else tc_commit(empty_bar(stage));
           if (++stage == STAGES) { stage = 0; phase ^= 1u; }
         }
         if (!ok) break;
-        if (elect_one()) {
-          if (CTAS == 2) tc_commit2(tfull_bar(acc), (uint16_t)3);
-          else tc_commit(tfull_bar(acc));
-        }
-        __syncwarp();
+        if (CTAS == 2) tc_commit2(tfull_bar(acc), (uint16_t)3);
+        else tc_commit(tfull_bar(acc));
       }
     }
   } else {

@@ -16,7 +16,8 @@
 //     blocks per loading warp.  Usually every block of a step has a slot of its own, so all loads of a step are in
 //     flight together; a slice so large that fewer slots fit re-uses them within the step.  The warp that loads a
 //     quarter also issues its products (tcgen05.mma, M = 64 or 128, N = 4 U, accumulators in tensor memory,
-//     double-buffered over steps); the copies are requested by the lanes of a warp, ~70 SM cycles apart;
+//     double-buffered over steps): one thread issuing box after box paces at ~410 SM cycles per box, the lanes of a
+//     warp ~70 cycles apart, and a tcgen05.mma this narrow costs its issuing thread ~110 cycles;
 //   - the accumulator rows move to shared memory, then all 11 compute warps apply the cell
 //     update to the (batch row, unit) pairs, keep c in registers, and write h_t (bf16) into the operand
 //     of step t+1 and, after signalling, c_t and the gate activations for BPTT;
@@ -174,51 +175,36 @@ __device__ __forceinline__ void lstm_sum_groups(uint32_t taddr, int stride, int 
       if (c < groups) z[i] += __uint_as_float(y[c][i]);
   }
 }
-// One step's blocks [0, n) of a loading warp, called by all its lanes.  Usually every block has a slot of its own: lane i
-// requests block i, and once all are there one thread issues all products (35 steps, 20 rows, 750 of 1500 units kept,
-// forward plus BPTT: 426 us; product by product as the blocks arrive 439, requests from one thread 454, products behind
-// a test of the lane number 443).  Where fewer slots fit, the blocks are multiplied as they arrive and the later ones
-// requested into the slots that fell free; a slot's barriers are phased by how often it has been used, `step` steps
-// before this one.  request(block, slot) issues the copies of a block (and announces their bytes), multiply(block, slot,
-// first) its products.
+// One step's blocks [0, n) of a loading warp, called by all its lanes: lane i requests block i into slot i while slots
+// last; lane 0 multiplies the blocks as they arrive and requests the later ones into the slots that fell free.  A slot's
+// barriers are phased by how often it has been used: `step` steps before this one.  request(block, slot) issues the
+// copies of a block (and announces their bytes); multiply(block, slot, first) its products.  ok: lane 0's verdict.
 template <typename Request, typename Multiply, typename FullBar, typename FreeBar>
-__device__ __forceinline__ bool lstm_stream_blocks(int n, int cap, int step, FullBar full_bar, FreeBar free_bar,
+__device__ __forceinline__ bool lstm_stream_blocks(int n, int cap, int step, int lane, bool ok, FullBar full_bar, FreeBar free_bar,
                                                    volatile int* abort_flag, int* status, Request request, Multiply multiply) {
-  const int lane = threadIdx.x & 31;
   if (lane < n && lane < cap) request(lane, lane);
   __syncwarp();
-  auto count = [&](int slot, int i) { return (uint32_t)(step * ((n - 1 - slot) / cap + 1) + i / cap); };
-  if (n <= cap) {
-    for (int i = 0; i < n; ++i)
-      if (!mbar_wait_warp(full_bar(i), (uint32_t)step & 1u, abort_flag, status)) return false;
-    tc_fence_after();
-    if (elect_one()) {
-      for (int i = 0; i < n; ++i) multiply(i, i, i == 0);
-    }
-    __syncwarp();
-    return true;
-  }
-  for (int i = 0; i < n; ++i) {
-    const int slot = i % cap;
-    if (!mbar_wait_warp(full_bar(slot), count(slot, i) & 1u, abort_flag, status)) return false;
-    tc_fence_after();
-    if (elect_one()) {
+  if (lane == 0 && ok) {
+    auto count = [&](int slot, int i) { return (uint32_t)(step * ((n - 1 - slot) / cap + 1) + i / cap); };
+    for (int i = 0; i < n; ++i) {
+      const int slot = i % cap;
+      if (!mbar_wait(full_bar(slot), count(slot, i) & 1u, abort_flag, status)) { ok = false; break; }
+      tc_fence_after();
       multiply(i, slot, i == 0);
-      if (n > cap) tc_commit(free_bar(slot));
-    }
-    __syncwarp();
-    if (n > cap) {
-      // refill the slot of the block before this one, whose products were issued a block ago (with one slot: of this one)
-      const int j = cap > 1 ? i - 1 : i;
-      if (j >= 0 && j + cap < n) {
-        const int sj = j % cap;
-        if (!mbar_wait_warp(free_bar(sj), count(sj, j) & 1u, abort_flag, status)) return false;
-        if (elect_one()) request(j + cap, sj);
-        __syncwarp();
+      if (n > cap) {
+        // refill the slot of the block before this one, whose products were issued a block ago (with one slot: of this one)
+        tc_commit(free_bar(slot));
+        const int j = cap > 1 ? i - 1 : i;
+        if (j >= 0 && j + cap < n) {
+          const int sj = j % cap;
+          if (!mbar_wait(free_bar(sj), count(sj, j) & 1u, abort_flag, status)) { ok = false; break; }
+          request(j + cap, sj);
+        }
       }
     }
   }
-  return true;
+  __syncwarp();
+  return ok;
 }
 
 // The gate functions of the per-step kernels (aux_kernels.cu), so that a layer's results do not depend on the path it takes.
@@ -367,9 +353,9 @@ __device__ __forceinline__ void lstm_forward_body(const LstmFwdParams& p, uint8_
 #pragma unroll
           for (int s = 0; s < LP_BK / 16; ++s) tc_mma_bf16(d_tmem, ad + 2 * s, bd + 2 * s, idesc, (!first || s != 0) ? 1u : 0u);
         };
-        ok = lstm_stream_blocks(n, cap, t, [&](int s) { return full_bar(g, s); }, [&](int s) { return free_bar(g, s); },
+        ok = lstm_stream_blocks(n, cap, t, lane, ok, [&](int s) { return full_bar(g, s); }, [&](int s) { return free_bar(g, s); },
                                 abort_flag, p.status, request, multiply);
-        if (ok && elect_one()) tc_commit(tfull_bar(acc));  // this quarter is complete
+        if (lane == 0 && ok) tc_commit(tfull_bar(acc));  // this quarter is complete
         __syncwarp();
       }
     } else {
@@ -842,9 +828,9 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
 #pragma unroll
         for (int s = 0; s < LP_BK / 16; ++s) tc_mma_bf16(d_tmem, ad + 2 * s, bd + 2 * s, idesc, (!first || s != 0) ? 1u : 0u);
       };
-      ok = lstm_stream_blocks(n, cap, k - 1, [&](int s) { return full_bar(g4, s); }, [&](int s) { return free_bar(g4, s); },
+      ok = lstm_stream_blocks(n, cap, k - 1, lane, ok, [&](int s) { return full_bar(g4, s); }, [&](int s) { return free_bar(g4, s); },
                               abort_flag, p.status, request, multiply);
-      if (ok && elect_one()) {
+      if (lane == 0 && ok) {
         if (n > 0) tc_commit(tfull_bar);
         else mbar_arrive(tfull_bar);
       }

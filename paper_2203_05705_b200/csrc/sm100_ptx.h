@@ -73,25 +73,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
-// The same by all 32 lanes of a warp, one verdict for all of them.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
-  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, status));
-}
-
-// True in one lane of the warp, always the same one; called by all 32.  Tensor-core and TMA instructions are issued
-// behind this and not behind a test of the lane number: only then does the compiler know that one thread runs them and
-// drops the loop over active lanes around each.  Cycles per instruction of one issuing thread: tcgen05.mma 136 behind
-// `lane == 0`, 63 - 75 behind this (the tensor core needs 64 for 128 x 128 x 16, 128 for 128 x 256 x 16), the commit of a
-// block 213 and 108.  Such a region uses registers that the whole warp shares, so it holds the instructions only: the
-// waits around it are the whole warp's, a __syncwarp() follows it at once, and nothing between two regions of a loop calls
-// a function that is not inlined (the iteration kernel, whose waits do, lost the context now and then: it keeps the test
-// of the lane number).
-__device__ __forceinline__ bool elect_one() {
-  uint32_t p;
-  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.b32 %0, 1, 0, P;\n\t}" : "=r"(p) : : "memory");
-  return p != 0;
-}
-
 __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
