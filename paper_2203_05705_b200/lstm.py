@@ -43,6 +43,10 @@ class LstmLayer:
     def backward(self, alpha, dH):
         """dH: fp32 [T][B][H], gradient with respect to every h_t.  Returns (dX [T][B][I] fp32 view, dW)."""
         ctx, pat, T, B, H, KH, I = self.ctx, self.pat, self.T, self.B, self.H, self.KH, self.I
+        if tuple(dH.shape) != (T, B, H):
+            raise ValueError("dH has shape %s, the layer's is %s" % (tuple(dH.shape), (T, B, H)))
+        if dH.device != self.D.device:
+            raise ValueError("dH is on %s, the layer on %s" % (dH.device, self.D.device))
         dH = dH.to(torch.float32).contiguous()
         ard.ard_lstm_backward_dh(ctx, pat, T, B, I, H, alpha, self.XH, self.W, KH, self.C, self.G, dH, self.D, self.dc, self.DZ,
                                  self.dW)
