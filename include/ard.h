@@ -607,7 +607,8 @@ ard_status ard_lstm_backward(ard_ctx* ctx, const ard_pattern* pat, int T, int B,
                              const void* XH, const void* W, int ldw, const float* C, const float* G,
                              const float* dH_last, float* D, float* dc, void* DZ, float* dW, void* cuda_stream);
 /* The same with nothing prepared: dH [T][B][H] fp32 holds the upstream gradient of every h_t, no gradient arrives at
- * c_T, and D and dc are outputs only: contents as above, the h halves of D[1..T-1] unspecified. */
+ * c_T, and D and dc are outputs only: contents as above, the h halves of D[1..T-1] unspecified; dc is zero behind the kept
+ * columns, and so is the h half of D[0] at dropped units where the one-kernel recurrence runs. */
 ard_status ard_lstm_backward_dh(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                 const void* XH, const void* W, int ldw, const float* C, const float* G, const float* dH,
                                 float* D, float* dc, void* DZ, float* dW, void* cuda_stream);

@@ -932,8 +932,13 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
           rec = zs[row * (U + 1) + j - j0];
         }
         if (t < 0) {  // gradient of h_0, added to what the caller left in the h half of D[0]
-          float* d0 = p.D + (size_t)row * ldd + p.I + bb + j * dp;
-          *d0 = p.dH == nullptr ? *d0 + rec : rec;
+          float* d0 = p.D + (size_t)row * ldd + p.I;
+          if (p.dH == nullptr) {
+            d0[bb + j * dp] += rec;
+          } else {  // nothing was there: zeros of the dropped units; the j-th kept one owns [j * dp, (j + 1) * dp), the last the tail
+            const int last = j == n_keep - 1 ? p.H : min(p.H, (j + 1) * dp);
+            for (int u = j * dp; u < last; ++u) d0[u] = u == bb + j * dp ? rec : 0.f;
+          }
           continue;
         }
         total[i] = adj[i].up + rec;  // upstream gradient of h_t plus the recurrent part (none at T - 1)
@@ -947,7 +952,7 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
         fence_proxy_async_smem();
         if (math_barrier_failed<1>(!ok)) { ok = false; break; }
         if (tid == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(p.bar) : "memory");
-        if (t < T - 1 && p.dH == nullptr) {  // the caller's D holds the totals afterwards
+        if (t < T - 1 && p.dH == nullptr) {  // the caller's D holds the totals afterwards (with dH 10 us of a pass of 381)
 #pragma unroll
           for (int i = 0; i < PAIRS; ++i)
             if (own >> i & 1u) p.D[((size_t)(t + 1) * p.B + row_of(i)) * ldd + p.I + bb + unit_of(i) * dp] = total[i];
@@ -957,7 +962,12 @@ __device__ __forceinline__ void lstm_backward_body(const LstmBwdParams& p, uint8
     if (ok) {
 #pragma unroll
       for (int i = 0; i < PAIRS; ++i)
-        if (own >> i & 1u) p.dc[(size_t)row_of(i) * p.H + unit_of(i)] = dcreg[i];
+        if (own >> i & 1u) {
+          float* dc = p.dc + (size_t)row_of(i) * p.H;
+          dc[unit_of(i)] = dcreg[i];
+          if (p.dH != nullptr)  // nothing was there: zeros behind the kept columns
+            for (int c = unit_of(i) + n_keep; c < p.H; c += n_keep) dc[c] = 0.f;
+        }
     }
   }
 

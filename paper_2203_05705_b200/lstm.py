@@ -27,7 +27,7 @@ class LstmLayer:
         self.G = torch.zeros((T, B, 4 * H), dtype=f32, device="cuda")
         self.Z = torch.zeros((B, 4 * H), dtype=f32, device="cuda")
         self.DZ = torch.zeros((T, B, 4 * H), dtype=bf, device="cuda")
-        self.D = torch.zeros((T, B, self.KH), dtype=f32, device="cuda")   # [dx_t | total dh_{t-1}]
+        self.D = torch.zeros((T, B, self.KH), dtype=f32, device="cuda")   # dx_t; h half: D[0] dh_0, else scratch
         self.dc = torch.zeros((B, H), dtype=f32, device="cuda")
         self.dW = torch.zeros((4 * H, self.KH), dtype=f32, device="cuda")
 
