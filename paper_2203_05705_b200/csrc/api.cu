@@ -1220,10 +1220,12 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
     DeviceGuard guard(ctx->device);
     const bool tma = tc_eligible(ctx, pat, ARD_BF16, T * B, KH, H, DZ, 4 * H, W, ldw, D, KH, 4) == ARD_OK &&
                      ((size_t)H * ldw * 2) % 16 == 0 && I % 8 == 0;
+    // dz is the one operand that the kernel reads through descriptors: a copy only where its own rows are off the grid
+    const bool copy = !aligned16(DZ) || H % 8 != 0;
     const int padded = (H + 7) / 8 * 8;
-    const bool room = tma || (size_t)T * B * 4 * padded * 2 <= sk_ws_bytes(ctx->sm_count);
+    const bool room = !copy || (size_t)T * B * 4 * padded * 2 <= sk_ws_bytes(ctx->sm_count);
     if (lstm_persistent_bwd_fits(ctx, B, H) && room && (tma || ctx->path == ARD_PATH_AUTO)) {
-      if (!tma) {
+      if (copy) {
         dz = ctx->d_sk_ws;
         gs = padded;
       }

@@ -48,3 +48,37 @@ def test_buffers_after_a_backward_pass(T, B, I, H):
             assert bool((D1[:, drop] == 0).all()), dp
     finally:
         ctx.close()
+
+
+# 148 SMs hold 38.8 MB of gate gradients in context scratch (T * B * 4 * H bf16, H rounded up to 8) for layers whose own are off
+# the 16-byte grid: the last length that fits and the first that does not; and a layer off the grid for its inputs alone, whose
+# gate gradients need no copy however many there are
+@pytest.mark.parametrize("T,I,H,one_kernel", [(34, 20, 1092, True), (35, 20, 1092, False), (35, 20, 1096, True)])
+def test_gate_gradients_around_the_limit_of_the_scratch(T, I, H, one_kernel):
+    B = 128
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("the scratch is sized by the number of SMs")
+    g = torch.Generator(device="cuda").manual_seed(T + H)
+    W = (torch.rand((4 * H, I + H), device="cuda", generator=g) * 0.12 - 0.06).to(BF)
+    X = torch.randn((T, B, I), device="cuda", generator=g).to(BF)
+    dH = torch.randn((T, B, H), device="cuda", generator=g) / 8
+    ctx = Ctx(1 << 20)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, I + H, H)
+        layer = LstmLayer(ctx.h, pat, T, B, I, H, W)
+        ard.ard_pattern_set(ctx.h, pat, 2, 2)
+        res = []
+        for persistent in (0, 1):
+            ard.ard_set_lstm_persistent(ctx.h, persistent)
+            layer.load_inputs(X)
+            layer.forward(1.5)
+            n0 = ard.ard_launch_count(ctx.h)
+            dX, dW = layer.backward(1.5, dH)
+            n = ard.ard_launch_count(ctx.h) - n0
+            assert (n <= 9) == (bool(persistent) and one_kernel), n
+            assert ard.ard_last_device_status(ctx.h) == 0
+            res.append((dX.double().clone(), dW.double().clone()))
+        for a, r in zip(res[1], res[0]):
+            assert (a - r).norm() <= TOL[ard.ARD_BF16] * r.norm()
+    finally:
+        ctx.close()
