@@ -224,6 +224,15 @@ def oracle_sample_seconds(wl, d, rows=256):
     return dt, flops, threads, f"{len(sel)} of {B} batch rows (fwd, bwd-data) + {len(cols)} of {N} neurons (bwd-weight), dp=2"
 
 
+def emit(line, args):
+    """Prints the result line.  Its "detail" (tables of tens of kilobytes, more than a reader of one line keeps) goes to
+    the file that --detail names, together with the rest of the line."""
+    if getattr(args, "detail", None) and "detail" in line:
+        with open(args.detail, "w") as f:
+            json.dump(line, f)
+    print(json.dumps({k: v for k, v in line.items() if k != "detail"}))
+
+
 def run_reference(args, wl):
     """--impl reference: the CPU oracle on the host cores, bounded sample per step."""
     rank = int(os.environ.get("RANK", "0"))
@@ -410,7 +419,7 @@ def run_lstm(args, wl):
                    "rate_sweep": sweep, "per_dp": per_dp},
         "device_status": int(status),
     }
-    print(json.dumps(line))
+    emit(line, args)
     ard.ard_pattern_destroy(pat)
     ard.ard_destroy(ctx)
 
@@ -564,7 +573,7 @@ def run_lstm_stack(args, wl):
                    "kept_fraction_of_outputs": {str(p): [float(x) for x in np.mean(np.array(fracs), axis=0)]}},
         "device_status": int(status),
     }
-    print(json.dumps(line))
+    emit(line, args)
     stack.close()
     ard.ard_destroy(ctx)
 
@@ -835,7 +844,7 @@ def run_mlp_step(args, wl):
                        launches_per_step=launches_per_step),
         "device_status": int(status),
     }
-    print(json.dumps(line))
+    emit(line, args)
 
 
 def run_conv_rows(args, wl):
@@ -1005,7 +1014,7 @@ def run_conv_rows(args, wl):
                      "note": "whole step incl. sensitivity prediction, row sampling and zero fill of the dropped rows"},
         "cpu_baseline": cpu, "detail": detail, "device_status": int(status),
     }
-    print(json.dumps(line))
+    emit(line, args)
     ard.ard_rows_destroy(rows)
     ard.ard_destroy(ctx)
 
@@ -1140,7 +1149,7 @@ def run_conv_blocks(args, wl):
                      "note": "whole step incl. sensitivity counts, labels, block draws, lists and zero fill of the dropped blocks"},
         "cpu_baseline": cpu, "detail": detail, "device_status": int(status),
     }
-    print(json.dumps(line))
+    emit(line, args)
     ard.ard_blocks_destroy(blocks)
     ard.ard_destroy(ctx)
 
@@ -1528,6 +1537,7 @@ def main():
     ap.add_argument("--impl", default="ours", choices=["ours", "reference"])
     ap.add_argument("--workload", default="mlp8192_row", choices=sorted(WORKLOADS))
     ap.add_argument("--no-cpu-baseline", action="store_true")
+    ap.add_argument("--detail", metavar="FILE", help="write the result with its tables (per period, rates, graphs) to FILE as JSON")
     ap.add_argument("--quick", action="store_true", help="headline region only (for profiler captures)")
     ap.add_argument("--conv-run-len", type=int, default=0,
                     help="conv workloads: values per sampled run of the sensitivity prediction (1 = single values, "
@@ -1798,7 +1808,7 @@ def main():
             "dense_equiv_tflops": h["dense_equiv"], "clocks": clk, "e2e": e2e, "gpu_launches": h["launches"],
             "roofline": roofline, "cpu_baseline": cpu, "detail": detail, "device_status": h["status"],
         }
-        print(json.dumps(line))
+        emit(line, args)
     lb.close()
     if world > 1:
         dist.destroy_process_group()
