@@ -12,7 +12,6 @@ import ctypes as C
 import os
 
 import numpy as np
-import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libard.so")
@@ -171,11 +170,26 @@ def _ptr(t):
     return t.data_ptr()
 
 
+_current_stream = None
+
+
+def _current_stream_getter():
+    """The current stream's handle as torch's binding has it: torch.cuda.current_stream() builds an object around it (3.3 us a
+    call against 0.3, where the native call that follows takes 5).  The name is private, so the public call stands in for it.
+    torch is looked for by the first call without a stream only: callers with streams of their own do without it."""
+    import torch
+    raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), torch.cuda.current_device
+    if raw is None:
+        return lambda: torch.cuda.current_stream().cuda_stream
+    return lambda: raw(device())
+
+
 def _stream(stream):
+    global _current_stream
     if stream is None:
-        # the current stream's handle itself: torch.cuda.current_stream() builds an object around it (3.3 us a call
-        # against 0.3, where the native call that follows takes 5)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        if _current_stream is None:
+            _current_stream = _current_stream_getter()
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
