@@ -99,8 +99,8 @@ ard_status ard_set_path(ard_ctx* ctx, ard_path path);
  *                                 the kept units alone when the pattern drops any: forward over a compact copy of
  *                                 h_{t-1} in context scratch, BPTT with whole contractions in every CTA where few
  *                                 units are kept (0: forward over all H columns, the dropped ones being zero, BPTT's
- *                                 contraction always shared by a cluster of CTAs); same results up to the order of
- *                                 fp32 additions
+ *                                 contraction shared by a cluster of CTAs whatever is kept, where the device holds
+ *                                 all of the layer's CTAs in clusters); same results up to the order of fp32 additions
  * Errors: ARD_ERR_INVALID_ARG (unknown option, negative value). */
 typedef enum { ARD_OPT_PDL = 0, ARD_OPT_PDL_IN_CAPTURE = 1, ARD_OPT_SIDE_STREAMS = 2, ARD_OPT_CTA_PAIRS = 3,
                ARD_OPT_BAND_ROWS = 4, ARD_OPT_MLP_PERSISTENT = 5, ARD_OPT_LSTM_COMPACT_H = 6 } ard_option;
@@ -576,7 +576,7 @@ ard_status ard_lstm_gate_gemm_bwd(ard_ctx* ctx, const ard_pattern* pat, int B, i
 
 /* Whole-sequence forward: for t = 0..T-1, the gate product on XH[t] followed by the cell update, which writes
  * h_t into the h half of XH[t+1].  When the layer fits (B <= 128; 8 or 12 hidden units per SM, whose recurrent weight
- * rows fit in shared memory beside part of h; any alignment with ARD_PATH_AUTO) this
+ * rows fit in shared memory beside part of h: on 148 SMs 1664 units, 1776 with B <= 64; any alignment with ARD_PATH_AUTO) this
  * is ONE cooperative kernel that keeps the weight in shared memory and the cell state in registers for the
  * whole sequence and synchronises the SMs once per step (every wait bounded, see ARD_ERR_TIMEOUT); Z is
  * then not used.  Otherwise, or after ard_set_lstm_persistent(ctx, 0), it is a loop in native code that
@@ -596,8 +596,9 @@ ard_status ard_lstm_forward(ard_ctx* ctx, const ard_pattern* pat, int T, int B, 
  * half of D[0] the gradient of h_0.  dH_last [B][H] fp32 is the gradient of h_{T-1}; dc [B][H] fp32 must be
  * zero on entry (or hold the gradient of c_T) and returns the gradient of c_0; DZ [T][B][4H] bf16 scratch;
  * dW [4H][I+H] fp32 receives the weight gradient (dropped units' rows zero).
- * When the layer fits (as for ard_lstm_forward) and
- * ard_set_lstm_persistent is on, the recurrence dh_{t-1} = upstream + dz_t W_h with the cell adjoint is ONE
+ * When the layer fits (as for ard_lstm_forward, but on 148 SMs B <= 128 up to 1408 units, 85 up to 1536, 64 up to 1584, less
+ * beyond; and where DZ is not 16-byte aligned or H no multiple of 8, T * B * 8 * H bytes, H rounded up to a multiple of 8,
+ * must not exceed the 256 KB per SM of the context's scratch: 38.8 MB on 148 SMs) and ard_set_lstm_persistent is on, the recurrence dh_{t-1} = upstream + dz_t W_h with the cell adjoint is ONE
  * cooperative kernel (weight slices resident in shared memory, dc in registers, one bounded grid-wide synchronisation
  * per step) and the x halves come from one product over all T*B rows; otherwise a loop
  * in native code enqueues ard_lstm_gates_bwd and ard_lstm_gate_gemm_bwd per step.  In both cases the h

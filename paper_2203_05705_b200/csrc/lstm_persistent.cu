@@ -65,8 +65,8 @@ struct LstmPlan {
   int behind;     // bytes from the slice on, without the staged sums
   int bytes;      // everything behind the barriers
 };
-// The MMA always reads 128 rows, so what lies behind a slot has to exist: 16 KiB from the start of the last slot.  tail:
-// bytes that the MMA may read behind the slice.
+// An MMA reads 64 or 128 rows (lstm_mma_rows) however many the batch has, so what lies behind a slot has to exist: 16 KiB
+// from the start of the last slot serve both.  tail: bytes that the MMA may read behind the slice.
 __host__ __device__ inline LstmPlan lstm_plan(int blocks, int a_block, int w_block, int tail, int zs, int smem_bytes) {
   LstmPlan r;
   r.gsz = (blocks + LP_GROUPS - 1) / LP_GROUPS;
@@ -255,8 +255,7 @@ __device__ __forceinline__ void lstm_forward_body(const LstmFwdParams& p, uint8_
   const int nkb = ((compact ? n_keep : p.H) + LP_BK - 1) / LP_BK;
   // The staged pre-activations share the start of the ring where they fit: they are written after the step's MMAs
   // have completed and read before this CTA releases h_t, and the next loads are issued only after every CTA has
-  // released.  Without them the kernel stays below 196 KB of shared memory at H = 1024; one carve-out step higher
-  // (228 KB, next to no L1 left) this kernel was measured 1.5 % slower and the BPTT kernel 4 %.
+  // released.
   const LstmPlan plan = lstm_plan(nkb, (int)a_block, W_BLOCK, 0, (p.B + 31) / 32 * 32 * ZS_LD * 4, p.smem_bytes);
   const int gsz = plan.gsz, cap = plan.cap;
   const uint32_t sA = base + LP_BAR_BYTES;

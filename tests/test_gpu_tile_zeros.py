@@ -21,11 +21,12 @@ def test_dropped_tiles_are_zero(ts, rows, cols, dw):
     try:
         ard.ard_set_path(ctx.h, ard.ARD_PATH_TENSOR_CORE)
         pat = ctx.pattern(ard.ARD_TILE, K, N, ts)
-        for dp, b in [(2, 1), (2, 2), (3, 2), (7, 7), (rows * cols, rows * cols // 2)]:
+        for i, (dp, b) in enumerate([(2, 1), (2, 2), (3, 2), (7, 7), (rows * cols, rows * cols // 2)]):
             if dp > 64:
                 continue
             ard.ard_pattern_set(ctx.h, pat, dp, b)
-            res = run_three_gemms(ctx, pat, ard.ARD_TILE, ard.ARD_BF16, X, W, dY, dp, b, 2.0, ts=ts, zero_fill=True, dw_dtype=dw)
+            res = run_three_gemms(ctx, pat, ard.ARD_TILE, ard.ARD_BF16, X, W, dY, dp, b, 2.0, ts=ts, zero_fill=True, dw_dtype=dw,
+                                  lds={"w": K + 8 * (i % 2)})
             assert_ok(res, TOL[ard.ARD_BF16], (ts, dp, b))
     finally:
         ctx.close()
