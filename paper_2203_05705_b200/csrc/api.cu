@@ -752,8 +752,7 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
   g.out_is_f32 = dW_dtype == ARD_F32;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
   if (in_pat && zero_fill_dropped) return ARD_ERR_INVALID_ARG;  // the packed gradient has no rows of dropped neurons
-  // The kernels write the zeros of dropped rows and pattern tiles themselves, but for the tensor-core kernels of a fixed
-  // tile width (below).
+  // The kernels write the zeros of dropped rows and pattern tiles themselves.
   // Empty batch: the gradient of every kept weight is zero; the CUDA-core kernel writes exactly that.
   if (B == 0) return launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
 
@@ -781,10 +780,6 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     st = get_maps(ctx, dyc, B, N, ldc, N, MAP_COMPACT_COLS, pat->dp_bound, 64, 64, &t.mapA, dense, dense_ld);
     t.mapA_indexed = 1;
   } else {
-    if (zero_fill_dropped && t.bn != 0) {  // the class form (0) writes them itself
-      st = launch_zero_dropped_tiles(ctx, pat, dW, lddw, es_out, s);
-      if (st != ARD_OK) return st;
-    }
     st = get_maps(ctx, dY, B, N, lddy, 0, MAP_PLAIN, 0, 64, 64, &t.mapA);
     t.mapA_indexed = 0;
   }

@@ -275,9 +275,6 @@ ard_status launch_rows_gather(ard_ctx* ctx, const ard_rows* rows, const void* sr
 ard_status launch_zero_dropped_rows(ard_ctx* ctx, const ard_rows* rows, void* out, int ld_bytes, int row_bytes,
                                     cudaStream_t s);
 
-ard_status launch_zero_dropped_tiles(ard_ctx* ctx, const ard_pattern* pat, void* dW, int lddw, int elem_bytes,
-                                     cudaStream_t s);
-
 // Layer-step helpers (aux_kernels.cu); elem_bytes 2 or 4.
 ard_status launch_compact_weight_cols(ard_ctx* ctx, const int32_t* hdr, const int32_t* hdr_in, const void* W, int ldw,
                                       void* Wk, int ldwk, int N, int K, int elem_bytes, cudaStream_t s);

@@ -52,6 +52,14 @@ __device__ __forceinline__ uint64_t pack2(float lo, float hi) {
 }
 __device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) { asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b)); }
 
+// A call, not inlined: inlined, the loops take registers from the product's (4096 x 33 x 4096 in fp32, a dense draw, 63 -> 79 us).
+template <int KIND>
+__device__ __noinline__ void cc_zeros(const GemmArgs& g, int ts, int cols, int warps) {
+  const int warp = (int)blockIdx.x * warps + ((int)threadIdx.x >> 5), all = (int)gridDim.x * warps, lane = threadIdx.x & 31;
+  if (KIND == 1) zero_dropped_tiles(g, ts, warp, all, lane);
+  else zero_dropped_rows(g, cols, warp, all, lane);
+}
+
 // R: rows and columns of the output tile (64 or 32); a thread of the R / 4 x 8 grid owns 4 rows by R / 8 columns of it,
 // multiplied two columns an instruction.  The operands of a KT-deep block are staged k-major as fp32, [k][row], through registers, one block ahead of the
 // products.  KIND: 0 row, 1 tile.  OP: GemmOp.
@@ -88,8 +96,7 @@ __global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_con
   const bool whole = KIND == 0 || (p.ts & 3) == 0;  // four consecutive positions never leave a pattern tile
   const bool vec_a = (p.vec & 1) && step_a == 1 && whole, vec_b = (p.vec & 2) && whole;
 
-  if (KIND == 1 && OP == OP_BWD_WEIGHT && g.flag1)
-    sp_zero_dropped_tiles(g, p.ts, (int)blockIdx.x * (CC_THREADS / 32) + warp, (int)gridDim.x * (CC_THREADS / 32), lane);
+  if (OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1) cc_zeros<KIND>(g, p.ts, KIND == 0 ? s.N : 0, CC_THREADS / 32);
   for (int u = (int)blockIdx.x / CC_CLUSTER; u < units; u += n_cl) {
     const int t = u * groups + group;
     ProductTile ti = {};
@@ -201,7 +208,7 @@ __global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_con
     }
     if (s.S > 1) cluster_sync_all();  // the partial tiles of the group are complete
     else __syncthreads();
-    if (live) write_tile<KIND, OP, R, R, PITCH, CC_THREADS / 32, T>(g, s, ti, sm, smem_u32(sm), part, lead, warp, lane);
+    if (live) write_tile<KIND, OP, R, R, PITCH, CC_THREADS / 32, false, T>(g, s, ti, sm, smem_u32(sm), part, lead, warp, lane);
     __syncwarp();
     if (s.S > 1) cluster_sync_all();  // no CTA of the group reads this one's partial tile any more
     else __syncthreads();

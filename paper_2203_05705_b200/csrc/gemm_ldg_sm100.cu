@@ -123,11 +123,15 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
   const ProductPlan s = make_plan<KIND, OP, UMMA_BM, BN, LG_BK>(g, p.ts, (int)gridDim.x, p.cl);
   const int rank = (int)cluster_ctarank();
   const int part = rank & (s.S - 1);          // this CTA's share of the contraction
-  const int lead = rank - part;               // first CTA of the tile's group
-  const int group = rank / s.S, groups = p.cl / s.S;
+  const int lead = rank - part;               // first CTA of those that share it
+  const int rows = rank & (s.G - 1);          // this CTA's part of the tile's rows
+  const int group = rank / s.G, groups = p.cl / s.G;
   const int n_cl = (int)gridDim.x / p.cl, units = (s.tiles + groups - 1) / groups;
-  if (KIND == 1 && OP == OP_BWD_WEIGHT && g.flag1 && warp < LG_LOADERS / 32)
-    sp_zero_dropped_tiles(g, p.ts, (int)blockIdx.x * (LG_LOADERS / 32) + warp, (int)gridDim.x * (LG_LOADERS / 32), lane);
+  if (OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1 && warp < LG_LOADERS / 32) {
+    const int w = (int)blockIdx.x * (LG_LOADERS / 32) + warp, ws = (int)gridDim.x * (LG_LOADERS / 32);
+    if (KIND == 1) zero_dropped_tiles(g, p.ts, w, ws, lane);
+    else zero_dropped_rows(g, s.N, w, ws, lane);
+  }
   int blk = 0;        // blocks staged so far: stage = blk % STAGES
   int done = 0;       // accumulators finished so far
   bool ok = true;
@@ -352,7 +356,7 @@ __global__ void __launch_bounds__(LG_THREADS, 2) gemm_ldg_kernel(const __grid_co
 
     if (warp < 8 && live) {
       // ===================== epilogue =====================
-      write_tile<KIND, OP, UMMA_BM, BN, L::PITCH, LG_LOADERS / 32, __nv_bfloat16>(g, s, ti, reinterpret_cast<float*>(smem), base, part,
+      write_tile<KIND, OP, UMMA_BM, BN, L::PITCH, LG_LOADERS / 32, true, __nv_bfloat16>(g, s, ti, reinterpret_cast<float*>(smem), base, rows,
                                                                                  lead, warp, lane);
       if (s.S == 1) asm volatile("bar.sync 1, 256;" ::: "memory");  // the tile has been read: the stages may be filled again
     }

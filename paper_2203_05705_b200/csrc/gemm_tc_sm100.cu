@@ -22,6 +22,7 @@
 #include "ard_internal.h"
 #include <type_traits>
 
+#include "dropped_zeros.h"
 #include "sm100_ptx.h"
 
 namespace {
@@ -94,7 +95,7 @@ struct TcParams {
   int ldo;
   int out_is_f32;
   int scatter;    // row fwd: full-width output with zero fill
-  int zero_fill;  // row and class bwd-weight: write zeros to dropped rows / tiles
+  int zero_fill;  // bwd-weight: write zeros to dropped rows / tiles
   int force_bn;   // row modes: 0 = choose the N tile on the device, else a multiple of 32 in 64 .. 256
   int accumulate; // plain stores add to the existing output
   int band_m;     // M-tiles per raster band (0: one band)
@@ -1067,22 +1068,11 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
     int it = 0, nacc = 0;
     bool ok = true;
     Unit un;
-    if (MODE == M_TILEC_BWD_WEIGHT && !PLAIN && p.zero_fill) {
+    if (((MODE == M_TILEC_BWD_WEIGHT && !PLAIN) || MODE == M_TILE_BWD_WEIGHT) && p.zero_fill && dp > 1) {
       // The dropped tiles of dW are zero (Sec. 3.2).  These warps write them while the first tile's products run; a
       // launch of its own waited for SMs that the other products held and kept this kernel waiting (three products,
-      // 64-wide tiles of 4096 x 4096, batch 1024, a period of 4: 66 us with it, 60 without).  The j-th dropped tile: bb
-      // of them precede the first kept one, dp - 1 follow each kept one.
-      const int row_bytes = p.ts * (p.out_is_f32 ? 4 : 2), per_row = row_bytes >> 4;  // 8 .. 32 lanes per row
-      const int rows = 32 / per_row, n_drop = sch.Tr * sch.Tc - sch.n_keep;
-      for (int j = (int)blockIdx.x * EPI_WARPS + warp - 2; j < n_drop; j += (int)gridDim.x * EPI_WARPS) {
-        const int after = j - bb;
-        const int lin = after < 0 ? j : bb + after / (dp - 1) * dp + 1 + after % (dp - 1);
-        const int r = lin / sch.Tc, c = lin - r * sch.Tc;  // tile-row along the fan-in, tile-column along the neurons
-        char* tile = reinterpret_cast<char*>(p.out) + ((size_t)c * p.ts * p.ldo + (size_t)r * p.ts) * (p.out_is_f32 ? 4 : 2) +
-                     (lane % per_row) * 16;
-        for (int n = lane / per_row; n < p.ts; n += rows)
-          *reinterpret_cast<uint4*>(tile + (size_t)n * p.ldo * (p.out_is_f32 ? 4 : 2)) = make_uint4(0, 0, 0, 0);
-      }
+      // 64-wide tiles of 4096 x 4096, batch 1024, a period of 4: 66 us with it, 60 without).
+      zero_dropped_tiles(p, p.ts, (int)blockIdx.x * EPI_WARPS + warp - 2, (int)gridDim.x * EPI_WARPS, lane);
     }
     for (; ok && sch.unit(w0, it, un); ++it) {
       const TileInfo ti = sch.template tile<PLAIN>(p, un.t);

@@ -11,6 +11,7 @@
 #pragma once
 
 #include "ard_internal.h"
+#include "dropped_zeros.h"
 #include "sm100_ptx.h"
 
 namespace {
@@ -20,7 +21,8 @@ struct ProductPlan {
   int M, N, K;         // extents of the product (tile patterns: K is the batch for the weight gradient, else unused)
   int Mt;              // tiles along M
   int tiles;           // output tiles (weight gradient of a tile pattern: an upper bound, some may turn out empty)
-  int S;               // CTAs per output tile
+  int S;               // shares that a tile's contraction is cut into
+  int G;               // CTAs per output tile: S, or more that compute the same shares and write other rows
   // tile patterns: class c (tiles with equal number mod cstep) has q + (c < rmd) members
   int ts, lts;         // pattern tile, its log2 (-1: not a power of two)
   int cstep, q, rmd, nclass;
@@ -50,28 +52,6 @@ struct ProductTile {
 };
 
 __device__ __forceinline__ int sp_cdiv(int a, int b) { return (a + b - 1) / b; }
-
-// Tile patterns, weight gradient: zeros of the dropped tiles (Sec. 3.2), dealt to the grid's `warps` warps.  They go out
-// while the first blocks are on their way; a kernel of its own ahead of the product was one more dependent launch
-// (2048 x 2048, 32-wide tiles, batch 128, a period of 2, sampler and three products: 50.8 us with it, 48.5 without).  The j-th dropped tile: bb of them precede the first kept one, dp - 1 follow each kept one.
-__device__ __forceinline__ void sp_zero_dropped_tiles(const GemmArgs& g, int ts, int warp, int warps, int lane) {
-  const int dp = g.hdr[HDR_DP], bb = g.hdr[HDR_B] - 1, Tc = g.hdr[HDR_TC];
-  const int n_drop = g.hdr[HDR_TR] * Tc - g.hdr[HDR_NKEEP], es = g.out_is_f32 ? 4 : 2;
-  const size_t pitch = (size_t)g.ldo * es;
-  const bool wide = ((ts * es) & 15) == 0 && (pitch & 15) == 0 && (reinterpret_cast<uintptr_t>(g.out) & 15) == 0;
-  const int per_row = wide ? ts * es >> 4 : ts * es >> 1, piece = wide ? 16 : 2;
-  for (int j = warp; j < n_drop; j += warps) {
-    const int after = j - bb, lin = after < 0 ? j : bb + after / (dp - 1) * dp + 1 + after % (dp - 1);
-    const int r = lin / Tc, c = lin - r * Tc;  // tile-row along the fan-in, tile-column along the neurons
-    char* tile = reinterpret_cast<char*>(g.out) + (size_t)c * ts * pitch + (size_t)r * ts * es;
-    for (int e = lane; e < ts * per_row; e += 32) {
-      const int n = e / per_row, q = e - n * per_row;
-      char* d = tile + (size_t)n * pitch + (size_t)q * piece;
-      if (wide) *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
-      else *reinterpret_cast<uint16_t*>(d) = 0;
-    }
-  }
-}
 
 // want: CTAs the device has room for at once; cl: CTAs per cluster.
 template <int KIND, int OP, int BM, int BN, int BK>
@@ -125,6 +105,12 @@ __device__ __forceinline__ ProductPlan make_plan(const GemmArgs& g, int ts, int 
   // two cluster barriers and a pass of the partial tiles through shared memory.
   s.S = cl;
   while (s.S > 1 && (s.tiles * s.S > want || nkb < 2 * s.S)) s.S >>= 1;
+  // A full-width output under a long period is up to dp times as wide as what is multiplied: where the contraction is too
+  // short to be cut, CTAs that would be idle compute the tile once more and write a part of its rows (forward, 2000 x 129 ->
+  // 2047 under a period of 16: 103 -> 43 us).
+  s.G = s.S;
+  if (KIND == 0 && OP == OP_FWD && g.flag0 == ARD_OUT_SCATTER_ZEROFILL && s.dp > 1)
+    while (s.G < cl && s.tiles * s.G * 2 <= want) s.G <<= 1;
   return s;
 }
 
@@ -180,12 +166,14 @@ __device__ __forceinline__ float4 sum_shares(uint32_t off, int lead) {
 }
 
 // The CTA's rows of a finished tile (fp32, PITCH words per row in shared memory at T / address t_addr): rows
-// [part * BM / S, (part + 1) * BM / S), dealt to NW warps.  With S > 1 the group's shares are added into this CTA's
-// own copy first.  T_: operand type (the saved activation's).
-template <int KIND, int OP, int BM, int BN, int PITCH, int NW, typename T_>
+// [part * BM / G, (part + 1) * BM / G), dealt to NW warps.  With S > 1 the shares of CTAs lead .. lead + S - 1 are added
+// into this CTA's own copy first.  T_: operand type (the saved activation's).  SPREAD: G may exceed S, and rows off
+// the grid of four elements get wide stores between their edges (not for the CUDA-core kernels, whose loop lost a quarter of
+// its speed to the code's registers; there G is S).
+template <int KIND, int OP, int BM, int BN, int PITCH, int NW, bool SPREAD, typename T_>
 __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan& s, const ProductTile& ti, float* T, uint32_t t_addr,
                                            int part, int lead, int warp, int lane) {
-  const int rows_per = BM / s.S, r0 = part * rows_per;
+  const int rows_per = BM / (SPREAD ? s.G : s.S), r0 = part * rows_per;
   if (s.S > 1) {
     for (int i = lane; i < rows_per / NW * (BN / 4); i += 32) {  // this warp's rows r0 + warp, r0 + warp + NW, ...
       const int row = r0 + warp + NW * (i / (BN / 4)), w = row * PITCH + 4 * (i % (BN / 4));
@@ -206,16 +194,20 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
       *o = __float2bfloat16_rn(g.accumulate ? __bfloat162float(*o) + val : val);
     }
   };
+  // v to four consecutive elements whose address is a multiple of four of them
+  auto put4_aligned = [&](size_t off, const float (&v)[4]) {
+    if (g.out_is_f32) {
+      *reinterpret_cast<float4*>(reinterpret_cast<float*>(g.out) + off) = make_float4(v[0], v[1], v[2], v[3]);
+    } else {
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
+      *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(g.out) + off) =
+          make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    }
+  };
   // v, the first nv of them, to four consecutive elements; off is a multiple of four
   auto put4 = [&](size_t off, const float (&v)[4], int nv) {
     if (vec && nv >= 4) {
-      if (g.out_is_f32) {
-        *reinterpret_cast<float4*>(reinterpret_cast<float*>(g.out) + off) = make_float4(v[0], v[1], v[2], v[3]);
-      } else {
-        const __nv_bfloat162 lo = __floats2bfloat162_rn(v[0], v[1]), hi = __floats2bfloat162_rn(v[2], v[3]);
-        *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(g.out) + off) =
-            make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-      }
+      put4_aligned(off, v);
       return;
     }
 #pragma unroll
@@ -235,8 +227,14 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
     for (int r = r0 + warp; r < r0 + rows_per && ti.m0 + r < s.M; r += NW) {
       const float* row = T + r * PITCH;
       const size_t base = (size_t)(ti.m0 + r) * g.ldo;
-      for (int c = lo + 4 * lane; c < hi; c += 128) {
-        const int rel = c - s.bb;
+      int first = lo;  // of the pieces of four columns; off the grid the piece before the first one on it reaches back past lo
+      if (SPREAD && !vec) {
+        const uintptr_t at = reinterpret_cast<uintptr_t>(g.out) + (base + lo) * es;
+        const int sh = (int)((0 - at) & (uintptr_t)(4 * es - 1)) / es;  // columns up to the grid
+        first = sh == 0 ? lo : lo + sh - 4;
+      }
+      for (int c = first + 4 * lane; c < hi; c += 128) {
+        const int rel = max(c, lo) - s.bb;
         int j = rel <= 0 ? 0 : (rel + s.dp - 1) / s.dp;  // first kept column at or after c
         int at = s.bb + j * s.dp - c;
         float v[4];
@@ -249,7 +247,17 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
             at += s.dp;
           }
         }
-        put4(base + c, v, hi - c);
+        if (SPREAD && !vec) {
+          if (c >= lo && hi - c >= 4 && !g.accumulate) {
+            put4_aligned(base + c, v);
+          } else {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (c + i >= lo && c + i < hi) put(base + c + i, v[i]);
+          }
+        } else {
+          put4(base + c, v, hi - c);
+        }
       }
     }
     return;
@@ -287,14 +295,6 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (i < nv) put(orow * g.ldo + pos(n + i), v[i]);
-    }
-    if (KIND == 0 && OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1) {
-      // compact row m owns output rows [m * dp, (m + 1) * dp), the last one the tail: zeros but for its own
-      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
-      const long long first = (long long)m * s.dp;
-      const long long last = m == s.M - 1 ? g.N : min((long long)g.N, first + s.dp);
-      for (long long z = first; z < last; ++z)
-        if (z != (long long)orow) put4((size_t)z * g.ldo + n, zero, nv);
     }
   }
 }
