@@ -11,8 +11,8 @@
 //
 // Bound: the load unit and the latency of its copies (two CTAs share an SM); the tensor
 // pipe is nearly idle.  Three products of a layer, against the CUDA-core kernel that took these shapes before:
-// 700 x 1500 x 1500 under a row pattern of period 2 463 -> 73 us, 128 x 2048 x 2048 under 32 x 32 tiles of period 2
-// 519 -> 51 us.
+// 700 x 1500 x 1500 under a row pattern of period 2 465 -> 69 us, 128 x 2048 x 2048 under 32 x 32 tiles of period 2
+// 519 -> 49 us (with the sampler's launch).
 #include "staged_product.h"
 
 namespace {
