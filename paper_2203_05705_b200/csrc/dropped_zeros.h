@@ -16,28 +16,33 @@ __device__ __forceinline__ int dropped_unit(int j, int bb, int dp) {
 // their way; a kernel of its own ahead of the product was one more dependent launch (2048 x 2048, 32-wide tiles, batch 128, a
 // period of 2, sampler and three products: 50.8 us with it, 48.5 without).
 // Tile patterns (Sec. 3.2): a warp takes up to ZERO_PIECES pieces of a tile at a time, so that a few large tiles find as many
-// warps as many small ones.
+// warps as many small ones, and a tile of up to 64 x 64 bf16 values stays with one warp (pieces of a quarter of that: three
+// products of 4096 x 4096 with 64-wide tiles, batch 1024, a period of 4, 60 -> 65 us).
 template <typename Args>
 __device__ __forceinline__ void zero_dropped_tiles(const Args& g, int ts, int warp, int warps, int lane) {
-  constexpr int ZERO_PIECES = 128;
+  constexpr int ZERO_PIECES = 512;
   const int dp = g.hdr[HDR_DP], bb = g.hdr[HDR_B] - 1, Tc = g.hdr[HDR_TC];
   const int n_drop = g.hdr[HDR_TR] * Tc - g.hdr[HDR_NKEEP], es = g.out_is_f32 ? 4 : 2;
   const size_t pitch = (size_t)g.ldo * es;
   const bool wide = ((ts * es) & 15) == 0 && (pitch & 15) == 0 && (reinterpret_cast<uintptr_t>(g.out) & 15) == 0;
   const int per_row = wide ? ts * es >> 4 : ts * es >> 1, piece = wide ? 16 : 2;
-  const long long per_tile = (long long)ts * per_row, chunks = (per_tile + ZERO_PIECES - 1) / ZERO_PIECES;
-  for (long long u = warp; u < n_drop * chunks; u += warps) {
-    const int j = (int)(u / chunks);
-    const long long e0 = (u - j * chunks) * ZERO_PIECES;
+  const int step_n = 32 / per_row, step_q = 32 - step_n * per_row;
+  // 32 bits: a matrix of 180 GB has fewer than 1e9 such units
+  const int chunks = (int)(((long long)ts * per_row + ZERO_PIECES - 1) / ZERO_PIECES);
+  for (int u = warp; u < n_drop * chunks; u += warps) {
+    const int j = u / chunks;
+    const unsigned long long e = (unsigned long long)(u - j * chunks) * ZERO_PIECES + lane;
     const int lin = dropped_unit(j, bb, dp);
     const int r = lin / Tc, c = lin - r * Tc;  // tile-row along the fan-in, tile-column along the neurons
     char* tile = reinterpret_cast<char*>(g.out) + (size_t)c * ts * pitch + (size_t)r * ts * es;
-    int n = (int)((e0 + lane) / per_row), q = (int)(e0 + lane - (long long)n * per_row);
+    int n = (int)(e >> 32 ? e / per_row : (unsigned)e / (unsigned)per_row), q = (int)(e - (unsigned long long)n * per_row);
     for (int i = 0; i < ZERO_PIECES / 32 && n < ts; ++i) {
       char* d = tile + (size_t)n * pitch + (size_t)q * piece;
       if (wide) *reinterpret_cast<uint4*>(d) = make_uint4(0u, 0u, 0u, 0u);
       else *reinterpret_cast<uint16_t*>(d) = 0;
-      for (q += 32; q >= per_row; q -= per_row) ++n;
+      n += step_n;
+      q += step_q;
+      if (q >= per_row) { q -= per_row; ++n; }
     }
   }
 }

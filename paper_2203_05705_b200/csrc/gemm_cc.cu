@@ -96,7 +96,10 @@ __global__ void __launch_bounds__(cc_threads(R)) gemm_cc_kernel(const __grid_con
   const bool whole = KIND == 0 || (p.ts & 3) == 0;  // four consecutive positions never leave a pattern tile
   const bool vec_a = (p.vec & 1) && step_a == 1 && whole, vec_b = (p.vec & 2) && whole;
 
-  if (OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1) cc_zeros<KIND>(g, p.ts, KIND == 0 ? s.N : 0, CC_THREADS / 32);
+  // Rows: dealt to all warps by the small tile where the contraction is not cut; else each row's zeros are left to the CTAs of
+  // its tile (fp32, weight gradient, dealt and left: 16 x 2047 -> 2045, a period of 3, 15 and 23 us; 2000 x 129 -> 2047 39
+  // and 30; and the call alone costs the large tile's loop 2 % and more).
+  if (OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1 && (KIND == 1 || (R == 32 && s.S == 1))) cc_zeros<KIND>(g, p.ts, KIND == 0 ? s.N : 0, CC_THREADS / 32);
   for (int u = (int)blockIdx.x / CC_CLUSTER; u < units; u += n_cl) {
     const int t = u * groups + group;
     ProductTile ti = {};

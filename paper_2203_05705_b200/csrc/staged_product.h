@@ -169,7 +169,7 @@ __device__ __forceinline__ float4 sum_shares(uint32_t off, int lead) {
 // [part * BM / G, (part + 1) * BM / G), dealt to NW warps.  With S > 1 the shares of CTAs lead .. lead + S - 1 are added
 // into this CTA's own copy first.  T_: operand type (the saved activation's).  SPREAD: G may exceed S, and rows off
 // the grid of four elements get wide stores between their edges (not for the CUDA-core kernels, whose loop lost a quarter of
-// its speed to the code's registers; there G is S).
+// its speed to the code's registers; there G is S, and the CTAs that share a tile write the zeros that belong to its rows).
 template <int KIND, int OP, int BM, int BN, int PITCH, int NW, bool SPREAD, typename T_>
 __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan& s, const ProductTile& ti, float* T, uint32_t t_addr,
                                            int part, int lead, int warp, int lane) {
@@ -295,6 +295,14 @@ __device__ __forceinline__ void write_tile(const GemmArgs& g, const ProductPlan&
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         if (i < nv) put(orow * g.ldo + pos(n + i), v[i]);
+    }
+    if (!SPREAD && KIND == 0 && OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1 && (BM == 64 || s.S > 1)) {
+      // compact row m owns output rows [m * dp, (m + 1) * dp), the last one the tail: zeros but for its own
+      const float zero[4] = {0.f, 0.f, 0.f, 0.f};
+      const long long first = (long long)m * s.dp;
+      const long long last = m == s.M - 1 ? g.N : min((long long)g.N, first + s.dp);
+      for (long long z = first; z < last; ++z)
+        if (z != (long long)orow) put4((size_t)z * g.ldo + n, zero, nv);
     }
   }
 }
