@@ -29,8 +29,11 @@
  *     the device can see (a wait inside a kernel that ran out of patience) set a sticky device
  *     status word, read with ard_last_device_status; the kernel then exits normally and the output
  *     of that call is unspecified.  Nothing aborts or traps.
- *   - Arithmetic: ARD_F32 operands are multiplied and accumulated in fp32 on the CUDA cores;
- *     ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
+ *   - Arithmetic: ARD_F32 operands are multiplied and accumulated in fp32 on the CUDA cores, or, in products of
+ *     more than 1.5e8 kept operations under ARD_PATH_AUTO, split into three bf16 parts each and multiplied on the
+ *     tensor cores with fp32 accumulation (an error no larger than the CUDA cores' against fp64; elements below
+ *     2^-109 lose what a bf16 subnormal cannot hold, 2^-134 in absolute terms; results that are infinite or NaN are
+ *     those of the CUDA cores).  ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
  *   - There is no CPU fallback.
  */
 #ifndef ARD_H_

@@ -80,6 +80,7 @@ ard_status check_common(ard_ctx* ctx, const ard_pattern* pat, int B, int K, int 
 }
 
 void fill_common(GemmArgs& g, ard_ctx* ctx, const ard_pattern* pat, int B, int K, int N, float alpha) {
+  g.keep = pat->keep;
   g.hdr = pat->d_hdr;
   g.idx = pat->d_idx;
   g.col_ptr = pat->d_col_ptr;
@@ -372,6 +373,9 @@ ard_status ard_set_distribution(ard_ctx* ctx, int dist_id, const double* K, int 
   ARD_CUDA_OK(cudaMemcpy(d.d_cdf, cdf.data(), sizeof(unsigned long long) * ndp, cudaMemcpyHostToDevice));
   d.h_cdf = cdf;
   d.ndp = ndp;
+  double keep = 0.0;
+  for (int i = 0; i < ndp; ++i) keep += (double)(cdf[i] - (i > 0 ? cdf[i - 1] : 0ull)) / 4294967296.0 / (i + 1);
+  d.keep = (float)keep;
   return ARD_OK;
 }
 
@@ -406,6 +410,7 @@ ard_status ard_pattern_create(ard_ctx* ctx, ard_pattern** out, ard_kind kind, in
   if (units > (1ll << 30)) { delete p; return ARD_ERR_UNSUPPORTED; }
   p->units = (int)units;
   p->dp_bound = 1;
+  p->keep = 1.f;
   p->generation = 0;
   size_t words = HDR_WORDS + (size_t)p->units;
   if (kind == ARD_TILE) words += (size_t)(p->Tc + 1) + (size_t)(p->Tr + 1) + 2 * (size_t)p->units;
@@ -444,6 +449,7 @@ ard_status ard_sample_pattern(ard_ctx* ctx, ard_pattern* pat, int dist_id, uint6
   if (d.ndp == 0 || d.ndp > pat->units) return ARD_ERR_DISTRIBUTION;
   DeviceGuard guard(ctx->device);
   pat->dp_bound = d.ndp;
+  pat->keep = d.keep;
   pat->generation++;
   return launch_sampler(ctx, pat, d.d_cdf, d.ndp, seed, iteration, stream_id, 0, 0, (cudaStream_t)cuda_stream);
 }
@@ -453,6 +459,7 @@ ard_status ard_pattern_set(ard_ctx* ctx, ard_pattern* pat, int dp, int b, void* 
   if (dp < 1 || b < 1 || b > dp || dp > pat->units) return ARD_ERR_INVALID_ARG;
   DeviceGuard guard(ctx->device);
   pat->dp_bound = dp;
+  pat->keep = 1.f / (float)dp;
   pat->generation++;
   return launch_sampler(ctx, pat, nullptr, 0, 0, 0, 0, dp, b, (cudaStream_t)cuda_stream);
 }
@@ -529,6 +536,7 @@ static ard_status fwd_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_patte
   g.out_is_f32 = out_f32;
   g.accumulate = accumulate;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
+  if (in_pat) g.keep *= in_pat->keep;
   g.bias = bias;
   g.relu = relu ? 1 : 0;
   if (accumulate && (bias != nullptr || relu)) return ARD_ERR_INVALID_ARG;
@@ -590,7 +598,7 @@ ard_status ard_layer_fwd(ard_ctx* ctx, const ard_pattern* pat, const ard_pattern
 // with_dense: a dense pattern is copied too (the caller reads the copy in every case).
 static ard_status compact_dy(ard_ctx* ctx, const ard_pattern* pat, int B, int N, const void* dY, int lddy,
                              int dy_is_compact, const void** out_ptr, int* out_ld, const void** dense_ptr,
-                             int* dense_ld, cudaStream_t s, int with_dense = 0) {
+                             int* dense_ld, cudaStream_t s, int with_dense = 0, int es = 2) {
   *dense_ptr = nullptr;
   *dense_ld = 0;
   if (dy_is_compact) {
@@ -602,15 +610,15 @@ static ard_status compact_dy(ard_ctx* ctx, const ard_pattern* pat, int B, int N,
   *dense_ptr = dY;
   *dense_ld = lddy;
   const int ldc = (N + 7) / 8 * 8;
-  if ((size_t)B * ldc * 2 > ctx->workspace_bytes) return ARD_ERR_NOMEM;
+  if ((size_t)B * ldc * es > ctx->workspace_bytes) return ARD_ERR_NOMEM;
   *out_ptr = ctx->d_workspace;
   *out_ld = ldc;
   auto& lg = ctx->last_gather;
   if (ctx->reuse_compact && lg.src == dY && lg.ld == lddy && lg.B == B && lg.N == N && lg.pat == pat &&
-      lg.gen == pat->generation && lg.stream == s && lg.with_dense >= with_dense)
+      lg.gen == pat->generation && lg.stream == s && lg.with_dense >= with_dense && lg.es == es)
     return ARD_OK;  // the previous backward call on this stream already compacted this dY for this pattern
-  lg = {dY, lddy, B, N, pat, pat->generation, s, with_dense};
-  ard_status st = launch_gather_cols(ctx, pat->d_hdr, pat->d_idx, dY, lddy, ctx->d_workspace, ldc, B, 2, N, !with_dense, s);
+  lg = {dY, lddy, B, N, pat, pat->generation, s, with_dense, es};
+  ard_status st = launch_gather_cols(ctx, pat->d_hdr, pat->d_idx, dY, lddy, ctx->d_workspace, ldc, B, es, N, !with_dense, s);
   *out_ptr = ctx->d_workspace;
   *out_ld = ldc;
   return st;
@@ -632,6 +640,25 @@ static ard_status bwd_staged_by_threads(ard_ctx* ctx, const ard_pattern* pat, Ge
     g.flag0 = 1;
   }
   return launch_gemm_ldg(ctx, pat->kind, op, g, pat->ts, s);
+}
+
+// A backward product of an fp32 layer.  Columns of a full-width dY lie dp apart; from 2e9 kept operations on the product reads
+// them often enough that a compact copy in the workspace, where it fits, is the faster way (1024 x 4096 x 4096, a period of 2,
+// the two backward products 278 and 265 us without it, 189 and 196 with it, its launches included).
+static ard_status bwd_f32(ard_ctx* ctx, const ard_pattern* pat, GemmOp op, GemmArgs g, cudaStream_t s) {
+  if (pat->kind == ARD_ROW && !g.flag0 && g.keep < 1.f && 2.0 * g.B * g.K * g.N * g.keep >= 2e9 && f32_takes(ctx, pat->kind, op, g, pat->ts)) {
+    const void *dyc, *dense;
+    int ldc, dense_ld;
+    const ard_status st = compact_dy(ctx, pat, g.B, g.N, g.A0, g.lda0, 0, &dyc, &ldc, &dense, &dense_ld, s, 1, 4);
+    if (st == ARD_OK) {
+      g.A0 = dyc;
+      g.lda0 = ldc;
+      g.flag0 = 1;
+    } else if (st != ARD_ERR_NOMEM) {
+      return st;
+    }
+  }
+  return launch_gemm_cc(ctx, pat->kind, op, ARD_F32, g, pat->ts, s);
 }
 
 static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_pattern* in_pat, ard_dtype dtype, int B,
@@ -663,6 +690,7 @@ static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_
   g.accumulate = (flags & ARD_FLAG_ACCUMULATE) != 0;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
   g.act = act;
+  if (in_pat) g.keep *= in_pat->keep;
   g.ldact = ldact;
   if (g.accumulate && act != nullptr) return ARD_ERR_INVALID_ARG;
 
@@ -677,6 +705,7 @@ static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
     st = bwd_staged_by_threads(ctx, pat, OP_BWD_DATA, dtype, g, s);
+    if (dtype == ARD_F32) return bwd_f32(ctx, pat, OP_BWD_DATA, g, s);
     return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_DATA, dtype, g, pat->ts, s);
   }
   TcArgs t = {};
@@ -753,6 +782,7 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
   if (in_pat && zero_fill_dropped) return ARD_ERR_INVALID_ARG;  // the packed gradient has no rows of dropped neurons
   // The kernels write the zeros of dropped rows and pattern tiles themselves.
+  if (in_pat) g.keep *= in_pat->keep;
   // Empty batch: the gradient of every kept weight is zero; the CUDA-core kernel writes exactly that.
   if (B == 0) return launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
 
@@ -766,6 +796,7 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
     st = bwd_staged_by_threads(ctx, pat, OP_BWD_WEIGHT, dtype, g, s);
     return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
+    if (dtype == ARD_F32) return bwd_f32(ctx, pat, OP_BWD_WEIGHT, g, s);
   }
   TcArgs t = {};
   t.ts = pat->ts;
@@ -928,6 +959,7 @@ ard_status ard_lstm_gate_gemm(ard_ctx* ctx, const ard_pattern* pat, int B, int K
                               const void* W, int ldw, float* Z, int ldz_gate, void* cuda_stream) {
   ard_status st = check_common(ctx, pat, B, KH, H);
   if (st != ARD_OK) return st;
+  pat->keep = d.keep;
   if (!XH || !W || !Z) return ARD_ERR_INVALID_ARG;
   if (pat->kind != ARD_ROW) return ARD_ERR_INVALID_ARG;
   if (ldxh < KH || ldw < KH || ldz_gate < H) return ARD_ERR_SHAPE;

@@ -31,6 +31,7 @@ struct ard_pattern {
   ard_kind kind;
   int K_dim, N_dim, ts, Tr, Tc, units;
   int dp_bound;        // largest dp the last sample/set call can have produced
+  float keep;          // share of the units that the last sample/set call keeps in the mean
   unsigned long long generation;  // bumped by every sample / set call
   int32_t* d_hdr;      // device: header
   int32_t* d_idx;      // device: kept list (row: neuron index; tile: t-1), capacity `units`
@@ -55,6 +56,7 @@ struct ard_rows {
 
 struct ArdDistribution {
   int ndp = 0;
+  float keep = 1.f;  // kept share of the units in the mean
   unsigned long long* d_cdf = nullptr;  // device: ndp entries
   std::vector<unsigned long long> h_cdf;
 };
@@ -118,7 +120,7 @@ struct ard_ctx {
   int sk_min_gain;    // fewest blocks the sharing must save per worker to be used
   void* d_sk_ws;      // partial accumulators of the shared tail, sk_ws_bytes(sm_count)
   int* d_sk_cnt;      // arrival counters, zero between launches
-  struct { const void* src; int ld, B, N; const ard_pattern* pat; unsigned long long gen; cudaStream_t stream; int with_dense; } last_gather;
+  struct { const void* src; int ld, B, N; const ard_pattern* pat; unsigned long long gen; cudaStream_t stream; int with_dense, es; } last_gather;
   size_t workspace_bytes;
   void* d_workspace;
   int* d_status;
@@ -221,6 +223,7 @@ ard_status launch_gemm_cc(ard_ctx* ctx, ard_kind kind, GemmOp op, ard_dtype dtyp
                           cudaStream_t s);
 
 // tcgen05 products whose operands the CTA's threads stage themselves: bf16 operands of any alignment under a row pattern
+  float keep;  // share of the whole layer's products that the pattern leaves in the mean (0: not known); fp32 only
 // (dY compact), pattern tiles of 8 to 64 columns.  ldg_takes: can it take these operands?
 bool ldg_takes(const ard_ctx* ctx, ard_kind kind, const GemmArgs& g, int ts);
 ard_status launch_gemm_ldg(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
@@ -234,6 +237,10 @@ struct TcArgs {
   int mapA_indexed, mapB_indexed;  // 0: used as encoded, 1: specialised to the pattern, 2: to the input pattern
   GemmArgs g;
   int ts;
+// fp32 layers on the tensor cores, operands split into three bf16 parts.  f32_takes: can, and should, it take this call?
+bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts);
+ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
+
   int bn;  // N tile: 64, 128 or 256
 };
 int tc_pick_bn(ard_ctx* ctx, ard_kind kind, GemmOp op, int dp_bound, int ts);

@@ -1,7 +1,6 @@
 // CUDA-core family of the compacted GEMMs: fp32 (or bf16) operands, fp32 FFMA accumulation.
 //
-// This is the path of the fp32 layers (a single tcgen05 tf32 pass keeps 10 mantissa bits and
-// cannot reach 1e-5) and the fall-back for bf16 shapes whose alignment no tensor-core kernel can take.
+// This is the path of the smaller fp32 layers (the larger ones: gemm_f32_sm100.cu) and the fall-back for bf16 shapes whose alignment no tensor-core kernel can take.
 // One shared-memory tiled kernel; what differs per product is only how the logical operand element (m, k), (n, k)
 // maps to memory and which contraction indices exist: dropped neurons / tiles are skipped through the pattern,
 // never multiplied by zero.  Tiling, cut contractions and the rows' way out: staged_product.h.
@@ -379,6 +378,8 @@ ard_status launch_gemm_cc(ard_ctx* ctx, ard_kind kind, GemmOp op, ard_dtype dtyp
   } else if (kind == ARD_ROW && a.N <= SKINNY_N && op == OP_BWD_WEIGHT) {
     if (dtype == ARD_F32) (void)ard_launch(ctx, skinny_bwd_weight_kernel<float>, dim3((a.K + 31) / 32), dim3(256), 0, s, a);
     else (void)ard_launch(ctx, skinny_bwd_weight_kernel<__nv_bfloat16>, dim3((a.K + 31) / 32), dim3(256), 0, s, a);
+  } else if (dtype == ARD_F32 && f32_takes(ctx, kind, op, a, ts)) {
+    return launch_gemm_f32(ctx, kind, op, a, ts, s);
   } else if (dtype == ARD_F32) {
     dispatch<float>(ctx, kind, op, a, ts, s);
   } else {

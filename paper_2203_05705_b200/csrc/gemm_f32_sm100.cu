@@ -1,0 +1,568 @@
+// fp32 layers on the tensor cores: every operand element is split into three bf16 numbers that add up to it,
+// x = h + m + l (8 bits each, rounded to nearest, so 24 in all), and a product is taken as h h' + h m' + m h' + h l' + m m' + l h'.
+// What is left out (m l', l m', l l') is below 2^-25 of |x y|, half of what rounding one fp32 product costs.  The
+// tensor core truncates its sums, so the accumulators are taken out of tensor memory after every 64 contraction indices
+// and added in fp32 registers, rounded to nearest: four truncations per sum instead of K / 16.
+//
+// One CTA per SM, 128 x 64 output tiles.  Warps 0..7 load (registers, the next block's piece requested as soon as this block's
+// has been split) and write the six planes in the 128-byte-swizzled layout; warps 8 and 9 issue the products of the even and
+// the odd blocks, each into accumulators of its own (an issued product costs its thread 136 cycles whatever its size, so one
+// thread could not keep up); warps 10..13 take the accumulators out, add them up and write the tile.
+// The three planes of B lie behind one another, so that one instruction multiplies a plane of A with up to all three:
+//   A.h x [B.h B.m B.l] -> columns 0..191,  A.m x [B.h B.m] -> 64..191,  A.l x B.h -> 128..191.
+//
+// Bound: shared memory.  A block (128 + 64 rows, 64 contraction indices) takes 48 KB through L1, 72 KB of stores of the planes
+// and 98 KB of operand reads, about 1730 cycles at 128 bytes a cycle, next to 768 tensor-core cycles.
+//
+// Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l.  Blocks in which that happens are noticed by the
+// loading warps, and the tile (its share of the contraction) is multiplied again on the CUDA cores.
+#include "staged_product.h"
+
+#include <type_traits>
+
+namespace {
+
+constexpr int F3_LOADERS = 256;
+constexpr int F3_ISSUE_WARP = 8, F3_DRAIN_WARP = 10, F3_DRAINS = 4;
+constexpr int F3_THREADS = 32 * (F3_DRAIN_WARP + F3_DRAINS);
+constexpr int F3_BK = 64, F3_BN = 64;
+constexpr int F3_A_PLANE = UMMA_BM * F3_BK * 2, F3_B_PLANE = F3_BN * F3_BK * 2;
+constexpr int F3_STAGE = 3 * (F3_A_PLANE + F3_B_PLANE);
+constexpr int F3_PITCH = F3_BN + 4;
+constexpr int F3_TILE_OFF = 2 * F3_STAGE;
+constexpr int F3_BAR_OFF = F3_TILE_OFF + UMMA_BM * F3_PITCH * 4;
+constexpr int F3_SMEM = F3_BAR_OFF + 128 + 1024;
+constexpr int F3_TMEM = 512;           // two blocks' accumulators of 3 * F3_BN columns each, rounded up to a power of two
+constexpr double F3_LEAST_FLOPS = 1.5e8;  // kept operations, see f32_takes
+constexpr int F3_RING = 8;             // blocks between a loader and the warps that add up: at most four
+
+struct F32Params {
+  GemmArgs g;
+  int ts;
+  int cl;   // CTAs per cluster
+  int vec;  // bit 0 / 1: rows of operand A / B start on 16-byte boundaries
+};
+
+// Four elements as two pairs; `pred`: zeros where it does not hold
+struct Quad { uint64_t lo, hi; };
+__device__ __forceinline__ Quad ld4(const float* p) {
+  Quad v;
+  asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.lo), "=l"(v.hi) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ Quad ld4(const float* p, bool pred) {
+  Quad v;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %3, 0;\n\tmov.b64 %0, 0;\n\tmov.b64 %1, 0;\n\t@p ld.global.v2.u64 {%0, %1}, [%2];\n\t}"
+      : "=&l"(v.lo), "=&l"(v.hi) : "l"(p), "r"((int)pred));
+  return v;
+}
+__device__ __forceinline__ float ld1(const float* p) {
+  float v;
+  asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float ld1(const float* p, bool pred) {
+  float v;
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %2, 0;\n\tmov.b32 %0, 0;\n\t@p ld.global.f32 %0, [%1];\n\t}"
+               : "=&f"(v) : "l"(p), "r"((int)pred));
+  return v;
+}
+__device__ __forceinline__ void sts8(uint32_t a, uint32_t x, uint32_t y) {
+  asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(x), "r"(y) : "memory");
+}
+__device__ __forceinline__ uint64_t pair(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint32_t round2(uint64_t x) {
+  float a, b;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
+  uint32_t h;
+  asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(h) : "f"(b), "f"(a));
+  return h;
+}
+// The pair rounded to bf16, and what that leaves of it (exact)
+__device__ __forceinline__ uint32_t take_bf16(uint64_t& x) {
+  const uint32_t h = round2(x);
+  x = fma2(pair(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), pair(-1.f, -1.f), x);
+  return h;
+}
+__device__ __forceinline__ void split2(uint64_t x, uint32_t& h, uint32_t& m, uint32_t& l, uint64_t& bad) {
+  h = take_bf16(x);
+  m = take_bf16(x);
+  l = round2(x);
+  bad = fma2(x, 0ull, bad);  // zero, and NaN from here on if a part was not finite
+}
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+
+// Where operand elements are: r = position inside the tile, k = contraction index.
+template <int KIND, int OP>
+struct Operands {
+  static constexpr bool A_MN = OP == OP_BWD_WEIGHT, B_MN = OP != OP_FWD;
+  const float *PA, *PB;
+  size_t lda, ldb, step_a;  // step_a: columns of a full-width dY from one kept neuron to the next
+  bool vec_a, vec_b;        // pieces of four contiguous elements are whole and on the 16-byte grid, or do not exist
+
+  __device__ __forceinline__ Operands(const GemmArgs& g, const ProductPlan& s, int vec) {
+    PA = reinterpret_cast<const float*>(g.A0);
+    PB = reinterpret_cast<const float*>(g.A1);
+    const bool strided_a = KIND == 0 && OP != OP_FWD && !g.flag0;
+    lda = (size_t)g.lda0;
+    step_a = strided_a ? (size_t)s.dp : 1;
+    if (strided_a) PA += s.bb;
+    // kept neurons are rows bb + i * dp of the weight (unless packed for a feeding pattern)
+    const bool strided_b = KIND == 0 && OP != OP_BWD_WEIGHT && g.hdr_in == nullptr;
+    ldb = strided_b ? (size_t)g.lda1 * s.dp : (size_t)g.lda1;
+    if (strided_b) PB += (size_t)s.bb * g.lda1;
+    const int along_a = KIND == 1 ? 0 : (A_MN ? s.M : s.K), along_b = KIND == 1 ? 0 : (B_MN ? s.N : s.K);
+    vec_a = (vec & 1) && step_a == 1 && (along_a & 3) == 0;
+    vec_b = (vec & 2) && (along_b & 3) == 0;
+  }
+  __device__ __forceinline__ int a_lim(const ProductPlan& s, const ProductTile& ti) const {
+    return (KIND == 0 || OP != OP_BWD_WEIGHT ? s.M : ti.cnt * s.ts) - ti.m0;
+  }
+  __device__ __forceinline__ int b_lim(const ProductPlan& s, const ProductTile& ti) const {
+    return (KIND == 0 ? s.N : (OP == OP_BWD_WEIGHT ? ti.len : ti.cnt) * s.ts) - ti.n0;
+  }
+  __device__ __forceinline__ const float* a(const ProductPlan& s, const ProductTile& ti, int r, int k) const {
+    const int m = ti.m0 + r;
+    if (KIND == 0) return PA + (A_MN ? (size_t)k * lda + (size_t)m * step_a : (size_t)m * lda + (size_t)k * step_a);
+    return PA + (A_MN ? (size_t)k * lda + ti.class_pos(s, m) : (size_t)m * lda + ti.list_pos(s, k));
+  }
+  __device__ __forceinline__ const float* b(const ProductPlan& s, const ProductTile& ti, int r, int k) const {
+    const int n = ti.n0 + r;
+    if (KIND == 0) return PB + (B_MN ? (size_t)k * ldb + n : (size_t)n * ldb + k);
+    if (OP == OP_FWD) return PB + (size_t)ti.class_pos(s, n) * ldb + ti.list_pos(s, k);
+    if (OP == OP_BWD_DATA) return PB + (size_t)ti.list_pos(s, k) * ldb + ti.class_pos(s, n);
+    return PB + (size_t)k * ldb + ti.list_pos(s, n);
+  }
+};
+
+// Row r of the tile's sums over contraction indices [k0, k1) on the CUDA cores, for operands that are not finite.
+template <int KIND, int OP>
+__device__ __noinline__ void multiply_again(const Operands<KIND, OP>& o, const ProductPlan& s, const ProductTile& ti, int r, int k0, int k1,
+                                            float* T) {
+  const int nb = min(F3_BN, o.b_lim(s, ti));
+  for (int j = 0; j < F3_BN; ++j) {
+    float acc = 0.f;
+    if (j < nb && r < o.a_lim(s, ti))
+      for (int k = k0; k < k1; ++k) acc = fmaf(*o.a(s, ti, r, k), *o.b(s, ti, j, k), acc);
+    T[j] = acc;
+  }
+}
+
+template <int KIND, int OP>
+__global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_constant__ F32Params p) {
+  using O = Operands<KIND, OP>;
+  constexpr bool A_MN = O::A_MN, B_MN = O::B_MN;
+  constexpr int NA = 8, NB = 4;  // four-element pieces per loading thread and block
+  const GemmArgs& g = p.g;
+
+  extern __shared__ uint8_t smem_raw[];
+  const uint32_t raw_addr = smem_u32(smem_raw);
+  const uint32_t base = (raw_addr + 1023u) & ~1023u;
+  uint8_t* smem = smem_raw + (base - raw_addr);
+  const uint32_t bars = base + F3_BAR_OFF;
+  // of half h of stage i and of accumulators i, i = block & 1: operands written; multiplied (for the loaders and, the second
+  // half, for the warps that add up); added up
+  auto full_bar = [&](int i, int h) { return bars + 8u * (2 * i + h); };
+  auto done_bar = [&](int i, int h) { return bars + 8u * (4 + 2 * i + h); };
+  auto free_bar = [&](int i) { return bars + 8u * (8 + i); };
+  volatile uint32_t* tmem_ptr = reinterpret_cast<volatile uint32_t*>(smem + F3_BAR_OFF + 80);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + F3_BAR_OFF + 84);
+  volatile int* bad_ring = reinterpret_cast<volatile int*>(smem + F3_BAR_OFF + 96);  // [block % F3_RING] = block + 1: not finite
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_launch_dependents();
+  if (tid == 0) {
+    for (int i = 0; i < 2; ++i) {
+      for (int h = 0; h < 2; ++h) {
+        mbar_init(full_bar(i, h), F3_LOADERS / 64);
+        mbar_init(done_bar(i, h), 1 + h);
+      }
+      mbar_init(free_bar(i), F3_DRAINS);
+    }
+    *abort_flag = 0;
+    for (int i = 0; i < F3_RING; ++i) bad_ring[i] = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == F3_ISSUE_WARP) {
+    tmem_alloc(smem_u32(const_cast<uint32_t*>(tmem_ptr)), F3_TMEM);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_ptr;
+  pdl_wait_prior_grids();
+
+  const ProductPlan s = make_plan<KIND, OP, UMMA_BM, F3_BN, F3_BK>(g, p.ts, (int)gridDim.x, p.cl);
+  const O o(g, s, p.vec);
+  const int rank = (int)cluster_ctarank();
+  const int lS = 31 - __clz(s.S), lG = 31 - __clz(s.G);
+  const int part = rank & (s.S - 1);          // this CTA's share of the contraction
+  const int lead = rank - part;               // first CTA of those that share it
+  const int rows = rank & (s.G - 1);          // this CTA's part of the tile's rows
+  const int group = rank >> lG, groups = p.cl >> lG;
+  const int n_cl = (int)gridDim.x / p.cl, units = (s.tiles + groups - 1) / groups, u0 = (int)blockIdx.x / p.cl;
+
+  // Unit u's tile and this CTA's blocks [kb0, kb1) of it; nkb < 0: nothing there.
+  auto unit = [&](int u, int& kb0, int& kb1) {
+    const int t = u * groups + group;
+    ProductTile ti = {};
+    ti.nkb = -1;
+    if (t < s.tiles) ti = make_tile<KIND, OP, UMMA_BM, F3_BN, F3_BK>(g, s, t);
+    kb0 = ti.nkb > 0 ? (ti.nkb * part) >> lS : 0;
+    kb1 = ti.nkb > 0 ? (ti.nkb * (part + 1)) >> lS : 0;
+    return ti;
+  };
+  float* T = reinterpret_cast<float*>(smem + F3_TILE_OFF);
+  bool ok = true;
+
+  if (warp < F3_ISSUE_WARP) {
+    // ===================== loads =====================
+    // Warps 0..3 bring the first half of every block (32 contraction indices), warps 4..7 the second: while one group waits for
+    // its stage or its stores, the other splits.  A thread owns NA four-element pieces of A and NB of B.
+    // K-major: 8 lanes read a row's 32 elements, piece i is row 16 i + r (the two rows of a half warp are four apart, so that
+    // their halves of the 128-byte rows of the stage lie in different banks).  MN-major: 16 lanes read 64 columns of one
+    // contraction row, piece i is row 8 (i & 3) + r of the half and, of A, box i / 4.
+    const int h = warp >> 2, grp = (tid >> 3) & 15, kr = (grp >> 3) * 8 + (grp & 1) * 4 + ((grp >> 1) & 3);
+    const int ra = A_MN ? (tid >> 4) & 7 : kr, rb = B_MN ? (tid >> 4) & 7 : kr;
+    const int ca = 4 * (tid & (A_MN ? 15 : 7)), cb = 4 * (tid & (B_MN ? 15 : 7));
+    ProductTile ti;
+    int kb = 0, kb1 = 0, u = u0 - n_cl;     // the block in registers: block kb of unit u
+    const float *ta[2] = {}, *tb[NB] = {};  // of the tile: see at()
+    int na = 0, nb = 0;                     // K-major: rows that exist from the first piece's on; MN-major: columns
+    Quad v[NA + NB];
+    uint64_t bad = 0ull;
+    // Moves on to the next block; false: there is none.
+    auto advance = [&]() {
+      if (++kb < kb1) return true;
+      for (;;) {
+        u += n_cl;
+        if (u >= units) return false;
+        ti = unit(u, kb, kb1);
+        if (kb < kb1) break;
+      }
+      na = o.a_lim(s, ti) - (A_MN ? ca : ra);
+      nb = o.b_lim(s, ti) - (B_MN ? cb : rb);
+      if (KIND == 0) {
+        ta[0] = o.a(s, ti, A_MN ? ca : ra, A_MN ? ra : ca);
+        tb[0] = o.b(s, ti, B_MN ? cb : rb, B_MN ? rb : cb);
+      } else if (OP == OP_BWD_WEIGHT) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) ta[i] = o.PA + (size_t)ra * o.lda + (na > 64 * i ? ti.class_pos(s, ti.m0 + 64 * i + ca) : 0);
+        tb[0] = o.PB + (size_t)rb * o.ldb + (nb > 0 ? ti.list_pos(s, ti.n0 + cb) : 0);
+      } else {
+        ta[0] = o.PA + (size_t)(ti.m0 + ra) * o.lda;
+        if (OP == OP_FWD) {
+#pragma unroll
+          for (int i = 0; i < NB; ++i) tb[i] = o.PB + (size_t)(nb > 16 * i ? ti.class_pos(s, ti.n0 + 16 * i + rb) : 0) * o.ldb;
+        } else {
+          tb[0] = o.PB + (nb > 0 ? ti.class_pos(s, ti.n0 + cb) : 0);
+        }
+      }
+      return true;
+    };
+    int kfirst = 0, kleft = 0;  // first contraction index of the half block, and how many there are from it on
+    int kpos = 0;               // tile patterns: coordinate of contraction index kfirst + ca
+    bool whole = false;         // every element of the half block exists
+    auto begin_block = [&]() {
+      kfirst = kb * F3_BK + 32 * h;
+      kleft = ti.kext - kfirst;
+      whole = kleft >= 32 && o.a_lim(s, ti) >= UMMA_BM && o.b_lim(s, ti) >= F3_BN;
+      if (KIND == 1 && OP != OP_BWD_WEIGHT) kpos = ca < kleft ? ti.list_pos(s, kfirst + ca) : 0;
+    };
+    // Piece i: address, and whether / how many of its elements exist (<= 0: none).
+    auto at = [&](int i, int& n) -> const float* {
+      if (i < NA) {
+        const int row = A_MN ? 8 * (i & 3) : 16 * i;
+        if (A_MN) n = row + ra < kleft ? na - 64 * (i >> 2) : 0;
+        else n = row < na ? kleft - ca : 0;
+        if (KIND == 0) {
+          if (A_MN) return ta[0] + (size_t)(kfirst + row) * o.lda + (size_t)((i >> 2) * 64) * o.step_a;
+          return ta[0] + (size_t)row * o.lda + (size_t)kfirst * o.step_a;
+        }
+        if (A_MN) return ta[i >> 2] + (size_t)(kfirst + row) * o.lda;
+        return ta[0] + (size_t)row * o.lda + kpos;
+      }
+      const int ib = i - NA, row = B_MN ? 8 * ib : 16 * ib;
+      if (B_MN) n = row + rb < kleft ? nb : 0;
+      else n = row < nb ? kleft - cb : 0;
+      if (KIND == 0) return B_MN ? tb[0] + (size_t)(kfirst + row) * o.ldb : tb[0] + (size_t)row * o.ldb + kfirst;
+      if (OP == OP_FWD) return tb[ib] + kpos;
+      if (OP == OP_BWD_DATA) return tb[0] + (size_t)(row + rb < kleft ? ti.list_pos(s, kfirst + row + rb) : 0) * o.ldb;
+      return tb[0] + (size_t)(kfirst + row) * o.ldb;
+    };
+    // VEC: 1 pieces on the 16-byte grid, 0 not, -1 to be looked at, and whether their elements exist too
+    auto load = [&](auto vec, int i) {
+      constexpr int VEC = decltype(vec)::value;
+      int n;
+      const float* q = at(i, n);
+      const size_t st = i < NA ? o.step_a : 1;
+      Quad& x = v[i];
+      if (VEC == 1) {
+        x = ld4(q);
+      } else if (VEC == 0) {
+        x.lo = pair(ld1(q), ld1(q + st));
+        x.hi = pair(ld1(q + 2 * st), ld1(q + 3 * st));
+      } else if (i < NA ? o.vec_a : o.vec_b) {
+        x = ld4(q, n > 0);
+      } else {
+        x.lo = pair(ld1(q, n > 0), ld1(q + st, n > 1));
+        x.hi = pair(ld1(q + 2 * st, n > 2), ld1(q + 3 * st, n > 3));
+      }
+    };
+    auto place = [&](bool mn, int r, int c) {  // of piece 0
+      const uint32_t d = (uint32_t)r * 128u + (uint32_t)(((c >> 3) ^ (r & 7)) << 4) + (uint32_t)(c & 4) * 2u;
+      return base + (mn ? d + (uint32_t)h * 4096u : d ^ ((uint32_t)h * 64u));
+    };
+    const uint32_t pa = place(A_MN, ra, ca), pb = place(B_MN, rb, cb) + 3 * F3_A_PLANE;
+    auto split = [&](int i, uint32_t stage) {
+      uint32_t h0, m0, l0, h1, m1, l1;
+      split2(v[i].lo, h0, m0, l0, bad);
+      split2(v[i].hi, h1, m1, l1, bad);
+      const int ib = i - NA;
+      const uint32_t d = i < NA ? pa + stage + (uint32_t)(A_MN ? (i >> 2) * 8192 + (i & 3) * 1024 : i * 2048)
+                                : pb + stage + (uint32_t)(B_MN ? ib * 1024 : ib * 2048);
+      const uint32_t plane = i < NA ? F3_A_PLANE : F3_B_PLANE;
+      sts8(d, h0, h1);
+      sts8(d + plane, m0, m1);
+      sts8(d + 2 * plane, l0, l1);
+    };
+    // The half block in registers goes to its stage while the next block's takes its place
+    auto swap = [&](auto va, auto vb, uint32_t stage) {
+#pragma unroll
+      for (int i = 0; i < NA + NB; ++i) {
+        split(i, stage);
+        if (i < NA) load(va, i); else load(vb, i);
+      }
+    };
+    using Yes = std::integral_constant<int, 1>;
+    using No = std::integral_constant<int, 0>;
+    using Look = std::integral_constant<int, -1>;
+    int it = 0;
+    bool more = advance();
+    if (more) {
+      begin_block();
+#pragma unroll
+      for (int i = 0; i < NA + NB; ++i) load(Look{}, i);
+    }
+    for (int w = u0; w < units; w += n_cl) {
+      while (more && u == w && ok) {
+        const int st = it & 1;
+        const uint32_t stage = (uint32_t)st * F3_STAGE;
+        bad = 0ull;
+        more = advance();
+        if (more) begin_block();
+        else { whole = false; na = nb = kleft = 0; }  // nothing exists
+        if (it >= 2 && !mbar_wait(done_bar(st, h), (uint32_t)((it >> 1) - 1) & 1u, abort_flag, g.status)) ok = false;
+        ok = __all_sync(0xffffffffu, ok);
+        if (!ok) break;
+        if (whole && o.vec_b && o.vec_a) swap(Yes{}, Yes{}, stage);
+        else if (whole && o.vec_b) swap(No{}, Yes{}, stage);
+        else if (whole && !o.vec_a) swap(No{}, No{}, stage);
+        else swap(Look{}, Look{}, stage);
+        if (__any_sync(0xffffffffu, bad != 0ull) && lane == 0) bad_ring[it % F3_RING] = it + 1;
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full_bar(st, h));
+        ++it;
+      }
+      __syncwarp();
+      if (s.S > 1) {
+        cluster_sync_all();  // the partial tiles of the group are complete
+        int k0, k1;
+        const ProductTile tw = unit(w, k0, k1);
+        if (tw.nkb >= 0)
+          write_tile<KIND, OP, UMMA_BM, F3_BN, F3_PITCH, F3_LOADERS / 32, true, float>(g, s, tw, T, base + F3_TILE_OFF, rows, lead, warp, lane);
+        __syncwarp();
+        cluster_sync_all();  // no CTA of the group reads this one's partial tile any more
+      }
+    }
+  } else {
+    const bool drain = warp >= F3_DRAIN_WARP;
+    const int dw = warp - F3_DRAIN_WARP, quad = warp & 3;  // a warp reads the 32 lanes of tensor memory of its number modulo 4
+    if (drain && OP == OP_BWD_WEIGHT && g.flag1 && s.dp > 1) {
+      const int w = (int)blockIdx.x * F3_DRAINS + dw, ws = (int)gridDim.x * F3_DRAINS;
+      if (KIND == 1) zero_dropped_tiles(g, p.ts, w, ws, lane);
+      else zero_dropped_rows(g, s.N, w, ws, lane);
+    }
+    int it = 0;  // blocks of this CTA so far
+    for (int u = u0; u < units; u += n_cl) {
+      int kb0, kb1;
+      const ProductTile ti = unit(u, kb0, kb1);
+      if (!drain) {
+        // ===================== products =====================
+        const int mine = warp - F3_ISSUE_WARP;
+        if (lane == 0 && ok) {
+          const uint64_t desc_a = A_MN ? make_desc(0, 64 * F3_BK * 2, 1024) : make_desc(0, 16, 1024);
+          const uint64_t desc_b = B_MN ? make_desc(0, 64 * F3_BK * 2, 1024) : make_desc(0, 16, 1024);
+          const uint32_t sA = base + (uint32_t)mine * F3_STAGE, sB = sA + 3 * F3_A_PLANE;
+          const uint64_t ad = desc_a | (uint64_t)((sA & 0x3FFFFu) >> 4), bd = desc_b | (uint64_t)((sB & 0x3FFFFu) >> 4);
+          const uint32_t d = tmem + (uint32_t)mine * 256u;
+          for (int b = it; b < it + kb1 - kb0; ++b) {
+            if ((b & 1) != mine) continue;
+            const uint32_t par = (uint32_t)(b >> 1) & 1u;
+            if (!mbar_wait(free_bar(mine), par ^ 1u, abort_flag, g.status)) { ok = false; break; }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              if (!mbar_wait(full_bar(mine, h), par, abort_flag, g.status)) { ok = false; break; }
+              tc_fence_after();
+#pragma unroll
+              for (int k = 2 * h; k < 2 * h + 2; ++k) {
+                const uint64_t ak = ad + (uint64_t)(k * (A_MN ? 128 : 2)), bk = bd + (uint64_t)(k * (B_MN ? 128 : 2));
+                tc_mma_bf16(d, ak, bk, make_idesc(3 * F3_BN, A_MN, B_MN), k != 0 ? 1u : 0u);
+                tc_mma_bf16(d + F3_BN, ak + (F3_A_PLANE >> 4), bk, make_idesc(2 * F3_BN, A_MN, B_MN), 1u);
+                tc_mma_bf16(d + 2 * F3_BN, ak + 2 * (F3_A_PLANE >> 4), bk, make_idesc(F3_BN, A_MN, B_MN), 1u);
+              }
+              tc_commit(done_bar(mine, h));
+            }
+            if (!ok) break;
+            mbar_arrive(done_bar(mine, 1));  // passes on what the loaders said of the block
+          }
+        }
+        __syncwarp();
+      } else if (ti.nkb >= 0) {
+        // ===================== sums =====================
+        uint64_t acc[F3_BN / 2];
+#pragma unroll
+        for (int i = 0; i < F3_BN / 2; ++i) acc[i] = 0ull;
+        bool again = false;
+        for (int b = it; b < it + kb1 - kb0 && ok; ++b) {
+          const int i = b & 1;
+          if (!mbar_wait(done_bar(i, 1), (uint32_t)(b >> 1) & 1u, abort_flag, g.status)) ok = false;
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
+          tc_fence_after();
+          again = again || bad_ring[b % F3_RING] == b + 1;
+          const uint32_t from = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)i * 256u;
+#pragma unroll
+          for (int cc = 0; cc < F3_BN; cc += 16) {
+            uint32_t x[16], y[16], z[16];
+            tmem_ld16(from + cc, x);
+            tmem_ld16(from + F3_BN + cc, y);
+            tmem_ld16(from + 2 * F3_BN + cc, z);
+            tmem_ld_wait();
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              auto two = [&](const uint32_t (&r)[16]) { return pair(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])); };
+              acc[cc / 2 + q] = add2(acc[cc / 2 + q], add2(two(x), add2(two(y), two(z))));
+            }
+          }
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(free_bar(i));
+        }
+        float* row = T + (quad * 32 + lane) * F3_PITCH;
+        if (again) {
+          multiply_again(o, s, ti, quad * 32 + lane, kb0 * F3_BK, min(kb1 * F3_BK, ti.kext), row);
+        } else {
+#pragma unroll
+          for (int i = 0; i < F3_BN / 4; ++i) *reinterpret_cast<ulonglong2*>(row + 4 * i) = make_ulonglong2(acc[2 * i], acc[2 * i + 1]);
+        }
+        if (s.S == 1) asm volatile("bar.sync 1, 128;" ::: "memory");
+      }
+      it += kb1 - kb0;
+      __syncwarp();
+      if (s.S > 1) {  // the loading warps, twice as many, add up the shares and write the tile
+        cluster_sync_all();
+        cluster_sync_all();
+      } else if (drain && ti.nkb >= 0) {
+        write_tile<KIND, OP, UMMA_BM, F3_BN, F3_PITCH, F3_DRAINS, true, float>(g, s, ti, T, base + F3_TILE_OFF, rows, lead, dw, lane);
+        asm volatile("bar.sync 1, 128;" ::: "memory");  // the tile has been read
+        __syncwarp();
+      }
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == F3_ISSUE_WARP) {
+    tc_fence_after();
+    tmem_dealloc(tmem, F3_TMEM);
+  }
+}
+
+inline int cdiv(int a, int b) { return (a + b - 1) / b; }
+
+template <int KIND, int OP>
+ard_status launch_f32(ard_ctx* ctx, F32Params p, cudaStream_t s) {
+  auto kern = gemm_f32_kernel<KIND, OP>;
+  static bool attr_done[64] = {};
+  const int dev = ctx->device & 63;
+  if (!attr_done[dev]) {
+    ARD_CUDA_OK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F3_SMEM));
+    attr_done[dev] = true;
+  }
+  const GemmArgs& g = p.g;
+  const int M = OP == OP_BWD_WEIGHT ? g.N : g.B, N = OP == OP_FWD ? g.N : g.K;
+  const int nkb = cdiv(OP == OP_FWD ? g.K : (OP == OP_BWD_DATA ? g.N : g.B), F3_BK);
+  const int tiles = cdiv(M, UMMA_BM) * cdiv(N, F3_BN);
+  p.cl = tiles * 8 <= ctx->sm_count ? 8 : 4;
+  static int room[2][64] = {};
+  int& r = room[p.cl == 8][dev];
+  if (r == 0) r = ard_cluster_room(ctx, kern, p.cl, F3_THREADS, F3_SMEM);
+  int ctas = r;
+  if (KIND == 0) {  // no more than the densest pattern's tiles, cut as often as its contraction allows
+    int S = p.cl;
+    while (S > 1 && nkb < 2 * S) S >>= 1;
+    const int n = cdiv(tiles * S, p.cl) * p.cl;
+    if (n < ctas) ctas = n;
+  }
+  ARD_CUDA_OK(ard_launch_cluster(ctx, kern, p.cl, dim3(ctas), dim3(F3_THREADS), F3_SMEM, s, p));
+  ctx->launches++;
+  ARD_CUDA_OK(cudaGetLastError());
+  return ARD_OK;
+}
+
+}  // namespace
+
+// A product of up to 1.5e8 kept operations stays on the CUDA cores: about 5 us of every launch here go to the tables of the tile, the
+// first loads and the way out, which the lighter kernel does faster.  Three products, CUDA cores and here, in us (graph replays):
+//   kept operations of one product   dense    dp 2    dp 5    dp 16
+//   64 x 784 x 256        2.6e7      19, 30   20, 33  21, 30  18, 28
+//   100 x 1001 x 777      1.6e8      61, 43   46, 46  39, 45  41, 39
+//   128 x 2048 x 2048     1.1e9     105, 57   82, 53  69, 56  56, 64
+//   1024 x 4096 x 4096    3.4e10   2730, 963 1601, 710 806, 460 332, 247
+// Error against fp64 (2-norm) there and here: 7e-8 .. 1.2e-6 and 3.5e-8 .. 1.7e-7, never larger here.
+bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts) {
+  if (ctx->path != ARD_PATH_AUTO || ctx->encode_fn == nullptr || g.B < 1 || g.K < 1 || g.N < 1) return false;
+  if (kind == ARD_TILE && ts % 4 != 0) return false;  // four consecutive positions never leave a pattern tile
+  return 2.0 * g.B * g.K * g.N * g.keep >= F3_LEAST_FLOPS;
+}
+
+ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s) {
+  F32Params p = {};
+  p.g = g;
+  p.ts = ts;
+  p.vec = ((reinterpret_cast<uintptr_t>(g.A0) & 15) == 0 && g.lda0 % 4 == 0 ? 1 : 0) |
+          ((reinterpret_cast<uintptr_t>(g.A1) & 15) == 0 && g.lda1 % 4 == 0 ? 2 : 0);
+  if (kind == ARD_ROW) {
+    if (op == OP_FWD) return launch_f32<0, OP_FWD>(ctx, p, s);
+    if (op == OP_BWD_DATA) return launch_f32<0, OP_BWD_DATA>(ctx, p, s);
+    return launch_f32<0, OP_BWD_WEIGHT>(ctx, p, s);
+  }
+  if (op == OP_FWD) return launch_f32<1, OP_FWD>(ctx, p, s);
+  if (op == OP_BWD_DATA) return launch_f32<1, OP_BWD_DATA>(ctx, p, s);
+  return launch_f32<1, OP_BWD_WEIGHT>(ctx, p, s);
+}

@@ -1203,6 +1203,7 @@ ard_status launch_mlp_persistent(ard_ctx* ctx, const ard_mlp_layer* layers, int 
   for (int l = 0; l < H; ++l) {
     if (!layers[l].sample) continue;
     layers[l].pat->dp_bound = d->ndp;
+    layers[l].pat->keep = d->keep;
     layers[l].pat->generation++;
   }
   return ARD_OK;

@@ -87,6 +87,7 @@ extern "C" ard_status ard_bwd_data_static_scratch(ard_ctx* ctx, const ard_patter
       g.idx = pat->d_idx;
       g.col_ptr = g.col_idx = g.row_ptr = g.row_idx = nullptr;
       g.B = B; g.K = K; g.N = N;
+      g.keep = pat->keep;
       g.alpha = alpha;
       g.A0 = scratch; g.lda0 = ldc;   // compact dY
       g.A1 = W; g.lda1 = ldw;

@@ -1,0 +1,84 @@
+"""fp32 layers large enough for the tensor cores (operands split into three bf16 parts) against the oracle: edges of the 128 x 64
+tiles and of the contraction blocks, rows on and off the 16-byte grid, cut and whole contractions, a compact copy of dY or none,
+and operands that are not finite."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2203_05705_b200 import ard
+from gpu_helpers import Ctx, run_three_gemms, assert_ok
+
+pytestmark = pytest.mark.gpu
+
+# What is left out of a product of two elements is below 2^-25 of it; sums of 64 products lose up to four truncations (2^-22 of a
+# partial sum) and are added with round to nearest.  The operands are random, so the errors of a sum's terms are too: 1e-6.
+TOL = 1e-6
+
+
+def _layer(B, K, N):
+    rng = np.random.default_rng(B + K + N)
+    X, W, dY = (rng.standard_normal(s).astype(np.float32) for s in ((B, K), (K, N), (B, N)))
+    return X, W / np.float32(np.sqrt(K)), dY
+
+
+@pytest.mark.parametrize("B,K,N", [(128, 2048, 2048), (129, 2087, 1531), (5, 6001, 8193), (4097, 65, 1201), (4100, 700, 130)])
+@pytest.mark.parametrize("workspace", [0, 32 << 20])
+def test_row_pattern(B, K, N, workspace):
+    X, W, dY = _layer(B, K, N)
+    ctx = Ctx(workspace)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        for i, (dp, b) in enumerate([(1, 1), (2, 2), (3, 1)]):
+            ard.ard_pattern_set(ctx.h, pat, dp, b)
+            res = run_three_gemms(ctx, pat, ard.ARD_ROW, ard.ARD_F32, X, W, dY, dp, b, 1.5, compact=(i == 1), zero_fill=(i != 2),
+                                  lds={"x": K + i, "w": (K + 3) // 4 * 4, "y": N + 5 * (i & 1)})
+            assert_ok(res, TOL, (B, K, N, dp, b))
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("ts,B,Tr,Tc", [(32, 129, 64, 33), (12, 200, 90, 101), (128, 260, 9, 10), (200, 130, 6, 7)])
+def test_tile_pattern(ts, B, Tr, Tc):
+    K, N = Tr * ts, Tc * ts
+    X, W, dY = _layer(B, K, N)
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_TILE, K, N, ts)
+        for i, dp in enumerate([1, 2, 3, 5]):
+            b = 1 + i % dp
+            ard.ard_pattern_set(ctx.h, pat, dp, b)
+            res = run_three_gemms(ctx, pat, ard.ARD_TILE, ard.ARD_F32, X, W, dY, dp, b, 2.0, ts=ts, zero_fill=(i % 2 == 0),
+                                  lds={"x": K + 4 * (i & 1), "w": K, "y": N + i // 3})
+            assert_ok(res, TOL, (ts, B, Tr, Tc, dp, b))
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.395e38])
+@pytest.mark.parametrize("kind,ts,dp", [(ard.ARD_ROW, 0, 1), (ard.ARD_ROW, 0, 2), (ard.ARD_TILE, 64, 3)])
+def test_not_finite(value, kind, ts, dp):
+    """An infinity, a NaN or a value that no bf16 holds ends up where the CUDA-core kernel has it."""
+    B, K, N = 200, 1536, 1088
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(kind, K, N, ts)
+        ard.ard_pattern_set(ctx.h, pat, dp, 1)
+        for where in range(3):
+            g = torch.Generator(device="cuda").manual_seed(where)
+            ops = [torch.randn(s, device="cuda", generator=g) * 0.1 for s in ((B, K), (N, K), (B, N))]
+            ops[where][130, 66 if where == 2 else 700] = value  # row 130 of the weight and column 66 of dY are kept neurons
+            X, W, dY = ops
+            outs = []
+            for path in (ard.ARD_PATH_CUDA_CORE, ard.ARD_PATH_AUTO):
+                ard.ard_set_path(ctx.h, path)
+                Y, dX, dW = (torch.full(s, 7.0, device="cuda") for s in ((B, N), (B, K), (N, K)))
+                ard.ard_fwd(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, X, K, W, K, Y, N, ard.ARD_OUT_SCATTER_ZEROFILL)
+                ard.ard_bwd_data(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, dY, N, 0, W, K, dX, K)
+                ard.ard_bwd_weight(ctx.h, pat, ard.ARD_F32, ard.ARD_F32, B, K, N, 1.0, X, K, dY, N, 0, dW, K, 1)
+                outs.append([Y, dX, dW])
+            for cc, tc in zip(*outs):
+                fin = cc.isfinite()
+                assert torch.equal(fin, tc.isfinite()) and torch.equal(cc.isnan(), tc.isnan()) and torch.equal(cc[cc.isinf()], tc[tc.isinf()])
+                assert (cc[fin].double() - tc[fin].double()).norm() <= 2e-6 * cc[fin].double().norm()
+    finally:
+        ctx.close()
