@@ -689,8 +689,8 @@ static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_
   g.out_is_f32 = out_f32;
   g.accumulate = (flags & ARD_FLAG_ACCUMULATE) != 0;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
-  g.act = act;
   if (in_pat) g.keep *= in_pat->keep;
+  g.act = act;
   g.ldact = ldact;
   if (g.accumulate && act != nullptr) return ARD_ERR_INVALID_ARG;
 
@@ -704,8 +704,8 @@ static ard_status bwd_data_impl(ard_ctx* ctx, const ard_pattern* pat, const ard_
     el = ARD_ERR_NOMEM;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
-    st = bwd_staged_by_threads(ctx, pat, OP_BWD_DATA, dtype, g, s);
     if (dtype == ARD_F32) return bwd_f32(ctx, pat, OP_BWD_DATA, g, s);
+    st = bwd_staged_by_threads(ctx, pat, OP_BWD_DATA, dtype, g, s);
     return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_DATA, dtype, g, pat->ts, s);
   }
   TcArgs t = {};
@@ -780,9 +780,9 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
   g.flag1 = zero_fill_dropped ? 1 : 0;
   g.out_is_f32 = dW_dtype == ARD_F32;
   g.hdr_in = in_pat ? in_pat->d_hdr : nullptr;
+  if (in_pat) g.keep *= in_pat->keep;
   if (in_pat && zero_fill_dropped) return ARD_ERR_INVALID_ARG;  // the packed gradient has no rows of dropped neurons
   // The kernels write the zeros of dropped rows and pattern tiles themselves.
-  if (in_pat) g.keep *= in_pat->keep;
   // Empty batch: the gradient of every kept weight is zero; the CUDA-core kernel writes exactly that.
   if (B == 0) return launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
 
@@ -794,9 +794,9 @@ static ard_status bwd_weight_impl(ard_ctx* ctx, const ard_pattern* pat, const ar
     el = ARD_ERR_NOMEM;
   if (el != ARD_OK) {
     if (ctx->path == ARD_PATH_TENSOR_CORE) return el;
+    if (dtype == ARD_F32) return bwd_f32(ctx, pat, OP_BWD_WEIGHT, g, s);
     st = bwd_staged_by_threads(ctx, pat, OP_BWD_WEIGHT, dtype, g, s);
     return st != ARD_ERR_UNSUPPORTED ? st : launch_gemm_cc(ctx, pat->kind, OP_BWD_WEIGHT, dtype, g, pat->ts, s);
-    if (dtype == ARD_F32) return bwd_f32(ctx, pat, OP_BWD_WEIGHT, g, s);
   }
   TcArgs t = {};
   t.ts = pat->ts;
@@ -946,6 +946,7 @@ ard_status ard_sample_pattern_counter(ard_ctx* ctx, ard_pattern* pat, int dist_i
   if (d.ndp == 0 || d.ndp > pat->units) return ARD_ERR_DISTRIBUTION;
   DeviceGuard guard(ctx->device);
   pat->dp_bound = d.ndp;
+  pat->keep = d.keep;
   pat->generation++;
   return launch_sampler(ctx, pat, d.d_cdf, d.ndp, seed, iteration_base, stream_id, 0, 0, (cudaStream_t)cuda_stream,
                         reinterpret_cast<unsigned long long*>(iteration_counter), advance ? 1 : 0);
@@ -959,7 +960,6 @@ ard_status ard_lstm_gate_gemm(ard_ctx* ctx, const ard_pattern* pat, int B, int K
                               const void* W, int ldw, float* Z, int ldz_gate, void* cuda_stream) {
   ard_status st = check_common(ctx, pat, B, KH, H);
   if (st != ARD_OK) return st;
-  pat->keep = d.keep;
   if (!XH || !W || !Z) return ARD_ERR_INVALID_ARG;
   if (pat->kind != ARD_ROW) return ARD_ERR_INVALID_ARG;
   if (ldxh < KH || ldw < KH || ldz_gate < H) return ARD_ERR_SHAPE;

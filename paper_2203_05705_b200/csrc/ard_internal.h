@@ -214,6 +214,7 @@ struct GemmArgs {
   // ext_mode 2: hdr's count is the length of the contraction (weight gradient).
   int ext_mode;
   const int32_t* ridx;
+  float keep;  // share of the whole layer's products that the pattern leaves in the mean (0: not known); fp32 only
 };
 
 enum GemmOp { OP_FWD = 0, OP_BWD_DATA = 1, OP_BWD_WEIGHT = 2 };
@@ -223,10 +224,13 @@ ard_status launch_gemm_cc(ard_ctx* ctx, ard_kind kind, GemmOp op, ard_dtype dtyp
                           cudaStream_t s);
 
 // tcgen05 products whose operands the CTA's threads stage themselves: bf16 operands of any alignment under a row pattern
-  float keep;  // share of the whole layer's products that the pattern leaves in the mean (0: not known); fp32 only
 // (dY compact), pattern tiles of 8 to 64 columns.  ldg_takes: can it take these operands?
 bool ldg_takes(const ard_ctx* ctx, ard_kind kind, const GemmArgs& g, int ts);
 ard_status launch_gemm_ldg(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
+
+// fp32 layers on the tensor cores, operands split into three bf16 parts.  f32_takes: can, and should, it take this call?
+bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts);
+ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
 
 // tcgen05 family (bf16 operands, fp32 accumulate in TMEM).
 struct TcArgs {
@@ -237,10 +241,6 @@ struct TcArgs {
   int mapA_indexed, mapB_indexed;  // 0: used as encoded, 1: specialised to the pattern, 2: to the input pattern
   GemmArgs g;
   int ts;
-// fp32 layers on the tensor cores, operands split into three bf16 parts.  f32_takes: can, and should, it take this call?
-bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts);
-ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
-
   int bn;  // N tile: 64, 128 or 256
 };
 int tc_pick_bn(ard_ctx* ctx, ard_kind kind, GemmOp op, int dp_bound, int ts);
