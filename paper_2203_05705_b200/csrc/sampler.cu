@@ -10,7 +10,6 @@
 namespace {
 
 constexpr int SAMPLER_THREADS = 1024;  // tile patterns; row patterns launch 256 (fewer lists to fill)
-constexpr int SCAN_CAP = 2048;  // tile-columns whose running count fits in shared memory
 
 __global__ void __launch_bounds__(SAMPLER_THREADS)
 ard_sample_kernel(int32_t* __restrict__ hdr, int32_t* __restrict__ idx, int32_t* __restrict__ col_ptr,
@@ -83,46 +82,65 @@ ard_sample_kernel(int32_t* __restrict__ hdr, int32_t* __restrict__ idx, int32_t*
     if (lim > b - 1) cnt = (int)((lim - 1 - (b - 1)) / dp) + 1;
     row_ptr[r] = cnt;
   }
-  // Group by tile-column: count, prefix-sum, fill.  A warp takes a column at a time with its lanes across
-  // the tile-rows, so a column costs Tr/32 ballots instead of a serial walk; the running sum over the
-  // columns lives in shared memory when the grid is narrow enough (a dependent chain through global
-  // memory would cost a round trip per column).
-  __shared__ int s_cnt[SCAN_CAP];
-  const bool in_smem = Tc <= SCAN_CAP;
+  // Grouped by tile-column.  Tile (r, c) is kept iff r * Tc + c = b - 1 (mod dp), so walking down a column adds Tc mod dp to a
+  // residue: a thread per column finds its first kept row and the distance to the next in at most 2 dp steps, and the rest
+  // follows.  Then a scan over the columns, and a warp per column writes its rows.  (4096 tiles, a period of 4: 5.0 us; ballots over
+  // every tile of a column, twice, and one thread's running sum took 6.2.)
+  __shared__ int s_first[SAMPLER_THREADS], s_step[SAMPLER_THREADS], s_ptr[SAMPLER_THREADS], s_sum[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = nthreads / 32;
-  auto kept = [&](int r, int c) {
-    const int lin = r * Tc + c - (b - 1);
-    return r < Tr && lin >= 0 && lin % dp == 0;
-  };
-  for (int c = warp; c < Tc; c += nwarps) {
-    int cnt = 0;
-    for (int r0 = 0; r0 < Tr; r0 += 32) cnt += __popc(__ballot_sync(0xffffffffu, kept(r0 + lane, c)));
-    if (lane == 0) { if (in_smem) s_cnt[c] = cnt; else col_ptr[c + 1] = cnt; }
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int run = 0;
-    if (in_smem) {
-      for (int c = 0; c < Tc; ++c) { const int n = s_cnt[c]; s_cnt[c] = run; run += n; }
-    } else {
-      col_ptr[0] = 0;
-      for (int c = 0; c < Tc; ++c) { run += col_ptr[c + 1]; col_ptr[c + 1] = run; }
+  const int t = Tc % dp;
+  int before = 0;  // kept tiles in the columns of earlier rounds
+  for (int c0 = 0; c0 < Tc; c0 += nthreads) {
+    const int c = c0 + (int)threadIdx.x;
+    int first = Tr, step = Tr, cnt = 0;
+    if (c < Tc) {
+      int v = (c - (b - 1)) % dp;
+      if (v < 0) v += dp;
+      int r = 0;
+      auto down = [&]() { ++r; v += t; if (v >= dp) v -= dp; };
+      const int most = min(dp, Tr);  // dp rows on, the residue is the same again
+      while (v != 0 && r < most) down();
+      if (v == 0 && r < Tr) {
+        first = r;
+        do down(); while (v != 0 && r < Tr);
+        step = r - first;
+        cnt = v == 0 ? (Tr - 1 - first) / step + 1 : 1;
+      }
     }
-  }
-  __syncthreads();
-  if (in_smem) {
-    for (int c = threadIdx.x; c < Tc; c += nthreads) col_ptr[c] = s_cnt[c];
-    if (threadIdx.x == 0) col_ptr[Tc] = n_keep;
-  }
-  for (int c = warp; c < Tc; c += nwarps) {
-    int o = in_smem ? s_cnt[c] : col_ptr[c];
-    for (int r0 = 0; r0 < Tr; r0 += 32) {
-      const bool k = kept(r0 + lane, c);
-      const unsigned m = __ballot_sync(0xffffffffu, k);
-      if (k) col_idx[o + __popc(m & ((1u << lane) - 1u))] = r0 + lane;  // ascending rows
-      o += __popc(m);
+    int x = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, d);
+      if (lane >= d) x += y;
     }
+    if (lane == 31) s_sum[warp] = x;
+    __syncthreads();
+    int base = before, all = 0;
+    {
+      int w = lane < nwarps ? s_sum[lane] : 0;
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, w, d);
+        if (lane >= d) w += y;
+      }
+      all = __shfl_sync(0xffffffffu, w, 31);
+      const int mine = __shfl_sync(0xffffffffu, w, warp > 0 ? warp - 1 : 0);
+      if (warp > 0) base += mine;
+    }
+    base += x - cnt;
+    if (c < Tc) col_ptr[c] = base;
+    s_first[threadIdx.x] = first;
+    s_step[threadIdx.x] = step;
+    s_ptr[threadIdx.x] = base;
+    __syncthreads();
+    for (int i = warp; i < min(nthreads, Tc - c0); i += nwarps) {
+      int32_t* to = col_idx + s_ptr[i];
+      for (int r = s_first[i] + lane * s_step[i], j = lane; r < Tr; r += 32 * s_step[i], j += 32) to[j] = r;  // ascending rows
+    }
+    before += all;
+    __syncthreads();
   }
+  if (threadIdx.x == 0) col_ptr[Tc] = before;
 }
 
 }  // namespace
