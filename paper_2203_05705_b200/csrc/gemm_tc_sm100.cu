@@ -1116,6 +1116,25 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
         if (FUSED && (MODE == M_ROW_FWD || MODE == M_ROW_BWD_DATA) && p.ridx != nullptr && row_ok) out_row = p.ridx[m];
       }
 
+      constexpr bool ZERO_ROWS = MODE == M_ROW_BWD_WEIGHT || MODE == M_LSTM_BWD_WEIGHT;
+      constexpr int LINES_AT_ONCE = ZERO_ROWS ? 2 : 8;  // what fits the registers
+      // the class form keeps its list in the staging area, the row lists' weight gradient its row addresses
+      constexpr bool F32_LINES = !(is_class_mode(MODE) && !PLAIN) && !is_rows_mode(MODE);
+      // Zeros of the dropped neurons' rows beside this warp's row rr (output row `own`): 16 bytes of each from column n on, so that the
+      // eight lanes of a row write whole lines.  Compact row m owns output rows [m * dp, (m + 1) * dp), the last one also the tail.
+      // With a row to a thread these stores were most of a sparse product's time (2048 x 512 -> 4096, a period of 16, sampler and three
+      // products 78.4 -> 63.0 us; 4096 x 2048 x 2048 98.7 -> 85.3; LSTM layer of 1500 units, batch 20, a period of 8 361 -> 338).
+      auto zero_beside = [&](int rr, long long own, int n) {
+        const int mm = ti.m0 + q * 32 + rr;
+        const long long goff = (MODE == M_LSTM_BWD_WEIGHT) ? ti.out_row0 : 0;  // the gate's block of rows
+        const long long first = (long long)mm * dp;
+        const long long last = mm == sch.M_gemm - 1 ? (long long)p.N - 1 : min(first + dp - 1, (long long)p.N - 1);
+        char* o = reinterpret_cast<char*>(p.out) + ((size_t)(goff + first) * p.ldo + n) * (p.out_is_f32 ? 4 : 2);
+        const size_t pitch = (size_t)p.ldo * (p.out_is_f32 ? 4 : 2);
+        for (long long rz = goff + first; rz <= goff + last; ++rz, o += pitch)
+          if (rz != own) *reinterpret_cast<uint4*>(o) = make_uint4(0u, 0u, 0u, 0u);
+      };
+
       // The values of one 32-column chunk of this thread's accumulator row (already loaded into r[]), whose
       // first output column is n: rescale, and for the layer-step kernels bias / activation / ReLU adjoint.
       auto values = [&](const uint32_t (&r)[32], int n, float (&v)[32]) {
@@ -1257,9 +1276,30 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
           const int nvalid = (is_class_mode(MODE) && !PLAIN) ? 32
                              : (MODE == M_LSTM_FWD ? min(32, sch.n_keep - (ti.n0 + (ch & 1) * 32))
                                                    : min(32, sch.N_gemm - n));
-          if (row_ok && nvalid > 0) {
+          if (F32_LINES && p.out_is_f32 && !p.accumulate && nvalid >= 32) {
+            // fp32 rows go out through the warp's staging block as well, eight lanes to a row's 128 bytes (see the bf16 pairs below;
+            // gate products of 35 x 64 rows, 512 of 1024 units kept, forward 19.1 -> 16.5 us, input gradient 25.4 -> 23.3)
+            const unsigned rows_ok = __ballot_sync(0xffffffffu, row_ok);
+            float* sf = stg + lane * 33;
+#pragma unroll
+            for (int i = 0; i < 32; ++i) sf[i] = v[i];
+            __syncwarp();
+            const int piece = lane & 7;
+#pragma unroll LINES_AT_ONCE
+            for (int it8 = 0; it8 < 8; ++it8) {
+              const int rr = it8 * 4 + (lane >> 3);
+              const long long orow = __shfl_sync(0xffffffffu, out_row, rr);
+              const float* f = stg + rr * 33 + piece * 4;
+              const float4 w = make_float4(f[0], f[1], f[2], f[3]);
+              if ((rows_ok >> rr) & 1u) {
+                *reinterpret_cast<float4*>(reinterpret_cast<float*>(p.out) + (size_t)orow * p.ldo + n + piece * 4) = w;
+                if (ZERO_ROWS && p.zero_fill && dp > 1) zero_beside(rr, orow, n + piece * 4);
+              }
+            }
+            __syncwarp();
+          } else if (row_ok && nvalid > 0) {
             store_row32(p.out, (size_t)out_row * p.ldo, n, v, nvalid, p.out_is_f32, p.accumulate);
-            if ((MODE == M_ROW_BWD_WEIGHT || MODE == M_LSTM_BWD_WEIGHT) && p.zero_fill) {
+            if (ZERO_ROWS && p.zero_fill) {
               // Compact row m owns output rows [m*dp, (m+1)*dp); the last one also owns the tail.
               const long long goff = (MODE == M_LSTM_BWD_WEIGHT) ? ti.out_row0 : 0;  // the gate's block of rows
               const long long first = goff + (long long)m * dp;
@@ -1363,8 +1403,7 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
         // kept it at 6.4 us per 256 x 256 tile where the products and loads need 4.1.
         constexpr bool PAIR_MODES = MODE == M_ROW_FWD || MODE == M_ROW_BWD_DATA || MODE == M_ROW_BWD_WEIGHT ||
                                     (is_class_mode(MODE) && PLAIN);
-        const bool pair_ok = PAIR_MODES && !p.out_is_f32 && !p.accumulate && !(MODE == M_ROW_FWD && p.scatter && dp > 1) &&
-                             !(MODE == M_ROW_BWD_WEIGHT && p.zero_fill);
+        const bool pair_ok = PAIR_MODES && !p.out_is_f32 && !p.accumulate && !(MODE == M_ROW_FWD && p.scatter && dp > 1);
         const unsigned okmask = __ballot_sync(0xffffffffu, row_ok);
         // The class tiling keeps its list in the first part of the staging area: its warps stage one chunk
         // (32 rows x 17 words) behind it and write 64-byte row segments, four lanes per row.
@@ -1408,14 +1447,16 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
         auto flush_pair = [&](int n) {  // 32 rows x 64 columns starting at output column n
           __syncwarp();
           const int piece = lane & 7;
-#pragma unroll
+#pragma unroll LINES_AT_ONCE
           for (int it8 = 0; it8 < 8; ++it8) {
             const int rr = it8 * 4 + (lane >> 3);
             const long long orow = __shfl_sync(0xffffffffu, out_row, rr);
             const uint32_t* q = stw + rr * SW + piece * 4;
             const uint4 w = make_uint4(q[0], q[1], q[2], q[3]);
-            if ((okmask >> rr) & 1u)
+            if ((okmask >> rr) & 1u) {
               *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (size_t)orow * p.ldo + n + piece * 8) = w;
+              if (ZERO_ROWS && p.zero_fill && dp > 1) zero_beside(rr, orow, n + piece * 8);
+            }
           }
           __syncwarp();
         };
