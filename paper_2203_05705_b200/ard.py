@@ -157,6 +157,20 @@ def lib():
     return L
 
 
+_native = None
+
+
+def _calls():
+    """The calls of a training iteration, which take tensors as they are: an extension module beside the library
+    (csrc/python_calls.cpp).  Handing their arguments over through ctypes took 2.9 us of an ard_fwd, now 1.1."""
+    global _native
+    if _native is None:
+        lib()  # says what is missing where nothing has been built
+        from . import _calls as module
+        _native = module
+    return _native
+
+
 def _check(st, where):
     if st != ARD_OK:
         raise ArdError(st, where)
@@ -274,12 +288,12 @@ def ard_pattern_destroy(pat):
 
 
 def ard_sample_pattern(ctx, pat, dist_id, seed, iteration, stream_id, stream=None):
-    _check(lib().ard_sample_pattern(ctx, pat, dist_id, seed, iteration, stream_id, _stream(stream)),
+    _check(_calls().ard_sample_pattern(ctx, pat, dist_id, seed, iteration, stream_id, _stream(stream)),
            "ard_sample_pattern")
 
 
 def ard_pattern_set(ctx, pat, dp, b, stream=None):
-    _check(lib().ard_pattern_set(ctx, pat, dp, b, _stream(stream)), "ard_pattern_set")
+    _check(_calls().ard_pattern_set(ctx, pat, dp, b, _stream(stream)), "ard_pattern_set")
 
 
 def ard_pattern_to_host(pat, capacity, stream=None):
@@ -305,67 +319,67 @@ def ard_pattern_tile_lists_to_host(pat, Tr, Tc, stream=None):
 
 
 def ard_fwd(ctx, pat, dtype, B, K, N, alpha, X, ldx, W, ldw, Y, ldy, outmode, stream=None):
-    _check(lib().ard_fwd(ctx, pat, dtype, B, K, N, alpha, _ptr(X), ldx, _ptr(W), ldw, _ptr(Y), ldy, outmode,
+    _check(_calls().ard_fwd(ctx, pat, dtype, B, K, N, alpha, X, ldx, W, ldw, Y, ldy, outmode,
                          _stream(stream)), "ard_fwd")
 
 
 def ard_bwd_data(ctx, pat, dtype, B, K, N, alpha, dY, lddy, dy_is_compact, W, ldw, dX, lddx, stream=None):
-    _check(lib().ard_bwd_data(ctx, pat, dtype, B, K, N, alpha, _ptr(dY), lddy, dy_is_compact, _ptr(W), ldw,
-                              _ptr(dX), lddx, _stream(stream)), "ard_bwd_data")
+    _check(_calls().ard_bwd_data(ctx, pat, dtype, B, K, N, alpha, dY, lddy, dy_is_compact, W, ldw,
+                              dX, lddx, _stream(stream)), "ard_bwd_data")
 
 
 def ard_bwd_data_static_scratch(ctx, pat, dtype, B, K, N, alpha, dY, lddy, W, ldw, dX, lddx, stream=None):
     """Backward-data for callers that must not allocate: same result as ard_bwd_data (row pattern,
     full-width dY), with the compacted dY kept in the library's fixed device array."""
-    _check(lib().ard_bwd_data_static_scratch(ctx, pat, dtype, B, K, N, alpha, _ptr(dY), lddy, _ptr(W), ldw,
-                                             _ptr(dX), lddx, _stream(stream)), "ard_bwd_data_static_scratch")
+    _check(_calls().ard_bwd_data_static_scratch(ctx, pat, dtype, B, K, N, alpha, dY, lddy, W, ldw,
+                                             dX, lddx, _stream(stream)), "ard_bwd_data_static_scratch")
 
 
 def ard_bwd_weight(ctx, pat, dtype, dW_dtype, B, K, N, alpha, X, ldx, dY, lddy, dy_is_compact, dW, lddw,
                    zero_fill_dropped, stream=None):
-    _check(lib().ard_bwd_weight(ctx, pat, dtype, dW_dtype, B, K, N, alpha, _ptr(X), ldx, _ptr(dY), lddy,
-                                dy_is_compact, _ptr(dW), lddw, zero_fill_dropped, _stream(stream)),
+    _check(_calls().ard_bwd_weight(ctx, pat, dtype, dW_dtype, B, K, N, alpha, X, ldx, dY, lddy,
+                                dy_is_compact, dW, lddw, zero_fill_dropped, _stream(stream)),
            "ard_bwd_weight")
 
 
 def ard_layer_fwd(ctx, pat, in_pat, dtype, B, K, N, alpha, X, ldx, Wk, ldw, bias, A, lda, outmode_and_flags,
                   stream=None):
-    _check(lib().ard_layer_fwd(ctx, pat, in_pat, dtype, B, K, N, alpha, _ptr(X), ldx, _ptr(Wk), ldw, _ptr(bias),
-                               _ptr(A), lda, outmode_and_flags, _stream(stream)), "ard_layer_fwd")
+    _check(_calls().ard_layer_fwd(ctx, pat, in_pat, dtype, B, K, N, alpha, X, ldx, Wk, ldw, bias,
+                               A, lda, outmode_and_flags, _stream(stream)), "ard_layer_fwd")
 
 
 def ard_layer_bwd_data(ctx, pat, in_pat, dtype, B, K, N, alpha, dZ, lddz, dz_is_compact_and_flags, Wk, ldw, act_prev,
                        ldact, dX, lddx, stream=None):
-    _check(lib().ard_layer_bwd_data(ctx, pat, in_pat, dtype, B, K, N, alpha, _ptr(dZ), lddz, dz_is_compact_and_flags,
-                                    _ptr(Wk), ldw, _ptr(act_prev), ldact, _ptr(dX), lddx, _stream(stream)),
+    _check(_calls().ard_layer_bwd_data(ctx, pat, in_pat, dtype, B, K, N, alpha, dZ, lddz, dz_is_compact_and_flags,
+                                    Wk, ldw, act_prev, ldact, dX, lddx, _stream(stream)),
            "ard_layer_bwd_data")
 
 
 def ard_layer_bwd_weight(ctx, pat, in_pat, dtype, dW_dtype, B, K, N, alpha, X, ldx, dZ, lddz, dz_is_compact, dWk, lddw,
                          zero_fill_dropped, stream=None):
-    _check(lib().ard_layer_bwd_weight(ctx, pat, in_pat, dtype, dW_dtype, B, K, N, alpha, _ptr(X), ldx, _ptr(dZ), lddz,
-                                      dz_is_compact, _ptr(dWk), lddw, zero_fill_dropped, _stream(stream)),
+    _check(_calls().ard_layer_bwd_weight(ctx, pat, in_pat, dtype, dW_dtype, B, K, N, alpha, X, ldx, dZ, lddz,
+                                      dz_is_compact, dWk, lddw, zero_fill_dropped, _stream(stream)),
            "ard_layer_bwd_weight")
 
 
 def ard_compact_weight_cols(ctx, pat, in_pat, dtype, K, N, W, ldw, Wk, ldwk, stream=None):
-    _check(lib().ard_compact_weight_cols(ctx, pat, in_pat, dtype, K, N, _ptr(W), ldw, _ptr(Wk), ldwk, _stream(stream)),
+    _check(_calls().ard_compact_weight_cols(ctx, pat, in_pat, dtype, K, N, W, ldw, Wk, ldwk, _stream(stream)),
            "ard_compact_weight_cols")
 
 
 def ard_expand_weight_grad_cols(ctx, pat, in_pat, dtype, K, N, dWk, lddwk, dW, lddw, zero_fill, stream=None):
-    _check(lib().ard_expand_weight_grad_cols(ctx, pat, in_pat, dtype, K, N, _ptr(dWk), lddwk, _ptr(dW), lddw,
+    _check(_calls().ard_expand_weight_grad_cols(ctx, pat, in_pat, dtype, K, N, dWk, lddwk, dW, lddw,
                                              zero_fill, _stream(stream)), "ard_expand_weight_grad_cols")
 
 
 def ard_bias_grad(ctx, pat, dtype, B, N, dZ, lddz, dz_is_compact, db, zero_fill_dropped, stream=None):
-    _check(lib().ard_bias_grad(ctx, pat, dtype, B, N, _ptr(dZ), lddz, dz_is_compact, _ptr(db), zero_fill_dropped,
+    _check(_calls().ard_bias_grad(ctx, pat, dtype, B, N, dZ, lddz, dz_is_compact, db, zero_fill_dropped,
                                _stream(stream)), "ard_bias_grad")
 
 
 def ard_sample_pattern_counter(ctx, pat, dist_id, seed, iteration_base, iteration_counter, advance, stream_id,
                                stream=None):
-    _check(lib().ard_sample_pattern_counter(ctx, pat, dist_id, seed, iteration_base, _ptr(iteration_counter),
+    _check(_calls().ard_sample_pattern_counter(ctx, pat, dist_id, seed, iteration_base, iteration_counter,
                                             1 if advance else 0, stream_id, _stream(stream)),
            "ard_sample_pattern_counter")
 
@@ -411,7 +425,7 @@ def ard_blocks_destroy(blocks):
 
 def ard_blocks_predict(ctx, blocks, dtype, A, lda, k_frac, run_len, t_frac, threshold, cap, seed, iteration, stream_id,
                        stream=None):
-    _check(lib().ard_blocks_predict(ctx, blocks, dtype, _ptr(A), lda, k_frac, run_len, t_frac, threshold, cap, seed,
+    _check(_calls().ard_blocks_predict(ctx, blocks, dtype, A, lda, k_frac, run_len, t_frac, threshold, cap, seed,
                                     iteration, stream_id, _stream(stream)), "ard_blocks_predict")
 
 
@@ -420,29 +434,29 @@ def ard_blocks_set_label(ctx, blocks, sensitive, stream=None):
 
 
 def ard_blocks_sample(ctx, blocks, m_prob, n_prob, seed, iteration, stream_id, stream=None):
-    _check(lib().ard_blocks_sample(ctx, blocks, m_prob, n_prob, seed, iteration, stream_id, _stream(stream)),
+    _check(_calls().ard_blocks_sample(ctx, blocks, m_prob, n_prob, seed, iteration, stream_id, _stream(stream)),
            "ard_blocks_sample")
 
 
 def ard_blocks_fwd(ctx, blocks, N, alpha, A, lda, W, ldw, Yt, ldyt, stream=None):
-    _check(lib().ard_blocks_fwd(ctx, blocks, N, alpha, _ptr(A), lda, _ptr(W), ldw, _ptr(Yt), ldyt, _stream(stream)),
+    _check(_calls().ard_blocks_fwd(ctx, blocks, N, alpha, A, lda, W, ldw, Yt, ldyt, _stream(stream)),
            "ard_blocks_fwd")
 
 
 def ard_blocks_bwd_weight(ctx, blocks, N, alpha, A, lda, dYt, lddyt, dW, lddw, stream=None):
-    _check(lib().ard_blocks_bwd_weight(ctx, blocks, N, alpha, _ptr(A), lda, _ptr(dYt), lddyt, _ptr(dW), lddw,
+    _check(_calls().ard_blocks_bwd_weight(ctx, blocks, N, alpha, A, lda, dYt, lddyt, dW, lddw,
                                        _stream(stream)), "ard_blocks_bwd_weight")
 
 
 def ard_blocks_bwd_input(ctx, blocks, dA_dtype, N, alpha, dYt, lddyt, W, ldw, dA, ldda, zero_fill_dropped, stream=None):
-    _check(lib().ard_blocks_bwd_input(ctx, blocks, dA_dtype, N, alpha, _ptr(dYt), lddyt, _ptr(W), ldw, _ptr(dA), ldda,
+    _check(_calls().ard_blocks_bwd_input(ctx, blocks, dA_dtype, N, alpha, dYt, lddyt, W, ldw, dA, ldda,
                                       zero_fill_dropped, _stream(stream)), "ard_blocks_bwd_input")
 
 
 def ard_blocks_products(ctx, blocks, dA_dtype, N, alpha, A, lda, W, ldw, dYt, lddyt, Yt, ldyt, dW, lddw, dA, ldda,
                         zero_fill_dropped, stream=None):
-    _check(lib().ard_blocks_products(ctx, blocks, dA_dtype, N, alpha, _ptr(A), lda, _ptr(W), ldw, _ptr(dYt), lddyt,
-                                     _ptr(Yt), ldyt, _ptr(dW), lddw, _ptr(dA), ldda, zero_fill_dropped, _stream(stream)),
+    _check(_calls().ard_blocks_products(ctx, blocks, dA_dtype, N, alpha, A, lda, W, ldw, dYt, lddyt,
+                                     Yt, ldyt, dW, lddw, dA, ldda, zero_fill_dropped, _stream(stream)),
            "ard_blocks_products")
 
 
@@ -473,7 +487,7 @@ def ard_rows_destroy(rows):
 
 def ard_sensitivity_predict(ctx, rows, dtype, A, lda, Kc, k_frac, run_len, t_frac, threshold, m_prob, n_prob, seed,
                             iteration, stream_id, stream=None):
-    _check(lib().ard_sensitivity_predict(ctx, rows, dtype, _ptr(A), lda, Kc, k_frac, run_len, t_frac, threshold, m_prob,
+    _check(_calls().ard_sensitivity_predict(ctx, rows, dtype, A, lda, Kc, k_frac, run_len, t_frac, threshold, m_prob,
                                          n_prob, seed, iteration, stream_id, _stream(stream)), "ard_sensitivity_predict")
 
 
@@ -482,7 +496,7 @@ def ard_rows_set_probability(ctx, rows, p, stream=None):
 
 
 def ard_rows_sample(ctx, rows, seed, iteration, stream_id, stream=None):
-    _check(lib().ard_rows_sample(ctx, rows, seed, iteration, stream_id, _stream(stream)), "ard_rows_sample")
+    _check(_calls().ard_rows_sample(ctx, rows, seed, iteration, stream_id, _stream(stream)), "ard_rows_sample")
 
 
 def ard_rows_to_host(rows, M, regions=0, stream=None):
@@ -497,112 +511,112 @@ def ard_rows_to_host(rows, M, regions=0, stream=None):
 
 
 def ard_rows_fwd(ctx, rows, M, K, N, alpha, A, lda, W, ldw, Y, ldy, stream=None):
-    _check(lib().ard_rows_fwd(ctx, rows, M, K, N, alpha, _ptr(A), lda, _ptr(W), ldw, _ptr(Y), ldy, _stream(stream)),
+    _check(_calls().ard_rows_fwd(ctx, rows, M, K, N, alpha, A, lda, W, ldw, Y, ldy, _stream(stream)),
            "ard_rows_fwd")
 
 
 def ard_rows_bwd_data(ctx, rows, M, K, N, alpha, dY, lddy, W, ldw, dA, ldda, stream=None):
-    _check(lib().ard_rows_bwd_data(ctx, rows, M, K, N, alpha, _ptr(dY), lddy, _ptr(W), ldw, _ptr(dA), ldda,
+    _check(_calls().ard_rows_bwd_data(ctx, rows, M, K, N, alpha, dY, lddy, W, ldw, dA, ldda,
                                    _stream(stream)), "ard_rows_bwd_data")
 
 
 def ard_rows_bwd_weight(ctx, rows, dW_dtype, M, K, N, alpha, A, lda, dY, lddy, dW, lddw, stream=None):
-    _check(lib().ard_rows_bwd_weight(ctx, rows, dW_dtype, M, K, N, alpha, _ptr(A), lda, _ptr(dY), lddy, _ptr(dW), lddw,
+    _check(_calls().ard_rows_bwd_weight(ctx, rows, dW_dtype, M, K, N, alpha, A, lda, dY, lddy, dW, lddw,
                                      _stream(stream)), "ard_rows_bwd_weight")
 
 
 def ard_layer_products(ctx, pat, dtype, dW_dtype, B, K, N, alpha, X, ldx, W, ldw, dY, lddy, Y, ldy, outmode, dX, lddx,
                        dW, lddw, zero_fill_dropped, stream=None):
-    _check(lib().ard_layer_products(ctx, pat, dtype, dW_dtype, B, K, N, alpha, _ptr(X), ldx, _ptr(W), ldw, _ptr(dY),
-                                    lddy, _ptr(Y), ldy, outmode, _ptr(dX), lddx, _ptr(dW), lddw, zero_fill_dropped,
+    _check(_calls().ard_layer_products(ctx, pat, dtype, dW_dtype, B, K, N, alpha, X, ldx, W, ldw, dY,
+                                    lddy, Y, ldy, outmode, dX, lddx, dW, lddw, zero_fill_dropped,
                                     _stream(stream)), "ard_layer_products")
 
 
 def ard_rows_products(ctx, rows, dW_dtype, M, K, N, alpha, A, lda, W, ldw, dY, lddy, Ak, ldak, dYk, lddyk, Y, ldy, dA,
                       ldda, dW, lddw, stream=None):
-    _check(lib().ard_rows_products(ctx, rows, dW_dtype, M, K, N, alpha, _ptr(A), lda, _ptr(W), ldw, _ptr(dY), lddy,
-                                   _ptr(Ak), ldak, _ptr(dYk), lddyk, _ptr(Y), ldy, _ptr(dA), ldda, _ptr(dW), lddw,
+    _check(_calls().ard_rows_products(ctx, rows, dW_dtype, M, K, N, alpha, A, lda, W, ldw, dY, lddy,
+                                   Ak, ldak, dYk, lddyk, Y, ldy, dA, ldda, dW, lddw,
                                    _stream(stream)), "ard_rows_products")
 
 
 def ard_rows_gather(ctx, rows, M, width, src, ld_src, dst, ld_dst, stream=None):
-    _check(lib().ard_rows_gather(ctx, rows, M, width, _ptr(src), ld_src, _ptr(dst), ld_dst, _stream(stream)),
+    _check(_calls().ard_rows_gather(ctx, rows, M, width, src, ld_src, dst, ld_dst, _stream(stream)),
            "ard_rows_gather")
 
 
 def ard_rows_fwd_compact(ctx, rows, M, K, N, alpha, Ak, ldak, W, ldw, Y, ldy, stream=None):
-    _check(lib().ard_rows_fwd_compact(ctx, rows, M, K, N, alpha, _ptr(Ak), ldak, _ptr(W), ldw, _ptr(Y), ldy,
+    _check(_calls().ard_rows_fwd_compact(ctx, rows, M, K, N, alpha, Ak, ldak, W, ldw, Y, ldy,
                                       _stream(stream)), "ard_rows_fwd_compact")
 
 
 def ard_rows_bwd_data_compact(ctx, rows, M, K, N, alpha, dYk, lddyk, W, ldw, dA, ldda, stream=None):
-    _check(lib().ard_rows_bwd_data_compact(ctx, rows, M, K, N, alpha, _ptr(dYk), lddyk, _ptr(W), ldw, _ptr(dA), ldda,
+    _check(_calls().ard_rows_bwd_data_compact(ctx, rows, M, K, N, alpha, dYk, lddyk, W, ldw, dA, ldda,
                                            _stream(stream)), "ard_rows_bwd_data_compact")
 
 
 def ard_rows_bwd_weight_compact(ctx, rows, dW_dtype, M, K, N, alpha, Ak, ldak, dYk, lddyk, dW, lddw, stream=None):
-    _check(lib().ard_rows_bwd_weight_compact(ctx, rows, dW_dtype, M, K, N, alpha, _ptr(Ak), ldak, _ptr(dYk), lddyk,
-                                             _ptr(dW), lddw, _stream(stream)), "ard_rows_bwd_weight_compact")
+    _check(_calls().ard_rows_bwd_weight_compact(ctx, rows, dW_dtype, M, K, N, alpha, Ak, ldak, dYk, lddyk,
+                                             dW, lddw, _stream(stream)), "ard_rows_bwd_weight_compact")
 
 
 def ard_lstm_gate_gemm(ctx, pat, B, KH, H, XH, ldxh, W, ldw, Z, ldz_gate, stream=None):
-    _check(lib().ard_lstm_gate_gemm(ctx, pat, B, KH, H, _ptr(XH), ldxh, _ptr(W), ldw, _ptr(Z), ldz_gate,
+    _check(_calls().ard_lstm_gate_gemm(ctx, pat, B, KH, H, XH, ldxh, W, ldw, Z, ldz_gate,
                                     _stream(stream)), "ard_lstm_gate_gemm")
 
 
 def ard_lstm_gate_gemm_bwd(ctx, pat, B, KH, H, dZ, ldz_gate, W, ldw, dXH, lddxh, accumulate, stream=None):
-    _check(lib().ard_lstm_gate_gemm_bwd(ctx, pat, B, KH, H, _ptr(dZ), ldz_gate, _ptr(W), ldw, _ptr(dXH), lddxh,
+    _check(_calls().ard_lstm_gate_gemm_bwd(ctx, pat, B, KH, H, dZ, ldz_gate, W, ldw, dXH, lddxh,
                                         accumulate, _stream(stream)), "ard_lstm_gate_gemm_bwd")
 
 
 def ard_lstm_forward(ctx, pat, T, B, I, H, alpha, XH, W, ldw, bias, C, G, Z, stream=None):
-    _check(lib().ard_lstm_forward(ctx, pat, T, B, I, H, alpha, _ptr(XH), _ptr(W), ldw, _ptr(bias), _ptr(C), _ptr(G),
-                                  _ptr(Z), _stream(stream)), "ard_lstm_forward")
+    _check(_calls().ard_lstm_forward(ctx, pat, T, B, I, H, alpha, XH, W, ldw, bias, C, G,
+                                  Z, _stream(stream)), "ard_lstm_forward")
 
 
 def ard_lstm_backward(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH_last, D, dc, DZ, dW, stream=None):
-    _check(lib().ard_lstm_backward(ctx, pat, T, B, I, H, alpha, _ptr(XH), _ptr(W), ldw, _ptr(C), _ptr(G),
-                                   _ptr(dH_last), _ptr(D), _ptr(dc), _ptr(DZ), _ptr(dW), _stream(stream)),
+    _check(_calls().ard_lstm_backward(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G,
+                                   dH_last, D, dc, DZ, dW, _stream(stream)),
            "ard_lstm_backward")
 
 
 def ard_lstm_backward_dh(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH, D, dc, DZ, dW, stream=None):
-    _check(lib().ard_lstm_backward_dh(ctx, pat, T, B, I, H, alpha, _ptr(XH), _ptr(W), ldw, _ptr(C), _ptr(G), _ptr(dH), _ptr(D),
-                                      _ptr(dc), _ptr(DZ), _ptr(dW), _stream(stream)), "ard_lstm_backward_dh")
+    _check(_calls().ard_lstm_backward_dh(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH, D,
+                                      dc, DZ, dW, _stream(stream)), "ard_lstm_backward_dh")
 
 
 def ard_lstm_forward_from_gates(ctx, pat, T, B, I, H, alpha, XH, W, ldw, bias, C, G, stream=None):
-    _check(lib().ard_lstm_forward_from_gates(ctx, pat, T, B, I, H, alpha, _ptr(XH), _ptr(W), ldw, _ptr(bias), _ptr(C),
-                                             _ptr(G), _stream(stream)), "ard_lstm_forward_from_gates")
+    _check(_calls().ard_lstm_forward_from_gates(ctx, pat, T, B, I, H, alpha, XH, W, ldw, bias, C,
+                                             G, _stream(stream)), "ard_lstm_forward_from_gates")
 
 
 def ard_lstm_backward_recurrent(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G, dH_last, D, dc, DZ, dW, stream=None):
-    _check(lib().ard_lstm_backward_recurrent(ctx, pat, T, B, I, H, alpha, _ptr(XH), _ptr(W), ldw, _ptr(C), _ptr(G),
-                                             _ptr(dH_last), _ptr(D), _ptr(dc), _ptr(DZ), _ptr(dW), _stream(stream)),
+    _check(_calls().ard_lstm_backward_recurrent(ctx, pat, T, B, I, H, alpha, XH, W, ldw, C, G,
+                                             dH_last, D, dc, DZ, dW, _stream(stream)),
            "ard_lstm_backward_recurrent")
 
 
 def ard_compact_cols(ctx, pat, dtype, rows, N, src, ld_src, dst, ld_dst, stream=None):
-    _check(lib().ard_compact_cols(ctx, pat, dtype, rows, N, _ptr(src), ld_src, _ptr(dst), ld_dst, _stream(stream)),
+    _check(_calls().ard_compact_cols(ctx, pat, dtype, rows, N, src, ld_src, dst, ld_dst, _stream(stream)),
            "ard_compact_cols")
 
 
 def ard_expand_cols(ctx, pat, src_dtype, rows, N, alpha, src, ld_src, dst, ld_dst, stream=None):
-    _check(lib().ard_expand_cols(ctx, pat, src_dtype, rows, N, alpha, _ptr(src), ld_src, _ptr(dst), ld_dst,
+    _check(_calls().ard_expand_cols(ctx, pat, src_dtype, rows, N, alpha, src, ld_src, dst, ld_dst,
                                  _stream(stream)), "ard_expand_cols")
 
 
 def ard_lstm_gates(ctx, pat, h_dtype, B, H, alpha, Z, ldz_gate, bias, c_prev, ldc, c, h, ldh, h_scatter,
                    gates_saved, stream=None):
-    _check(lib().ard_lstm_gates(ctx, pat, h_dtype, B, H, alpha, _ptr(Z), ldz_gate, _ptr(bias), _ptr(c_prev), ldc,
-                                _ptr(c), _ptr(h), ldh, h_scatter, _ptr(gates_saved), _stream(stream)),
+    _check(_calls().ard_lstm_gates(ctx, pat, h_dtype, B, H, alpha, Z, ldz_gate, bias, c_prev, ldc,
+                                c, h, ldh, h_scatter, gates_saved, _stream(stream)),
            "ard_lstm_gates")
 
 
 def ard_lstm_gates_bwd(ctx, pat, dz_dtype, B, H, alpha, gates_saved, c_prev, c, ldc, dh, lddh, dh_scatter,
                        dc_inout, dZ, ldz_gate, stream=None):
-    _check(lib().ard_lstm_gates_bwd(ctx, pat, dz_dtype, B, H, alpha, _ptr(gates_saved), _ptr(c_prev), _ptr(c), ldc,
-                                    _ptr(dh), lddh, dh_scatter, _ptr(dc_inout), _ptr(dZ), ldz_gate,
+    _check(_calls().ard_lstm_gates_bwd(ctx, pat, dz_dtype, B, H, alpha, gates_saved, c_prev, c, ldc,
+                                    dh, lddh, dh_scatter, dc_inout, dZ, ldz_gate,
                                     _stream(stream)), "ard_lstm_gates_bwd")
 
 

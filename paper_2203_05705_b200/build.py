@@ -1,4 +1,4 @@
-"""Builds libard.so in-tree with nvcc for sm_100a (cross-compiles without a GPU).
+"""Builds libard.so and the Python functions of its hot calls in-tree with nvcc for sm_100a (cross-compiles without a GPU).
 
     python -m paper_2203_05705_b200.build [--force] [--verbose]
 """
@@ -8,6 +8,7 @@ import hashlib
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 PKG = os.path.dirname(os.path.abspath(__file__))
@@ -15,6 +16,8 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "build")
 LIB = os.path.join(PKG, "libard.so")
+CALLS_SRC = os.path.join(CSRC, "python_calls.cpp")
+CALLS = os.path.join(PKG, "_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))  # one per interpreter
 SOURCES = ["api.cu", "sampler.cu", "gemm_cc.cu", "gemm_tc_sm100.cu", "gemm_ldg_sm100.cu", "gemm_f32_sm100.cu", "aux_kernels.cu", "no_alloc.cu",
            "distribution_search.cu", "lstm_persistent.cu", "mlp_step.cu", "mlp_persistent.cu", "rows.cu", "blocks.cu", "dropout_schedule.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
@@ -74,7 +77,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     def run(cmd):
         r = subprocess.run(cmd, capture_output=True, text=True)
         if r.returncode != 0:
-            raise RuntimeError("nvcc failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
+            raise RuntimeError(cmd[0] + " failed:\n" + " ".join(cmd) + "\n" + r.stdout + r.stderr)
         return r.stderr
 
     def compile_one(job):
@@ -90,6 +93,15 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 print(out)
     if jobs or force or _stale(LIB, objs):
         run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs)
+    # the Python functions of the hot calls; found beside the library at run time
+    flags = ["-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"]]
+    deps = [CALLS_SRC, os.path.join(ROOT, "include", "ard.h")]
+    mark = os.path.join(OBJ, os.path.basename(CALLS) + ".key")
+    want = _sha(deps, " ".join(flags))
+    if force or not os.path.exists(CALLS) or not os.path.exists(mark) or open(mark).read() != want + _sha([CALLS]):
+        run([os.environ.get("CXX", "g++")] + flags + [CALLS_SRC, "-o", CALLS, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
+        with open(mark, "w") as f:
+            f.write(want + _sha([CALLS]))
     return LIB
 
 
