@@ -429,16 +429,16 @@ struct Sched {
     total = __shfl_sync(0xffffffffu, x, 31);
     return x - v;
   }
-  __device__ void build_class_table(const TcParams& p, int4* tab, int* out, int lane) const {
-    const int32_t* ptr = (MODE == M_TILEC_BWD_DATA) ? p.row_ptr : p.col_ptr;
+  // ptr: list pointers of classes lane and lane + 32 and behind them.
+  __device__ void build_class_table(const TcParams& p, const int (&ptr)[2][2], int4* tab, int* out, int lane) const {
     int off[2], len[2], cnt[2], items[2];
     bool valid[2], full[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int c = lane + 32 * h;
       valid[h] = c < nclass;
-      off[h] = valid[h] ? ptr[c] : 0;
-      len[h] = valid[h] ? ptr[c + 1] - off[h] : 0;
+      off[h] = valid[h] ? ptr[h][0] : 0;
+      len[h] = valid[h] ? ptr[h][1] - off[h] : 0;
       cnt[h] = valid[h] ? class_members(c) : 0;
       items[h] = valid[h] ? class_items(cnt[h], len[h]) : 0;
       full[h] = valid[h] && len[h] != 0;
@@ -447,11 +447,13 @@ struct Sched {
     const unsigned mf0 = __ballot_sync(0xffffffffu, full[0]), mf1 = __ballot_sync(0xffffffffu, full[1]);
     const unsigned me0 = __ballot_sync(0xffffffffu, valid[0] && !full[0]), me1 = __ballot_sync(0xffffffffu, valid[1] && !full[1]);
     const int n_full = __popc(mf0) + __popc(mf1);
-    int tA, tB, tC, tD;
+    int tA, tB = 0, tC, tD = 0, sB = 0, sD = 0;
     const int sA = warp_excl_scan(full[0] ? items[0] : 0, lane, tA);
-    const int sB = warp_excl_scan(full[1] ? items[1] : 0, lane, tB);
     const int sC = warp_excl_scan(valid[0] && !full[0] ? items[0] : 0, lane, tC);
-    const int sD = warp_excl_scan(valid[1] && !full[1] ? items[1] : 0, lane, tD);
+    if (nclass > 32) {
+      sB = warp_excl_scan(full[1] ? items[1] : 0, lane, tB);
+      sD = warp_excl_scan(valid[1] && !full[1] ? items[1] : 0, lane, tD);
+    }
     if (valid[0]) {
       const int slot = full[0] ? __popc(mf0 & lt) : n_full + __popc(me0 & lt);
       const int run = full[0] ? sA : tA + tB + sC;
@@ -743,6 +745,27 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
   // what earlier kernels of the stream wrote (the pattern, the operands) and overwrites what they read.
   pdl_wait_prior_grids();
 
+  // Class form: what the table of classes and the list's copy are made of is asked for together with the header they are cut by, not a
+  // round trip or two after it (lists hold garbage behind their last entry, which nobody looks at).  From the wait to the first tile,
+  // 4096 x 4096 under 64-wide tiles, a period of 4: 3700 - 4600 cycles before, 2500 - 3900 so.
+  constexpr int AHEAD = 4;
+  int ahead[AHEAD], ptrs[2][2];
+  if (is_class_mode(MODE)) {
+    const int lts = 31 - __clz(p.ts), Tr = p.K >> lts, Tc = p.N >> lts;
+    const int32_t* all = (MODE == M_TILEC_BWD_DATA) ? p.row_idx : p.col_idx;
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i) ahead[i] = threadIdx.x + i * blockDim.x < (unsigned)(Tr * Tc) ? all[threadIdx.x + i * blockDim.x] : 0;
+    if (warp == 0) {
+      const int32_t* ptr = (MODE == M_TILEC_BWD_DATA) ? p.row_ptr : p.col_ptr;
+      const int extent = (MODE == M_TILEC_BWD_DATA) ? Tr : Tc;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = lane + 32 * h;
+        ptrs[h][0] = c < extent ? ptr[c] : 0;
+        ptrs[h][1] = c < extent ? ptr[c + 1] : 0;
+      }
+    }
+  }
   Sched<BN, MODE, CTAS, SHARE> sch;
   sch.init(p, (int)rank, (FUSED && p.hdr_in != nullptr) ? p.hdr_in[HDR_NKEEP] : p.K, FUSED ? p.ext_mode : 0);
   if (is_class_mode(MODE) && !sch.dense) {
@@ -756,9 +779,13 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
     int* total_smem = reinterpret_cast<int*>(smem + L::MISC_OFF + 8);  // [3]: items, items of non-empty classes, light_q
     int32_t* slist = reinterpret_cast<int32_t*>(smem + L::STG_OFF);
     const bool fits = n_list * 4 <= CLASS_LIST_BYTES - 1024;
-    if (warp == 0) sch.build_class_table(p, tab, total_smem, lane);
-    if (fits)
-      for (int i = threadIdx.x; i < n_list; i += (int)blockDim.x) slist[i] = sch.list[i];
+    if (fits) {
+#pragma unroll
+      for (int i = 0; i < AHEAD; ++i)
+        if ((int)(threadIdx.x + i * blockDim.x) < n_list) slist[threadIdx.x + i * blockDim.x] = ahead[i];
+      for (int i = threadIdx.x + AHEAD * blockDim.x; i < n_list; i += (int)blockDim.x) slist[i] = sch.list[i];
+    }
+    if (warp == 0) sch.build_class_table(p, ptrs, tab, total_smem, lane);
     __syncthreads();
     sch.ctab = tab;
     sch.total = total_smem[0];
@@ -1079,6 +1106,25 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
       // An empty contraction leaves zeros: such a tile has no accumulator and no barrier traffic, these warps
       // just write it (the same way as any other tile, from zeros instead of the accumulator).
       const bool has_acc = (un.kb1 < 0 ? ti.nkb : un.kb1) > un.kb0;
+      if ((MODE == M_TILEC_FWD || MODE == M_TILEC_BWD_DATA) && !PLAIN && !has_acc) {
+        // Its columns come in groups of 64: eight lanes write a row's 128 bytes of one (or of half of one, in fp32).  As a tile of zeros
+        // on the ordinary way out a pair's tile took 7900 cycles, and with an even period (forward) most tiles are of this kind.
+        if (!p.accumulate) {
+          const int es = p.out_is_f32 ? 4 : 2;
+#pragma unroll 1
+          for (int j = 0; j < ti.bn / 64; ++j) {
+            const int oc = sel4(ti.ocol, j);
+            if (oc < 0) continue;  // padding
+            for (int r = (warp - 2) * (BM / EPI_WARPS) + (lane >> 3); r < (warp - 1) * (BM / EPI_WARPS); r += 4) {
+              if (ti.m0 + r >= sch.M_gemm) break;
+              uint4* o = reinterpret_cast<uint4*>(reinterpret_cast<char*>(p.out) + ((size_t)(ti.m0 + r) * p.ldo + oc) * es) + (lane & 7);
+              o[0] = make_uint4(0u, 0u, 0u, 0u);
+              if (p.out_is_f32) o[8] = make_uint4(0u, 0u, 0u, 0u);
+            }
+          }
+        }
+        continue;
+      }
       const int acc = nacc & 1;
       const uint32_t acc_phase = (uint32_t)(nacc >> 1) & 1u;
       if (has_acc) {
