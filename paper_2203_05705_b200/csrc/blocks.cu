@@ -32,16 +32,8 @@ template <> __device__ __forceinline__ float val_f<__nv_bfloat16>(__nv_bfloat16 
 // One warp per block (g, j); lane l takes the runs l, l + 32, ...: run d is chosen by word (d mod 4) of the
 // Philox block (d div 4) as run number floor(word * Cn / 2^32), runs numbered row-major inside the block.
 template <typename T>
-__global__ void __launch_bounds__(256) block_count_kernel(const T* A, int lda, int ts, int Q, int nblocks, int c,
-                                                          int n_runs, float threshold, unsigned long long seed,
-                                                          unsigned long long iteration, uint32_t stream_id,
-                                                          int32_t* counts) {
-  pdl_launch_dependents();
-  pdl_wait_prior_grids();
-  const int lane = threadIdx.x & 31;
-  const int blk = blockIdx.x * 8 + (threadIdx.x >> 5);
-  if (blk >= nblocks) return;
-  const int g = blk / Q, j = blk - g * Q;
+__device__ __forceinline__ int block_count(const T* A, int lda, int ts, int blk, int g, int j, int lane, int c, int n_runs, float threshold,
+                                           unsigned long long seed, unsigned long long iteration, uint32_t stream_id) {
   const T* base = A + (size_t)g * ts * lda + (size_t)j * ts;
   const unsigned int per_row = (unsigned int)(ts / c);
   const unsigned long long Cn = (unsigned long long)ts * per_row;
@@ -70,7 +62,38 @@ __global__ void __launch_bounds__(256) block_count_kernel(const T* A, int lda, i
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+  return count;
+}
+template <typename T>
+__global__ void __launch_bounds__(256) block_count_kernel(const T* A, int lda, int ts, int Q, int nblocks, int c,
+                                                          int n_runs, float threshold, unsigned long long seed,
+                                                          unsigned long long iteration, uint32_t stream_id,
+                                                          int32_t* counts) {
+  pdl_launch_dependents();
+  pdl_wait_prior_grids();
+  const int lane = threadIdx.x & 31;
+  const int blk = blockIdx.x * 8 + (threadIdx.x >> 5);
+  if (blk >= nblocks) return;
+  const int g = blk / Q, j = blk - g * Q;
+  const int count = block_count<T>(A, lda, ts, blk, g, j, lane, c, n_runs, threshold, seed, iteration, stream_id);
   if (lane == 0) counts[blk] = count;
+}
+// Counts and labels of a group by one CTA, a warp per block: groups of 4 to 32 blocks (see block_label_kernel for the rule).  With the
+// labels in a launch of their own the lists began 2 us later (4608 blocks in groups of 18).
+template <typename T>
+__global__ void __launch_bounds__(1024, 2) block_predict_kernel(const T* A, int lda, int ts, int Q, int c, int n_runs, float threshold,
+                                                             unsigned long long seed, unsigned long long iteration, uint32_t stream_id,
+                                                             int need, int cap, int32_t* counts, uint8_t* sens) {
+  __shared__ int s_count[32];
+  pdl_launch_dependents();
+  pdl_wait_prior_grids();
+  const int lane = threadIdx.x & 31, j = threadIdx.x >> 5, g = blockIdx.x, blk = g * Q + j;
+  const int count = block_count<T>(A, lda, ts, blk, g, j, lane, c, n_runs, threshold, seed, iteration, stream_id);
+  if (lane == 0) s_count[j] = counts[blk] = count;
+  __syncthreads();
+  const int other = lane < Q ? s_count[lane] : -1;
+  const int before = __popc(__ballot_sync(0xffffffffu, other > count || (other == count && lane < j)));
+  if (lane == 0) sens[blk] = (count >= need && before < cap) ? 1 : 0;
 }
 
 // Sec. 5.2.2: in its group a block is sensitive iff its count reaches `need` and fewer than `cap` blocks
@@ -165,6 +188,16 @@ __global__ void __launch_bounds__(LIST_THREADS) block_lists_kernel(uint8_t* keep
   __shared__ int s_warp[33];
   extern __shared__ int32_t s_dyn[];
   pdl_launch_dependents();
+  // the random words depend on nothing that an earlier kernel writes: the first of them are drawn while that one ends
+  constexpr int AHEAD = 6;
+  auto word = [&](int blk) {
+    uint32_t c[4] = {(uint32_t)iteration, (uint32_t)(iteration >> 32), (uint32_t)blk, (stream_id << 16) | 0xFFFFu};
+    philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
+    return c[0];
+  };
+  uint32_t ahead[AHEAD];
+#pragma unroll
+  for (int i = 0; i < AHEAD; ++i) ahead[i] = draw && (int)threadIdx.x + i * LIST_THREADS < G * Q ? word(threadIdx.x + i * LIST_THREADS) : 0u;
   pdl_wait_prior_grids();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = LIST_THREADS / 32;
   const int nblocks = G * Q;
@@ -173,13 +206,18 @@ __global__ void __launch_bounds__(LIST_THREADS) block_lists_kernel(uint8_t* keep
   uint8_t* s_keep = reinterpret_cast<uint8_t*>(s_dyn + (G + 1) + (Q + 1));
   const uint8_t* kp = in_smem ? s_keep : keep;
   if (draw) {
-    for (int blk = tid; blk < nblocks; blk += LIST_THREADS) {
-      uint32_t c[4] = {(uint32_t)iteration, (uint32_t)(iteration >> 32), (uint32_t)blk, (stream_id << 16) | 0xFFFFu};
-      philox4x32_10(c, (uint32_t)seed, (uint32_t)(seed >> 32));
-      const uint8_t k = (c[0] < (sens[blk] ? P_sens : P_insens)) ? 0 : 1;
+    auto put = [&](int blk, uint32_t w, uint8_t label) {
+      const uint8_t k = (w < (label ? P_sens : P_insens)) ? 0 : 1;
       keep[blk] = k;
       if (in_smem) s_keep[blk] = k;
-    }
+    };
+    uint8_t label[AHEAD];
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i) label[i] = tid + i * LIST_THREADS < nblocks ? sens[tid + i * LIST_THREADS] : 0;
+#pragma unroll
+    for (int i = 0; i < AHEAD; ++i)
+      if (tid + i * LIST_THREADS < nblocks) put(tid + i * LIST_THREADS, ahead[i], label[i]);
+    for (int blk = tid + AHEAD * LIST_THREADS; blk < nblocks; blk += LIST_THREADS) put(blk, word(blk), sens[blk]);
     __syncthreads();
   } else if (in_smem) {
     for (int blk = tid; blk < nblocks; blk += LIST_THREADS) s_keep[blk] = keep[blk];
@@ -356,6 +394,17 @@ ard_status ard_blocks_predict(ard_ctx* ctx, ard_blocks* b, ard_dtype dtype, cons
   DevGuard guard(ctx->device);
   cudaStream_t s = (cudaStream_t)cuda_stream;
   const int nblocks = b->G * b->Q;
+  if (b->Q >= 4 && b->Q <= 32) {
+    auto launch = [&](auto kern, auto* a) {
+      return ard_launch(ctx, kern, dim3(b->G), dim3(32 * b->Q), 0, s, a, lda, b->ts, b->Q, c, n_runs, threshold, (unsigned long long)seed,
+                        (unsigned long long)iteration, stream_id, need, cap, b->d_count, b->d_sens);
+    };
+    ARD_CUDA_OK(dtype == ARD_F32 ? launch(block_predict_kernel<float>, (const float*)A)
+                                 : launch(block_predict_kernel<__nv_bfloat16>, (const __nv_bfloat16*)A));
+    ctx->launches++;
+    ARD_CUDA_OK(cudaGetLastError());
+    return ARD_OK;
+  }
   if (dtype == ARD_F32)
     ARD_CUDA_OK(ard_launch(ctx, block_count_kernel<float>, dim3((nblocks + 7) / 8), dim3(256), 0, s, (const float*)A, lda,
                            b->ts, b->Q, nblocks, c, n_runs, threshold, (unsigned long long)seed,
