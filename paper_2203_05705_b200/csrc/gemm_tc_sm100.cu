@@ -313,12 +313,19 @@ struct Sched {
           constexpr bool FLEX = CTAS == 2 && MODE == M_ROW_FWD;  // single CTAs: small, latency-bound problems
           const int kt = (Kc + BK - 1) / BK;
           int best_cost = 0x7fffffff;
+          // every thread works this out between the header and the first load: divisions by constants (unrolled), and by the workers through
+          // one reciprocal (sampler and three products, 1024 x 1024 x 1024, a period of 2: 43.1 -> 42.7 us; the unrolled form costs the kernels that
+          // share tiles registers)
+          const float per_worker = 1.f / (float)workers;
+#pragma unroll (SK_MODE ? 1 : 8)
           for (int cand = BN; cand >= 64 * CTAS; cand = FLEX ? cand - 32 : cand >> 1) {
             const int tiles = Mt * ((N_gemm + cand - 1) / cand);
             const int wpair = cand == 256 ? 100 : (cand == 224 ? 92 : (cand == 192 ? 83 : (cand == 160 ? 78 : 76)));
             const int wone = cand == 256 ? 100 : (cand == 128 ? 70 : 55);
             const int w16 = 16 * (FLEX ? wpair : wone);
-            const int full = tiles / workers, rem = tiles % workers;
+            int full = (int)((float)tiles * per_worker), rem = tiles - full * workers;
+            while (rem < 0) { rem += workers; --full; }
+            while (rem >= workers) { rem -= workers; ++full; }
             const int S = (SK_MODE && p.sk_ws != nullptr && kt > 0)
                               ? sharing_workers(full, rem, kt, workers, p.sk_min_blocks, p.sk_min_gain, p.sk_any) : 0;
             int cost = full * w16;
@@ -1163,9 +1170,10 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
       }
 
       constexpr bool ZERO_ROWS = MODE == M_ROW_BWD_WEIGHT || MODE == M_LSTM_BWD_WEIGHT;
-      constexpr int LINES_AT_ONCE = ZERO_ROWS ? 2 : 8;  // what fits the registers
-      // the class form keeps its list in the staging area, the row lists' weight gradient its row addresses
-      constexpr bool F32_LINES = !(is_class_mode(MODE) && !PLAIN) && !is_rows_mode(MODE);
+      constexpr int LINES_AT_ONCE = ZERO_ROWS && !SHARE ? 2 : 8;  // what fits the registers
+      // the class form keeps its list in the staging area, the row lists' weight gradient its row addresses; the kernels that share tiles
+      // have no registers for it (weight gradient over 17700 kept rows, 512 x 2304: 69.8 -> 72.1 us)
+      constexpr bool F32_LINES = !(is_class_mode(MODE) && !PLAIN) && !is_rows_mode(MODE) && !SHARE;
       // Zeros of the dropped neurons' rows beside this warp's row rr (output row `own`): 16 bytes of each from column n on, so that the
       // eight lanes of a row write whole lines.  Compact row m owns output rows [m * dp, (m + 1) * dp), the last one also the tail.
       // With a row to a thread these stores were most of a sparse product's time (2048 x 512 -> 4096, a period of 16, sampler and three
@@ -1449,7 +1457,8 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
         // kept it at 6.4 us per 256 x 256 tile where the products and loads need 4.1.
         constexpr bool PAIR_MODES = MODE == M_ROW_FWD || MODE == M_ROW_BWD_DATA || MODE == M_ROW_BWD_WEIGHT ||
                                     (is_class_mode(MODE) && PLAIN);
-        const bool pair_ok = PAIR_MODES && !p.out_is_f32 && !p.accumulate && !(MODE == M_ROW_FWD && p.scatter && dp > 1);
+        const bool pair_ok = PAIR_MODES && !p.out_is_f32 && !p.accumulate && !(MODE == M_ROW_FWD && p.scatter && dp > 1) &&
+                             !(SHARE && MODE == M_ROW_BWD_WEIGHT && p.zero_fill);
         const unsigned okmask = __ballot_sync(0xffffffffu, row_ok);
         // The class tiling keeps its list in the first part of the staging area: its warps stage one chunk
         // (32 rows x 17 words) behind it and write 64-byte row segments, four lanes per row.
@@ -1501,7 +1510,7 @@ ard_gemm_tc_kernel(const __grid_constant__ TcParamsT<nmaps(MODE)> p) {
             const uint4 w = make_uint4(q[0], q[1], q[2], q[3]);
             if ((okmask >> rr) & 1u) {
               *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(p.out) + (size_t)orow * p.ldo + n + piece * 8) = w;
-              if (ZERO_ROWS && p.zero_fill && dp > 1) zero_beside(rr, orow, n + piece * 8);
+              if (ZERO_ROWS && !SHARE && p.zero_fill && dp > 1) zero_beside(rr, orow, n + piece * 8);
             }
           }
           __syncwarp();
