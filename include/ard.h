@@ -32,8 +32,8 @@
  *   - Arithmetic: ARD_F32 operands are multiplied and accumulated in fp32 on the CUDA cores, or, in products of
  *     more than 1.5e8 kept operations under ARD_PATH_AUTO, split into three bf16 parts each and multiplied on the
  *     tensor cores with fp32 accumulation (an error no larger than the CUDA cores' against fp64; elements below
- *     2^-109 lose what a bf16 subnormal cannot hold, 2^-134 in absolute terms; results that are infinite or NaN are
- *     those of the CUDA cores).  ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
+ *     2^-109 lose what a bf16 subnormal cannot hold, 2^-134 in absolute terms; sums that would be infinite or NaN are taken
+ *     with fp32 multiply-adds instead).  ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
  *   - There is no CPU fallback.
  */
 #ifndef ARD_H_

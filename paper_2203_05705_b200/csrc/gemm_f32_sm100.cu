@@ -15,7 +15,9 @@
 // and 98 KB of operand reads, about 1730 cycles at 128 bytes a cycle, next to 768 tensor-core cycles.
 //
 // Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l.  Blocks in which that happens are noticed by the
-// loading warps, and the tile (its share of the contraction) is multiplied again on the CUDA cores.
+// loading warps, and the tile (its share of the contraction) is multiplied again on the CUDA cores.  Finite operands can leave an
+// infinity or a NaN too where a product is near the largest fp32 number or beyond it: h h' may round past it, and h m' and m h' of
+// an infinite product may have the other sign.  A row of sums that are not all finite is therefore multiplied again as well.
 #include "staged_product.h"
 
 #include <type_traits>
@@ -474,7 +476,10 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
           if (lane == 0) mbar_arrive(free_bar(i));
         }
         float* row = T + (quad * 32 + lane) * F3_PITCH;
-        if (again) {
+        uint64_t bad = 0ull;  // NaN once a sum is not finite
+#pragma unroll
+        for (int i = 0; i < F3_BN / 2; ++i) bad = fma2(acc[i], 0ull, bad);
+        if (again || bad != 0ull) {
           multiply_again(o, s, ti, quad * 32 + lane, kb0 * F3_BK, min(kb1 * F3_BK, ti.kext), row);
         } else {
 #pragma unroll

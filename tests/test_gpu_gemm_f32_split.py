@@ -82,3 +82,41 @@ def test_not_finite(value, kind, ts, dp):
                 assert (cc[fin].double() - tc[fin].double()).norm() <= 2e-6 * cc[fin].double().norm()
     finally:
         ctx.close()
+
+
+def _both_paths(ctx, pat, B, K, N, X, W, dY, relu=False):
+    outs = []
+    for path in (ard.ARD_PATH_CUDA_CORE, ard.ARD_PATH_AUTO):
+        ard.ard_set_path(ctx.h, path)
+        Y, dX, dW = (torch.full(s, 7.0, device="cuda") for s in ((B, N), (B, K), (N, K)))
+        if relu:
+            ard.ard_layer_fwd(ctx.h, pat, None, ard.ARD_F32, B, K, N, 1.0, X, K, W, K, None, Y, N,
+                              ard.ARD_OUT_SCATTER_ZEROFILL | ard.ARD_FLAG_RELU)
+        else:
+            ard.ard_fwd(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, X, K, W, K, Y, N, ard.ARD_OUT_SCATTER_ZEROFILL)
+        ard.ard_bwd_data(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, dY, N, 0, W, K, dX, K)
+        ard.ard_bwd_weight(ctx.h, pat, ard.ARD_F32, ard.ARD_F32, B, K, N, 1.0, X, K, dY, N, 0, dW, K, 1)
+        outs.append([Y, dX, dW])
+    return list(zip(*outs))
+
+
+@pytest.mark.parametrize("x,w", [(1e30, 1e30), (-1e25, 3e20), (3e20, -1e25), (2.0 ** 64 * (1 - 2 ** -10), 2.0 ** 64 * (1 - 2 ** -10)),
+                                 (2.0 ** 70 * (1 - 2 ** -10), 2.0 ** 70 * (1 - 2 ** -10)), (2.0 ** 63 * (2 - 2 ** -9), 2.0 ** 64 * (1 - 2 ** -20))])
+@pytest.mark.parametrize("kind,ts,dp,relu", [(ard.ARD_ROW, 0, 1, False), (ard.ARD_ROW, 0, 2, True), (ard.ARD_TILE, 64, 3, False)])
+def test_products_near_and_beyond_the_largest_number(x, w, kind, ts, dp, relu):
+    """Finite operands whose product overflows, or only just does not: as the CUDA-core kernel has it."""
+    B, K, N = 200, 1536, 1088
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(kind, K, N, ts)
+        ard.ard_pattern_set(ctx.h, pat, dp, 1)
+        g = torch.Generator(device="cuda").manual_seed(1)
+        X, W, dY = (torch.randn(s, device="cuda", generator=g) * 0.1 for s in ((B, K), (N, K), (B, N)))
+        X[130, 700], dY[130, 66], W[66, 700] = x, x, w  # kept under every pattern here
+        for cc, tc in _both_paths(ctx, pat, B, K, N, X, W, dY, relu):
+            fin = cc.isfinite()
+            assert not tc.isnan().any() and torch.equal(fin, tc.isfinite()) and torch.equal(cc[~fin], tc[~fin])
+            assert (cc[fin].double() - tc[fin].double()).norm() <= 2e-6 * cc[fin].double().norm()
+        assert ard.ard_last_device_status(ctx.h) == 0
+    finally:
+        ctx.close()
