@@ -17,7 +17,7 @@
 // Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l.  Blocks in which that happens are noticed by the
 // loading warps, and the tile (its share of the contraction) is multiplied again on the CUDA cores.  Finite operands can leave an
 // infinity or a NaN too where a product is near the largest fp32 number or beyond it: h h' may round past it, and h m' and m h' of
-// an infinite product may have the other sign.  A row of sums that are not all finite is therefore multiplied again as well.
+// an infinite product may have the other sign.  A tile whose sums are not all finite is therefore multiplied again as well.
 #include "staged_product.h"
 
 #include <type_traits>
@@ -159,17 +159,89 @@ struct Operands {
   }
 };
 
-// Row r of the tile's sums over contraction indices [k0, k1) on the CUDA cores, for operands that are not finite.
+// True in all threads of the warps that add up if it is in any.
+__device__ __forceinline__ bool any_drain(bool x) {
+  uint32_t r;
+  asm volatile("{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbarrier.cta.red.or.pred q, 1, 128, p;\n\tselp.u32 %0, 1, 0, q;\n\t}"
+               : "=r"(r) : "r"((uint32_t)x) : "memory");
+  return r != 0;
+}
+__device__ __forceinline__ void sync_drain() { asm volatile("barrier.cta.sync 1, 128;" ::: "memory"); }
+
+// The tile's sums over contraction indices [k0, k1) on the CUDA cores, for operands or sums that are not finite, into T: thread t of
+// the 128 that add up owns 8 x 8 of them, and blocks of 32 indices of both operands pass through T itself.  A training run that has
+// diverged puts every tile through this (NaN in a column of each operand, 256 x 2048 x 2048, forward: 208 us; the CUDA-core kernel
+// takes 74; a thread for a row's 64 sums, one after the other, took 4500).
 template <int KIND, int OP>
-__device__ __noinline__ void multiply_again(const Operands<KIND, OP>& o, const ProductPlan& s, const ProductTile& ti, int r, int k0, int k1,
+__device__ __noinline__ void multiply_again(const Operands<KIND, OP>& o_, const ProductPlan& s_, const ProductTile& ti_, int t, int k0, int k1,
                                             float* T) {
-  const int nb = min(F3_BN, o.b_lim(s, ti));
-  for (int j = 0; j < F3_BN; ++j) {
-    float acc = 0.f;
-    if (j < nb && r < o.a_lim(s, ti))
-      for (int k = k0; k < k1; ++k) acc = fmaf(*o.a(s, ti, r, k), *o.b(s, ti, j, k), acc);
-    T[j] = acc;
+  using O = Operands<KIND, OP>;
+  const O o = o_;
+  const ProductPlan s = s_;
+  const ProductTile ti = ti_;
+  constexpr int KT = 32, PA = UMMA_BM + 4, PB = F3_BN + 4;
+  static_assert(KT * (PA + PB) <= UMMA_BM * F3_PITCH, "both blocks fit the tile's place");
+  float *bA = T, *bB = T + KT * PA;
+  const int na = min(UMMA_BM, o.a_lim(s, ti)), nb = min(F3_BN, o.b_lim(s, ti));
+  const int r0 = t >> 3 << 3, c0 = (t & 7) << 3;
+  uint64_t acc[8][4];
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
+  for (int kk = k0; kk < k1; kk += KT) {
+    sync_drain();  // nobody reads the block before this one any more
+    // sixteen elements on their way at a time
+#pragma unroll 1
+    for (int i0 = 0; i0 < KT * UMMA_BM / 128; i0 += 16) {
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int e = (i0 + i) * 128 + t, r = O::A_MN ? e & (UMMA_BM - 1) : e / KT, k = O::A_MN ? e / UMMA_BM : e & (KT - 1);
+        v[i] = r < na && kk + k < k1 ? ld1(o.a(s, ti, r, kk + k)) : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int e = (i0 + i) * 128 + t;
+        bA[O::A_MN ? e / UMMA_BM * PA + (e & (UMMA_BM - 1)) : (e & (KT - 1)) * PA + e / KT] = v[i];
+      }
+    }
+    {
+      static_assert(KT * F3_BN == 16 * 128, "one batch");
+      float v[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int e = i * 128 + t, r = O::B_MN ? e & (F3_BN - 1) : e / KT, k = O::B_MN ? e / F3_BN : e & (KT - 1);
+        v[i] = r < nb && kk + k < k1 ? ld1(o.b(s, ti, r, kk + k)) : 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < 16; ++i) {
+        const int e = i * 128 + t;
+        bB[O::B_MN ? e / F3_BN * PB + (e & (F3_BN - 1)) : (e & (KT - 1)) * PB + e / KT] = v[i];
+      }
+    }
+    sync_drain();
+#pragma unroll 2
+    for (int k = 0; k < KT; ++k) {
+      const float4 x = *reinterpret_cast<const float4*>(bA + k * PA + r0), y = *reinterpret_cast<const float4*>(bA + k * PA + r0 + 4);
+      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(bB + k * PB + c0), v = *reinterpret_cast<const ulonglong2*>(bB + k * PB + c0 + 4);
+      const float a[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const uint64_t aa = pair(a[i], a[i]);
+        acc[i][0] = fma2(aa, u.x, acc[i][0]);
+        acc[i][1] = fma2(aa, u.y, acc[i][1]);
+        acc[i][2] = fma2(aa, v.x, acc[i][2]);
+        acc[i][3] = fma2(aa, v.y, acc[i][3]);
+      }
+    }
   }
+  sync_drain();
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+#pragma unroll
+    for (int j = 0; j < 2; ++j)
+      *reinterpret_cast<ulonglong2*>(T + (r0 + i) * F3_PITCH + c0 + 4 * j) = make_ulonglong2(acc[i][2 * j], acc[i][2 * j + 1]);
 }
 
 template <int KIND, int OP>
@@ -479,13 +551,13 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
         uint64_t bad = 0ull;  // NaN once a sum is not finite
 #pragma unroll
         for (int i = 0; i < F3_BN / 2; ++i) bad = fma2(acc[i], 0ull, bad);
-        if (again || bad != 0ull) {
-          multiply_again(o, s, ti, quad * 32 + lane, kb0 * F3_BK, min(kb1 * F3_BK, ti.kext), row);
+        if (any_drain(again || bad != 0ull)) {
+          multiply_again(o, s, ti, tid - 32 * F3_DRAIN_WARP, kb0 * F3_BK, min(kb1 * F3_BK, ti.kext), T);
         } else {
 #pragma unroll
           for (int i = 0; i < F3_BN / 4; ++i) *reinterpret_cast<ulonglong2*>(row + 4 * i) = make_ulonglong2(acc[2 * i], acc[2 * i + 1]);
         }
-        if (s.S == 1) asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (s.S == 1) sync_drain();
       }
       it += kb1 - kb0;
       __syncwarp();
@@ -494,7 +566,7 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
         cluster_sync_all();
       } else if (drain && ti.nkb >= 0) {
         write_tile<KIND, OP, UMMA_BM, F3_BN, F3_PITCH, F3_DRAINS, true, float>(g, s, ti, T, base + F3_TILE_OFF, rows, lead, dw, lane);
-        asm volatile("bar.sync 1, 128;" ::: "memory");  // the tile has been read
+        sync_drain();  // the tile has been read
         __syncwarp();
       }
     }

@@ -120,3 +120,44 @@ def test_products_near_and_beyond_the_largest_number(x, w, kind, ts, dp, relu):
         assert ard.ard_last_device_status(ctx.h) == 0
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("B,K,N,kind,ts,dp", [(131, 1547, 1091, ard.ARD_ROW, 0, 1), (131, 1547, 1091, ard.ARD_ROW, 0, 2),
+                                              (1029, 67, 1201, ard.ARD_ROW, 0, 1), (133, 1080, 1212, ard.ARD_TILE, 12, 1),
+                                              (4101, 480, 312, ard.ARD_TILE, 12, 5)])
+def test_not_finite_at_the_edges(B, K, N, kind, ts, dp):
+    """Infinities in the last row, column and index of ragged tiles: what the repeated products read and write."""
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(kind, K, N, ts)
+        ard.ard_pattern_set(ctx.h, pat, dp, 1)
+        X, W, dY = (torch.randn(s, device="cuda") * 0.1 for s in ((B, K), (N, K), (B, N)))
+        last = (N - 1) // dp * dp if kind == ard.ARD_ROW else N - 1  # kept neuron
+        X[-1, -1] = X[0, 0] = float("inf")
+        W[last, -1], dY[-1, last], dY[0, 0] = float("-inf"), float("inf"), float("nan")
+        for cc, tc in _both_paths(ctx, pat, B, K, N, X, W, dY):
+            fin = cc.isfinite()
+            assert torch.equal(fin, tc.isfinite()) and torch.equal(cc.isnan(), tc.isnan()) and torch.equal(cc[cc.isinf()], tc[tc.isinf()])
+            assert (cc[fin].double() - tc[fin].double()).norm() <= 2e-6 * cc[fin].double().norm()
+        assert ard.ard_last_device_status(ctx.h) == 0
+    finally:
+        ctx.close()
+
+
+def test_not_finite_in_a_long_contraction():
+    """A weight gradient over a million rows, its contraction not cut: the repeat ends well before the kernel's waits give up."""
+    B, K, N = 1 << 20, 1216, 512
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        ard.ard_pattern_set(ctx.h, pat, 1, 1)
+        X, dY = torch.full((B, K), 0.5, device="cuda"), torch.full((B, N), 0.25, device="cuda")
+        X[B // 2, 1] = dY[7, 2] = float("nan")
+        dW = torch.zeros((N, K), device="cuda")
+        ard.ard_bwd_weight(ctx.h, pat, ard.ARD_F32, ard.ARD_F32, B, K, N, 1.0, X, K, dY, N, 0, dW, K, 1)
+        assert ard.ard_last_device_status(ctx.h) == 0
+        want = torch.full((N, K), 0.125 * B, device="cuda")  # exact in fp32
+        want[:, 1] = want[2, :] = float("nan")
+        assert torch.equal(want.isnan(), dW.isnan()) and torch.equal(want.nan_to_num(), dW.nan_to_num())
+    finally:
+        ctx.close()
