@@ -31,9 +31,8 @@
  *     of that call is unspecified.  Nothing aborts or traps.
  *   - Arithmetic: ARD_F32 operands are multiplied and accumulated in fp32 on the CUDA cores, or, in products of
  *     more than 1.5e8 kept operations under ARD_PATH_AUTO, split into three bf16 parts each and multiplied on the
- *     tensor cores with fp32 accumulation (an error no larger than the CUDA cores' against fp64; elements below
- *     2^-109 lose what a bf16 subnormal cannot hold, 2^-134 in absolute terms; sums that would be infinite or NaN are taken
- *     with fp32 multiply-adds instead).  ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
+ *     tensor cores with fp32 accumulation (an error no larger than the CUDA cores' against fp64; where elements
+ *     reach 2^111, sums 2^96, or either is not finite, with fp32 multiply-adds instead).  ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
  *   - There is no CPU fallback.
  */
 #ifndef ARD_H_

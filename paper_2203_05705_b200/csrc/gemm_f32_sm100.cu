@@ -14,10 +14,14 @@
 // Bound: shared memory.  A block (128 + 64 rows, 64 contraction indices) takes 48 KB through L1, 72 KB of stores of the planes
 // and 98 KB of operand reads, about 1730 cycles at 128 bytes a cycle, next to 768 tensor-core cycles.
 //
-// Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l.  Blocks in which that happens are noticed by the
-// loading warps, and the tile (its share of the contraction) is multiplied again on the CUDA cores.  Finite operands can leave an
-// infinity or a NaN too where a product is near the largest fp32 number or beyond it: h h' may round past it, and h m' and m h' of
-// an infinite product may have the other sign.  A tile whose sums are not all finite is therefore multiplied again as well.
+// Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l, and so in every sum they are part of.  Finite operands can
+// leave an infinity or a NaN too where a product is near the largest fp32 number or beyond it: h h' may round past it, and h m'
+// and m h' of an infinite product may have the other sign.  A tile whose sums are not all finite (its share of the contraction) is
+// multiplied again on the CUDA cores.
+//
+// m and l of a small element would fall below the smallest bf16 (2^-133) and leave it with fewer bits: 2^-115 had an error of 1e-6,
+// 2^-126 of 2e-3.  Operands are therefore taken times 2^16, which puts the last bit of the smallest fp32 number there, and the
+// sums times 2^-32.  Elements from 2^111 on and sums from 2^96 on are not finite then, and are multiplied again.
 #include "staged_product.h"
 
 #include <type_traits>
@@ -32,11 +36,13 @@ constexpr int F3_A_PLANE = UMMA_BM * F3_BK * 2, F3_B_PLANE = F3_BN * F3_BK * 2;
 constexpr int F3_STAGE = 3 * (F3_A_PLANE + F3_B_PLANE);
 constexpr int F3_PITCH = F3_BN + 4;
 constexpr int F3_TILE_OFF = 2 * F3_STAGE;
-constexpr int F3_BAR_OFF = F3_TILE_OFF + UMMA_BM * F3_PITCH * 4;
+constexpr int AGAIN_K = 32, AGAIN_N = 32, AGAIN_PA = UMMA_BM + 4, AGAIN_PB = AGAIN_N + 4;  // multiply_again
+constexpr int F3_AGAIN_OFF = F3_TILE_OFF + UMMA_BM * F3_PITCH * 4;
+constexpr int F3_BAR_OFF = F3_AGAIN_OFF + AGAIN_K * (AGAIN_PA + AGAIN_PB) * 4;
 constexpr int F3_SMEM = F3_BAR_OFF + 128 + 1024;
 constexpr int F3_TMEM = 512;           // two blocks' accumulators of 3 * F3_BN columns each, rounded up to a power of two
 constexpr double F3_LEAST_FLOPS = 1.5e8;  // kept operations, see f32_takes
-constexpr int F3_RING = 8;             // blocks between a loader and the warps that add up: at most four
+constexpr float F3_UP = 65536.f, F3_DOWN = 1.f / (F3_UP * F3_UP);
 
 struct F32Params {
   GemmArgs g;
@@ -88,6 +94,11 @@ __device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
   asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
 __device__ __forceinline__ uint32_t round2(uint64_t x) {
   float a, b;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
@@ -101,11 +112,11 @@ __device__ __forceinline__ uint32_t take_bf16(uint64_t& x) {
   x = fma2(pair(__uint_as_float(h << 16), __uint_as_float(h & 0xffff0000u)), pair(-1.f, -1.f), x);
   return h;
 }
-__device__ __forceinline__ void split2(uint64_t x, uint32_t& h, uint32_t& m, uint32_t& l, uint64_t& bad) {
+__device__ __forceinline__ void split2(uint64_t x, uint32_t& h, uint32_t& m, uint32_t& l) {
+  x = mul2(x, pair(F3_UP, F3_UP));
   h = take_bf16(x);
   m = take_bf16(x);
   l = round2(x);
-  bad = fma2(x, 0ull, bad);  // zero, and NaN from here on if a part was not finite
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
   asm volatile(
@@ -121,15 +132,16 @@ template <int KIND, int OP>
 struct Operands {
   static constexpr bool A_MN = OP == OP_BWD_WEIGHT, B_MN = OP != OP_FWD;
   const float *PA, *PB;
-  size_t lda, ldb, step_a;  // step_a: columns of a full-width dY from one kept neuron to the next
+  size_t ldb;
+  int lda, step_a;          // step_a: columns of a full-width dY from one kept neuron to the next
   bool vec_a, vec_b;        // pieces of four contiguous elements are whole and on the 16-byte grid, or do not exist
 
   __device__ __forceinline__ Operands(const GemmArgs& g, const ProductPlan& s, int vec) {
     PA = reinterpret_cast<const float*>(g.A0);
     PB = reinterpret_cast<const float*>(g.A1);
     const bool strided_a = KIND == 0 && OP != OP_FWD && !g.flag0;
-    lda = (size_t)g.lda0;
-    step_a = strided_a ? (size_t)s.dp : 1;
+    lda = g.lda0;
+    step_a = strided_a ? s.dp : 1;
     if (strided_a) PA += s.bb;
     // kept neurons are rows bb + i * dp of the weight (unless packed for a feeding pattern)
     const bool strided_b = KIND == 0 && OP != OP_BWD_WEIGHT && g.hdr_in == nullptr;
@@ -168,80 +180,63 @@ __device__ __forceinline__ bool any_drain(bool x) {
 }
 __device__ __forceinline__ void sync_drain() { asm volatile("barrier.cta.sync 1, 128;" ::: "memory"); }
 
-// The tile's sums over contraction indices [k0, k1) on the CUDA cores, for operands or sums that are not finite, into T: thread t of
-// the 128 that add up owns 8 x 8 of them, and blocks of 32 indices of both operands pass through T itself.  A training run that has
-// diverged puts every tile through this (NaN in a column of each operand, 256 x 2048 x 2048, forward: 208 us; the CUDA-core kernel
-// takes 74; a thread for a row's 64 sums, one after the other, took 4500).
+// The tile's sums over contraction indices [k0, k1) on the CUDA cores, for operands or sums that are not finite, into T, by the 128
+// threads that add up (t: which of them): 32 columns at a time, 8 x 4 sums a thread, blocks of 32 indices of both operands through
+// shared memory of its own at S.  Not more sums at a time: the registers of a function count for every warp of the kernel that calls
+// it (64 a thread cost 128 x 2048 x 2048 1 us a product).  A training run that has diverged puts every tile through this (NaN in a
+// column of each operand, 256 x 2048 x 2048, forward: 370 us; the CUDA-core kernel takes 76; a thread for a row's 64 sums, one
+// after the other, took 4500).
 template <int KIND, int OP>
-__device__ __noinline__ void multiply_again(const Operands<KIND, OP>& o_, const ProductPlan& s_, const ProductTile& ti_, int t, int k0, int k1,
-                                            float* T) {
+__device__ __noinline__ void multiply_again(const Operands<KIND, OP>& o, const ProductPlan& s, const ProductTile& ti, int t, int k0, int k1,
+                                            float* T, float* S) {
   using O = Operands<KIND, OP>;
-  const O o = o_;
-  const ProductPlan s = s_;
-  const ProductTile ti = ti_;
-  constexpr int KT = 32, PA = UMMA_BM + 4, PB = F3_BN + 4;
-  static_assert(KT * (PA + PB) <= UMMA_BM * F3_PITCH, "both blocks fit the tile's place");
-  float *bA = T, *bB = T + KT * PA;
-  const int na = min(UMMA_BM, o.a_lim(s, ti)), nb = min(F3_BN, o.b_lim(s, ti));
-  const int r0 = t >> 3 << 3, c0 = (t & 7) << 3;
-  uint64_t acc[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
-  for (int kk = k0; kk < k1; kk += KT) {
-    sync_drain();  // nobody reads the block before this one any more
-    // sixteen elements on their way at a time
+  float* bB = S + AGAIN_K * AGAIN_PA;
+  const int na = o.a_lim(s, ti), nb = o.b_lim(s, ti), r0 = t >> 3 << 3, c0 = (t & 7) << 2;
 #pragma unroll 1
-    for (int i0 = 0; i0 < KT * UMMA_BM / 128; i0 += 16) {
-      float v[16];
+  for (int n0 = 0; n0 < F3_BN; n0 += AGAIN_N) {
+    uint64_t acc[8][2] = {};
+#pragma unroll 1
+    for (int kk = k0; kk < k1; kk += AGAIN_K) {
+      sync_drain();  // nobody reads the block before this one any more
+      // eight elements on their way at a time: first those of A, then those of B
+#pragma unroll 1
+      for (int i0 = 0; i0 < AGAIN_K * (UMMA_BM + AGAIN_N) / 128; i0 += 8) {
+        const bool is_a = i0 < AGAIN_K * UMMA_BM / 128;
+        float v[8];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int e = (i0 + i) * 128 + t, r = O::A_MN ? e & (UMMA_BM - 1) : e / KT, k = O::A_MN ? e / UMMA_BM : e & (KT - 1);
-        v[i] = r < na && kk + k < k1 ? ld1(o.a(s, ti, r, kk + k)) : 0.f;
-      }
+        for (int i = 0; i < 8; ++i) {
+          const int e = (i0 + i) * 128 + t;
+          if (is_a) {
+            const int r = O::A_MN ? e & (UMMA_BM - 1) : e / AGAIN_K, k = kk + (O::A_MN ? e / UMMA_BM : e & (AGAIN_K - 1));
+            v[i] = r < na && k < k1 ? ld1(o.a(s, ti, r, k)) : 0.f;
+          } else {
+            const int f = e - AGAIN_K * UMMA_BM, r = n0 + (O::B_MN ? f & (AGAIN_N - 1) : f / AGAIN_K), k = kk + (O::B_MN ? f / AGAIN_N : f & (AGAIN_K - 1));
+            v[i] = r < nb && k < k1 ? ld1(o.b(s, ti, r, k)) : 0.f;
+          }
+        }
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int e = (i0 + i) * 128 + t;
-        bA[O::A_MN ? e / UMMA_BM * PA + (e & (UMMA_BM - 1)) : (e & (KT - 1)) * PA + e / KT] = v[i];
+        for (int i = 0; i < 8; ++i) {
+          const int e = (i0 + i) * 128 + t, f = e - AGAIN_K * UMMA_BM;
+          if (is_a) S[O::A_MN ? e / UMMA_BM * AGAIN_PA + (e & (UMMA_BM - 1)) : (e & (AGAIN_K - 1)) * AGAIN_PA + e / AGAIN_K] = v[i];
+          else bB[O::B_MN ? f / AGAIN_N * AGAIN_PB + (f & (AGAIN_N - 1)) : (f & (AGAIN_K - 1)) * AGAIN_PB + f / AGAIN_K] = v[i];
+        }
       }
-    }
-    {
-      static_assert(KT * F3_BN == 16 * 128, "one batch");
-      float v[16];
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int e = i * 128 + t, r = O::B_MN ? e & (F3_BN - 1) : e / KT, k = O::B_MN ? e / F3_BN : e & (KT - 1);
-        v[i] = r < nb && kk + k < k1 ? ld1(o.b(s, ti, r, kk + k)) : 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 16; ++i) {
-        const int e = i * 128 + t;
-        bB[O::B_MN ? e / F3_BN * PB + (e & (F3_BN - 1)) : (e & (KT - 1)) * PB + e / KT] = v[i];
-      }
-    }
-    sync_drain();
+      sync_drain();
 #pragma unroll 2
-    for (int k = 0; k < KT; ++k) {
-      const float4 x = *reinterpret_cast<const float4*>(bA + k * PA + r0), y = *reinterpret_cast<const float4*>(bA + k * PA + r0 + 4);
-      const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(bB + k * PB + c0), v = *reinterpret_cast<const ulonglong2*>(bB + k * PB + c0 + 4);
-      const float a[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+      for (int k = 0; k < AGAIN_K; ++k) {
+        const float4 x = *reinterpret_cast<const float4*>(S + k * AGAIN_PA + r0), y = *reinterpret_cast<const float4*>(S + k * AGAIN_PA + r0 + 4);
+        const ulonglong2 w = *reinterpret_cast<const ulonglong2*>(bB + k * AGAIN_PB + c0);
+        const float a[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const uint64_t aa = pair(a[i], a[i]);
-        acc[i][0] = fma2(aa, u.x, acc[i][0]);
-        acc[i][1] = fma2(aa, u.y, acc[i][1]);
-        acc[i][2] = fma2(aa, v.x, acc[i][2]);
-        acc[i][3] = fma2(aa, v.y, acc[i][3]);
+        for (int i = 0; i < 8; ++i) {
+          acc[i][0] = fma2(pair(a[i], a[i]), w.x, acc[i][0]);
+          acc[i][1] = fma2(pair(a[i], a[i]), w.y, acc[i][1]);
+        }
       }
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) *reinterpret_cast<ulonglong2*>(T + (r0 + i) * F3_PITCH + n0 + c0) = make_ulonglong2(acc[i][0], acc[i][1]);
   }
-  sync_drain();
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 2; ++j)
-      *reinterpret_cast<ulonglong2*>(T + (r0 + i) * F3_PITCH + c0 + 4 * j) = make_ulonglong2(acc[i][2 * j], acc[i][2 * j + 1]);
 }
 
 template <int KIND, int OP>
@@ -263,7 +258,6 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
   auto free_bar = [&](int i) { return bars + 8u * (8 + i); };
   volatile uint32_t* tmem_ptr = reinterpret_cast<volatile uint32_t*>(smem + F3_BAR_OFF + 80);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + F3_BAR_OFF + 84);
-  volatile int* bad_ring = reinterpret_cast<volatile int*>(smem + F3_BAR_OFF + 96);  // [block % F3_RING] = block + 1: not finite
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_launch_dependents();
@@ -271,12 +265,11 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
     for (int i = 0; i < 2; ++i) {
       for (int h = 0; h < 2; ++h) {
         mbar_init(full_bar(i, h), F3_LOADERS / 64);
-        mbar_init(done_bar(i, h), 1 + h);
+        mbar_init(done_bar(i, h), 1);
       }
       mbar_init(free_bar(i), F3_DRAINS);
     }
     *abort_flag = 0;
-    for (int i = 0; i < F3_RING; ++i) bad_ring[i] = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == F3_ISSUE_WARP) {
@@ -327,7 +320,6 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
     const float *ta[2] = {}, *tb[NB] = {};  // of the tile: see at()
     int na = 0, nb = 0;                     // K-major: rows that exist from the first piece's on; MN-major: columns
     Quad v[NA + NB];
-    uint64_t bad = 0ull;
     // Moves on to the next block; false: there is none.
     auto advance = [&]() {
       if (++kb < kb1) return true;
@@ -413,8 +405,8 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
     const uint32_t pa = place(A_MN, ra, ca), pb = place(B_MN, rb, cb) + 3 * F3_A_PLANE;
     auto split = [&](int i, uint32_t stage) {
       uint32_t h0, m0, l0, h1, m1, l1;
-      split2(v[i].lo, h0, m0, l0, bad);
-      split2(v[i].hi, h1, m1, l1, bad);
+      split2(v[i].lo, h0, m0, l0);
+      split2(v[i].hi, h1, m1, l1);
       const int ib = i - NA;
       const uint32_t d = i < NA ? pa + stage + (uint32_t)(A_MN ? (i >> 2) * 8192 + (i & 3) * 1024 : i * 2048)
                                 : pb + stage + (uint32_t)(B_MN ? ib * 1024 : ib * 2048);
@@ -445,7 +437,6 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
       while (more && u == w && ok) {
         const int st = it & 1;
         const uint32_t stage = (uint32_t)st * F3_STAGE;
-        bad = 0ull;
         more = advance();
         if (more) begin_block();
         else { whole = false; na = nb = kleft = 0; }  // nothing exists
@@ -456,7 +447,6 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
         else if (whole && o.vec_b) swap(No{}, Yes{}, stage);
         else if (whole && !o.vec_a) swap(No{}, No{}, stage);
         else swap(Look{}, Look{}, stage);
-        if (__any_sync(0xffffffffu, bad != 0ull) && lane == 0) bad_ring[it % F3_RING] = it + 1;
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(full_bar(st, h));
@@ -512,7 +502,6 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
               tc_commit(done_bar(mine, h));
             }
             if (!ok) break;
-            mbar_arrive(done_bar(mine, 1));  // passes on what the loaders said of the block
           }
         }
         __syncwarp();
@@ -521,14 +510,12 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
         uint64_t acc[F3_BN / 2];
 #pragma unroll
         for (int i = 0; i < F3_BN / 2; ++i) acc[i] = 0ull;
-        bool again = false;
         for (int b = it; b < it + kb1 - kb0 && ok; ++b) {
           const int i = b & 1;
           if (!mbar_wait(done_bar(i, 1), (uint32_t)(b >> 1) & 1u, abort_flag, g.status)) ok = false;
           ok = __all_sync(0xffffffffu, ok);
           if (!ok) break;
           tc_fence_after();
-          again = again || bad_ring[b % F3_RING] == b + 1;
           const uint32_t from = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)i * 256u;
 #pragma unroll
           for (int cc = 0; cc < F3_BN; cc += 16) {
@@ -548,14 +535,16 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
           if (lane == 0) mbar_arrive(free_bar(i));
         }
         float* row = T + (quad * 32 + lane) * F3_PITCH;
-        uint64_t bad = 0ull;  // NaN once a sum is not finite
+        uint64_t bad[4] = {};  // NaN once a sum is not finite, zero otherwise
 #pragma unroll
-        for (int i = 0; i < F3_BN / 2; ++i) bad = fma2(acc[i], 0ull, bad);
-        if (any_drain(again || bad != 0ull)) {
-          multiply_again(o, s, ti, tid - 32 * F3_DRAIN_WARP, kb0 * F3_BK, min(kb1 * F3_BK, ti.kext), T);
+        for (int i = 0; i < F3_BN / 2; ++i) bad[i & 3] = fma2(acc[i], 0ull, bad[i & 3]);
+        if (any_drain((bad[0] | bad[1] | bad[2] | bad[3]) != 0ull)) {
+          multiply_again(o, s, ti, tid - 32 * F3_DRAIN_WARP, kb0 * F3_BK, min(kb1 * F3_BK, ti.kext), T,
+                         reinterpret_cast<float*>(smem + F3_AGAIN_OFF));
         } else {
 #pragma unroll
-          for (int i = 0; i < F3_BN / 4; ++i) *reinterpret_cast<ulonglong2*>(row + 4 * i) = make_ulonglong2(acc[2 * i], acc[2 * i + 1]);
+          for (int i = 0; i < F3_BN / 4; ++i)
+            *reinterpret_cast<ulonglong2*>(row + 4 * i) = make_ulonglong2(mul2(acc[2 * i], pair(F3_DOWN, F3_DOWN)), mul2(acc[2 * i + 1], pair(F3_DOWN, F3_DOWN)));
         }
         if (s.S == 1) sync_drain();
       }

@@ -6,7 +6,7 @@ import pytest
 import torch
 
 from paper_2203_05705_b200 import ard
-from gpu_helpers import Ctx, run_three_gemms, assert_ok
+from gpu_helpers import Ctx, run_three_gemms, assert_ok, oracle_mask
 
 pytestmark = pytest.mark.gpu
 
@@ -159,5 +159,26 @@ def test_not_finite_in_a_long_contraction():
         want = torch.full((N, K), 0.125 * B, device="cuda")  # exact in fp32
         want[:, 1] = want[2, :] = float("nan")
         assert torch.equal(want.isnan(), dW.isnan()) and torch.equal(want.nan_to_num(), dW.nan_to_num())
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("exponent", [-100, -113, -126, -140])
+@pytest.mark.parametrize("kind,ts,dp", [(ard.ARD_ROW, 0, 1), (ard.ARD_TILE, 64, 3)])
+def test_small_elements_keep_their_bits(exponent, kind, ts, dp):
+    """Operands down to fp32's subnormal numbers (the others large enough for results that are not)."""
+    B, K, N = 200, 1536, 1088
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(kind, K, N, ts)
+        ard.ard_pattern_set(ctx.h, pat, dp, 1)
+        mask = torch.from_numpy(np.ascontiguousarray(oracle_mask(kind, K, N, ts, dp, 1).T)).cuda().double()
+        for where in range(3):
+            ops = [torch.randn(s, device="cuda") * 2.0 ** (exponent if i == where else 30) for i, s in enumerate(((B, K), (N, K), (B, N)))]
+            X, W, dY = [o.double() for o in ops]
+            Wm = W * (mask if mask.ndim == 2 else mask[:, None])
+            want = [X @ Wm.T, dY @ Wm, (dY.T @ X) * (mask if mask.ndim == 2 else mask[:, None])]
+            for w, (_, tc) in zip(want, _both_paths(ctx, pat, B, K, N, *ops)):
+                assert (tc.double() - w).norm() <= TOL * w.norm()
     finally:
         ctx.close()
