@@ -2,17 +2,20 @@
 // x = h + m + l (8 bits each, rounded to nearest, so 24 in all), and a product is taken as h h' + h m' + m h' + h l' + m m' + l h'.
 // What is left out (m l', l m', l l') is below 2^-25 of |x y|, half of what rounding one fp32 product costs.  The
 // tensor core truncates its sums, so the accumulators are taken out of tensor memory after every 64 contraction indices
-// and added in fp32 registers, rounded to nearest: four truncations per sum instead of K / 16.
+// and added in fp32 registers, rounded to nearest, and h h' of a block's two halves has columns of its own: two truncations per
+// sum instead of K / 16.  With four, operands of one sign, whose truncations add up, had a larger error than on the CUDA cores
+// where those cut a contraction eight ways (512 x 384 x 512, uniform in 0 .. 1: 8.0e-8 against 6.1e-8, now 5.5e-8).
 //
 // One CTA per SM, 128 x 64 output tiles.  Warps 0..7 load (registers, the next block's piece requested as soon as this block's
 // has been split) and write the six planes in the 128-byte-swizzled layout; warps 8 and 9 issue the products of the even and
 // the odd blocks, each into accumulators of its own (an issued product costs its thread 136 cycles whatever its size, so one
 // thread could not keep up); warps 10..13 take the accumulators out, add them up and write the tile.
 // The three planes of B lie behind one another, so that one instruction multiplies a plane of A with up to all three:
-//   A.h x [B.h B.m B.l] -> columns 0..191,  A.m x [B.h B.m] -> 64..191,  A.l x B.h -> 128..191.
+//   A.h x [B.h B.m B.l] -> columns 0..191,  A.m x [B.h B.m] -> 64..191,  A.l x B.h -> 128..191;
+// in the second half of a block A.h x B.h -> 192..255 and A.h x [B.m B.l] -> 64..191.
 //
 // Bound: shared memory.  A block (128 + 64 rows, 64 contraction indices) takes 48 KB through L1, 72 KB of stores of the planes
-// and 98 KB of operand reads, about 1730 cycles at 128 bytes a cycle, next to 768 tensor-core cycles.
+// and 106 KB of operand reads, about 1810 cycles at 128 bytes a cycle, next to 768 tensor-core cycles.
 //
 // Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l, and so in every sum they are part of.  Finite operands can
 // leave an infinity or a NaN too where a product is near the largest fp32 number or beyond it: h h' may round past it, and h m'
@@ -40,7 +43,7 @@ constexpr int AGAIN_K = 32, AGAIN_N = 32, AGAIN_PA = UMMA_BM + 4, AGAIN_PB = AGA
 constexpr int F3_AGAIN_OFF = F3_TILE_OFF + UMMA_BM * F3_PITCH * 4;
 constexpr int F3_BAR_OFF = F3_AGAIN_OFF + AGAIN_K * (AGAIN_PA + AGAIN_PB) * 4;
 constexpr int F3_SMEM = F3_BAR_OFF + 128 + 1024;
-constexpr int F3_TMEM = 512;           // two blocks' accumulators of 3 * F3_BN columns each, rounded up to a power of two
+constexpr int F3_TMEM = 512;           // two blocks' accumulators of 4 * F3_BN columns each
 constexpr double F3_LEAST_FLOPS = 1.5e8;  // kept operations, see f32_takes
 constexpr float F3_UP = 65536.f, F3_DOWN = 1.f / (F3_UP * F3_UP);
 
@@ -495,7 +498,12 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
 #pragma unroll
               for (int k = 2 * h; k < 2 * h + 2; ++k) {
                 const uint64_t ak = ad + (uint64_t)(k * (A_MN ? 128 : 2)), bk = bd + (uint64_t)(k * (B_MN ? 128 : 2));
-                tc_mma_bf16(d, ak, bk, make_idesc(3 * F3_BN, A_MN, B_MN), k != 0 ? 1u : 0u);
+                if (h == 0) {
+                  tc_mma_bf16(d, ak, bk, make_idesc(3 * F3_BN, A_MN, B_MN), k != 0 ? 1u : 0u);
+                } else {
+                  tc_mma_bf16(d + 3 * F3_BN, ak, bk, make_idesc(F3_BN, A_MN, B_MN), k != 2 ? 1u : 0u);
+                  tc_mma_bf16(d + F3_BN, ak, bk + (F3_B_PLANE >> 4), make_idesc(2 * F3_BN, A_MN, B_MN), 1u);
+                }
                 tc_mma_bf16(d + F3_BN, ak + (F3_A_PLANE >> 4), bk, make_idesc(2 * F3_BN, A_MN, B_MN), 1u);
                 tc_mma_bf16(d + 2 * F3_BN, ak + 2 * (F3_A_PLANE >> 4), bk, make_idesc(F3_BN, A_MN, B_MN), 1u);
               }
@@ -519,15 +527,16 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
           const uint32_t from = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)i * 256u;
 #pragma unroll
           for (int cc = 0; cc < F3_BN; cc += 16) {
-            uint32_t x[16], y[16], z[16];
+            uint32_t x[16], w[16], y[16], z[16];
             tmem_ld16(from + cc, x);
+            tmem_ld16(from + 3 * F3_BN + cc, w);
             tmem_ld16(from + F3_BN + cc, y);
             tmem_ld16(from + 2 * F3_BN + cc, z);
             tmem_ld_wait();
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
               auto two = [&](const uint32_t (&r)[16]) { return pair(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1])); };
-              acc[cc / 2 + q] = add2(acc[cc / 2 + q], add2(two(x), add2(two(y), two(z))));
+              acc[cc / 2 + q] = add2(acc[cc / 2 + q], add2(add2(two(x), two(w)), add2(two(y), two(z))));
             }
           }
           tc_fence_before();
@@ -610,7 +619,8 @@ ard_status launch_f32(ard_ctx* ctx, F32Params p, cudaStream_t s) {
 //   100 x 1001 x 777      1.6e8      61, 43   46, 46  39, 45  41, 39
 //   128 x 2048 x 2048     1.1e9     105, 57   82, 53  69, 56  56, 64
 //   1024 x 4096 x 4096    3.4e10   2730, 963 1601, 710 806, 460 332, 247
-// Error against fp64 (2-norm) there and here: 7e-8 .. 1.2e-6 and 3.5e-8 .. 1.7e-7, never larger here.
+// Error against fp64 (2-norm) there and here, 12 shapes with contractions of 64 to 4096: operands of both signs 1.5e-7 .. 4.1e-7 and
+// 5.4e-8 .. 1.0e-7, of one sign 6.1e-8 .. 2.5e-7 and 3.1e-8 .. 6.5e-8; at most 0.9 of the CUDA cores' in each.
 bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts) {
   if (ctx->path != ARD_PATH_AUTO || ctx->encode_fn == nullptr || g.B < 1 || g.K < 1 || g.N < 1) return false;
   if (kind == ARD_TILE && ts % 4 != 0) return false;  // four consecutive positions never leave a pattern tile

@@ -182,3 +182,21 @@ def test_small_elements_keep_their_bits(exponent, kind, ts, dp):
                 assert (tc.double() - w).norm() <= TOL * w.norm()
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("K,M,N", [(64, 1088, 1088), (512, 384, 512), (1024, 256, 384)])
+def test_operands_of_one_sign(K, M, N):
+    """Truncated sums of terms of one sign lose in one direction: still no larger an error than the CUDA-core kernel's (shapes whose
+    contraction that one cuts eight ways among them, where its error is smallest)."""
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        ard.ard_pattern_set(ctx.h, pat, 1, 1)
+        g = torch.Generator(device="cuda").manual_seed(K)
+        for draw in (lambda s: torch.rand(s, device="cuda", generator=g), lambda s: torch.randn(s, device="cuda", generator=g).abs()):
+            X, W, dY = draw((M, K)), draw((N, K)), draw((M, N))
+            want = [X.double() @ W.double().T, dY.double() @ W.double(), dY.double().T @ X.double()]
+            for w, (cc, tc) in zip(want, _both_paths(ctx, pat, M, K, N, X, W, dY)):
+                assert (tc.double() - w).norm() <= (cc.double() - w).norm()
+    finally:
+        ctx.close()
