@@ -107,7 +107,7 @@ ard_status ard_set_path(ard_ctx* ctx, ard_path path);
 typedef enum { ARD_OPT_PDL = 0, ARD_OPT_PDL_IN_CAPTURE = 1, ARD_OPT_SIDE_STREAMS = 2, ARD_OPT_CTA_PAIRS = 3,
                ARD_OPT_BAND_ROWS = 4, ARD_OPT_MLP_PERSISTENT = 5, ARD_OPT_LSTM_COMPACT_H = 6 } ard_option;
 ard_status ard_set_option(ard_ctx* ctx, ard_option option, int value);
-/* Opt-in for training loops.  The tensor-core backward GEMMs of a row pattern read a compacted copy
+/* Opt-in for training loops, bf16 layers.  The tensor-core backward GEMMs of a row pattern read a compacted copy
  * of a full-width dY (kept columns only) that the library makes in the context workspace.  With
  * enable != 0, a backward call whose dY pointer, leading dimension, batch size, pattern sample and
  * stream equal those of the previous backward call on this context reuses that copy instead of

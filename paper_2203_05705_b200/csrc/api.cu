@@ -614,7 +614,8 @@ static ard_status compact_dy(ard_ctx* ctx, const ard_pattern* pat, int B, int N,
   *out_ptr = ctx->d_workspace;
   *out_ld = ldc;
   auto& lg = ctx->last_gather;
-  if (ctx->reuse_compact && lg.src == dY && lg.ld == lddy && lg.B == B && lg.N == N && lg.pat == pat &&
+  // fp32 copies are taken again within one ard_layer_products only: ard_set_compact_reuse speaks of bf16 calls
+  if (ctx->reuse_compact >= (es == 2 ? 1 : 2) && lg.src == dY && lg.ld == lddy && lg.B == B && lg.N == N && lg.pat == pat &&
       lg.gen == pat->generation && lg.stream == s && lg.with_dense >= with_dense && lg.es == es)
     return ARD_OK;  // the previous backward call on this stream already compacted this dY for this pattern
   lg = {dY, lddy, B, N, pat, pat->generation, s, with_dense, es};
@@ -852,7 +853,7 @@ ard_status ard_layer_products(ard_ctx* ctx, const ard_pattern* pat, ard_dtype dt
   if (!streams) {
     // one stream: the calls in order, the second backward product reusing the first one's compact dY
     const int reuse = ctx->reuse_compact;
-    ctx->reuse_compact = 1;
+    ctx->reuse_compact = 2;
     ard_status st = fwd_impl(ctx, pat, nullptr, dtype, B, K, N, alpha, X, ldx, W, ldw, nullptr, 0, Y, ldy, (int)outmode, s);
     if (st == ARD_OK)
       st = bwd_data_impl(ctx, pat, nullptr, dtype, B, K, N, alpha, dY, lddy, 0, W, ldw, nullptr, 0, dX, lddx, s);
@@ -872,7 +873,7 @@ ard_status ard_layer_products(ard_ctx* ctx, const ard_pattern* pat, ard_dtype dt
   if (three) ARD_CUDA_OK(cudaStreamWaitEvent(aux, ctx->ev[100], 0));
   ard_status st = fwd_impl(ctx, pat, nullptr, dtype, B, K, N, alpha, X, ldx, W, ldw, nullptr, 0, Y, ldy, (int)outmode, s);
   const int reuse = ctx->reuse_compact;
-  ctx->reuse_compact = 1;
+  ctx->reuse_compact = 2;
   ard_status st2 = bwd_data_impl(ctx, pat, nullptr, dtype, B, K, N, alpha, dY, lddy, 0, W, ldw, nullptr, 0, dX, lddx, side);
   ard_status st3 = bwd_weight_impl(ctx, pat, nullptr, dtype, dW_dtype, B, K, N, alpha, X, ldx, dY, lddy, 0, dW, lddw,
                                    zero_fill_dropped, three ? aux : side);

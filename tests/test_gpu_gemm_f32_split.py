@@ -200,3 +200,28 @@ def test_operands_of_one_sign(K, M, N):
                 assert (tc.double() - w).norm() <= (cc.double() - w).norm()
     finally:
         ctx.close()
+
+
+def _tensors(B, K, N, seed=0):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    return [torch.randn(s, device="cuda", generator=g) * (K ** -0.5 if i == 1 else 1.0) for i, s in enumerate(((B, K), (N, K), (B, N)))]
+
+
+def test_the_compact_copy_is_not_kept_between_calls():
+    """ard_set_compact_reuse is for bf16 calls: an fp32 layer's dY may be written between its two backward calls."""
+    B, K, N = 1025, 2049, 2051
+    ctx = Ctx(4 * B * (N + 8))
+    try:
+        ard.ard_set_compact_reuse(ctx.h, True)
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        ard.ard_pattern_set(ctx.h, pat, 2, 1)
+        X, W, dY = _tensors(B, K, N)
+        dX, dW = torch.zeros((B, K), device="cuda"), torch.zeros((N, K), device="cuda")
+        ard.ard_bwd_data(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, dY, N, 0, W, K, dX, K)
+        dY.mul_(-3.0)
+        ard.ard_bwd_weight(ctx.h, pat, ard.ARD_F32, ard.ARD_F32, B, K, N, 1.0, X, K, dY, N, 0, dW, K, 1)
+        want = dY.double().T @ X.double()
+        want[1::2] = 0.0
+        assert (dW.double() - want).norm() <= TOL * want.norm()
+    finally:
+        ctx.close()
