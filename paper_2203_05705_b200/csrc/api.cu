@@ -647,7 +647,7 @@ static ard_status bwd_staged_by_threads(ard_ctx* ctx, const ard_pattern* pat, Ge
 // them often enough that a compact copy in the workspace, where it fits, is the faster way (1024 x 4096 x 4096, a period of 2,
 // the two backward products 278 and 265 us without it, 189 and 196 with it, its launches included).
 static ard_status bwd_f32(ard_ctx* ctx, const ard_pattern* pat, GemmOp op, GemmArgs g, cudaStream_t s) {
-  if (pat->kind == ARD_ROW && !g.flag0 && g.keep < 1.f && 2.0 * g.B * g.K * g.N * g.keep >= 2e9 && f32_takes(ctx, pat->kind, op, g, pat->ts)) {
+  if (pat->kind == ARD_ROW && !g.flag0 && g.keep < 1.f && 2.0 * g.B * g.K * g.N * g.keep >= F32_COMPACT_FLOPS && f32_takes(ctx, pat->kind, op, g, pat->ts)) {
     const void *dyc, *dense;
     int ldc, dense_ld;
     const ard_status st = compact_dy(ctx, pat, g.B, g.N, g.A0, g.lda0, 0, &dyc, &ldc, &dense, &dense_ld, s, 1, 4);

@@ -229,6 +229,7 @@ bool ldg_takes(const ard_ctx* ctx, ard_kind kind, const GemmArgs& g, int ts);
 ard_status launch_gemm_ldg(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
 
 // fp32 layers on the tensor cores, operands split into three bf16 parts.  f32_takes: can, and should, it take this call?
+constexpr double F32_COMPACT_FLOPS = 2e9;  // kept operations from which its backward products get a compact dY, see bwd_f32
 bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts);
 ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s);
 

@@ -27,6 +27,8 @@
 // sums times 2^-32.  Elements from 2^111 on and sums from 2^96 on are not finite then, and are multiplied again.
 #include "staged_product.h"
 
+#include <math.h>
+
 #include <type_traits>
 
 namespace {
@@ -580,6 +582,30 @@ __global__ void __launch_bounds__(F3_THREADS, 1) gemm_f32_kernel(const __grid_co
 
 inline int cdiv(int a, int b) { return (a + b - 1) / b; }
 
+inline int cluster_size(const ard_ctx* ctx, int M, int N) { return (long long)cdiv(M, UMMA_BM) * cdiv(N, F3_BN) * 8 <= ctx->sm_count ? 8 : 4; }
+
+// CTAs that the device holds at once in clusters of cl (all kernels here have the same registers, threads and shared memory)
+int room(const ard_ctx* ctx, int cl) {
+  static int known[2][64] = {};
+  int& r = known[cl == 8][ctx->device & 63];
+  if (r == 0) {
+    auto kern = gemm_f32_kernel<0, OP_FWD>;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, F3_SMEM) != cudaSuccess) (void)cudaGetLastError();
+    r = ard_cluster_room(ctx, kern, cl, F3_THREADS, F3_SMEM);
+  }
+  return r;
+}
+
+// How make_plan cuts a product: blocks that a CTA takes one after the other, tiles among them, and blocks of all CTAs.
+struct Cut { double serial, waves, total; };
+Cut cut(double M, double N, double K, int BM, int BN, int BK, int places, int cl) {
+  const double tiles = ceil(M / BM) * ceil(N / BN), nkb = ceil(K / BK);
+  int S = cl;
+  while (S > 1 && (tiles * S > places || nkb < 2 * S)) S >>= 1;
+  const double waves = ceil(tiles * S / places), share = ceil(nkb / S);
+  return {waves * share, waves, tiles * S * share};
+}
+
 template <int KIND, int OP>
 ard_status launch_f32(ard_ctx* ctx, F32Params p, cudaStream_t s) {
   auto kern = gemm_f32_kernel<KIND, OP>;
@@ -593,11 +619,8 @@ ard_status launch_f32(ard_ctx* ctx, F32Params p, cudaStream_t s) {
   const int M = OP == OP_BWD_WEIGHT ? g.N : g.B, N = OP == OP_FWD ? g.N : g.K;
   const int nkb = cdiv(OP == OP_FWD ? g.K : (OP == OP_BWD_DATA ? g.N : g.B), F3_BK);
   const int tiles = cdiv(M, UMMA_BM) * cdiv(N, F3_BN);
-  p.cl = tiles * 8 <= ctx->sm_count ? 8 : 4;
-  static int room[2][64] = {};
-  int& r = room[p.cl == 8][dev];
-  if (r == 0) r = ard_cluster_room(ctx, kern, p.cl, F3_THREADS, F3_SMEM);
-  int ctas = r;
+  p.cl = cluster_size(ctx, M, N);
+  int ctas = room(ctx, p.cl);
   if (KIND == 0) {  // no more than the densest pattern's tiles, cut as often as its contraction allows
     int S = p.cl;
     while (S > 1 && nkb < 2 * S) S >>= 1;
@@ -613,18 +636,43 @@ ard_status launch_f32(ard_ctx* ctx, F32Params p, cudaStream_t s) {
 }  // namespace
 
 // A product of up to 1.5e8 kept operations stays on the CUDA cores: about 5 us of every launch here go to the tables of the tile, the
-// first loads and the way out, which the lighter kernel does faster.  Three products, CUDA cores and here, in us (graph replays):
-//   kept operations of one product   dense    dp 2    dp 5    dp 16
-//   64 x 784 x 256        2.6e7      19, 30   20, 33  21, 30  18, 28
-//   100 x 1001 x 777      1.6e8      61, 43   46, 46  39, 45  41, 39
-//   128 x 2048 x 2048     1.1e9     105, 57   82, 53  69, 56  56, 64
-//   1024 x 4096 x 4096    3.4e10   2730, 963 1601, 710 806, 460 332, 247
+// first loads and the way out, which the lighter kernel does faster.  Above, the rule is an estimate of both kernels' times from how
+// they cut the product, its constants (us) fitted to 4400 products (batches of 16 to 4096, 128 to 4096 units, odd ones among
+// them, periods of 1 to 16, both kinds of pattern, graph replays).  It is off by 14 % here and 11 % there (rms), hence the
+// margin of a fifth.  Operations alone do not decide: a batch of 16 leaves a weight gradient a single block to a tile (16 x
+// 4096 x 4096: 34 us there, 66 here), 94 tiles cannot be cut and leave 38 places idle (192 x 3000 x 3000, a period of 2, input gradient:
+// 65, 79), columns of dY a period apart cost 8 sectors where one would do (512 x 3000 x 3000, a period of 16, weight gradient: 39, 80).
+// With operations alone 14 % of the products were slower here by 3 % and more, up to 2.2x; with this rule 0.8 %, up to 1.2x (of 1600
+// others five by 8 % and more, up to 1.3x), at the same gain in the mean (1.3x; 1.36x if the faster kernel were always taken).
+// Three products of a dense layer, CUDA cores and here: 128 x 2048 x 2048 105 and 62 us, 1024 x 4096 x 4096 2730 and 951.
 // Error against fp64 (2-norm) there and here, 12 shapes with contractions of 64 to 4096: operands of both signs 1.5e-7 .. 4.1e-7 and
 // 5.4e-8 .. 1.0e-7, of one sign 6.1e-8 .. 2.5e-7 and 3.1e-8 .. 6.5e-8; at most 0.9 of the CUDA cores' in each.
 bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts) {
   if (ctx->path != ARD_PATH_AUTO || ctx->encode_fn == nullptr || g.B < 1 || g.K < 1 || g.N < 1) return false;
   if (kind == ARD_TILE && ts % 4 != 0) return false;  // four consecutive positions never leave a pattern tile
-  return 2.0 * g.B * g.K * g.N * g.keep >= F3_LEAST_FLOPS;
+  const double kept = 2.0 * g.B * g.K * g.N * g.keep;
+  if (kept < F3_LEAST_FLOPS) return false;
+  const bool row = kind == ARD_ROW;
+  const double n = row ? ceil(g.N * (double)g.keep) : g.N, keep_tile = row ? 1.0 : g.keep;
+  const double M = op == OP_BWD_WEIGHT ? n : g.B, N = op == OP_FWD ? n : g.K * (op == OP_BWD_WEIGHT ? keep_tile : 1.0);
+  const double K = op == OP_FWD ? g.K * keep_tile : (op == OP_BWD_DATA ? n * keep_tile : g.B);
+  const int cl = cluster_size(ctx, op == OP_BWD_WEIGHT ? g.N : g.B, op == OP_FWD ? g.N : g.K);
+  const Cut tc = cut(M, N, K, UMMA_BM, F3_BN, F3_BK, room(ctx, cl), cl), cc = cut(M, N, K, 64, 64, 16, 4 * ctx->sm_count, 8);
+  const double cc_blocks = cc.total / (4 * ctx->sm_count);
+  // columns of dY, a period apart (up to 8 elements to a sector) unless a compact copy will be read; zeros of dropped outputs, in MB
+  const bool dropped = row && g.keep < 1.f, full_dy = op != OP_FWD && !g.flag0;
+  const double apart = dropped && full_dy && kept < F32_COMPACT_FLOPS ? fmin(1.0 / g.keep, 8.0) - 1.0 : 0.0;
+  const double mb_fwd = dropped && op == OP_FWD && g.flag0 == ARD_OUT_SCATTER_ZEROFILL ? 4e-6 * g.B * g.N : 0.0;
+  const double mb_dw = op == OP_BWD_WEIGHT ? 4e-6 * g.N * g.K : 0.0;
+  // contiguous pieces off the 16-byte grid
+  auto off = [](const void* p, int ld, int along) { return ((reinterpret_cast<uintptr_t>(p) & 15) != 0 || ld % 4 != 0 || along % 4 != 0) ? 1.0 : 0.0; };
+  const double off_a = row && apart == 0.0 ? off(g.A0, g.lda0, op == OP_FWD ? g.K : g.N) : 0.0;
+  const double off_b = row ? off(g.A1, g.lda1, g.K) : 0.0;
+  const double tc_off = op == OP_FWD ? 0.2 * off_a : (op == OP_BWD_DATA ? 0.55 * off_a + 0.15 * off_b : 0.9 * off_a + 0.3 * off_b);
+  const double cc_off = op == OP_FWD ? 0.7 * off_a : 0.13 * (off_a + off_b);
+  const double t_tc = 7.4 + 1.4 * tc.waves + tc.serial * (1.55 + 0.44 * apart + tc_off) + 1.1 * mb_fwd + 0.19 * mb_dw;
+  const double t_cc = 7.4 + 0.74 * cc.serial + cc_blocks * (1.45 + 0.2 * apart + cc_off) + 0.36 * mb_fwd + 0.14 * mb_dw;
+  return 1.2 * t_tc < t_cc;
 }
 
 ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s) {

@@ -21,7 +21,12 @@ def _layer(B, K, N):
     return X, W / np.float32(np.sqrt(K)), dY
 
 
-@pytest.mark.parametrize("B,K,N", [(128, 2048, 2048), (129, 2087, 1531), (5, 6001, 8193), (4097, 65, 1201), (4100, 700, 130)])
+# contractions cut eight, four and two ways and not at all
+ROWS = [(250, 4099, 510), (250, 510, 4099), (4099, 250, 510), (257, 2051, 701), (385, 3001, 1003), (513, 2087, 1531)]
+TILES = [(32, 700, 36, 35), (12, 800, 90, 101), (128, 520, 9, 10), (200, 520, 6, 7), (4, 500, 300, 300)]
+
+
+@pytest.mark.parametrize("B,K,N", [(128, 2048, 2048), (129, 2087, 1531), (5, 6001, 8193), (4097, 65, 1201), (4100, 700, 130)] + ROWS)
 @pytest.mark.parametrize("workspace", [0, 32 << 20])
 def test_row_pattern(B, K, N, workspace):
     X, W, dY = _layer(B, K, N)
@@ -37,7 +42,7 @@ def test_row_pattern(B, K, N, workspace):
         ctx.close()
 
 
-@pytest.mark.parametrize("ts,B,Tr,Tc", [(32, 129, 64, 33), (12, 200, 90, 101), (128, 260, 9, 10), (200, 130, 6, 7)])
+@pytest.mark.parametrize("ts,B,Tr,Tc", [(32, 129, 64, 33), (12, 200, 90, 101), (128, 260, 9, 10), (200, 130, 6, 7)] + TILES)
 def test_tile_pattern(ts, B, Tr, Tc):
     K, N = Tr * ts, Tc * ts
     X, W, dY = _layer(B, K, N)
@@ -56,9 +61,10 @@ def test_tile_pattern(ts, B, Tr, Tc):
 
 @pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.395e38])
 @pytest.mark.parametrize("kind,ts,dp", [(ard.ARD_ROW, 0, 1), (ard.ARD_ROW, 0, 2), (ard.ARD_TILE, 64, 3)])
-def test_not_finite(value, kind, ts, dp):
+@pytest.mark.parametrize("B", [200, 700])
+def test_not_finite(value, kind, ts, dp, B):
     """An infinity, a NaN or a value that no bf16 holds ends up where the CUDA-core kernel has it."""
-    B, K, N = 200, 1536, 1088
+    K, N = 1536, 1088
     ctx = Ctx(0)
     try:
         pat = ctx.pattern(kind, K, N, ts)
@@ -105,7 +111,7 @@ def _both_paths(ctx, pat, B, K, N, X, W, dY, relu=False):
 @pytest.mark.parametrize("kind,ts,dp,relu", [(ard.ARD_ROW, 0, 1, False), (ard.ARD_ROW, 0, 2, True), (ard.ARD_TILE, 64, 3, False)])
 def test_products_near_and_beyond_the_largest_number(x, w, kind, ts, dp, relu):
     """Finite operands whose product overflows, or only just does not: as the CUDA-core kernel has it."""
-    B, K, N = 200, 1536, 1088
+    B, K, N = 700, 1536, 1088
     ctx = Ctx(0)
     try:
         pat = ctx.pattern(kind, K, N, ts)
@@ -122,9 +128,9 @@ def test_products_near_and_beyond_the_largest_number(x, w, kind, ts, dp, relu):
         ctx.close()
 
 
-@pytest.mark.parametrize("B,K,N,kind,ts,dp", [(131, 1547, 1091, ard.ARD_ROW, 0, 1), (131, 1547, 1091, ard.ARD_ROW, 0, 2),
-                                              (1029, 67, 1201, ard.ARD_ROW, 0, 1), (133, 1080, 1212, ard.ARD_TILE, 12, 1),
-                                              (4101, 480, 312, ard.ARD_TILE, 12, 5)])
+@pytest.mark.parametrize("B,K,N,kind,ts,dp", [(513, 2087, 1531, ard.ARD_ROW, 0, 1), (513, 2087, 1531, ard.ARD_ROW, 0, 2),
+                                              (4099, 250, 510, ard.ARD_ROW, 0, 1), (800, 1080, 1212, ard.ARD_TILE, 12, 1),
+                                              (500, 1200, 1200, ard.ARD_TILE, 4, 5)])
 def test_not_finite_at_the_edges(B, K, N, kind, ts, dp):
     """Infinities in the last row, column and index of ragged tiles: what the repeated products read and write."""
     ctx = Ctx(0)
@@ -167,7 +173,7 @@ def test_not_finite_in_a_long_contraction():
 @pytest.mark.parametrize("kind,ts,dp", [(ard.ARD_ROW, 0, 1), (ard.ARD_TILE, 64, 3)])
 def test_small_elements_keep_their_bits(exponent, kind, ts, dp):
     """Operands down to fp32's subnormal numbers (the others large enough for results that are not)."""
-    B, K, N = 200, 1536, 1088
+    B, K, N = 700, 1536, 1088
     ctx = Ctx(0)
     try:
         pat = ctx.pattern(kind, K, N, ts)
@@ -184,8 +190,8 @@ def test_small_elements_keep_their_bits(exponent, kind, ts, dp):
         ctx.close()
 
 
-@pytest.mark.parametrize("K,M,N", [(64, 1088, 1088), (512, 384, 512), (1024, 256, 384)])
-def test_operands_of_one_sign(K, M, N):
+@pytest.mark.parametrize("M,K,N", [(256, 4096, 512), (256, 512, 4096), (4096, 256, 512), (1024, 1024, 1024)])
+def test_operands_of_one_sign(M, K, N):
     """Truncated sums of terms of one sign lose in one direction: still no larger an error than the CUDA-core kernel's (shapes whose
     contraction that one cuts eight ways among them, where its error is smallest)."""
     ctx = Ctx(0)
@@ -223,5 +229,17 @@ def test_the_compact_copy_is_not_kept_between_calls():
         want = dY.double().T @ X.double()
         want[1::2] = 0.0
         assert (dW.double() - want).norm() <= TOL * want.norm()
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("B,K,N,ts", [r + (0,) for r in ROWS] + [(B, Tr * ts, Tc * ts, ts) for ts, B, Tr, Tc in TILES])
+def test_these_layers_reach_the_kernel(B, K, N, ts):
+    """Other sums than the CUDA-core kernel's, bit for bit, from at least two of the three products."""
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_TILE if ts else ard.ARD_ROW, K, N, ts)
+        ard.ard_pattern_set(ctx.h, pat, 1, 1)
+        assert sum(not torch.equal(cc, tc) for cc, tc in _both_paths(ctx, pat, B, K, N, *_tensors(B, K, N))) >= 2
     finally:
         ctx.close()
