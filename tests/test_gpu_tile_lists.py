@@ -24,3 +24,18 @@ def test_every_kind_of_period(Tr, Tc):
                     assert np.array_equal(g, o), (Tr, Tc, dp, b)
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("dp,b", [(2 ** 26, 1), (2 ** 26 + 1, 6), (2 ** 25, 1)])
+def test_rows_whose_distance_times_a_warp_is_no_int(dp, b):
+    Tr = 2 ** 26 + 1
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_TILE, Tr, 1, 1)
+        ard.ard_pattern_set(ctx.h, pat, dp, b)
+        col_ptr, col_idx, row_ptr, row_idx = ard.ard_pattern_tile_lists_to_host(pat, Tr, 1)
+        rows = np.arange(b - 1, Tr, dp)
+        assert np.array_equal(col_ptr, [0, len(rows)]) and np.array_equal(col_idx[:len(rows)], rows)
+        assert row_ptr[-1] == len(rows) and not row_idx[:len(rows)].any()
+    finally:
+        ctx.close()
