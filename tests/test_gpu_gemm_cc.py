@@ -28,11 +28,15 @@ def ctx():
 def test_row_pattern(ctx, B, K, N):
     X, W, dY = _layer(B, K, N, B + K + N)
     pat = ctx.pattern(ard.ARD_ROW, K, N)
-    for i, (dp, b) in enumerate([(1, 1), (2, 2), (3, 1), (16, 7)]):
-        ard.ard_pattern_set(ctx.h, pat, dp, b)
-        res = run_three_gemms(ctx, pat, ard.ARD_ROW, ard.ARD_F32, X, W, dY, dp, b, 1.5, compact=(i % 2 == 1), zero_fill=(i != 2),
-                              lds={"x": K + i, "w": K + 3 * (i & 1), "y": N + 5 * (i & 2)})
-        assert_ok(res, TOL[ard.ARD_F32], (B, K, N, dp, b))
+    ard.ard_set_path(ctx.h, ard.ARD_PATH_CUDA_CORE)
+    try:
+        for i, (dp, b) in enumerate([(1, 1), (2, 2), (3, 1), (16, 7)]):
+            ard.ard_pattern_set(ctx.h, pat, dp, b)
+            res = run_three_gemms(ctx, pat, ard.ARD_ROW, ard.ARD_F32, X, W, dY, dp, b, 1.5, compact=(i % 2 == 1), zero_fill=(i != 2),
+                                  lds={"x": K + i, "w": K + 3 * (i & 1), "y": N + 5 * (i & 2)})
+            assert_ok(res, TOL[ard.ARD_F32], (B, K, N, dp, b))
+    finally:
+        ard.ard_set_path(ctx.h, ard.ARD_PATH_AUTO)
 
 
 @pytest.mark.parametrize("dtype", [ard.ARD_F32, ard.ARD_BF16])

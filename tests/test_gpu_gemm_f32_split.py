@@ -1,6 +1,6 @@
 """fp32 layers large enough for the tensor cores (operands split into three bf16 parts) against the oracle: edges of the 128 x 64
 tiles and of the contraction blocks, rows on and off the 16-byte grid, cut and whole contractions, a compact copy of dY or none,
-and operands that are not finite."""
+operands and sums that are not finite, very small or of one sign."""
 import numpy as np
 import pytest
 import torch
@@ -215,7 +215,7 @@ def _tensors(B, K, N, seed=0):
 
 def test_the_compact_copy_is_not_kept_between_calls():
     """ard_set_compact_reuse is for bf16 calls: an fp32 layer's dY may be written between its two backward calls."""
-    B, K, N = 1025, 2049, 2051
+    B, K, N = 1017, 2049, 1481
     ctx = Ctx(4 * B * (N + 8))
     try:
         ard.ard_set_compact_reuse(ctx.h, True)
@@ -241,5 +241,102 @@ def test_these_layers_reach_the_kernel(B, K, N, ts):
         pat = ctx.pattern(ard.ARD_TILE if ts else ard.ARD_ROW, K, N, ts)
         ard.ard_pattern_set(ctx.h, pat, 1, 1)
         assert sum(not torch.equal(cc, tc) for cc, tc in _both_paths(ctx, pat, B, K, N, *_tensors(B, K, N))) >= 2
+    finally:
+        ctx.close()
+
+
+# from 2e9 kept operations on the backward products of a row pattern read a compact copy of dY, where the workspace has room for it
+COMPACTED = [(1017, 2049, 1481), (1030, 2052, 2308)]
+
+
+@pytest.mark.parametrize("B,K,N", COMPACTED)
+@pytest.mark.parametrize("room", [0, -1])
+def test_compact_copy_of_a_full_width_gradient(B, K, N, room):
+    X, W, dY = _layer(B, K, N)
+    ctx = Ctx(4 * B * ((N + 7) // 8 * 8) + room)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        for dp, b in [(2, 2), (3, 1)]:
+            ard.ard_pattern_set(ctx.h, pat, dp, b)
+            before = ard.ard_launch_count(ctx.h)
+            res = run_three_gemms(ctx, pat, ard.ARD_ROW, ard.ARD_F32, X, W, dY, dp, b, 1.5, lds={"y": N + 3})
+            assert_ok(res, TOL, (B, K, N, dp, b))
+            assert ard.ard_launch_count(ctx.h) - before in ((4, 5) if room == 0 else (3,))
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("side_streams", [0, 1])
+def test_compact_copy_over_a_distribution(side_streams):
+    """Dense draws of a distribution that drops something go through the copy too; ard_layer_products makes one for both products."""
+    B, K, N = COMPACTED[1]
+    ctx = Ctx(4 * B * (N + 8))
+    try:
+        ard.ard_set_option(ctx.h, ard.ARD_OPT_SIDE_STREAMS, side_streams)
+        ard.ard_set_distribution(ctx.h, 0, [0.4, 0.3, 0.3])
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        X, W, dY = _tensors(B, K, N)
+        seen = set()
+        for it in range(12):
+            ard.ard_sample_pattern(ctx.h, pat, 0, 1, it, 0)
+            dp, _, _, keep = ard.ard_pattern_to_host(pat, N)
+            if dp in seen:
+                continue
+            seen.add(dp)
+            mask = torch.zeros(N, dtype=torch.float64, device="cuda")
+            mask[torch.from_numpy(keep).long().cuda()] = 1.0
+            dY.mul_(-1.5)  # another gradient in the same buffer
+            Y, dX, dW = (torch.full(s, float("nan"), device="cuda") for s in ((B, N), (B, K), (N, K)))
+            ard.ard_layer_products(ctx.h, pat, ard.ARD_F32, ard.ARD_F32, B, K, N, 2.0, X, K, W, K, dY, N, Y, N,
+                                   ard.ARD_OUT_SCATTER_ZEROFILL, dX, K, dW, K, 1)
+            dYm = dY.double() * mask
+            for got, want in zip((Y, dX, dW), (X.double() @ W.double().T * mask, dYm @ W.double(), dYm.T @ X.double())):
+                assert (got.double() - 2.0 * want).norm() <= TOL * 2.0 * want.norm(), dp
+        assert seen == {1, 2, 3}
+        assert ard.ard_last_device_status(ctx.h) == 0
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("B,K,N", [(513, 2087, 1531), (700, 1536, 1088)])
+def test_accumulate(B, K, N):
+    """ARD_FLAG_ACCUMULATE: compact forward and input gradient added to what is there."""
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        X, W, dY = _tensors(B, K, N)
+        for dp in (1, 2):
+            ard.ard_pattern_set(ctx.h, pat, dp, 1)
+            n = (N - 1) // dp + 1
+            Y, dX = torch.randn((B, N), device="cuda"), torch.randn((B, K), device="cuda")
+            wantY, wantdX = Y.double(), dX.double()
+            wantY[:, :n] += X.double() @ W[::dp].double().T
+            wantdX += dY[:, ::dp].double() @ W[::dp].double()
+            ard.ard_fwd(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, X, K, W, K, Y, N, ard.ARD_OUT_COMPACT | ard.ARD_FLAG_ACCUMULATE)
+            ard.ard_bwd_data(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, dY, N, ard.ARD_FLAG_ACCUMULATE, W, K, dX, K)
+            for got, want in ((Y, wantY), (dX, wantdX)):
+                assert (got.double() - want).norm() <= TOL * want.norm()
+    finally:
+        ctx.close()
+
+
+def test_static_scratch():
+    """The entry point without a workspace, at a size that the tensor cores take (B * N * 4 bytes fit its fixed array)."""
+    B, K, N = 700, 2048, 1531
+    ctx = Ctx(0)
+    try:
+        pat = ctx.pattern(ard.ARD_ROW, K, N)
+        X, W, dY = _tensors(B, K, N)
+        for dp in (1, 2):
+            ard.ard_pattern_set(ctx.h, pat, dp, 1)
+            outs = []
+            for path in (ard.ARD_PATH_CUDA_CORE, ard.ARD_PATH_AUTO):
+                ard.ard_set_path(ctx.h, path)
+                dX = torch.full((B, K), float("nan"), device="cuda")
+                ard.ard_bwd_data_static_scratch(ctx.h, pat, ard.ARD_F32, B, K, N, 1.0, dY, N, W, K, dX, K)
+                outs.append(dX)
+            want = dY[:, ::dp].double() @ W[::dp].double()
+            assert (outs[1].double() - want).norm() <= TOL * want.norm()
+            assert not torch.equal(*outs)  # not the CUDA-core kernel's sums
     finally:
         ctx.close()
