@@ -1,4 +1,4 @@
-"""Thin ctypes binding over libard.so: argument marshalling only.
+"""Thin binding over libard.so (ctypes; native functions for the calls of a training iteration): argument marshalling only.
 
 Every function here has the name and the argument order of its C counterpart in
 include/ard.h; tensors are torch CUDA tensors (used for device memory and
@@ -9,7 +9,9 @@ raises -- there is no CPU fallback.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
+import warnings
 
 import numpy as np
 
@@ -157,16 +159,37 @@ def lib():
     return L
 
 
+_FED = {"ard_layer_fwd", "ard_layer_bwd_data", "ard_layer_bwd_weight", "ard_compact_weight_cols", "ard_expand_weight_grad_cols"}
 _native = None
+
+
+def _through_ctypes(name, *args):
+    """A call by its ctypes signature: pointers behind the handles (context, pattern or the like, feeding pattern) and before the
+    stream are device memory."""
+    fn = getattr(lib(), name)
+    first, last = 3 if name in _FED else 2, len(args) - 1
+    return fn(*(_ptr(a) if first <= i < last and fn.argtypes[i] is C.c_void_p else a for i, a in enumerate(args)))
+
+
+class _CtypesCalls:
+    def __getattr__(self, name):
+        return functools.partial(_through_ctypes, name)
 
 
 def _calls():
     """The calls of a training iteration, which take tensors as they are: an extension module beside the library
-    (csrc/python_calls.cpp).  Handing their arguments over through ctypes took 2.9 us of an ard_fwd, now 1.1."""
+    (csrc/python_calls.cpp).  Handing their arguments over through ctypes took 2.9 us of an ard_fwd, now 1.1.  Where the module was
+    built for another interpreter, or not at all, the calls go through ctypes."""
     global _native
     if _native is None:
         lib()  # says what is missing where nothing has been built
-        from . import _calls as module
+        try:
+            from . import _calls as module
+            module.fall_back(_through_ctypes)
+        except (ImportError, AttributeError) as e:
+            warnings.warn(f"calls go through ctypes, some 2 us slower each: no native functions for this interpreter ({e}); build "
+                          "them with `python -m paper_2203_05705_b200.build`", RuntimeWarning, stacklevel=3)
+            module = _CtypesCalls()
         _native = module
     return _native
 

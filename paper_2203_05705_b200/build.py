@@ -6,6 +6,7 @@ from __future__ import annotations
 
 import hashlib
 import os
+import shutil
 import subprocess
 import sys
 import sysconfig
@@ -93,13 +94,18 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 print(out)
     if jobs or force or _stale(LIB, objs):
         run([NVCC, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", LIB] + objs)
-    # the Python functions of the hot calls; found beside the library at run time
-    flags = ["-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", sysconfig.get_paths()["include"]]
+    # the Python functions of the hot calls; found beside the library at run time.  Without a compiler or Python's headers the calls
+    # go through ctypes.
+    cxx, include = os.environ.get("CXX", "g++"), sysconfig.get_paths()["include"]
+    if shutil.which(cxx) is None or not os.path.exists(os.path.join(include, "Python.h")):
+        print(f"{os.path.basename(CALLS)} not built: needs {cxx} and {include}/Python.h", file=sys.stderr)
+        return LIB
+    flags = ["-O2", "-std=c++17", "-shared", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", include]
     deps = [CALLS_SRC, os.path.join(ROOT, "include", "ard.h")]
     mark = os.path.join(OBJ, os.path.basename(CALLS) + ".key")
     want = _sha(deps, " ".join(flags))
     if force or not os.path.exists(CALLS) or not os.path.exists(mark) or open(mark).read() != want + _sha([CALLS]):
-        run([os.environ.get("CXX", "g++")] + flags + [CALLS_SRC, "-o", CALLS, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
+        run([cxx] + flags + [CALLS_SRC, "-o", CALLS, "-L", PKG, "-l:" + os.path.basename(LIB), "-Wl,-rpath,$ORIGIN"])
         with open(mark, "w") as f:
             f.write(want + _sha([CALLS]))
     return LIB

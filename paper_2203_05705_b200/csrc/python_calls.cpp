@@ -1,5 +1,7 @@
 // The C ABI's calls of a training iteration as Python functions: the arguments of include/ard.h in their order, device
 // memory as torch tensors (data_ptr() is asked for here), integers or None, handles as ctypes.c_void_p.  Returns the ard_status.
+// Arguments of any other kind go to the function given to fall_back(), which makes the call through ctypes: that takes, or refuses
+// in its own words, whatever it always did.
 //
 // An iteration of a small layer is bound by the host: a call through ctypes spent 2.9 us on its arguments where the native
 // call behind it takes 4.
@@ -8,6 +10,7 @@
 #include <stdint.h>
 
 #include <tuple>
+#include <type_traits>
 #include <utility>
 
 #include "ard.h"
@@ -15,6 +18,9 @@
 namespace {
 
 PyObject *g_void_p, *g_data_ptr;  // ctypes.c_void_p; the method's name
+PyObject* g_fall_back;            // (name, arguments...)
+
+// Each convert() returns false for what it does not take, an error set or not.
 
 bool convert(PyObject* o, int& v) {
   const unsigned long x = PyLong_AsUnsignedLongMask(o);  // what does not fit is cut off, as ctypes does
@@ -49,17 +55,37 @@ bool convert(PyObject* o, E& v) {
   v = (E)x;
   return true;
 }
+// Handles and streams
 template <typename T>
-bool convert(PyObject* o, T*& v) {
+bool convert_handle(PyObject* o, T*& v) {
   if (o == Py_None) {
     v = nullptr;
     return true;
   }
+  uint64_t x;
   if ((PyObject*)Py_TYPE(o) == g_void_p) {  // its memory holds the pointer
     Py_buffer b;
     if (PyObject_GetBuffer(o, &b, PyBUF_SIMPLE) != 0) return false;
     v = *(T**)b.buf;
     PyBuffer_Release(&b);
+    return true;
+  }
+  if (!PyLong_Check(o) || !convert(o, x)) return false;
+  v = (T*)(uintptr_t)x;
+  return true;
+}
+bool convert(PyObject* o, ard_ctx*& v) { return convert_handle(o, v); }
+bool convert(PyObject* o, const ard_pattern*& v) { return convert_handle(o, v); }
+bool convert(PyObject* o, ard_pattern*& v) { return convert_handle(o, v); }
+bool convert(PyObject* o, const ard_rows*& v) { return convert_handle(o, v); }
+bool convert(PyObject* o, ard_rows*& v) { return convert_handle(o, v); }
+bool convert(PyObject* o, const ard_blocks*& v) { return convert_handle(o, v); }
+bool convert(PyObject* o, ard_blocks*& v) { return convert_handle(o, v); }
+// Device memory
+template <typename T>
+bool convert(PyObject* o, T*& v) {
+  if (o == Py_None) {
+    v = nullptr;
     return true;
   }
   uint64_t x;
@@ -68,18 +94,38 @@ bool convert(PyObject* o, T*& v) {
   } else {
     PyObject* p = PyObject_CallMethodNoArgs(o, g_data_ptr);
     if (p == nullptr) return false;
-    const bool ok = convert(p, x);
+    const bool ok = PyLong_Check(p) && convert(p, x);
     Py_DECREF(p);
     if (!ok) return false;
   }
   v = (T*)(uintptr_t)x;
   return true;
 }
+// Argument i of n: a pointer in the last place is the stream.
+template <typename T>
+bool convert_argument(PyObject* o, T& v, size_t i, size_t n) {
+  if constexpr (std::is_same<T, void*>::value) {
+    if (i + 1 == n) return convert_handle(o, v);
+  }
+  return convert(o, v);
+}
 
 template <typename... A, size_t... I>
-PyObject* call(ard_status (*f)(A...), PyObject* const* args, std::index_sequence<I...>) {
+PyObject* call(ard_status (*f)(A...), const char* name, PyObject* const* args, std::index_sequence<I...>) {
   std::tuple<std::remove_const_t<A>...> v;
-  if (!(convert(args[I], std::get<I>(v)) && ...)) return nullptr;
+  if (!(convert_argument(args[I], std::get<I>(v), I, sizeof...(A)) && ...)) {
+    if (g_fall_back == nullptr) {
+      if (!PyErr_Occurred()) PyErr_Format(PyExc_TypeError, "%s: argument of a type that is not taken", name);
+      return nullptr;
+    }
+    PyErr_Clear();
+    PyObject* n = PyUnicode_FromString(name);
+    if (n == nullptr) return nullptr;
+    PyObject* all[] = {n, args[I]...};
+    PyObject* r = PyObject_Vectorcall(g_fall_back, all, 1 + sizeof...(A), nullptr);
+    Py_DECREF(n);
+    return r;
+  }
   ard_status st;
   Py_BEGIN_ALLOW_THREADS
   st = f(std::get<I>(v)...);
@@ -87,20 +133,24 @@ PyObject* call(ard_status (*f)(A...), PyObject* const* args, std::index_sequence
   return PyLong_FromLong((long)st);
 }
 template <typename... A>
-PyObject* call(ard_status (*f)(A...), PyObject* const* args, Py_ssize_t n) {
+PyObject* call(ard_status (*f)(A...), const char* name, PyObject* const* args, Py_ssize_t n) {
   if (n != (Py_ssize_t)sizeof...(A)) {
-    PyErr_Format(PyExc_TypeError, "%zd arguments expected, %zd given", (Py_ssize_t)sizeof...(A), n);
+    PyErr_Format(PyExc_TypeError, "%s: %zd arguments expected, %zd given", name, (Py_ssize_t)sizeof...(A), n);
     return nullptr;
   }
-  return call(f, args, std::index_sequence_for<A...>{});
+  return call(f, name, args, std::index_sequence_for<A...>{});
 }
-template <auto F>
-PyObject* entry(PyObject*, PyObject* const* args, Py_ssize_t n) {
-  return call(F, args, n);
+PyObject* fall_back(PyObject*, PyObject* f) {
+  Py_INCREF(f);
+  Py_XSETREF(g_fall_back, f);
+  Py_RETURN_NONE;
 }
 
-#define CALL(name) {#name, (PyCFunction)(void (*)(void))entry<&name>, METH_FASTCALL, nullptr}
+#define CALL(name)                                                                                            \
+  {#name, (PyCFunction)(void (*)(void))+[](PyObject*, PyObject* const* a, Py_ssize_t n) { return call(&name, #name, a, n); }, \
+   METH_FASTCALL, nullptr}
 PyMethodDef g_methods[] = {
+    {"fall_back", fall_back, METH_O, nullptr},
     CALL(ard_sample_pattern), CALL(ard_sample_pattern_counter), CALL(ard_pattern_set), CALL(ard_fwd), CALL(ard_bwd_data),
     CALL(ard_bwd_weight), CALL(ard_bwd_data_static_scratch), CALL(ard_layer_fwd), CALL(ard_layer_bwd_data),
     CALL(ard_layer_bwd_weight), CALL(ard_layer_products), CALL(ard_compact_weight_cols), CALL(ard_expand_weight_grad_cols),
