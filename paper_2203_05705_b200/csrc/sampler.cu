@@ -86,7 +86,7 @@ ard_sample_kernel(int32_t* __restrict__ hdr, int32_t* __restrict__ idx, int32_t*
   // residue: a thread per column finds its first kept row and the distance to the next in at most 2 dp steps, and the rest
   // follows.  Then a scan over the columns, and a warp per column writes its rows.  (4096 tiles, a period of 4: 5.0 us; ballots over
   // every tile of a column, twice, and one thread's running sum took 6.2.)
-  __shared__ int s_first[SAMPLER_THREADS], s_step[SAMPLER_THREADS], s_cnt[SAMPLER_THREADS], s_ptr[SAMPLER_THREADS], s_sum[32];
+  __shared__ int s_first[SAMPLER_THREADS], s_step[SAMPLER_THREADS], s_ptr[SAMPLER_THREADS], s_sum[32];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = nthreads / 32;
   const int t = Tc % dp;
   int before = 0;  // kept tiles in the columns of earlier rounds
@@ -131,14 +131,19 @@ ard_sample_kernel(int32_t* __restrict__ hdr, int32_t* __restrict__ idx, int32_t*
     if (c < Tc) col_ptr[c] = base;
     s_first[threadIdx.x] = first;
     s_step[threadIdx.x] = step;
-    s_cnt[threadIdx.x] = cnt;
     s_ptr[threadIdx.x] = base;
     __syncthreads();
-    for (int i = warp; i < min(nthreads, Tc - c0); i += nwarps) {
-      int32_t* to = col_idx + s_ptr[i];
-      // by entries: a row beyond the last one may not be an int
-      for (int j = lane; j < s_cnt[i]; j += 32) to[j] = s_first[i] + j * s_step[i];  // ascending rows
-    }
+    auto fill = [&](auto zero) {  // ascending rows, counted in the type of `zero`
+      using Row = decltype(zero);
+      for (int i = warp; i < min(nthreads, Tc - c0); i += nwarps) {
+        int32_t* to = col_idx + s_ptr[i];
+        int j = lane;
+        for (Row r = s_first[i] + lane * (Row)s_step[i]; r < Tr; r += 32 * (Row)s_step[i], j += 32) to[j] = (int)r;
+      }
+    };
+    // beyond 2^25 rows 32 times a distance may be no int (64 bits, or entries counted instead of rows, for all: 0.2 us)
+    if (Tr <= 1 << 25) fill(0);
+    else fill(0ll);
     before += all;
     __syncthreads();
   }
