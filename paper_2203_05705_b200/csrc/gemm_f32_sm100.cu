@@ -15,7 +15,8 @@
 // in the second half of a block A.h x B.h -> 192..255 and A.h x [B.m B.l] -> 64..191.
 //
 // Bound: shared memory.  A block (128 + 64 rows, 64 contraction indices) takes 48 KB through L1, 72 KB of stores of the planes
-// and 106 KB of operand reads, about 1810 cycles at 128 bytes a cycle, next to 768 tensor-core cycles.
+// and 106 KB of operand reads, 1810 cycles if all took turns at 128 bytes a cycle, next to 768 tensor-core cycles.  Measured 1724 (1024 x
+// 4096 x 4096, forward), the threads' data pipe busy for 49 % of the time, the issue slots for 55 %, the tensor pipe for 39 %.
 //
 // Infinities, NaN and magnitudes that a bf16 cannot hold leave a NaN in l, and so in every sum they are part of.  Finite operands can
 // leave an infinity or a NaN too where a product is near the largest fp32 number or beyond it: h h' may round past it, and h m'
@@ -638,12 +639,13 @@ ard_status launch_f32(ard_ctx* ctx, F32Params p, cudaStream_t s) {
 // A product of up to 1.5e8 kept operations stays on the CUDA cores: about 5 us of every launch here go to the tables of the tile, the
 // first loads and the way out, which the lighter kernel does faster.  Above, the rule is an estimate of both kernels' times from how
 // they cut the product, its constants (us) fitted to 4400 products (batches of 16 to 4096, 128 to 4096 units, odd ones among
-// them, periods of 1 to 16, both kinds of pattern, graph replays).  It is off by 14 % here and 11 % there (rms), hence the
-// margin of a fifth.  Operations alone do not decide: a batch of 16 leaves a weight gradient a single block to a tile (16 x
+// them, periods of 1 to 16, both kinds of pattern, graph replays).  It is off by 14 % here and 11 % there (rms).
+// Operations alone do not decide: a batch of 16 leaves a weight gradient a single block to a tile (16 x
 // 4096 x 4096: 34 us there, 66 here), 94 tiles cannot be cut and leave 38 places idle (192 x 3000 x 3000, a period of 2, input gradient:
 // 65, 79), columns of dY a period apart cost 8 sectors where one would do (512 x 3000 x 3000, a period of 16, weight gradient: 39, 80).
-// With operations alone 14 % of the products were slower here by 3 % and more, up to 2.2x; with this rule 0.8 %, up to 1.2x (of 1600
-// others five by 8 % and more, up to 1.3x), at the same gain in the mean (1.3x; 1.36x if the faster kernel were always taken).
+// Of 1452 others, operations alone made 135 slower than on the CUDA cores by a tenth and more, up to 2.2x, and this rule 20, up to 1.3x; the
+// gain in the mean is 1.43x and 1.46x.  The margin of 5 % balances what is lost by being here (one in a hundred by a tenth) and there
+// (two); a margin of a fifth 0.2 and 9.
 // Three products of a dense layer, CUDA cores and here: 128 x 2048 x 2048 105 and 62 us, 1024 x 4096 x 4096 2730 and 951.
 // Error against fp64 (2-norm) there and here, 12 shapes with contractions of 64 to 4096: operands of both signs 1.5e-7 .. 4.1e-7 and
 // 5.4e-8 .. 1.0e-7, of one sign 6.1e-8 .. 2.5e-7 and 3.1e-8 .. 6.5e-8; at most 0.9 of the CUDA cores' in each.
@@ -670,9 +672,9 @@ bool f32_takes(const ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, 
   const double off_b = row ? off(g.A1, g.lda1, g.K) : 0.0;
   const double tc_off = op == OP_FWD ? 0.2 * off_a : (op == OP_BWD_DATA ? 0.55 * off_a + 0.15 * off_b : 0.9 * off_a + 0.3 * off_b);
   const double cc_off = op == OP_FWD ? 0.7 * off_a : 0.13 * (off_a + off_b);
-  const double t_tc = 7.4 + 1.4 * tc.waves + tc.serial * (1.55 + 0.44 * apart + tc_off) + 1.1 * mb_fwd + 0.19 * mb_dw;
+  const double t_tc = 7.4 + 1.4 * tc.waves + tc.serial * (1.55 + 0.44 * apart + tc_off) + 1.3 * mb_fwd + 0.19 * mb_dw;
   const double t_cc = 7.4 + 0.74 * cc.serial + cc_blocks * (1.45 + 0.2 * apart + cc_off) + 0.36 * mb_fwd + 0.14 * mb_dw;
-  return 1.2 * t_tc < t_cc;
+  return 1.05 * t_tc < t_cc;
 }
 
 ard_status launch_gemm_f32(ard_ctx* ctx, ard_kind kind, GemmOp op, const GemmArgs& g, int ts, cudaStream_t s) {

@@ -1,5 +1,5 @@
-// What the product kernels whose threads stage the operands themselves have in common (gemm_ldg_sm100.cu on the tensor
-// cores, gemm_cc.cu on the CUDA cores): the tiling worked out from the pattern header on the device, the sum of the
+// What the product kernels whose threads stage the operands themselves have in common (gemm_ldg_sm100.cu and, for fp32 operands,
+// gemm_f32_sm100.cu on the tensor cores, gemm_cc.cu on the CUDA cores): the tiling worked out from the pattern header on the device, the sum of the
 // partial tiles of a cut contraction, and the rows' way out.  Everything is static to the including translation unit.
 //
 // A tile pattern (Sec. 3.2) keeps tile (r, c) iff r * Tc + c = b - 1 (mod dp), so tile-columns with equal c mod dp share
