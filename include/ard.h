@@ -30,9 +30,11 @@
  *     status word, read with ard_last_device_status; the kernel then exits normally and the output
  *     of that call is unspecified.  Nothing aborts or traps.
  *   - Arithmetic: ARD_F32 operands are multiplied and accumulated in fp32 on the CUDA cores, or, in products of
- *     more than 1.5e8 kept operations under ARD_PATH_AUTO, split into three bf16 parts each and multiplied on the
- *     tensor cores with fp32 accumulation (an error no larger than the CUDA cores' against fp64; where elements
- *     reach 2^111, sums 2^96, or either is not finite, with fp32 multiply-adds instead).  ARD_BF16 operands are multiplied on the tensor cores with fp32 accumulation.
+ *     more than 1.5e8 kept operations that are faster so under ARD_PATH_AUTO, split into three bf16 parts each and
+ *     multiplied on the tensor cores with fp32 accumulation: an error against fp64 no larger than the CUDA cores' on
+ *     operands of both signs and of one, contractions of 64 to 4096.  Where elements reach 2^111, sums 2^96, or either is
+ *     not finite, the sums are taken again with fp32 multiply-adds.  ARD_BF16 operands are multiplied on the tensor
+ *     cores with fp32 accumulation.
  *   - There is no CPU fallback.
  */
 #ifndef ARD_H_
@@ -71,9 +73,9 @@ typedef enum { ARD_OUT_COMPACT = 0, ARD_OUT_SCATTER_ZEROFILL = 1 } ard_outmode;
 #define ARD_FLAG_ACCUMULATE 0x20 /* add the product to the existing output; not with ARD_OUT_SCATTER_ZEROFILL   */
 #define ARD_FLAG_RELU 0x40       /* ard_layer_fwd only: apply max(., 0) before the rescale                      */
 
-/* Selects the kernel family for ARD_BF16 calls.  AUTO picks the tcgen05 path when the shape and
- * alignment allow it and the CUDA-core path otherwise; the other two force one family (FORCE_TC
- * returns ARD_ERR_ALIGNMENT / ARD_ERR_UNSUPPORTED instead of falling back). */
+/* Selects the kernel family.  AUTO picks the tcgen05 path when the shape and alignment allow it (ARD_F32: when it is
+ * the faster one, too) and the CUDA-core path otherwise; the other two force one family (FORCE_TC returns
+ * ARD_ERR_ALIGNMENT / ARD_ERR_UNSUPPORTED instead of falling back, for ARD_F32 in any case). */
 typedef enum { ARD_PATH_AUTO = 0, ARD_PATH_CUDA_CORE = 1, ARD_PATH_TENSOR_CORE = 2 } ard_path;
 
 #define ARD_MAX_DISTRIBUTIONS 16
@@ -83,8 +85,9 @@ typedef enum { ARD_PATH_AUTO = 0, ARD_PATH_CUDA_CORE = 1, ARD_PATH_TENSOR_CORE =
 /* ---- context -------------------------------------------------------------------------------- */
 
 /* Creates a context on CUDA device `device` with `workspace_bytes` of device scratch memory (used
- * to compact a full-width dY for the tensor-core backward GEMMs; 2*B*N bytes suffice for one
- * layer).  Synchronous. */
+ * to compact a full-width dY for the tensor-core backward GEMMs; one layer needs 2 * B * N bytes, ARD_F32 layers
+ * from 2e9 kept operations on 4 * B * N, N rounded up to a multiple of 8.  With less, bf16 layers go to other kernels
+ * and fp32 ones read dY where it is, which is slower).  Synchronous. */
 ard_status ard_create(ard_ctx** ctx, int device, size_t workspace_bytes);
 ard_status ard_destroy(ard_ctx* ctx);
 ard_status ard_set_path(ard_ctx* ctx, ard_path path);
@@ -226,7 +229,8 @@ ard_status ard_bwd_data(ard_ctx* ctx, const ard_pattern* pat, ard_dtype dtype, i
  * ard_create allocated (and fails with ARD_ERR_NOMEM when that workspace is too small); this call needs no
  * workspace at all, and calls neither cudaMalloc / cudaFree nor any allocating library routine.
  *   Row patterns only, full-width dY [B][N] (lddy), W [N][K] (ldw), dX [B][K] (lddx); runs on the
- *   CUDA cores (fp32 accumulate) for both dtypes.  The compacted copy of dY is kept in a fixed
+ *   CUDA cores (fp32 accumulate), larger ARD_F32 products on the tensor cores as in ard_bwd_data.
+ *   The compacted copy of dY is kept in a fixed
  *   array inside the library image: ARD_STATIC_SCRATCH_BYTES per GPU that loads the library, held
  *   until the process exits.  B*N*sizeof(element) must not exceed that size, otherwise the call
  *   returns ARD_ERR_NOMEM and launches nothing.
