@@ -20,7 +20,7 @@ LIB = os.path.join(PKG, "libard.so")
 CALLS_SRC = os.path.join(CSRC, "python_calls.cpp")
 CALLS = os.path.join(PKG, "_calls" + (sysconfig.get_config_var("EXT_SUFFIX") or ".so"))  # one per interpreter
 SOURCES = ["api.cu", "sampler.cu", "gemm_cc.cu", "gemm_tc_sm100.cu", "gemm_ldg_sm100.cu", "gemm_f32_sm100.cu", "aux_kernels.cu", "no_alloc.cu",
-           "distribution_search.cu", "lstm_persistent.cu", "mlp_step.cu", "mlp_persistent.cu", "rows.cu", "blocks.cu", "dropout_schedule.cu"]
+           "distribution_search.cu", "lstm_persistent.cu", "lstm_cluster.cu", "mlp_step.cu", "mlp_persistent.cu", "rows.cu", "blocks.cu", "dropout_schedule.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
          "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]

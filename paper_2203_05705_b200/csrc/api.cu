@@ -376,6 +376,10 @@ ard_status ard_set_distribution(ard_ctx* ctx, int dist_id, const double* K, int 
   double keep = 0.0;
   for (int i = 0; i < ndp; ++i) keep += (double)(cdf[i] - (i > 0 ? cdf[i - 1] : 0ull)) / 4294967296.0 / (i + 1);
   d.keep = (float)keep;
+  d.least = 1;
+  while (d.least < ndp && cdf[d.least - 1] == 0ull) ++d.least;
+  d.most = ndp;
+  while (d.most > 1 && cdf[d.most - 1] == cdf[d.most - 2]) --d.most;
   return ARD_OK;
 }
 
@@ -411,6 +415,8 @@ ard_status ard_pattern_create(ard_ctx* ctx, ard_pattern** out, ard_kind kind, in
   p->units = (int)units;
   p->dp_bound = 1;
   p->keep = 1.f;
+  p->dp_least = p->dp_most = 1;
+  p->in_graph = 0;
   p->generation = 0;
   size_t words = HDR_WORDS + (size_t)p->units;
   if (kind == ARD_TILE) words += (size_t)(p->Tc + 1) + (size_t)(p->Tr + 1) + 2 * (size_t)p->units;
@@ -441,6 +447,18 @@ ard_status ard_pattern_destroy(ard_pattern* pat) {
   return ARD_OK;
 }
 
+// What the host knows of the period that the pattern's header holds when later calls run.  A captured call runs again with
+// every replay, unseen: from then on nothing is known.
+static bool stream_captures(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+static void note_periods(ard_pattern* pat, int least, int most, cudaStream_t s) {
+  if (stream_captures(s)) pat->in_graph = 1;
+  pat->dp_least = pat->in_graph ? 1 : least;
+  pat->dp_most = pat->in_graph ? pat->units : most;
+}
+
 ard_status ard_sample_pattern(ard_ctx* ctx, ard_pattern* pat, int dist_id, uint64_t seed, uint64_t iteration,
                               uint32_t stream_id, void* cuda_stream) {
   if (!ctx || !pat || pat->ctx != ctx) return ARD_ERR_INVALID_ARG;
@@ -450,6 +468,7 @@ ard_status ard_sample_pattern(ard_ctx* ctx, ard_pattern* pat, int dist_id, uint6
   DeviceGuard guard(ctx->device);
   pat->dp_bound = d.ndp;
   pat->keep = d.keep;
+  note_periods(pat, d.least, d.most, (cudaStream_t)cuda_stream);
   pat->generation++;
   return launch_sampler(ctx, pat, d.d_cdf, d.ndp, seed, iteration, stream_id, 0, 0, (cudaStream_t)cuda_stream);
 }
@@ -460,6 +479,7 @@ ard_status ard_pattern_set(ard_ctx* ctx, ard_pattern* pat, int dp, int b, void* 
   DeviceGuard guard(ctx->device);
   pat->dp_bound = dp;
   pat->keep = 1.f / (float)dp;
+  note_periods(pat, dp, dp, (cudaStream_t)cuda_stream);
   pat->generation++;
   return launch_sampler(ctx, pat, nullptr, 0, 0, 0, 0, dp, b, (cudaStream_t)cuda_stream);
 }
@@ -948,6 +968,7 @@ ard_status ard_sample_pattern_counter(ard_ctx* ctx, ard_pattern* pat, int dist_i
   DeviceGuard guard(ctx->device);
   pat->dp_bound = d.ndp;
   pat->keep = d.keep;
+  note_periods(pat, d.least, d.most, (cudaStream_t)cuda_stream);
   pat->generation++;
   return launch_sampler(ctx, pat, d.d_cdf, d.ndp, seed, iteration_base, stream_id, 0, 0, (cudaStream_t)cuda_stream,
                         reinterpret_cast<unsigned long long*>(iteration_counter), advance ? 1 : 0);
@@ -1141,6 +1162,13 @@ static ard_status lstm_input_half(ard_ctx* ctx, const ard_pattern* pat, int T, i
   return launch_lstm_tc(ctx, 0, t, s);
 }
 
+// Units that the pattern can keep at most, and at least, when a call enqueued, or captured, now runs.
+static int lstm_most_kept(const ard_pattern* pat, int H, cudaStream_t s) {
+  const int dp = stream_captures(s) ? 1 : pat->dp_least;
+  return (H + dp - 1) / dp;
+}
+static int lstm_least_kept(const ard_pattern* pat, int H, cudaStream_t s) { return stream_captures(s) ? 0 : H / pat->dp_most; }
+
 // Whole-sequence drivers: the time loop runs here, in native code, and only enqueues kernels.
 // gates_ready: the input half of every step's pre-activations is already in G (the caller multiplied it, e.g. over
 // the kept outputs of the layer below); only the recurrence runs, which needs the one-kernel form.
@@ -1190,8 +1218,19 @@ static ard_status lstm_forward_impl(ard_ctx* ctx, const ard_pattern* pat, int T,
         st = get_maps(ctx, ctx->d_lstm_hc, 2 * B, ARD_LSTM_HC_LD, ARD_LSTM_HC_LD, 0, MAP_PLAIN, 0, box, 64, &mapHc);
         if (st != ARD_OK) return st;
       }
+      // Where the kept weights fit a cluster of CTAs the steps hand over inside it; the device decides by the kept count, and
+      // only where the host knows that no pattern can keep more does the kernel over the whole grid stay out.
+      int done_to = 0;
+      const int n_max = lstm_most_kept(pat, H, s);
+      if (compact_h && lstm_least_kept(pat, H, s) <= (done_to = lstm_cluster_limit(ctx, B, n_max, false))) {
+        st = launch_lstm_forward_cluster(ctx, pat, n_max, T, B, I, H, I > 0 ? 1 : 0, alpha, W, ldw, XH, bias, C, G, s);
+        if (st == ARD_ERR_UNSUPPORTED) done_to = 0;
+        else if (st != ARD_OK || n_max <= done_to) return st;
+      } else {
+        done_to = 0;
+      }
       st = launch_lstm_forward_persistent(ctx, pat, T, B, I, H, I > 0 ? 1 : 0, alpha, tma ? &mapXH : nullptr, mapW,
-                                          compact_h ? &mapHc : nullptr, W, ldw, XH, bias, C, G, s);
+                                          compact_h ? &mapHc : nullptr, W, ldw, XH, bias, C, G, done_to, s);
       if (st != ARD_ERR_UNSUPPORTED) return st;
       // not launchable as one kernel right now: the per-step path below recomputes everything
     }
@@ -1263,7 +1302,15 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
                       pat->dp_bound, lstm_box_rows_of(B), 64, &mapDZ[gate]);
         if (st != ARD_OK) return st;
       }
-      st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, recurrent_only && dz != DZ ? DZ : nullptr, s);
+      void* dz_out = recurrent_only && dz != DZ ? DZ : nullptr;
+      int done_to = 0;
+      const int n_max = lstm_most_kept(pat, H, s);
+      st = ARD_ERR_UNSUPPORTED;
+      if (ctx->lstm_compact_h && lstm_least_kept(pat, H, s) <= (done_to = lstm_cluster_limit(ctx, B, n_max, true)))
+        st = launch_lstm_backward_cluster(ctx, pat, n_max, T, B, I, H, alpha, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out, s);
+      if (st == ARD_ERR_UNSUPPORTED) done_to = 0;
+      if (st == ARD_ERR_UNSUPPORTED || (st == ARD_OK && n_max > done_to))
+        st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out, done_to, s);
       if (st == ARD_OK) {
         recurrence_done = true;
         // dx_t for all t: the x halves of D are overwritten

@@ -32,6 +32,8 @@ struct ard_pattern {
   int K_dim, N_dim, ts, Tr, Tc, units;
   int dp_bound;        // largest dp the last sample/set call can have produced
   float keep;          // share of the units that the last sample/set call keeps in the mean
+  int dp_least, dp_most;  // smallest and largest dp the pattern can have; anything once a graph may draw it (its replays are not seen here)
+  int in_graph;        // a sample/set call of this pattern was captured
   unsigned long long generation;  // bumped by every sample / set call
   int32_t* d_hdr;      // device: header
   int32_t* d_idx;      // device: kept list (row: neuron index; tile: t-1), capacity `units`
@@ -57,6 +59,7 @@ struct ard_rows {
 struct ArdDistribution {
   int ndp = 0;
   float keep = 1.f;  // kept share of the units in the mean
+  int least = 1, most = 1;  // smallest and largest period with any weight
   unsigned long long* d_cdf = nullptr;  // device: ndp entries
   std::vector<unsigned long long> h_cdf;
 };
@@ -257,13 +260,22 @@ bool lstm_persistent_fits(ard_ctx* ctx, int B, int H, bool tma);
 bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H);
 // dH: gradients of every h_t, D and dc are then outputs only; nullptr: dH_last, D and dc as ard_lstm_backward has them.
 // DZ: gate blocks of width gs; DZ_out: a second copy with the caller's layout, or nullptr.
+// done_to: a pattern that keeps this many units or fewer has been served by another kernel.
 ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                            const TcMap mapDZ[4], const void* W, int ldw,
                                            const float* C, const float* G, const float* dH, const float* dH_last, float* D,
-                                           float* dc, void* DZ, int gs, void* DZ_out, cudaStream_t s);
+                                           float* dc, void* DZ, int gs, void* DZ_out, int done_to, cudaStream_t s);
 ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, int add_zx,
                                           float alpha, const TcMap* mapXH, const TcMap* mapW, const TcMap* mapHc, const void* W,
-                                          int ldw, void* XH, const float* bias, float* C, float* G, cudaStream_t s);
+                                          int ldw, void* XH, const float* bias, float* C, float* G, int done_to, cudaStream_t s);
+// The same recurrences inside clusters of CTAs (lstm_cluster.cu).  n_max: units that the pattern can keep at most.
+// lstm_cluster_limit: a pattern that keeps this many units or fewer is taken (0: none; with more the kernel does nothing).
+int lstm_cluster_limit(const ard_ctx* ctx, int B, int n_max, bool backward);
+ard_status launch_lstm_forward_cluster(ard_ctx* ctx, const ard_pattern* pat, int n_max, int T, int B, int I, int H, int add_zx, float alpha,
+                                       const void* W, int ldw, void* XH, const float* bias, float* C, float* G, cudaStream_t s);
+ard_status launch_lstm_backward_cluster(ard_ctx* ctx, const ard_pattern* pat, int n_max, int T, int B, int I, int H, float alpha,
+                                        const void* W, int ldw, const float* C, const float* G, const float* dH, const float* dH_last,
+                                        float* D, float* dc, void* DZ, int gs, void* DZ_out, cudaStream_t s);
 ard_status launch_gather_cols(ard_ctx* ctx, const int32_t* hdr, const int32_t* idx, const void* src, int ld_src,
                               void* dst, int ld_dst, int rows, int elem_bytes, int max_cols, int skip_dense,
                               cudaStream_t s);

@@ -205,6 +205,31 @@ __device__ __forceinline__ void cluster_sync_all() {
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_addr) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// 16 bytes into another CTA's shared memory, counted on that CTA's barrier.
+__device__ __forceinline__ void st_async_f4(uint32_t addr, uint32_t bar, float a, float b, float c, float d) {
+  asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%2, %3, %4, %5}, [%1];"
+               ::"r"(addr), "r"(bar), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
+}
+// Bounded wait for data that other CTAs of the cluster store into this one.
+__device__ __forceinline__ bool mbar_wait_cluster(uint32_t bar, uint32_t parity, volatile int* abort_flag, int* status) {
+  unsigned long long t0 = 0;
+  for (int spin = 0;; ++spin) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred P;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 P, [%1], %2, %3;\n\t"
+        "selp.b32 %0, 1, 0, P;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity), "r"(1000000u) : "memory");
+    if (ok) return true;
+    if (*abort_flag) return false;
+    if (spin == 0) t0 = global_ns();
+    else if (global_ns() - t0 > WAIT_LIMIT_NS) {
+      *abort_flag = 1;
+      atomicMax(status, (int)ARD_ERR_TIMEOUT);
+      return false;
+    }
+  }
+}
 // TMA load issued inside a CTA pair: the data lands in this CTA, the byte count is reported to the
 // mbarrier at `bar_cluster`, which may live in the peer CTA.  The data goes to this CTA only.
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar_cluster, int x,
