@@ -16,24 +16,26 @@
 // that an SM sends or receives (bulk copies of the same bytes 1280 and more).
 //
 // us, forward and BPTT recurrence of a sequence of 35 steps, all SMs meeting in L2 / here: 64 rows, 512 of 1024 units kept 140 and 143 / 78
-// and 70; 20 rows, 750 of 1500 kept 148 and 158 / 72 and 62; the whole pass 383 / 271 and 437 / 263.  Of a step's 2.1 us (64 rows) the
+// and 63; 20 rows, 750 of 1500 kept 148 and 158 / 72 and 62; the whole pass 383 / 266 and 437 / 263.  Of a step's 2.1 us (64 rows) the
 // products take 0.65, the cells 0.6, the exchange 0.55; the first 10 us of a launch are the weights' way in and cold code.
 //
 // Virtual units.  The kept units are numbered v = j + pad, j = 0 .. n_keep-1, with pad < 4 chosen so that at periods of 1 and
 // 2 four consecutive units begin on an 8 or 16 byte boundary of the weight's rows, and are gathered with one load.
 //
-// Clusters: 16 CTAs, or 8 where the layer is known to keep few units (more clusters, fewer rows each).  A wait that expires
+// Clusters: 16 CTAs, or 8 where the layer is known to keep few units (cluster_form).  A wait that expires
 // sets the status word; both kernels end by a cluster barrier, behind which nobody sends.
+#include <atomic>
+
 #include "ard_internal.h"
 #include "sm100_ptx.h"
 
 namespace {
 
-constexpr int LC_THREADS = 384, LC_WARPS = 12;
-constexpr int LC_UNITS = 48;          // units per CTA at most
+// W: warps of a CTA, 12, or 16 in one form of the backward kernel; each finishes the cells of 4 units.
+__host__ __device__ constexpr int lc_units(int W) { return 4 * W; }  // units per CTA at most
+constexpr int LC_REG = 8;                                     // 16 x 16 weight operands of a warp in registers; more in tensor memory,
+__host__ __device__ constexpr int lc_tmem_warp(int W) { return W == 12 ? 160 : 128; }  // ... 4 columns each: W / 4 warps share the 512 of a quarter of its lanes
 constexpr int LC_KQ = 12;             // forward: contraction steps (16 units) of a warp at most
-constexpr int LC_REG = 8;             // 16 x 16 weight operands of a warp in registers; up to 40 more in tensor memory,
-constexpr int LC_TMEM_WARP = 160;     // ... 4 columns each: three warps share the 512 columns of a quarter of its lanes
 constexpr int LC_HB = 4 * LC_KQ * 256;  // one copy of h for 8 batch rows, as the products read it
 constexpr int LC_BARS = 128;          // barriers and flags at the start of shared memory
 constexpr int LC_RING = 8;            // chunks of weight rows on their way at most
@@ -182,10 +184,10 @@ struct RowRing {
   int chunk, slot;       // the chunk that is read now, and its slot
   uint32_t phase;        // of that slot's barrier
 };
-// Row i of chunk `chunk` (its address in the weight: row(chunk, i)) into a slot, by lane i / 12 of warp i % 12.
-template <typename Row>
+// Row i of chunk `chunk` (its address in the weight: row(chunk, i)) into a slot, by lane i / W of warp i % W.
+template <int W, typename Row>
 __device__ __forceinline__ void ring_request(const RowRing& r, int chunk, int slot, Row row) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = lane * LC_WARPS + warp;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, i = lane * W + warp;
   const uint32_t bar = r.bars + 8u * (uint32_t)slot;
   if (i < r.rows) {
     const unsigned long long a = reinterpret_cast<unsigned long long>(row(chunk, i)), from = a & ~15ull;
@@ -195,7 +197,7 @@ __device__ __forceinline__ void ring_request(const RowRing& r, int chunk, int sl
                  ::"r"(r.base + (uint32_t)(slot * r.rows + i) * r.pitch), "l"(from), "r"(bytes), "r"(bar) : "memory");
   }
 }
-template <int PHASE, typename Row>  // PHASE: of the pitch modulo 128: conflict-free reads of two rows x 64 bytes (64) or four rows x 32 bytes (32)
+template <int W, int PHASE, typename Row>  // PHASE: of the pitch modulo 128: conflict-free reads of two rows x 64 bytes (64) or four rows x 32 bytes (32)
 __device__ __forceinline__ RowRing ring_start(const KeptWeights& k, uint32_t base, int rows, int chunks, Row row) {
   RowRing r;
   const int groups = ((k.nv - 1) >> 2) + 1;
@@ -212,7 +214,7 @@ __device__ __forceinline__ RowRing ring_start(const KeptWeights& k, uint32_t bas
     for (int i = 0; i < r.slots; ++i) mbar_init(r.bars + 8u * i, (uint32_t)rows);
   asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   __syncthreads();
-  for (int i = 0; i < r.slots; ++i) ring_request(r, i, i, row);
+  for (int i = 0; i < r.slots; ++i) ring_request<W>(r, i, i, row);
   return r;
 }
 __device__ __forceinline__ bool ring_wait(const RowRing& r, volatile int* abort_flag, int* status) {
@@ -221,13 +223,13 @@ __device__ __forceinline__ bool ring_wait(const RowRing& r, volatile int* abort_
   return ok;
 }
 // All threads, when they have read the chunk: another takes its place.  False: someone's wait failed.
-template <typename Row>
+template <int W, typename Row>
 __device__ __forceinline__ bool ring_next(RowRing& r, bool ok, Row row) {
-  if (barrier_failed(0, LC_THREADS, !ok)) {  // copies on their way have another millisecond before the block may end
+  if (barrier_failed(0, 32 * W, !ok)) {  // copies on their way have another millisecond before the block may end
     for (int x = 0; x < 1000; ++x) __nanosleep(1000);
     return false;
   }
-  if (r.chunk + r.slots < r.chunks) ring_request(r, r.chunk + r.slots, r.slot, row);
+  if (r.chunk + r.slots < r.chunks) ring_request<W>(r, r.chunk + r.slots, r.slot, row);
   ++r.chunk;
   if (++r.slot == r.slots) {
     r.slot = 0;
@@ -299,7 +301,9 @@ __device__ __forceinline__ void by_path(const KeptWeights& k, Run run) {
 }
 
 // The gate functions, without branches: a step's cells are a serial chain per thread, and behind the branches of tanhf and of an
-// IEEE division the chains of a thread's cells do not overlap (two cells 1150 cycles, so 400).  Errors in ulps over GATE_RANGE
+// IEEE division the chains of a thread's cells do not overlap (two cells 1150 cycles, so 400).  Errors against 64 bits in ulps:
+// tanh at most 1.64 for |x| up to 12 (tanhf 1.82); the sigmoid as the per-step kernels' 1 / (1 + __expf(-x)), 2.6 up to |x| = 1
+// and 14.4 at 12.
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
@@ -343,7 +347,8 @@ __device__ __forceinline__ float gate_tanh(float x) {
 // the cluster.  Column 2 c + b of a product is batch row c + 4 b of its group of 8, so that a warp's rows lie together.
 // NT: groups of 8 batch rows.
 template <int CL, int NT>
-__global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_forward_kernel(const __grid_constant__ LstmClusterParams p) {
+__global__ void __launch_bounds__(384, 1) ard_lstm_cluster_forward_kernel(const __grid_constant__ LstmClusterParams p) {
+  constexpr int W = 12, LC_THREADS = 32 * W, LC_WARPS = W, LC_UNITS = lc_units(W), LC_TMEM_WARP = lc_tmem_warp(W);
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + LC_BARS - 8);
@@ -390,7 +395,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_forward_kernel
   for (int i = 0; i < LC_REG * 4; ++i) w[i] = 0u;
   if (active) {
     auto row = [&](int chunk, int i) { return kept_row(k, chunk >> 1, rank * U + 16 * (i >> 3) + 8 * (chunk & 1) + (i & 7)); };
-    RowRing ring = ring_start<64>(k, base, 8 * (U >> 4), 8, row);
+    RowRing ring = ring_start<W, 64>(k, base, 8 * (U >> 4), 8, row);
     const int v0 = quarter * kq * 16 + 4 * c, last = (k.nv - 1) & ~3;
     const bool edge = (quarter == 0 && k.pad > 0) || (quarter + 1) * kq * 16 > k.nv || (kq & 3) != 0;  // some of this warp's units do not exist
     uint32_t a[LC_KQ][4];
@@ -412,7 +417,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_forward_kernel
     for (int g = 0; g < 4 && ok; ++g) {
       ok = ring_wait(ring, abort_flag, p.status);
       if (working) take(g, std::integral_constant<int, 0>{});
-      ok = ring_next(ring, ok, row);
+      ok = ring_next<W>(ring, ok, row);
       if (!ok) break;
       ok = ring_wait(ring, abort_flag, p.status);
       if (working) {
@@ -440,7 +445,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_forward_kernel
         for (int ib = 0; ib < LC_KQ / 4; ++ib)
           if (ib < blocks && 4 * ib + g >= 2) tmem_st16(my_w + (uint32_t)((4 * ib + g - 2) * 16), &a[4 * ib][0]);
       }
-      ok = ring_next(ring, ok, row);
+      ok = ring_next<W>(ring, ok, row);
     }
     if (!ok) working = false;
     tmem_st_wait();
@@ -638,7 +643,7 @@ __global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_forward_kernel
 // (unit, gate), so a thread's four gate gradients are the 8 bytes of the operand that another thread reads whole.
 // Tiles of 16 output units are dealt to the warps round-robin; row g of a tile is unit 2 g, row g + 8 unit 2 g + 1.  A tile's sums
 // lie as [column pair c][g][4]: 16 bytes of one thread, and the cells of warp (tile, c) are consecutive words.
-__host__ __device__ constexpr int lcb_tiles(int CL, int KS) { return (CL * KS / 4 + LC_WARPS - 1) / LC_WARPS; }  // per warp
+__host__ __device__ constexpr int lcb_tiles(int CL, int KS, int W) { return (CL * KS / 4 + W - 1) / W; }  // per warp
 __host__ __device__ constexpr int lcb_sums(int CL, int KS) { return CL * (KS / 4) * 512; }  // partial sums of 8 rows, one step
 __host__ __device__ constexpr int lcb_smem(int CL, int KS, int NT) { return LC_BARS + 2 * NT * lcb_sums(CL, KS) + 2 * NT * KS * 256; }
 
@@ -646,11 +651,12 @@ struct SavedCell {
   float gi, gf, gg, go, cp, up;
 };
 
-template <int CL, int NT, int KS>
+template <int CL, int NT, int W, int KS>
 __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterParams& p, uint8_t* smem, uint32_t base, uint32_t tmem_base,
                                                            volatile int* abort_flag, int rank, const KeptWeights& k, int n_keep) {
+  constexpr int LC_THREADS = 32 * W, LC_WARPS = W, LC_TMEM_WARP = lc_tmem_warp(W);
   constexpr int U = 4 * KS, TPC = KS / 4;  // units and tiles of a CTA
-  constexpr int TILES = lcb_tiles(CL, KS), OPS = TILES * KS, QUADS = OPS / 4;  // weight operands of a warp, fours of them
+  constexpr int TILES = lcb_tiles(CL, KS, W), OPS = TILES * KS, QUADS = OPS / 4;  // weight operands of a warp, fours of them
   static_assert(OPS >= LC_REG && 4 * (OPS - LC_REG) <= LC_TMEM_WARP, "weight operands");
   constexpr int SUMS = lcb_sums(CL, KS);
   const uint32_t s_p = base + LC_BARS, s_dz = s_p + 2 * NT * SUMS;
@@ -663,7 +669,7 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
   const int q = lane >> 2, c = lane & 3;
   const uint32_t my_w = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)((warp >> 2) * LC_TMEM_WARP);
 
-  // Weights: rows = output units, contraction = (own unit, gate).  Operand i * KS + ks is step ks of tile warp + 12 i, the first LC_REG in
+  // Weights: rows = output units, contraction = (own unit, gate).  Operand i * KS + ks is step ks of tile warp + W i, the first LC_REG in
   // registers.  A chunk holds the four gates' rows of the four units of a step.
   uint32_t w[LC_REG * 4];
 #pragma unroll
@@ -671,7 +677,7 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
   bool ok = true;
   if (active) {
     auto from_weight = [&](int ks, int i) { return kept_row(k, i >> 2, v_first + 4 * ks + (i & 3)); };
-    RowRing ring = ring_start<32>(k, base, 16, KS, from_weight);
+    RowRing ring = ring_start<W, 32>(k, base, 16, KS, from_weight);
 #pragma unroll 1
     for (int ks = 0; ks < KS && ok; ++ks) {
       ok = ring_wait(ring, abort_flag, p.status);
@@ -702,7 +708,7 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
           if (op >= LC_REG) tmem_st4(my_w + (uint32_t)((op - LC_REG) * 4), a);
         }
       });
-      ok = ring_next(ring, ok, from_weight);
+      ok = ring_next<W>(ring, ok, from_weight);
     }
     tmem_st_wait();
   }
@@ -893,8 +899,8 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
   }
 }
 
-template <int CL, int NT>
-__global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_backward_kernel(const __grid_constant__ LstmClusterParams p) {
+template <int CL, int NT, int W>
+__global__ void __launch_bounds__(32 * W, 1) ard_lstm_cluster_backward_kernel(const __grid_constant__ LstmClusterParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(smem + LC_BARS - 8);
@@ -918,14 +924,19 @@ __global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_backward_kerne
   const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP];
   if (n_keep <= p.limit) {  // the same for all CTAs
     const KeptWeights k = kept_weights(p, dp, bb, n_keep);
-    bool done = false;
+    bool done = false;  // four units a step: the fewest steps that the units fit
     if constexpr (CL == 16) {
       done = k.nv <= 16 * CL;
-      if (done) lstm_cluster_backward_body<CL, NT, 4>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+      if (done) lstm_cluster_backward_body<CL, NT, W, 4>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
     }
     if (done) {
-    } else if (k.nv <= 32 * CL) lstm_cluster_backward_body<CL, NT, 8>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
-    else lstm_cluster_backward_body<CL, NT, 12>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+    } else if (k.nv <= 32 * CL) {
+      lstm_cluster_backward_body<CL, NT, W, 8>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+    } else if (W == 12 || k.nv <= 48 * CL) {
+      lstm_cluster_backward_body<CL, NT, W, 12>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+    } else if constexpr (W == 16) {
+      lstm_cluster_backward_body<CL, NT, W, 16>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+    }
   } else if (p.alone && threadIdx.x == 0) {
     atomicMax(p.status, (int)ARD_ERR_UNSUPPORTED);
   }
@@ -939,71 +950,77 @@ __global__ void __launch_bounds__(LC_THREADS, 1) ard_lstm_cluster_backward_kerne
 }
 
 // ---- launch ----------------------------------------------------------------------------------------------------------
-constexpr int lcf_smem(int NT) { return LC_BARS + 2 * NT * LC_HB + LC_WARPS * NT * 4 * LC_SWAP; }
-constexpr int lcb_smem_max(int CL, int NT) { return lcb_smem(CL, LC_UNITS / 4, NT); }
-static_assert(lcf_smem(3) <= LC_SMEM_MAX && lcb_smem_max(16, 3) <= LC_SMEM_MAX, "shared memory of the cluster recurrences");
+constexpr int lcf_smem(int NT) { return LC_BARS + 2 * NT * LC_HB + 12 * NT * 4 * LC_SWAP; }
+static_assert(lcf_smem(3) <= LC_SMEM_MAX && lcb_smem(16, 12, 3) <= LC_SMEM_MAX && lcb_smem(8, 16, 1) <= LC_SMEM_MAX,
+              "shared memory of the cluster recurrences");
 
 using ClusterKernel = void (*)(LstmClusterParams);
 struct ClusterForm {
   ClusterKernel kern;  // nullptr: not taken
-  int cl, clusters, rows, limit, smem;
+  int cl, threads, nt, limit;
+  int clusters, rows;
 };
 
-// Clusters of `cl` CTAs of this kernel that the device holds at once; 0 where it holds none.
-int cluster_count(const ard_ctx* ctx, ClusterKernel kern, int cl, int smem) {
-  if (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) {
+// Clusters of this form that the device holds at once; 0 where it holds none.
+int cluster_count(const ard_ctx* ctx, const ClusterForm& f) {
+  if (cudaFuncSetAttribute((const void*)f.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaFuncSetAttribute((const void*)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LC_SMEM_MAX) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(ctx->sm_count / cl * cl);
-  cfg.blockDim = dim3(LC_THREADS);
-  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(ctx->sm_count / f.cl * f.cl);
+  cfg.blockDim = dim3(f.threads);
+  cfg.dynamicSmemBytes = LC_SMEM_MAX;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cl;
+  attr[0].val.clusterDim.x = f.cl;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, (const void*)kern, &cfg) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveClusters(&n, (const void*)f.kern, &cfg) != cudaSuccess) {
     (void)cudaGetLastError();
     return 0;
   }
   return n;
 }
 
-template <bool BWD, int CL, int NT>
-ClusterForm form_of() {
-  if constexpr (BWD) return {ard_lstm_cluster_backward_kernel<CL, NT>, CL, 0, 0, CL * LC_UNITS, LC_SMEM_MAX};
-  else return {ard_lstm_cluster_forward_kernel<CL, NT>, CL, 0, 0, CL * LC_UNITS, LC_SMEM_MAX};
-}
+template <int CL, int NT>
+ClusterForm forward_form() { return {ard_lstm_cluster_forward_kernel<CL, NT>, CL, 384, NT, CL * lc_units(12), 0, 0}; }
+template <int CL, int NT, int W>
+ClusterForm backward_form() { return {ard_lstm_cluster_backward_kernel<CL, NT, W>, CL, 32 * W, NT, CL * lc_units(W), 0, 0}; }
 
-// The form for a layer that keeps n_max units at most (0 units: nothing is known): clusters of 8 where its weights fit eight CTAs.
+// The form for a layer that keeps n_max units at most, in the order in which they are preferred: clusters of 8 where the weights fit eight
+// CTAs (more clusters, so fewer rows in each, and fewer CTAs to send to).  For 385 to 512 units the backward kernel has a form of 8 CTAs of 16
+// warps, better than 16 CTAs with a second group of rows (64 rows, 512 of 1024 units kept, 35 steps: 85 -> 78 us; the forward kernel that way
+// 99 -> 106: its exchange is not hidden), not better than 16 CTAs with one.
 template <bool BWD>
 ClusterForm cluster_form(const ard_ctx* ctx, int B, int n_max) {
-  static const ClusterForm forms[2][3] = {{form_of<BWD, 8, 1>(), form_of<BWD, 8, 2>(), {}},
-                                          {form_of<BWD, 16, 1>(), form_of<BWD, 16, 2>(), form_of<BWD, 16, 3>()}};
-  static int room[64][2][3] = {};  // clusters at once, plus one
-  for (int i = n_max <= forms[0][0].limit ? 0 : 1; i < 2; ++i)
-    for (int nt = 1; nt <= 3; ++nt) {
-      ClusterForm f = forms[i][nt - 1];
-      if (f.kern == nullptr) continue;
-      int& have = room[ctx->device & 63][i][nt - 1];
-      if (have == 0) have = 1 + cluster_count(ctx, f.kern, f.cl, f.smem);
-      if (have <= 1) continue;
-      f.rows = (B + have - 2) / (have - 1);
-      if (f.rows > 8 * nt) continue;
-      f.clusters = (B + f.rows - 1) / f.rows;
-      return f;
-    }
-  return {nullptr, 0, 0, 0, 0, 0};
+  static const ClusterForm forward[] = {forward_form<8, 1>(), forward_form<8, 2>(), forward_form<16, 1>(), forward_form<16, 2>(), forward_form<16, 3>(), {}};
+  static const ClusterForm backward[] = {backward_form<8, 1, 12>(), backward_form<8, 2, 12>(), backward_form<16, 1, 12>(),
+                                         backward_form<8, 1, 16>(), backward_form<16, 2, 12>(), backward_form<16, 3, 12>()};
+  constexpr int FORMS = 6;
+  const ClusterForm* forms = BWD ? backward : forward;
+  static std::atomic<int> room[64][FORMS];  // clusters at once, plus one; 0: not asked yet
+  for (int i = 0; i < FORMS; ++i) {
+    ClusterForm f = forms[i];
+    if (f.kern == nullptr || (n_max > f.limit && f.cl == 8)) continue;
+    std::atomic<int>& known = room[ctx->device & 63][i];
+    int have = known.load(std::memory_order_relaxed);
+    if (have == 0) known.store(have = 1 + cluster_count(ctx, f), std::memory_order_relaxed);
+    if (have <= 1) continue;
+    f.rows = (B + have - 2) / (have - 1);
+    if (f.rows > 8 * f.nt) continue;
+    f.clusters = (B + f.rows - 1) / f.rows;
+    return f;
+  }
+  return {nullptr, 0, 0, 0, 0, 0, 0};
 }
 
 ard_status launch_cluster(ard_ctx* ctx, const ClusterForm& f, const LstmClusterParams& p, cudaStream_t s) {
-  const cudaError_t err = ard_launch_cluster(ctx, f.kern, f.cl, dim3(f.cl * f.clusters), dim3(LC_THREADS), f.smem, s, p);
+  const cudaError_t err = ard_launch_cluster(ctx, f.kern, f.cl, dim3(f.cl * f.clusters), dim3(f.threads), LC_SMEM_MAX, s, p);
   if (err != cudaSuccess) {
     (void)cudaGetLastError();
     return err == cudaErrorLaunchOutOfResources || err == cudaErrorInvalidClusterSize ? ARD_ERR_UNSUPPORTED : ARD_ERR_CUDA;

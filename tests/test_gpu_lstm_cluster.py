@@ -21,7 +21,8 @@ BF = torch.bfloat16
     (3, 121, 16, 384, 1, 1), (3, 16, 20, 385, 1, 1), (3, 113, 40, 768, 1, 1), (2, 20, 40, 769, 1, 1), (3, 9, 8, 1536, 2, 2),
     (2, 60, 24, 1538, 2, 1), (3, 57, 52, 1504, 2, 2), (2, 5, 37, 769, 2, 2), (4, 1, 16, 17, 1, 1), (3, 2, 64, 12, 12, 7),
     (3, 8, 50, 122, 1, 1), (3, 8, 51, 121, 1, 1), (3, 64, 30, 506, 2, 1), (3, 64, 30, 506, 2, 2), (1, 30, 44, 260, 3, 3),
-    (3, 128, 24, 1024, 2, 1), (5, 64, 64, 400, 16, 16)])
+    (3, 128, 24, 1024, 2, 1), (5, 64, 64, 400, 16, 16),
+    (3, 57, 24, 1024, 2, 1), (3, 120, 40, 1023, 2, 2), (2, 120, 16, 385, 1, 1)])
 def test_edges_of_the_cluster_recurrences(T, B, I, H, dp, b):
     rng = np.random.default_rng(T * 1000 + B + H)
     W = inputs.bf16_round(rng.uniform(-0.06, 0.06, size=(I + H, 4 * H)).astype(np.float32))
