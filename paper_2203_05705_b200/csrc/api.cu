@@ -1278,7 +1278,16 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
   int gs = H;
   // One cooperative kernel for the recurrence of the whole sequence when the layer fits it, followed by the
   // input half of d[x, h] as one product over all T*B rows; otherwise the two kernels per time step below.
-  bool recurrence_done = false;
+  bool recurrence_done = false, zeros_done = false;  // zeros_done: those of dW's dropped rows
+  // the columns of dW that are computed (recurrent_only: the h half alone -- operand, output and fan-in extent start at column I), and
+  // whether the four gate blocks are one tensor-core launch
+  const int wcol0 = recurrent_only ? I : 0, wcols = recurrent_only ? H : KH;
+  const void* XHw = reinterpret_cast<const __nv_bfloat16*>(XH) + wcol0;
+  float* dWw = dW + wcol0;
+  auto weight_tc = [&](const void* z, int ldz_gate) {
+    return ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && B >= 1 && pat->kind == ARD_ROW && pat->dp_bound <= ARD_MAX_NDP_TC &&
+           aligned16(z) && ldz_gate % 8 == 0 && aligned16(XHw) && aligned16(dWw) && KH % 8 == 0;
+  };
   if (ctx->lstm_persistent && ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && B >= 1 && I > 0) {
     ard_status st = check_common(ctx, pat, B, KH, H);
     if (st != ARD_OK) return st;
@@ -1307,7 +1316,8 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
       const int n_max = lstm_most_kept(pat, H, s);
       st = ARD_ERR_UNSUPPORTED;
       if (ctx->lstm_compact_h && lstm_least_kept(pat, H, s) <= (done_to = lstm_cluster_limit(ctx, B, n_max, true)))
-        st = launch_lstm_backward_cluster(ctx, pat, n_max, T, B, I, H, alpha, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out, s);
+        st = launch_lstm_backward_cluster(ctx, pat, n_max, T, B, I, H, alpha, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out,
+                                          weight_tc(dz, gs) && lstm_least_kept(pat, H, s) < H ? dWw : nullptr, KH, wcols, &zeros_done, s);
       if (st == ARD_ERR_UNSUPPORTED) done_to = 0;
       if (st == ARD_ERR_UNSUPPORTED || (st == ARD_OK && n_max > done_to))
         st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out, done_to, s);
@@ -1355,21 +1365,15 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
   }
   // Weight gradient over all T*B rows: the four gate blocks in one tensor-core launch when the operands
   // allow it (the M tiles of the four gates share one tile loop), else one product per gate.
-  // (recurrent_only: the columns of the h half alone -- operand, output and fan-in extent start at column I)
-  const int wcol0 = recurrent_only ? I : 0, wcols = recurrent_only ? H : KH;
-  const void* XHw = reinterpret_cast<const __nv_bfloat16*>(XH) + wcol0;
-  float* dWw = dW + wcol0;
   const char* dzc = reinterpret_cast<const char*>(dz);
-  const bool w_tc = ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && B >= 1 && pat->kind == ARD_ROW &&
-                    pat->dp_bound <= ARD_MAX_NDP_TC && aligned16(dz) && gs % 8 == 0 && aligned16(XHw) && aligned16(dWw) && KH % 8 == 0;
   DeviceGuard guard(ctx->device);
-  if (w_tc) {
+  if (weight_tc(dz, gs)) {
     TcArgs t = {};
     GemmArgs g = {};
     fill_common(g, ctx, pat, T * B, wcols, H, 1.0f);
     g.A0 = dz; g.lda0 = 4 * gs; g.A1 = XHw; g.lda1 = KH; g.out = dWw; g.ldo = KH;
     g.flag0 = 1;
-    g.flag1 = 1;  // rows of dropped units are written as zero
+    g.flag1 = !zeros_done;  // rows of dropped units are written as zero
     g.out_is_f32 = 1;
     ard_status st = ARD_OK;
     for (int gate = 0; gate < 4 && st == ARD_OK; ++gate)

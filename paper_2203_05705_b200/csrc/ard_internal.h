@@ -269,13 +269,15 @@ ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, 
                                           float alpha, const TcMap* mapXH, const TcMap* mapW, const TcMap* mapHc, const void* W,
                                           int ldw, void* XH, const float* bias, float* C, float* G, int done_to, cudaStream_t s);
 // The same recurrences inside clusters of CTAs (lstm_cluster.cu).  n_max: units that the pattern can keep at most.
+// (backward: *zeros says whether it writes the zeros of the dropped rows of dW [4H][dw_cols]; dW nullptr: it does not)
 // lstm_cluster_limit: a pattern that keeps this many units or fewer is taken (0: none; with more the kernel does nothing).
 int lstm_cluster_limit(const ard_ctx* ctx, int B, int n_max, bool backward);
 ard_status launch_lstm_forward_cluster(ard_ctx* ctx, const ard_pattern* pat, int n_max, int T, int B, int I, int H, int add_zx, float alpha,
                                        const void* W, int ldw, void* XH, const float* bias, float* C, float* G, cudaStream_t s);
 ard_status launch_lstm_backward_cluster(ard_ctx* ctx, const ard_pattern* pat, int n_max, int T, int B, int I, int H, float alpha,
                                         const void* W, int ldw, const float* C, const float* G, const float* dH, const float* dH_last,
-                                        float* D, float* dc, void* DZ, int gs, void* DZ_out, cudaStream_t s);
+                                        float* D, float* dc, void* DZ, int gs, void* DZ_out, float* dW, int ld_dw, int dw_cols, bool* zeros,
+                                        cudaStream_t s);
 ard_status launch_gather_cols(ard_ctx* ctx, const int32_t* hdr, const int32_t* idx, const void* src, int ld_src,
                               void* dst, int ld_dst, int rows, int elem_bytes, int max_cols, int skip_dense,
                               cudaStream_t s);

@@ -15,9 +15,10 @@
 // the whole SM.  The exchange among 16 CTAs takes 400 cycles for one packet of 32 bytes each, and 1.7 cycles more for every packet
 // that an SM sends or receives (bulk copies of the same bytes 1280 and more).
 //
-// us, forward and BPTT recurrence of a sequence of 35 steps, all SMs meeting in L2 / here: 64 rows, 512 of 1024 units kept 140 and 143 / 78
-// and 63; 20 rows, 750 of 1500 kept 148 and 158 / 72 and 62; the whole pass 383 / 266 and 437 / 263.  Of a step's 2.1 us (64 rows) the
-// products take 0.65, the cells 0.6, the exchange 0.55; the first 10 us of a launch are the weights' way in and cold code.
+// us, forward and BPTT recurrence of a sequence of 35 steps, all SMs meeting in L2 / here: 64 rows, 512 of 1024 units kept 138 and 157 /
+// 99 and 78; 20 rows, 750 of 1500 kept 151 and 180 / 84 and 75; 64 rows, 64 of 1024 114 and 122 / 44 and 44; the whole pass of the first
+// two, what lies before and behind the recurrences included, 384 / 263 and 437 / 256.  Of a step's 2.1 us (64 rows, forward) the products
+// take 0.65, the cells 0.6, the exchange 0.55; the first 10 us of a launch are the weights' way in and cold code.
 //
 // Virtual units.  The kept units are numbered v = j + pad, j = 0 .. n_keep-1, with pad < 4 chosen so that at periods of 1 and
 // 2 four consecutive units begin on an 8 or 16 byte boundary of the weight's rows, and are gathered with one load.
@@ -66,6 +67,8 @@ struct LstmClusterParams {
   __nv_bfloat16* DZ;     // [T][B][4 * gs]: gate blocks of width gs, compact inside a block
   int gs;
   __nv_bfloat16* DZ_out; // a second copy for the caller, [T][B][4H] (nullptr: DZ is the caller's)
+  float* dW;             // weight gradient [4H][ld_dw]: the rows of dropped units become zero (the kernels that have it)
+  int ld_dw, dw_cols;    // multiples of 4, as dW of 16 bytes
 };
 
 __device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t* a, const uint32_t (&b)[2]) {
@@ -651,7 +654,20 @@ struct SavedCell {
   float gi, gf, gg, go, cp, up;
 };
 
-template <int CL, int NT, int W, int KS>
+// The zeros of the weight gradient's dropped rows are bulk copies from LC_ZERO bytes of zeros at the end of shared memory; this is the i-th
+// row of the CTA.
+constexpr int LC_ZERO = 16 * 1024;
+__device__ __forceinline__ void zero_dropped_weight_row(const LstmClusterParams& p, uint32_t zeros, int i, int dp, int bb) {
+  const int x = (int)blockIdx.x + (int)gridDim.x * i;
+  if (x >= 4 * p.H) return;
+  const int u = x % p.H;
+  if (u >= bb && (u - bb) % dp == 0) return;
+  char* d = reinterpret_cast<char*>(p.dW + (size_t)x * p.ld_dw);
+  for (int left = 4 * p.dw_cols; left > 0; left -= LC_ZERO, d += LC_ZERO) bulk_store(d, zeros, (uint32_t)min(left, LC_ZERO));
+}
+
+// ZEROS: with those of the weight gradient (a kernel of its own: the code alone costs the others 1.5 us, cold as it is).
+template <int CL, int NT, int W, int KS, bool ZEROS>
 __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterParams& p, uint8_t* smem, uint32_t base, uint32_t tmem_base,
                                                            volatile int* abort_flag, int rank, const KeptWeights& k, int n_keep) {
   constexpr int LC_THREADS = 32 * W, LC_WARPS = W, LC_TMEM_WARP = lc_tmem_warp(W);
@@ -715,8 +731,22 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
   __syncthreads();
   for (uint32_t o = threadIdx.x * 16u; o < 2u * NT * SUMS; o += LC_THREADS * 16u)
     *reinterpret_cast<uint4*>(smem + LC_BARS + o) = make_uint4(0u, 0u, 0u, 0u);
+  if constexpr (ZEROS) {
+    for (uint32_t o = threadIdx.x * 16u; o < (uint32_t)LC_ZERO; o += LC_THREADS * 16u)
+      *reinterpret_cast<uint4*>(smem + LC_SMEM_MAX - LC_ZERO + o) = make_uint4(0u, 0u, 0u, 0u);
+    fence_proxy_async_smem();  // (read by bulk copies)
+  }
   __syncwarp();
   cluster_sync_all();  // everyone's barriers and zeros are in place before anyone sends
+  // Zeros of the weight gradient: a burst of rows in every eighth step, or all here where a step has as many products as to have no room for
+  // the code (64 rows, 512 of 1024 units kept, us of the recurrence: 78 without zeros, 80.6 all here, 94 in bursts; 20 rows, 188 of 1500: 45, 61
+  // and 53; some rows in every step 56).
+  constexpr int BURST = KS <= 8 ? 8 : 0;
+  const uint32_t s_zeros = base + (uint32_t)(LC_SMEM_MAX - LC_ZERO);
+  const int zero_rows = dp > 1 ? (4 * p.H + (int)gridDim.x - 1) / (int)gridDim.x : 0;  // of this CTA
+  const int bursts = BURST > 0 ? (T + BURST - 1) / BURST : 1, zero_burst = (zero_rows + bursts - 1) / bursts;
+  if (ZEROS && (BURST == 0 || !active))
+    for (int i = warp + W * lane; i < zero_rows; i += 32 * W) zero_dropped_weight_row(p, s_zeros, i, dp, bb);
 
   // the cells of this thread: warps 0 .. 4 TPC - 1, unit lane / 2 of tile warp / 4, row 2 (warp % 4) + lane % 2 of a group
   const int ct = warp >> 2, n = 2 * (warp & 3) + (lane & 1);
@@ -872,6 +902,10 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
       for (int g = 0; g < 4; ++g) st16_if(cell[nt], d + 2 * g * p.gs, dz[nt][g >> 1] >> (16 * (g & 1)));
     }
     zp -= z_step;
+    if constexpr (ZEROS && BURST > 0) {
+      if (s % BURST == 0)
+        for (int i = warp + W * lane; i < zero_burst; i += 32 * W) zero_dropped_weight_row(p, s_zeros, s / BURST * zero_burst + i, dp, bb);
+    }
     if (p.dH == nullptr || p.DZ_out != nullptr) {
 #pragma unroll
       for (int nt = 0; nt < NT; ++nt) {
@@ -897,9 +931,13 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
           for (int x = j + n_keep; x < p.H; x += n_keep) dc[x] = 0.f;
       }
   }
+  if constexpr (ZEROS) {
+    bulk_commit();
+    bulk_wait_all();
+  }
 }
 
-template <int CL, int NT, int W>
+template <int CL, int NT, int W, bool ZEROS>
 __global__ void __launch_bounds__(32 * W, 1) ard_lstm_cluster_backward_kernel(const __grid_constant__ LstmClusterParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
@@ -927,15 +965,15 @@ __global__ void __launch_bounds__(32 * W, 1) ard_lstm_cluster_backward_kernel(co
     bool done = false;  // four units a step: the fewest steps that the units fit
     if constexpr (CL == 16) {
       done = k.nv <= 16 * CL;
-      if (done) lstm_cluster_backward_body<CL, NT, W, 4>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+      if (done) lstm_cluster_backward_body<CL, NT, W, 4, ZEROS>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
     }
     if (done) {
     } else if (k.nv <= 32 * CL) {
-      lstm_cluster_backward_body<CL, NT, W, 8>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+      lstm_cluster_backward_body<CL, NT, W, 8, ZEROS>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
     } else if (W == 12 || k.nv <= 48 * CL) {
-      lstm_cluster_backward_body<CL, NT, W, 12>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+      lstm_cluster_backward_body<CL, NT, W, 12, ZEROS>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
     } else if constexpr (W == 16) {
-      lstm_cluster_backward_body<CL, NT, W, 16>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
+      lstm_cluster_backward_body<CL, NT, W, 16, ZEROS>(p, smem, base, tmem_base, abort_flag, rank, k, n_keep);
     }
   } else if (p.alone && threadIdx.x == 0) {
     atomicMax(p.status, (int)ARD_ERR_UNSUPPORTED);
@@ -951,23 +989,24 @@ __global__ void __launch_bounds__(32 * W, 1) ard_lstm_cluster_backward_kernel(co
 
 // ---- launch ----------------------------------------------------------------------------------------------------------
 constexpr int lcf_smem(int NT) { return LC_BARS + 2 * NT * LC_HB + 12 * NT * 4 * LC_SWAP; }
-static_assert(lcf_smem(3) <= LC_SMEM_MAX && lcb_smem(16, 12, 3) <= LC_SMEM_MAX && lcb_smem(8, 16, 1) <= LC_SMEM_MAX,
+static_assert(lcf_smem(3) <= LC_SMEM_MAX && lcb_smem(16, 12, 3) + LC_ZERO <= LC_SMEM_MAX && lcb_smem(8, 16, 1) + LC_ZERO <= LC_SMEM_MAX,
               "shared memory of the cluster recurrences");
 
 using ClusterKernel = void (*)(LstmClusterParams);
 struct ClusterForm {
-  ClusterKernel kern;  // nullptr: not taken
+  ClusterKernel kern, kern_zeros;  // nullptr: not taken; the one that also writes zeros of the weight gradient
   int cl, threads, nt, limit;
   int clusters, rows;
 };
 
 // Clusters of this form that the device holds at once; 0 where it holds none.
 int cluster_count(const ard_ctx* ctx, const ClusterForm& f) {
-  if (cudaFuncSetAttribute((const void*)f.kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-      cudaFuncSetAttribute((const void*)f.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LC_SMEM_MAX) != cudaSuccess) {
-    (void)cudaGetLastError();
-    return 0;
-  }
+  for (ClusterKernel kern : {f.kern, f.kern_zeros})
+    if (kern != nullptr && (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                            cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LC_SMEM_MAX) != cudaSuccess)) {
+      (void)cudaGetLastError();
+      return 0;
+    }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(ctx->sm_count / f.cl * f.cl);
   cfg.blockDim = dim3(f.threads);
@@ -988,9 +1027,11 @@ int cluster_count(const ard_ctx* ctx, const ClusterForm& f) {
 }
 
 template <int CL, int NT>
-ClusterForm forward_form() { return {ard_lstm_cluster_forward_kernel<CL, NT>, CL, 384, NT, CL * lc_units(12), 0, 0}; }
+ClusterForm forward_form() { return {ard_lstm_cluster_forward_kernel<CL, NT>, nullptr, CL, 384, NT, CL * lc_units(12), 0, 0}; }
 template <int CL, int NT, int W>
-ClusterForm backward_form() { return {ard_lstm_cluster_backward_kernel<CL, NT, W>, CL, 32 * W, NT, CL * lc_units(W), 0, 0}; }
+ClusterForm backward_form() {
+  return {ard_lstm_cluster_backward_kernel<CL, NT, W, false>, ard_lstm_cluster_backward_kernel<CL, NT, W, true>, CL, 32 * W, NT, CL * lc_units(W), 0, 0};
+}
 
 // The form for a layer that keeps n_max units at most, in the order in which they are preferred: clusters of 8 where the weights fit eight
 // CTAs (more clusters, so fewer rows in each, and fewer CTAs to send to).  For 385 to 512 units the backward kernel has a form of 8 CTAs of 16
@@ -1016,7 +1057,7 @@ ClusterForm cluster_form(const ard_ctx* ctx, int B, int n_max) {
     f.clusters = (B + f.rows - 1) / f.rows;
     return f;
   }
-  return {nullptr, 0, 0, 0, 0, 0, 0};
+  return {};
 }
 
 ard_status launch_cluster(ard_ctx* ctx, const ClusterForm& f, const LstmClusterParams& p, cudaStream_t s) {
@@ -1060,8 +1101,10 @@ ard_status launch_lstm_forward_cluster(ard_ctx* ctx, const ard_pattern* pat, int
 
 ard_status launch_lstm_backward_cluster(ard_ctx* ctx, const ard_pattern* pat, int n_max, int T, int B, int I, int H, float alpha,
                                         const void* W, int ldw, const float* C, const float* G, const float* dH, const float* dH_last,
-                                        float* D, float* dc, void* DZ, int gs, void* DZ_out, cudaStream_t s) {
-  const ClusterForm f = cluster_form<true>(ctx, B, n_max);
+                                        float* D, float* dc, void* DZ, int gs, void* DZ_out, float* dW, int ld_dw, int dw_cols, bool* zeros,
+                                        cudaStream_t s) {
+  *zeros = false;
+  ClusterForm f = cluster_form<true>(ctx, B, n_max);
   if (!f.kern) return ARD_ERR_UNSUPPORTED;
   LstmClusterParams p = {};
   p.hdr = pat->d_hdr;
@@ -1079,5 +1122,17 @@ ard_status launch_lstm_backward_cluster(ard_ctx* ctx, const ard_pattern* pat, in
   p.DZ = reinterpret_cast<__nv_bfloat16*>(DZ);
   p.gs = gs;
   p.DZ_out = reinterpret_cast<__nv_bfloat16*>(DZ_out);
-  return launch_cluster(ctx, f, p, s);
+  // The zeros of dW's dropped rows pay here: the product that computes the kept rows takes 31.5 -> 25 us without them (33 MB of dW, half of it
+  // zero), 38 -> 25 (72 MB, half), 44 -> 17.5 (72 MB, seven eighths), this kernel 2.5, 6 and 8 us more with them.  The smallest layers that
+  // gained had 0.8 MB (12 steps, 87.3 -> 85.9 the whole pass); 0.5 MB lost (29 steps, 109.7 -> 111.7).
+  constexpr size_t least = 640u << 10;
+  if (p.alone && dW != nullptr && (uintptr_t)dW % 16 == 0 && ld_dw % 4 == 0 && dw_cols % 4 == 0 && (size_t)16 * H * dw_cols >= least) {
+    p.dW = dW;
+    p.ld_dw = ld_dw;
+    p.dw_cols = dw_cols;
+    f.kern = f.kern_zeros;
+  }
+  const ard_status st = launch_cluster(ctx, f, p, s);
+  *zeros = st == ARD_OK && p.dW != nullptr;
+  return st;
 }

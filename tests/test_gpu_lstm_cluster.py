@@ -1,6 +1,7 @@
 """Recurrences inside clusters of CTAs, forward and backward against the oracle, at the edges of the kernels: most units of a
 cluster of 8 and of 16 CTAs and one more, one unit, a second and a third group of 8 batch rows, the three ways the weights come in
-(periods of 1 and 2 with rows on the 8 and 16 byte grid, from every phase of it, and everything else).  What the weights of dropped
+(periods of 1 and 2 with rows on the 8 and 16 byte grid, from every phase of it, and everything else), weight-gradient rows longer than what a copy of
+zeros holds, and more steps than one burst of them.  What the weights of dropped
 units hold does not matter."""
 import numpy as np
 import pytest
@@ -22,7 +23,7 @@ BF = torch.bfloat16
     (2, 60, 24, 1538, 2, 1), (3, 57, 52, 1504, 2, 2), (2, 5, 37, 769, 2, 2), (4, 1, 16, 17, 1, 1), (3, 2, 64, 12, 12, 7),
     (3, 8, 50, 122, 1, 1), (3, 8, 51, 121, 1, 1), (3, 64, 30, 506, 2, 1), (3, 64, 30, 506, 2, 2), (1, 30, 44, 260, 3, 3),
     (3, 128, 24, 1024, 2, 1), (5, 64, 64, 400, 16, 16),
-    (3, 57, 24, 1024, 2, 1), (3, 120, 40, 1023, 2, 2), (2, 120, 16, 385, 1, 1)])
+    (3, 57, 24, 1024, 2, 1), (3, 120, 40, 1023, 2, 2), (2, 120, 16, 385, 1, 1), (18, 9, 4104, 120, 4, 3)])
 def test_edges_of_the_cluster_recurrences(T, B, I, H, dp, b):
     rng = np.random.default_rng(T * 1000 + B + H)
     W = inputs.bf16_round(rng.uniform(-0.06, 0.06, size=(I + H, 4 * H)).astype(np.float32))
