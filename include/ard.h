@@ -101,7 +101,8 @@ ard_status ard_set_path(ard_ctx* ctx, ard_path path);
  *   ARD_OPT_MLP_PERSISTENT [1]    ard_mlp_step runs the whole iteration in one cooperative kernel when the stack
  *                                 fits it (see ard_mlp_step); 0: always call by call
  *   ARD_OPT_LSTM_COMPACT_H [1]    the whole-sequence kernels of ard_lstm_forward / ard_lstm_backward contract over
- *                                 the kept units alone when the pattern drops any: forward over a compact copy of
+ *                                 the kept units alone when the pattern drops any: inside clusters of CTAs where the kept
+ *                                 units fit them, else forward over a compact copy of
  *                                 h_{t-1} in context scratch, BPTT with whole contractions in every CTA where few
  *                                 units are kept (0: forward over all H columns, the dropped ones being zero, BPTT's
  *                                 contraction shared by a cluster of CTAs whatever is kept, where the device holds
@@ -583,12 +584,15 @@ ard_status ard_lstm_gate_gemm_bwd(ard_ctx* ctx, const ard_pattern* pat, int B, i
 /* Whole-sequence forward: for t = 0..T-1, the gate product on XH[t] followed by the cell update, which writes
  * h_t into the h half of XH[t+1].  When the layer fits (B <= 128; 8 or 12 hidden units per SM, whose recurrent weight
  * rows fit in shared memory beside part of h: on 148 SMs 1664 units, 1776 with B <= 64; any alignment with ARD_PATH_AUTO) this
- * is ONE cooperative kernel that keeps the weight in shared memory and the cell state in registers for the
- * whole sequence and synchronises the SMs once per step (every wait bounded, see ARD_ERR_TIMEOUT); Z is
- * then not used.  Otherwise, or after ard_set_lstm_persistent(ctx, 0), it is a loop in native code that
+ * is ONE kernel for the whole sequence (every wait bounded, see ARD_ERR_TIMEOUT); Z is then not used.  A pattern that keeps
+ * 768 units or fewer (on 148 SMs) runs inside clusters of CTAs, each with some of the batch rows from the
+ * first step to the last, its weights in registers and tensor memory; the others run as a cooperative kernel that keeps the
+ * weight in shared memory and the cell state in registers and synchronises all SMs once per step.  Where the host cannot know
+ * how many units a pattern keeps (under stream capture, or a distribution with periods on both sides), both are enqueued and
+ * the one that the drawn pattern does not need returns at once.  Otherwise, or after ard_set_lstm_persistent(ctx, 0), it is a loop in native code that
  * enqueues ard_lstm_gate_gemm and ard_lstm_gates per step.  Both give the same C, G and XH up to
- * summation order.  Under a pattern that drops units the kernel contracts over the kept units of h_{t-1} only
- * (ARD_OPT_LSTM_COMPACT_H): it keeps a compact copy of h in scratch of the context, next to the grid-barrier
+ * summation order.  Under a pattern that drops units the kernels contract over the kept units of h_{t-1} only
+ * (ARD_OPT_LSTM_COMPACT_H); the cooperative one keeps a compact copy of h in scratch of the context, next to the grid-barrier
  * counter the whole-sequence kernels share, so one whole-sequence call at a time per context.
  *   XH [T+1][B][I+H] bf16: the caller fills the x halves of XH[0..T-1] and the h half of XH[0] (h_0, zeros at
  *   dropped units); C [T+1][B][H] fp32 compact cell states, C[0] = c_0; G [T][B][4H] fp32 saved gates;
@@ -605,8 +609,9 @@ ard_status ard_lstm_forward(ard_ctx* ctx, const ard_pattern* pat, int T, int B, 
  * When the layer fits (as for ard_lstm_forward, but on 148 SMs B <= 128 up to 1408 units, 85 up to 1536, 64 up to 1584, less
  * beyond; and where DZ is not 16-byte aligned or H no multiple of 8, T * B * 8 * H bytes, H rounded up to a multiple of 8,
  * must not exceed the 256 KB per SM of the context's scratch: 38.8 MB on 148 SMs) and ard_set_lstm_persistent is on, the recurrence dh_{t-1} = upstream + dz_t W_h with the cell adjoint is ONE
- * cooperative kernel (weight slices resident in shared memory, dc in registers, one bounded grid-wide synchronisation
- * per step) and the x halves come from one product over all T*B rows; otherwise a loop
+ * kernel, inside clusters of CTAs or cooperative as for ard_lstm_forward (the cooperative one: weight slices resident in
+ * shared memory, dc in registers, one bounded grid-wide synchronisation per step), and the x halves come from one product over
+ * all T*B rows; otherwise a loop
  * in native code enqueues ard_lstm_gates_bwd and ard_lstm_gate_gemm_bwd per step.  In both cases the h
  * halves of D[1..T-1] are overwritten (kept units: the total gradient of h_{t-1}; dropped units:
  * unspecified), and the h half of D[0] is meaningful at kept units only. */

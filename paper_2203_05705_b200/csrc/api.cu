@@ -1200,7 +1200,7 @@ static ard_status lstm_forward_impl(ard_ctx* ctx, const ard_pattern* pat, int T,
         st = lstm_input_half(ctx, pat, T, B, I, H, XH, W, ldw, G, s);
         if (st != ARD_OK) return st;
       }
-      // 2. The recurrence: one kernel, recurrent half of the weight resident in shared memory.
+      // 2. The recurrence: one kernel, recurrent half of the weight resident on the SMs.
       const int box = lstm_box_rows_of(B);
       if (tma) {
         st = get_maps(ctx, XH, (T + 1) * B, KH, KH, 0, MAP_PLAIN, 0, box, 64, &mapXH);

@@ -17,7 +17,7 @@
 //
 // us, forward and BPTT recurrence of a sequence of 35 steps, all SMs meeting in L2 / here: 64 rows, 512 of 1024 units kept 138 and 157 /
 // 99 and 78; 20 rows, 750 of 1500 kept 151 and 180 / 84 and 75; 64 rows, 64 of 1024 114 and 122 / 44 and 44; the whole pass of the first
-// two, what lies before and behind the recurrences included, 384 / 263 and 437 / 256.  Of a step's 2.1 us (64 rows, forward) the products
+// two, what lies before and behind the recurrences included, 384 / 258 and 437 / 251.  Of a step's 2.1 us (64 rows, forward) the products
 // take 0.65, the cells 0.6, the exchange 0.55; the first 10 us of a launch are the weights' way in and cold code.
 //
 // Virtual units.  The kept units are numbered v = j + pad, j = 0 .. n_keep-1, with pad < 4 chosen so that at periods of 1 and
