@@ -107,9 +107,12 @@ ard_status ard_set_path(ard_ctx* ctx, ard_path path);
  *                                 units are kept (0: forward over all H columns, the dropped ones being zero, BPTT's
  *                                 contraction shared by a cluster of CTAs whatever is kept, where the device holds
  *                                 all of the layer's CTAs in clusters); same results up to the order of fp32 additions
- * Errors: ARD_ERR_INVALID_ARG (unknown option, negative value). */
+ *   ARD_OPT_LSTM_REFUSE [0]       launches of the whole-sequence LSTM kernels that are answered as though the device could not
+ *                                 hold them now (SMs taken by another context, a smaller partition): 1 those in clusters of
+ *                                 CTAs, 2 the cooperative ones, 3 both; the calls take the way they have for that
+ * Errors: ARD_ERR_INVALID_ARG (unknown option, negative value, value of ARD_OPT_LSTM_REFUSE above 3). */
 typedef enum { ARD_OPT_PDL = 0, ARD_OPT_PDL_IN_CAPTURE = 1, ARD_OPT_SIDE_STREAMS = 2, ARD_OPT_CTA_PAIRS = 3,
-               ARD_OPT_BAND_ROWS = 4, ARD_OPT_MLP_PERSISTENT = 5, ARD_OPT_LSTM_COMPACT_H = 6 } ard_option;
+               ARD_OPT_BAND_ROWS = 4, ARD_OPT_MLP_PERSISTENT = 5, ARD_OPT_LSTM_COMPACT_H = 6, ARD_OPT_LSTM_REFUSE = 7 } ard_option;
 ard_status ard_set_option(ard_ctx* ctx, ard_option option, int value);
 /* Opt-in for training loops, bf16 layers.  The tensor-core backward GEMMs of a row pattern read a compacted copy
  * of a full-width dY (kept columns only) that the library makes in the context workspace.  With

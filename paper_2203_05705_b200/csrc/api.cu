@@ -1,5 +1,6 @@
 // C-ABI entry points: argument validation, context / pattern lifetime, the TMA descriptor cache and
 // the dispatch between the CUDA-core and tcgen05 kernel families.
+#include <limits.h>
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -151,6 +152,26 @@ bool ard_side_streams(ard_ctx* ctx, cudaStream_t main) {
   return true;
 }
 
+// The recurrence of a pattern that keeps `least` to `most` units: inside clusters of CTAs where it keeps `limit` or fewer (0: no form of
+// clusters serves the layer), else over the whole grid.  cluster() enqueues the one, grid(above, up_to) the other for patterns that keep more
+// than `above` and at most `up_to`.  The device decides by the kept count, and only what the host knows not to be needed stays out.
+// ARD_ERR_UNSUPPORTED: nothing has been enqueued.  Where both are needed the cooperative launch goes first, because it is the one that is
+// refused when SMs are taken (either kernel overwrites what the other, or the path of single steps, would begin from).
+template <typename Cluster, typename Grid>
+static ard_status lstm_recurrence(int least, int most, int limit, Cluster cluster, Grid grid) {
+  constexpr int any = INT_MAX;
+  if (limit == 0 || least > limit) return grid(0, any);
+  if (most <= limit) {
+    const ard_status st = cluster();
+    return st == ARD_ERR_UNSUPPORTED ? grid(0, any) : st;
+  }
+  ard_status st = grid(limit, any);
+  if (st != ARD_OK) return st;
+  st = cluster();
+  if (st == ARD_ERR_UNSUPPORTED) st = grid(0, limit);
+  return st == ARD_ERR_UNSUPPORTED ? ARD_ERR_CUDA : st;  // (what is enqueued cannot be taken back)
+}
+
 extern "C" {
 
 const char* ard_status_string(ard_status s) {
@@ -189,6 +210,7 @@ ard_status ard_create(ard_ctx** out, int device, size_t workspace_bytes) {
   ctx->d_grid_bar = nullptr;
   ctx->d_lstm_hc = nullptr;
   ctx->lstm_compact_h = 1;
+  ctx->lstm_refuse = 0;
   ctx->pdl_in_capture = 1;
   ctx->mlp_two_streams = 1;
   ctx->mlp_persistent = 1;
@@ -289,6 +311,10 @@ ard_status ard_set_option(ard_ctx* ctx, ard_option option, int value) {
     case ARD_OPT_BAND_ROWS: ctx->band_m = value; return ARD_OK;
     case ARD_OPT_MLP_PERSISTENT: ctx->mlp_persistent = value ? 1 : 0; return ARD_OK;
     case ARD_OPT_LSTM_COMPACT_H: ctx->lstm_compact_h = value ? 1 : 0; return ARD_OK;
+    case ARD_OPT_LSTM_REFUSE:
+      if (value > 3) return ARD_ERR_INVALID_ARG;
+      ctx->lstm_refuse = value;
+      return ARD_OK;
   }
   return ARD_ERR_INVALID_ARG;
 }
@@ -1218,19 +1244,14 @@ static ard_status lstm_forward_impl(ard_ctx* ctx, const ard_pattern* pat, int T,
         st = get_maps(ctx, ctx->d_lstm_hc, 2 * B, ARD_LSTM_HC_LD, ARD_LSTM_HC_LD, 0, MAP_PLAIN, 0, box, 64, &mapHc);
         if (st != ARD_OK) return st;
       }
-      // Where the kept weights fit a cluster of CTAs the steps hand over inside it; the device decides by the kept count, and
-      // only where the host knows that no pattern can keep more does the kernel over the whole grid stay out.
-      int done_to = 0;
-      const int n_max = lstm_most_kept(pat, H, s);
-      if (compact_h && lstm_least_kept(pat, H, s) <= (done_to = lstm_cluster_limit(ctx, B, n_max, false))) {
-        st = launch_lstm_forward_cluster(ctx, pat, n_max, T, B, I, H, I > 0 ? 1 : 0, alpha, W, ldw, XH, bias, C, G, s);
-        if (st == ARD_ERR_UNSUPPORTED) done_to = 0;
-        else if (st != ARD_OK || n_max <= done_to) return st;
-      } else {
-        done_to = 0;
-      }
-      st = launch_lstm_forward_persistent(ctx, pat, T, B, I, H, I > 0 ? 1 : 0, alpha, tma ? &mapXH : nullptr, mapW,
-                                          compact_h ? &mapHc : nullptr, W, ldw, XH, bias, C, G, done_to, s);
+      const int n_max = lstm_most_kept(pat, H, s), limit = compact_h ? lstm_cluster_limit(ctx, B, n_max, false) : 0;
+      st = lstm_recurrence(
+          lstm_least_kept(pat, H, s), n_max, limit,
+          [&] { return launch_lstm_forward_cluster(ctx, pat, n_max, T, B, I, H, I > 0 ? 1 : 0, alpha, W, ldw, XH, bias, C, G, s); },
+          [&](int above, int up_to) {
+            return launch_lstm_forward_persistent(ctx, pat, T, B, I, H, I > 0 ? 1 : 0, alpha, tma ? &mapXH : nullptr, mapW,
+                                                  compact_h ? &mapHc : nullptr, W, ldw, XH, bias, C, G, above, up_to, s);
+          });
       if (st != ARD_ERR_UNSUPPORTED) return st;
       // not launchable as one kernel right now: the per-step path below recomputes everything
     }
@@ -1312,15 +1333,17 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
         if (st != ARD_OK) return st;
       }
       void* dz_out = recurrent_only && dz != DZ ? DZ : nullptr;
-      int done_to = 0;
-      const int n_max = lstm_most_kept(pat, H, s);
-      st = ARD_ERR_UNSUPPORTED;
-      if (ctx->lstm_compact_h && lstm_least_kept(pat, H, s) <= (done_to = lstm_cluster_limit(ctx, B, n_max, true)))
-        st = launch_lstm_backward_cluster(ctx, pat, n_max, T, B, I, H, alpha, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out,
-                                          weight_tc(dz, gs) && lstm_least_kept(pat, H, s) < H ? dWw : nullptr, KH, wcols, &zeros_done, s);
-      if (st == ARD_ERR_UNSUPPORTED) done_to = 0;
-      if (st == ARD_ERR_UNSUPPORTED || (st == ARD_OK && n_max > done_to))
-        st = launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out, done_to, s);
+      const int n_min = lstm_least_kept(pat, H, s), n_max = lstm_most_kept(pat, H, s);
+      st = lstm_recurrence(
+          n_min, n_max, ctx->lstm_compact_h ? lstm_cluster_limit(ctx, B, n_max, true) : 0,
+          [&] {
+            return launch_lstm_backward_cluster(ctx, pat, n_max, T, B, I, H, alpha, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out,
+                                                weight_tc(dz, gs) && n_min < H ? dWw : nullptr, KH, wcols, &zeros_done, s);
+          },
+          [&](int above, int up_to) {
+            return launch_lstm_backward_persistent(ctx, pat, T, B, I, H, alpha, mapDZ, W, ldw, C, G, dH, dH_last, D, dc, dz, gs, dz_out, above,
+                                                   up_to, s);
+          });
       if (st == ARD_OK) {
         recurrence_done = true;
         // dx_t for all t: the x halves of D are overwritten

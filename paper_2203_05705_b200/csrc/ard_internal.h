@@ -116,6 +116,7 @@ struct ard_ctx {
   unsigned int* d_grid_bar;  // arrival counters of the cooperative kernels: word 0 ard_mlp_step, words 32, 33 LSTM (zero between launches)
   void* d_lstm_hc;           // compact copies of h_{t-1} and h_t of the whole-sequence forward kernel, lstm_hc_bytes()
   int lstm_compact_h;        // ... which contracts over the kept units of h alone under a pattern
+  int lstm_refuse;           // launches answered as though the device could not hold them: 1 clusters, 2 cooperative
   int use_pdl;        // launch kernels with programmatic stream serialization (see ard_launch)
   int pdl_in_capture; // ... also while the stream is being captured into a CUDA graph
   int stream_k;       // tensor-core row kernels: share the last, partial wave of tiles along the contraction
@@ -260,14 +261,14 @@ bool lstm_persistent_fits(ard_ctx* ctx, int B, int H, bool tma);
 bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H);
 // dH: gradients of every h_t, D and dc are then outputs only; nullptr: dH_last, D and dc as ard_lstm_backward has them.
 // DZ: gate blocks of width gs; DZ_out: a second copy with the caller's layout, or nullptr.
-// done_to: a pattern that keeps this many units or fewer has been served by another kernel.
+// A pattern that keeps `above` units or fewer, or more than `up_to`, is left to another kernel.
 ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                            const TcMap mapDZ[4], const void* W, int ldw,
                                            const float* C, const float* G, const float* dH, const float* dH_last, float* D,
-                                           float* dc, void* DZ, int gs, void* DZ_out, int done_to, cudaStream_t s);
+                                           float* dc, void* DZ, int gs, void* DZ_out, int above, int up_to, cudaStream_t s);
 ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, int add_zx,
                                           float alpha, const TcMap* mapXH, const TcMap* mapW, const TcMap* mapHc, const void* W,
-                                          int ldw, void* XH, const float* bias, float* C, float* G, int done_to, cudaStream_t s);
+                                          int ldw, void* XH, const float* bias, float* C, float* G, int above, int up_to, cudaStream_t s);
 // The same recurrences inside clusters of CTAs (lstm_cluster.cu).  n_max: units that the pattern can keep at most.
 // (backward: *zeros says whether it writes the zeros of the dropped rows of dW [4H][dw_cols]; dW nullptr: it does not)
 // lstm_cluster_limit: a pattern that keeps this many units or fewer is taken (0: none; with more the kernel does nothing).

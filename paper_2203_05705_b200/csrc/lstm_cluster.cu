@@ -1061,6 +1061,7 @@ ClusterForm cluster_form(const ard_ctx* ctx, int B, int n_max) {
 }
 
 ard_status launch_cluster(ard_ctx* ctx, const ClusterForm& f, const LstmClusterParams& p, cudaStream_t s) {
+  if (ctx->lstm_refuse & 1) return ARD_ERR_UNSUPPORTED;
   const cudaError_t err = ard_launch_cluster(ctx, f.kern, f.cl, dim3(f.cl * f.clusters), dim3(f.threads), LC_SMEM_MAX, s, p);
   if (err != cudaSuccess) {
     (void)cudaGetLastError();

@@ -110,7 +110,7 @@ struct LstmFwdParams {
   unsigned int* bar;  // arrival counter, zero at launch; [1]: CTAs that left
   int* status;
   int smem_bytes;     // dynamic shared memory of this launch
-  int done_to;        // a pattern that keeps this many units or fewer is another kernel's
+  int above, up_to;   // a pattern that keeps no more than the one, or more than the other, is another kernel's
 };
 
 __device__ __forceinline__ unsigned int ld_acquire_u32(const unsigned int* p) {
@@ -540,7 +540,7 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
 
   const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP], ctas = (int)gridDim.x;
   const bool compact = p.Hc != nullptr && (dp > 1 || p.always_compact);
-  if (n_keep <= p.done_to) {
+  if (n_keep <= p.above || n_keep > p.up_to) {
   } else if (compact && n_keep <= 4 * ctas) lstm_forward_body<4>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
   else if (U == 8 || (compact && n_keep <= 8 * ctas)) lstm_forward_body<8>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
   else lstm_forward_body<U>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
@@ -629,7 +629,7 @@ struct LstmBwdParams {
   int ldw;
   int whole_ok;            // a pattern that keeps few units may do without the exchange
   int smem_bytes;          // dynamic shared memory of this launch
-  int done_to;             // a pattern that keeps this many units or fewer is another kernel's
+  int above, up_to;        // a pattern that keeps no more than the one, or more than the other, is another kernel's
 };
 
 // What the cell adjoint of a (row, unit) pair reads besides the recurrent sum.
@@ -986,7 +986,7 @@ __global__ void __launch_bounds__(LB_THREADS, 1) ard_lstm_backward_kernel(const 
   const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP];
   const int ctas = (int)gridDim.x;
   // as few units per CTA as the grid allows (see the forward kernel; 64 rows, 512 kept: 4.9 us per step with 8, 4.2 with 4)
-  if (n_keep <= p.done_to) {
+  if (n_keep <= p.above || n_keep > p.up_to) {
   } else if (n_keep <= 4 * ctas) lstm_backward_body<4>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
   else if (U == 8 || n_keep <= 8 * ctas) lstm_backward_body<8>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
   else lstm_backward_body<U>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
@@ -1037,6 +1037,7 @@ bool lstm_probe(const ard_ctx* ctx, K kern, int* probed) {
 // context, a smaller partition).
 template <typename K, typename P>
 ard_status lstm_launch(ard_ctx* ctx, K kern, int cluster, int grid, int smem, const P& p, cudaStream_t s) {
+  if (ctx->lstm_refuse & 2) return ARD_ERR_UNSUPPORTED;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(LP_THREADS);
@@ -1082,7 +1083,7 @@ bool lstm_persistent_fits(ard_ctx* ctx, int B, int H, bool tma) {
 // gemm_ldg_sm100.cu, 0.45 ms with the whole-sequence kernels.
 ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, int add_zx, float alpha,
                                           const TcMap* mapXH, const TcMap* mapW, const TcMap* mapHc, const void* W, int ldw, void* XH,
-                                          const float* bias, float* C, float* G, int done_to, cudaStream_t s) {
+                                          const float* bias, float* C, float* G, int above, int up_to, cudaStream_t s) {
   const int U = lstm_units(H, ctx->sm_count);
   LstmFwdParams p = {};
   p.always_compact = mapXH == nullptr || U != 8;
@@ -1106,7 +1107,8 @@ ard_status launch_lstm_forward_persistent(ard_ctx* ctx, const ard_pattern* pat, 
   p.bar = ctx->d_grid_bar + LP_BAR_WORD;
   p.status = ctx->d_status;
   p.smem_bytes = lstm_fwd_smem_bytes(B, H, U);
-  p.done_to = done_to;
+  p.above = above;
+  p.up_to = up_to;
   const int grid = (H + U - 1) / U;  // sized for dp = 1
   static int probed[2][64] = {};
   if (U == 8) {
@@ -1151,7 +1153,7 @@ bool lstm_persistent_bwd_fits(ard_ctx* ctx, int B, int H) {
 ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat, int T, int B, int I, int H, float alpha,
                                            const TcMap mapDZ[4], const void* W, int ldw, const float* C, const float* G,
                                            const float* dH, const float* dH_last, float* D, float* dc, void* DZ, int gs,
-                                           void* DZ_out, int done_to, cudaStream_t s) {
+                                           void* DZ_out, int above, int up_to, cudaStream_t s) {
   const LstmBwdForm f = lstm_bwd_form(ctx, B, H);
   if (f.U == 0) return ARD_ERR_UNSUPPORTED;
   LstmBwdParams p = {};
@@ -1170,7 +1172,8 @@ ard_status launch_lstm_backward_persistent(ard_ctx* ctx, const ard_pattern* pat,
   p.ldw = ldw;
   p.whole_ok = ctx->lstm_compact_h || f.cl == 1;
   p.smem_bytes = f.smem;
-  p.done_to = done_to;
+  p.above = above;
+  p.up_to = up_to;
   const int grid = ((H + f.U - 1) / f.U + f.cl - 1) / f.cl * f.cl;
   return lstm_launch(ctx, f.U == 8 ? ard_lstm_backward_kernel<8> : ard_lstm_backward_kernel<12>, f.cl, grid, f.smem, p, s);
 }
