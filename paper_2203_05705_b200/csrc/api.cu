@@ -152,6 +152,17 @@ bool ard_side_streams(ard_ctx* ctx, cudaStream_t main) {
   return true;
 }
 
+static bool stream_captures(cudaStream_t s) {
+  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
+}
+
+void ard_note_periods(ard_pattern* pat, int least, int most, cudaStream_t s) {
+  if (stream_captures(s)) pat->in_graph = 1;
+  pat->dp_least = pat->in_graph ? 1 : least;
+  pat->dp_most = pat->in_graph ? pat->units : most;
+}
+
 // The recurrence of a pattern that keeps `least` to `most` units: inside clusters of CTAs where it keeps `limit` or fewer (0: no form of
 // clusters serves the layer), else over the whole grid.  cluster() enqueues the one, grid(above, up_to) the other for patterns that keep more
 // than `above` and at most `up_to`.  The device decides by the kept count, and only what the host knows not to be needed stays out.
@@ -473,18 +484,6 @@ ard_status ard_pattern_destroy(ard_pattern* pat) {
   return ARD_OK;
 }
 
-// What the host knows of the period that the pattern's header holds when later calls run.  A captured call runs again with
-// every replay, unseen: from then on nothing is known.
-static bool stream_captures(cudaStream_t s) {
-  cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-  return cudaStreamIsCapturing(s, &st) != cudaSuccess || st != cudaStreamCaptureStatusNone;
-}
-static void note_periods(ard_pattern* pat, int least, int most, cudaStream_t s) {
-  if (stream_captures(s)) pat->in_graph = 1;
-  pat->dp_least = pat->in_graph ? 1 : least;
-  pat->dp_most = pat->in_graph ? pat->units : most;
-}
-
 ard_status ard_sample_pattern(ard_ctx* ctx, ard_pattern* pat, int dist_id, uint64_t seed, uint64_t iteration,
                               uint32_t stream_id, void* cuda_stream) {
   if (!ctx || !pat || pat->ctx != ctx) return ARD_ERR_INVALID_ARG;
@@ -494,7 +493,7 @@ ard_status ard_sample_pattern(ard_ctx* ctx, ard_pattern* pat, int dist_id, uint6
   DeviceGuard guard(ctx->device);
   pat->dp_bound = d.ndp;
   pat->keep = d.keep;
-  note_periods(pat, d.least, d.most, (cudaStream_t)cuda_stream);
+  ard_note_periods(pat, d.least, d.most, (cudaStream_t)cuda_stream);
   pat->generation++;
   return launch_sampler(ctx, pat, d.d_cdf, d.ndp, seed, iteration, stream_id, 0, 0, (cudaStream_t)cuda_stream);
 }
@@ -505,7 +504,7 @@ ard_status ard_pattern_set(ard_ctx* ctx, ard_pattern* pat, int dp, int b, void* 
   DeviceGuard guard(ctx->device);
   pat->dp_bound = dp;
   pat->keep = 1.f / (float)dp;
-  note_periods(pat, dp, dp, (cudaStream_t)cuda_stream);
+  ard_note_periods(pat, dp, dp, (cudaStream_t)cuda_stream);
   pat->generation++;
   return launch_sampler(ctx, pat, nullptr, 0, 0, 0, 0, dp, b, (cudaStream_t)cuda_stream);
 }
@@ -994,7 +993,7 @@ ard_status ard_sample_pattern_counter(ard_ctx* ctx, ard_pattern* pat, int dist_i
   DeviceGuard guard(ctx->device);
   pat->dp_bound = d.ndp;
   pat->keep = d.keep;
-  note_periods(pat, d.least, d.most, (cudaStream_t)cuda_stream);
+  ard_note_periods(pat, d.least, d.most, (cudaStream_t)cuda_stream);
   pat->generation++;
   return launch_sampler(ctx, pat, d.d_cdf, d.ndp, seed, iteration_base, stream_id, 0, 0, (cudaStream_t)cuda_stream,
                         reinterpret_cast<unsigned long long*>(iteration_counter), advance ? 1 : 0);

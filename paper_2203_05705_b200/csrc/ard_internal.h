@@ -163,6 +163,10 @@ static inline long long ard_exact_need(double t, long long s) {
 // and cannot be created now (`main` is being captured into a graph: nothing may be created then).
 bool ard_side_streams(ard_ctx* ctx, cudaStream_t main);
 
+// For every call that draws or sets a pattern, on the stream it is enqueued on: what the host knows of the period that the header holds when
+// later calls run.  A captured call runs again with every replay, unseen: from then on nothing is known.
+void ard_note_periods(ard_pattern* pat, int least, int most, cudaStream_t s);
+
 // The shared tail of the row kernels parks partial sums in ONE scratch per context, so it must stay off while
 // products of the same context run side by side on several streams: calls that fork hold one of these.
 struct SharedTailOff {

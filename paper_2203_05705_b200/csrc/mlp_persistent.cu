@@ -1204,8 +1204,7 @@ ard_status launch_mlp_persistent(ard_ctx* ctx, const ard_mlp_layer* layers, int 
     if (!layers[l].sample) continue;
     layers[l].pat->dp_bound = d->ndp;
     layers[l].pat->keep = d->keep;
-    layers[l].pat->dp_least = 1;
-    layers[l].pat->dp_most = d->ndp;
+    ard_note_periods(layers[l].pat, d->least, d->most, s);
     layers[l].pat->generation++;
   }
   return ARD_OK;
