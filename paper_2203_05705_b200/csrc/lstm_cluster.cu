@@ -141,6 +141,14 @@ __device__ __forceinline__ bool barrier_failed(int id, int threads, bool failed)
   return r != 0;
 }
 
+// A kernel enqueued beside the one that takes the patterns of more units: is the drawn one among them?  The same for all CTAs, and asked before
+// anything is set up, because a launch that does nothing stands in front of the next one's work.  (These are kernels of their own: the question
+// alone cost the others, which take their pattern, 0.2 - 0.7 % of the pass.)
+__device__ __forceinline__ bool other_kernels_pattern(const LstmClusterParams& p) {
+  pdl_wait_prior_grids();
+  return p.hdr[HDR_NKEEP] > p.limit;
+}
+
 // Operand of 8 batch rows, 256 bytes for 16 contraction indices: thread (n = lane / 4, c = lane % 4) of a product reads the 8 bytes
 // of the four indices 4 c .. 4 c + 3 of row n.  The 64 bytes of a c lie together (one sender writes them: 32-byte packets), and
 // c = 2, 3 have their halves swapped so that 16 lanes' reads cover every bank once.
@@ -348,8 +356,8 @@ __device__ __forceinline__ float gate_tanh(float x) {
 // made it 16-byte pieces in 8 rows, and the loads and stores of a step took 1300 of its 4500 cycles).  A thread has all four
 // gates of its cell, keeps its c, and four threads put four units' h_t together (two shuffles), 8 bytes that go to every CTA of
 // the cluster.  Column 2 c + b of a product is batch row c + 4 b of its group of 8, so that a warp's rows lie together.
-// NT: groups of 8 batch rows.
-template <int CL, int NT>
+// NT: groups of 8 batch rows.  BESIDE: enqueued with the kernel over the whole grid.
+template <int CL, int NT, bool BESIDE>
 __global__ void __launch_bounds__(384, 1) ard_lstm_cluster_forward_kernel(const __grid_constant__ LstmClusterParams p) {
   constexpr int W = 12, LC_THREADS = 32 * W, LC_WARPS = W, LC_UNITS = lc_units(W), LC_TMEM_WARP = lc_tmem_warp(W);
   extern __shared__ __align__(128) uint8_t smem[];
@@ -361,6 +369,7 @@ __global__ void __launch_bounds__(384, 1) ard_lstm_cluster_forward_kernel(const 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int rank = (int)cluster_ctarank();
   pdl_launch_dependents();
+  if (BESIDE && other_kernels_pattern(p)) return;
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) mbar_init(base + 8u * i, 1);  // one per copy: h is complete
     *abort_flag = 0;
@@ -937,7 +946,7 @@ __device__ __forceinline__ void lstm_cluster_backward_body(const LstmClusterPara
   }
 }
 
-template <int CL, int NT, int W, bool ZEROS>
+template <int CL, int NT, int W, bool ZEROS, bool BESIDE>
 __global__ void __launch_bounds__(32 * W, 1) ard_lstm_cluster_backward_kernel(const __grid_constant__ LstmClusterParams p) {
   extern __shared__ __align__(128) uint8_t smem[];
   const uint32_t base = smem_u32(smem);
@@ -946,6 +955,7 @@ __global__ void __launch_bounds__(32 * W, 1) ard_lstm_cluster_backward_kernel(co
   const int warp = threadIdx.x >> 5;
   const int rank = (int)cluster_ctarank();
   pdl_launch_dependents();
+  if (BESIDE && other_kernels_pattern(p)) return;
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) mbar_init(base + 8u * i, 1);  // one per set of partial sums: they are complete
     *abort_flag = 0;
@@ -994,14 +1004,14 @@ static_assert(lcf_smem(3) <= LC_SMEM_MAX && lcb_smem(16, 12, 3) + LC_ZERO <= LC_
 
 using ClusterKernel = void (*)(LstmClusterParams);
 struct ClusterForm {
-  ClusterKernel kern, kern_zeros;  // nullptr: not taken; the one that also writes zeros of the weight gradient
+  ClusterKernel kern, kern_zeros, kern_beside;  // nullptr: not taken; the one that also writes zeros of the weight gradient; BESIDE
   int cl, threads, nt, limit;
   int clusters, rows;
 };
 
 // Clusters of this form that the device holds at once; 0 where it holds none.
 int cluster_count(const ard_ctx* ctx, const ClusterForm& f) {
-  for (ClusterKernel kern : {f.kern, f.kern_zeros})
+  for (ClusterKernel kern : {f.kern, f.kern_zeros, f.kern_beside})
     if (kern != nullptr && (cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
                             cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, LC_SMEM_MAX) != cudaSuccess)) {
       (void)cudaGetLastError();
@@ -1026,11 +1036,19 @@ int cluster_count(const ard_ctx* ctx, const ClusterForm& f) {
   return n;
 }
 
+// (the other kernel is needed only where 16 CTAs may not hold the kept units: cluster_form)
 template <int CL, int NT>
-ClusterForm forward_form() { return {ard_lstm_cluster_forward_kernel<CL, NT>, nullptr, CL, 384, NT, CL * lc_units(12), 0, 0}; }
+ClusterForm forward_form() {
+  ClusterForm f = {ard_lstm_cluster_forward_kernel<CL, NT, false>, nullptr, nullptr, CL, 384, NT, CL * lc_units(12), 0, 0};
+  if constexpr (CL == 16) f.kern_beside = ard_lstm_cluster_forward_kernel<CL, NT, true>;
+  return f;
+}
 template <int CL, int NT, int W>
 ClusterForm backward_form() {
-  return {ard_lstm_cluster_backward_kernel<CL, NT, W, false>, ard_lstm_cluster_backward_kernel<CL, NT, W, true>, CL, 32 * W, NT, CL * lc_units(W), 0, 0};
+  ClusterForm f = {ard_lstm_cluster_backward_kernel<CL, NT, W, false, false>, ard_lstm_cluster_backward_kernel<CL, NT, W, true, false>, nullptr, CL,
+                   32 * W, NT, CL * lc_units(W), 0, 0};
+  if constexpr (CL == 16) f.kern_beside = ard_lstm_cluster_backward_kernel<CL, NT, W, false, true>;
+  return f;
 }
 
 // The form for a layer that keeps n_max units at most, in the order in which they are preferred: clusters of 8 where the weights fit eight
@@ -1080,7 +1098,7 @@ int lstm_cluster_limit(const ard_ctx* ctx, int B, int n_max, bool backward) {
 
 ard_status launch_lstm_forward_cluster(ard_ctx* ctx, const ard_pattern* pat, int n_max, int T, int B, int I, int H, int add_zx, float alpha,
                                        const void* W, int ldw, void* XH, const float* bias, float* C, float* G, cudaStream_t s) {
-  const ClusterForm f = cluster_form<false>(ctx, B, n_max);
+  ClusterForm f = cluster_form<false>(ctx, B, n_max);
   if (!f.kern) return ARD_ERR_UNSUPPORTED;
   LstmClusterParams p = {};
   p.hdr = pat->d_hdr;
@@ -1088,6 +1106,7 @@ ard_status launch_lstm_forward_cluster(ard_ctx* ctx, const ard_pattern* pat, int
   p.rows = f.rows;
   p.limit = f.limit;
   p.alone = n_max <= f.limit;
+  if (!p.alone) f.kern = f.kern_beside;
   p.alpha = alpha;
   p.W = reinterpret_cast<const __nv_bfloat16*>(W);
   p.ldw = ldw;
@@ -1113,6 +1132,7 @@ ard_status launch_lstm_backward_cluster(ard_ctx* ctx, const ard_pattern* pat, in
   p.rows = f.rows;
   p.limit = f.limit;
   p.alone = n_max <= f.limit;
+  if (!p.alone) f.kern = f.kern_beside;
   p.alpha = alpha;
   p.W = reinterpret_cast<const __nv_bfloat16*>(W);
   p.ldw = ldw;

@@ -140,6 +140,24 @@ __device__ bool grid_wait(const unsigned int* bar, unsigned int target, volatile
 
 // The CTA that leaves last re-arms the grid-wide counter for the next launch.  Called by one thread per CTA after all
 // of its waits and arrivals.
+// Is the drawn pattern this launch's, with more than `above` units kept and at most `up_to`?  The same for all CTAs; asked before anything is
+// set up, because a launch that does nothing stands in front of the next one's work.
+__device__ __forceinline__ bool lstm_take_pattern(const int32_t* hdr, int above, int up_to) {
+  pdl_wait_prior_grids();
+  const int n_keep = hdr[HDR_NKEEP];
+  return n_keep > above && n_keep <= up_to;
+}
+
+// With `above`, the kernel of the patterns that keep fewer units is enqueued behind this one and has nothing to do: it may be scheduled while
+// this one runs, its CTAs then leave as soon as this one ends.  Only behind this one's allocation of tensor memory: a CTA of another kernel
+// on the same SM that held the columns while it waits for this kernel's end would wait for good (that kernel's CTAs need an SM of their own).
+// us of the whole pass, a dense draw of a distribution whose other draws are the clusters', 64 rows x 1024 units and 20 rows x 1500 over 35
+// steps, 16 x 1024 over 8: with the grid-wide kernels alone 509, 596 and 151; with the others behind them, both kinds asking for the pattern
+// once they are set up, 521, 609 and 156; as it is now 506, 595 and 151.
+__device__ __forceinline__ void lstm_next_launch(int above) {
+  if (above > 0) pdl_launch_dependents();
+}
+
 __device__ __forceinline__ void grid_leave(unsigned int* bar) {
   __threadfence();
   if (atomicAdd(bar + 1, 1u) == gridDim.x - 1) {
@@ -516,6 +534,7 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
   volatile uint32_t* tmem_ptr_smem = reinterpret_cast<volatile uint32_t*>(misc);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(misc + 4);
   const int warp = threadIdx.x >> 5;
+  if (!lstm_take_pattern(p.hdr, p.above, p.up_to)) return;
 
   if (threadIdx.x < 2 * LP_GROUPS * LP_SLOTS) mbar_init(base + 8u * threadIdx.x, 1);  // slots: full, free
   if (threadIdx.x == 0) {
@@ -536,12 +555,11 @@ __global__ void __launch_bounds__(LP_THREADS, 1) ard_lstm_forward_kernel(const _
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_smem;
-  pdl_wait_prior_grids();
+  lstm_next_launch(p.above);
 
   const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP], ctas = (int)gridDim.x;
   const bool compact = p.Hc != nullptr && (dp > 1 || p.always_compact);
-  if (n_keep <= p.above || n_keep > p.up_to) {
-  } else if (compact && n_keep <= 4 * ctas) lstm_forward_body<4>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
+  if (compact && n_keep <= 4 * ctas) lstm_forward_body<4>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
   else if (U == 8 || (compact && n_keep <= 8 * ctas)) lstm_forward_body<8>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
   else lstm_forward_body<U>(p, smem, base, tmem_base, abort_flag, dp, bb, n_keep, compact);
 
@@ -963,6 +981,7 @@ __global__ void __launch_bounds__(LB_THREADS, 1) ard_lstm_backward_kernel(const 
   const int warp = threadIdx.x >> 5;
   uint32_t cl;
   asm volatile("mov.u32 %0, %%cluster_nctaid.x;" : "=r"(cl));
+  if (!lstm_take_pattern(p.hdr, p.above, p.up_to)) return;
 
   if (threadIdx.x < 2 * LP_GROUPS * LP_SLOTS) mbar_init(base + 8u * threadIdx.x, 1);
   if (threadIdx.x == 0) {
@@ -981,13 +1000,12 @@ __global__ void __launch_bounds__(LB_THREADS, 1) ard_lstm_backward_kernel(const 
   tc_fence_after();
   const uint32_t tmem_base = *tmem_ptr_smem;
   if (cl > 1) cluster_sync_all();  // every CTA's barriers exist before anyone sends
-  pdl_wait_prior_grids();
+  lstm_next_launch(p.above);
 
   const int dp = p.hdr[HDR_DP], bb = p.hdr[HDR_B] - 1, n_keep = p.hdr[HDR_NKEEP];
   const int ctas = (int)gridDim.x;
   // as few units per CTA as the grid allows (see the forward kernel; 64 rows, 512 kept: 4.9 us per step with 8, 4.2 with 4)
-  if (n_keep <= p.above || n_keep > p.up_to) {
-  } else if (n_keep <= 4 * ctas) lstm_backward_body<4>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
+  if (n_keep <= 4 * ctas) lstm_backward_body<4>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
   else if (U == 8 || n_keep <= 8 * ctas) lstm_backward_body<8>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
   else lstm_backward_body<U>(p, smem, base, tmem_base, abort_flag, (int)cl, dp, bb, n_keep);
 
