@@ -31,6 +31,9 @@
 //     H = 1024: 218 -> 189 us at a period of 2, 204 -> 146 us at 8).  This form reads neither [x | h] nor the weight
 //     through a descriptor, so it also serves layers whose rows are off the 16-byte grid, dense draws included
 //     (1500 units, batch 20, 35 steps, a period of 2: see launch_lstm_forward_persistent).
+// Patterns that keep 768 units or fewer run in lstm_cluster.cu where the device has room for its clusters (on 148 SMs it has).  The forms
+// for few kept units here (U = 4; BPTT without the exchange) are for devices and partitions that have none, and for the option that refuses
+// those launches, with which their tests reach them.
 // The grid barrier is an arrival counter in global memory: after its stores and a fence each CTA adds 1,
 // and the relay thread of each CTA polls for t * (number of CTAs with units) before step t.  The CTA that leaves
 // last sets the counter back to zero.  The launch is cooperative, so all CTAs are resident; every wait is bounded
