@@ -6,19 +6,27 @@
 // descriptor in a step.  lstm_persistent.cu spreads the weights over the whole grid instead, so all SMs meet in L2 in every
 // step (about 2.8 us of its 4); it remains for the layers whose kept weights do not fit a cluster.
 //
-// Bound: latency, a chain of T steps.  A step's products have 8 columns or fewer (the cluster's rows of the batch), an eighth
-// of what the narrowest tcgen05.mma of 128 rows multiplies, and such an instruction costs its issuing thread 136 cycles, with
-// a commit, a wait and a load from tensor memory behind the last one.  mma.sync leaves the sums in the registers of the threads
-// that apply the cell update; it was measured at 8.1 cycles per 16 x 8 x 16 and SM quarter.  Its weights stay on the SM for the
+// Bound: latency, a chain of T steps.  A step's products have 8 columns for every group of 8 batch rows that the cluster has, one to three
+// groups.  Taken with one group: the narrowest tcgen05.mma has 128 rows and costs its issuing thread 136 cycles, with
+// a commit, a wait and a load from tensor memory behind the last one; mma.sync leaves the sums in the registers of the threads
+// that apply the cell update, at 8.1 cycles per 16 x 8 x 16 and SM quarter.  (With two and three groups, where mma.sync takes two and three
+// times as long, they were not compared.)  The weights stay on the SM for the
 // whole sequence, in TENSOR MEMORY used as a store: 12 warps with 48 operands each took 9.3 cycles per product with 8 operands in
 // registers and 40 streamed from tensor memory by tcgen05.ld, 17.4 with the 40 in shared memory, which gives 128 bytes a cycle to
 // the whole SM.  The exchange among 16 CTAs takes 400 cycles for one packet of 32 bytes each, and 1.7 cycles more for every packet
 // that an SM sends or receives (bulk copies of the same bytes 1280 and more).
 //
-// us, forward and BPTT recurrence of a sequence of 35 steps, all SMs meeting in L2 / here: 64 rows, 512 of 1024 units kept 138 and 157 /
-// 99 and 78; 20 rows, 750 of 1500 kept 151 and 180 / 84 and 75; 64 rows, 64 of 1024 114 and 122 / 44 and 44; the whole pass of the first
-// two, what lies before and behind the recurrences included, 384 / 258 and 437 / 251.  Of a step's 2.1 us (64 rows, forward) the products
-// take 0.65, the cells 0.6, the exchange 0.55; the first 10 us of a launch are the weights' way in and cold code.
+// us, forward and BPTT recurrence of a sequence of 35 steps, all SMs meeting in L2 / here, BPTT with the zeros of the weight gradient: 64 rows,
+// 512 of 1024 units kept 138 and 157 / 98 and 81; 20 rows, 750 of 1500 kept 151 and 180 / 82 and 81; 64 rows, 64 of 1024 114 and 122 / 44 and 48;
+// the whole pass of the first two, what lies before and behind the recurrences included, 384 / 254 and 437 / 247.  Of that the launch, the
+// weights' way in, cold code and the zeros take 13 and 22, 18 and 27, 14 and 18, a step 2.4 and 1.7, 1.8 and 1.5, 0.85 and 0.86 (sequences of 35
+// steps less those of 5).  Cycles of a forward step of 64 rows, 512 kept (two groups): products 1220, their sums through shared memory 300, cells
+// 1080, shuffles and sends 600, stores and the next gates' loads 575, the wait for the other CTAs 250; of 20 rows, 750 kept (one group) 1290,
+// 160, 680, 380, 700 and 220.
+//
+// Registers: 168 a thread in the forward kernels, of which all spill some.  With one and two groups the spills lie in front of the steps (as many
+// local loads and stores with 4 steps as with 24, in clusters of 16); with three, the form of more than 16 rows a cluster, a warp makes 9 loads and 4 stores a step.
+// Of the backward kernels only the one of 16 CTAs with three groups spills.
 //
 // Virtual units.  The kept units are numbered v = j + pad, j = 0 .. n_keep-1, with pad < 4 chosen so that at periods of 1 and
 // 2 four consecutive units begin on an 8 or 16 byte boundary of the weight's rows, and are gathered with one load.
