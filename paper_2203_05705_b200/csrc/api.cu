@@ -1204,7 +1204,7 @@ static ard_status lstm_forward_impl(ard_ctx* ctx, const ard_pattern* pat, int T,
   if (T < 0 || B < 0 || I < 0 || H < 1) return ARD_ERR_INVALID_ARG;
   const int KH = I + H;
   __nv_bfloat16* xh = reinterpret_cast<__nv_bfloat16*>(XH);
-  // One cooperative kernel for the whole sequence when the layer fits it (all units on the device at once, at most 128
+  // One kernel for the recurrence of the whole sequence (lstm_recurrence) when the layer fits it (all units on the device at once, at most 128
   // batch rows); otherwise one gate product and one cell kernel per time step.
   if (ctx->lstm_persistent && ctx->path != ARD_PATH_CUDA_CORE && ctx->encode_fn != nullptr && T >= 1 && B >= 1) {
     ard_status st = check_common(ctx, pat, B, KH, H);
@@ -1296,7 +1296,7 @@ static ard_status lstm_backward_impl(ard_ctx* ctx, const ard_pattern* pat, int T
   // gate gradients: the caller's DZ, or a copy in context scratch whose rows are padded to the 16-byte grid
   void* dz = DZ;
   int gs = H;
-  // One cooperative kernel for the recurrence of the whole sequence when the layer fits it, followed by the
+  // One kernel for the recurrence of the whole sequence (lstm_recurrence) when the layer fits it, followed by the
   // input half of d[x, h] as one product over all T*B rows; otherwise the two kernels per time step below.
   bool recurrence_done = false, zeros_done = false;  // zeros_done: those of dW's dropped rows
   // the columns of dW that are computed (recurrent_only: the h half alone -- operand, output and fan-in extent start at column I), and

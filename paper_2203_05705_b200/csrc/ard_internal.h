@@ -112,7 +112,7 @@ struct ard_ctx {
   int use_pairs;      // tensor-core row kernels: CTA pairs (cta_group::2) when the output has >= 2 row tiles
   int band_m;         // raster band height of the tensor-core kernels, in 128-row tiles
   int reuse_compact;  // 1: opt-in, consecutive backward calls share one compacted dY; 2: those of one ard_layer_products do
-  int lstm_persistent; // ard_lstm_forward: one cooperative kernel for the whole sequence when the layer fits
+  int lstm_persistent; // ard_lstm_forward: one kernel for the recurrence of the whole sequence when the layer fits
   unsigned int* d_grid_bar;  // arrival counters of the cooperative kernels: word 0 ard_mlp_step, words 32, 33 LSTM (zero between launches)
   void* d_lstm_hc;           // compact copies of h_{t-1} and h_t of the whole-sequence forward kernel, lstm_hc_bytes()
   int lstm_compact_h;        // ... which contracts over the kept units of h alone under a pattern

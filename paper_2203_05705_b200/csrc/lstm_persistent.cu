@@ -229,7 +229,8 @@ __device__ __forceinline__ bool lstm_stream_blocks(int n, int cap, int step, int
   return ok;
 }
 
-// The gate functions of the per-step kernels (aux_kernels.cu), so that a layer's results do not depend on the path it takes.
+// The gate functions of the per-step kernels (aux_kernels.cu), so that a layer's results do not depend on which of the two it takes (those in
+// lstm_cluster.cu have a tanh of their own, as close to the exact one).
 // 1 - 2 / (1 + exp(2x)) in tanhf's place cancels near zero: gates of size 0.01 were off by 7e-6 to 2e-5 of themselves, now by
 // 1e-7 to 9e-7 (the sums of the pre-activations among it), and it was no faster (35 steps, 64 rows, 512 of 1024 units kept,
 // forward plus BPTT 372.0 us, with tanhf 370.7; 20 rows, 750 of 1500 424.7 and 420.8).
